@@ -268,6 +268,24 @@ struct Workspace {
         cuda_check(cudaMallocFromPoolAsync(&p, size, device_pool(), s), "workspace allocation");
         base = static_cast<char*>(p);
     }
+    // As allocate, but an allocation that does not fit returns false when the
+    // caller has a smaller layout to try (`optional`).
+    bool try_allocate(cudaStream_t stream, bool optional) {
+        if (!optional || fault_alloc()) {
+            allocate(stream);
+            return true;
+        }
+        void* p = nullptr;
+        if (cudaMallocFromPoolAsync(&p, used, device_pool(), stream) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        s = stream;
+        size = used;
+        used = 0;
+        base = static_cast<char*>(p);
+        return true;
+    }
     ~Workspace() {
         if (base) cudaFreeAsync(base, s);
     }
@@ -1830,9 +1848,15 @@ int knng_exact(const float* data, int64_t n, int D, int k, const int32_t* sample
         DevBuf<float> X;
         DevBuf<int32_t> smp, oi;
         DevBuf<float> od;
-        uint64_t* keys = nullptr;
+        uint64_t *keys = nullptr, *part = nullptr;
         int* status = nullptr;
+        ScreenWork w{};
         const size_t sk = (size_t)s_rows * k;
+        const size_t batch = (size_t)exact_batch(s_rows);
+        const int nsplit = exact_splits(n, s_rows);
+        // the screen's copy and candidate lists come on top of what the FP32
+        // kernel needs; where they do not fit, the FP32 kernel runs alone
+        bool screen = exact_screened(n);
         for (int ps = 0; ps < 2; ++ps) {
             ws.used = 0;
             bind(ws, X, data, (size_t)n * D, ps);
@@ -1841,15 +1865,42 @@ int knng_exact(const float* data, int64_t n, int D, int k, const int32_t* sample
             bind(ws, od, out_dists, sk, ps);
             keys = ws.take<uint64_t>(std::max<size_t>(sk, 1));
             status = ws.take<int>(4);
-            if (ps == 0) ws.allocate(s);
+            if (screen) {
+                const size_t Dp = (size_t)lp_dim(D);
+                w.Xq = ws.take<uint16_t>((size_t)n * Dp);
+                w.nrm = ws.take<float>(n);
+                w.err = ws.take<float>(n);
+                if (sample) w.Qq = ws.take<uint16_t>(batch * Dp);
+                w.qn = ws.take<float>(batch);
+                w.qe = ws.take<float>(batch);
+                w.cg = ws.take<float>(batch * kScreenCap);
+                w.cid = ws.take<int32_t>(batch * kScreenCap);
+                w.cnt = ws.take<int32_t>(batch);
+                w.rowA = ws.take<float>(batch);
+                w.rowR = ws.take<float>(batch);
+                w.flags = ws.take<int>(2);
+                w.fb_list = ws.take<int32_t>(batch);
+                w.fb_flag = ws.take<int32_t>(batch);
+                w.part = ws.take<uint64_t>(batch * exact_splits(n, (int64_t)batch) * k);
+            } else if (nsplit > 1) {
+                part = ws.take<uint64_t>(sk * nsplit);
+            }
+            if (ps == 0 && !ws.try_allocate(s, screen)) {
+                screen = false;
+                ps = -1;
+            }
         }
         cuda_check(cudaMemsetAsync(status, 0, 4 * sizeof(int), s), "status clear");
         upload(X, s);
         if (sample) upload(smp, s);
-        launch_check_finite(X.dev, n * (int64_t)D, status, s);
         if (s_rows > 0) {
             if (sample) launch_check_ids(smp.dev, s_rows, 0, n, status, s);
-            launch_exact(X.dev, n, D, k, sample ? smp.dev : nullptr, s_rows, keys, status, s);
+            const int32_t* rows = sample ? smp.dev : nullptr;
+            if (!screen || !launch_exact_screened(X.dev, n, D, k, rows, s_rows, w, keys, status, s)) {
+                launch_check_finite(X.dev, n * (int64_t)D, status, s);
+                launch_exact(X.dev, n, D, k, rows, 0, s_rows, nullptr, nullptr, part ? nsplit : 1, part, keys, status,
+                             s);
+            }
             launch_unpack(keys, oi.dev, od.dev, (int64_t)sk, s);
         }
         download(oi, s);

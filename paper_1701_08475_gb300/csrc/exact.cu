@@ -2,6 +2,8 @@
 // problem statement of Sec. 1, each sampled point as a query against the
 // other n - 1), canonical FP32 distances, ties by id; recall of a graph on
 // those rows; and the input check.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -21,11 +23,19 @@ __host__ __device__ inline void exact_chunk(int D, int* dch, int* stride) {
     *stride = ((c / 4) & 1) ? c : c + 4;
 }
 
+// Query rows: row q is sample[q] (or row0 + q without a sample), q = list[r]
+// when a list is given (*list_count of them).  gridDim.y > 1 splits the
+// columns: split y writes its k best of list slot r to part, merged by
+// k7_merge; with one split the lists go straight to out.
 template <int NO>
 __global__ void __launch_bounds__(kNT) k7_exact(const float* __restrict__ X, int64_t n, int D, int k,
-                                               const int32_t* __restrict__ sample, int64_t s_rows,
-                                               uint64_t* __restrict__ out, const int* __restrict__ status) {
+                                               const int32_t* __restrict__ sample, int64_t row0, int64_t s_rows,
+                                               const int32_t* __restrict__ list, const int* __restrict__ list_count,
+                                               uint64_t* __restrict__ part, uint64_t* __restrict__ out,
+                                               const int* __restrict__ status) {
     if (*status & kStatusStop) return;  // a sampled id failed its check
+    if (list) s_rows = *list_count;
+    if ((int64_t)blockIdx.x * kQR >= s_rows) return;
     extern __shared__ float4 smem4[];
     int dch, stride;
     exact_chunk(D, &dch, &stride);
@@ -37,11 +47,27 @@ __global__ void __launch_bounds__(kNT) k7_exact(const float* __restrict__ X, int
     const int rg = tid % 16, cg = tid / 16;
     const int64_t q0 = (int64_t)blockIdx.x * kQR;
     const int nq = (int)min((int64_t)kQR, s_rows - q0);
-    for (int r = tid; r < kQR; r += kNT) qid[r] = r < nq ? (sample ? (int64_t)sample[q0 + r] : q0 + r) : -1;
+    for (int r = tid; r < kQR; r += kNT) {
+        const int64_t q = r < nq ? (list ? (int64_t)list[q0 + r] : q0 + r) : -1;
+        qid[r] = q < 0 ? -1 : sample ? (int64_t)sample[q] : row0 + q;
+    }
     __syncthreads();
     const bool one_chunk = dch >= D;
+    const bool vec = D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
     auto load_rows = [&](float* dst, int rows, int64_t first, bool query, int d0) {
         const int dl = min(dch, D - d0);
+        if (vec) {  // 16-byte pieces, a row's pieces by consecutive threads
+            const int q4 = dch / 4;
+            for (int e = tid; e < rows * q4; e += kNT) {
+                const int r = e / q4, c = e - r * q4;
+                const int64_t row = query ? qid[r] : first + r;
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (row >= 0 && row < n && 4 * c < dl)
+                    v = __ldg(reinterpret_cast<const float4*>(X + row * D + d0) + c);
+                *reinterpret_cast<float4*>(dst + r * stride + 4 * c) = v;
+            }
+            return;
+        }
         for (int e = tid; e < rows * dch; e += kNT) {
             const int r = e / dch, dd = e - r * dch;
             const int64_t row = query ? qid[r] : first + r;
@@ -57,7 +83,9 @@ __global__ void __launch_bounds__(kNT) k7_exact(const float* __restrict__ X, int
 #pragma unroll
         for (int o = 0; o < NO; ++o) run[rr][o] = kEmptyKey;
 
-    for (int64_t c0 = 0; c0 < n; c0 += kCT) {
+    const int64_t tiles = (n + kCT - 1) / kCT;
+    const int64_t t0 = tiles * blockIdx.y / gridDim.y, t1 = tiles * (blockIdx.y + 1) / gridDim.y;
+    for (int64_t c0 = t0 * kCT; c0 < min(n, t1 * kCT); c0 += kCT) {
         float acc[4][8];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -130,8 +158,42 @@ __global__ void __launch_bounds__(kNT) k7_exact(const float* __restrict__ X, int
         if (r >= nq) continue;
 #pragma unroll
         for (int o = 0; o < NO; ++o)
-            if (lane + 32 * o < k) out[(q0 + r) * k + lane + 32 * o] = run[rr][o];
+            if (lane + 32 * o < k) {
+                uint64_t* dst = gridDim.y > 1 ? part + ((q0 + r) * gridDim.y + blockIdx.y) * k
+                                              : out + (list ? (int64_t)list[q0 + r] : q0 + r) * k;
+                dst[lane + 32 * o] = run[rr][o];
+            }
     }
+}
+
+// One warp per list slot: the k best of its nsplit partial lists.
+template <int NO>
+__global__ void __launch_bounds__(256) k7_merge(const uint64_t* __restrict__ part, int nsplit, int k, int64_t s_rows,
+                                               const int32_t* __restrict__ list, const int* __restrict__ list_count,
+                                               uint64_t* __restrict__ out, const int* __restrict__ status) {
+    if (*status & kStatusStop) return;
+    if (list) s_rows = *list_count;
+    const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    if (r >= s_rows) return;
+    const int lane = threadIdx.x & 31;
+    uint64_t run[NO];
+#pragma unroll
+    for (int o = 0; o < NO; ++o) run[o] = kEmptyKey;
+    for (int y = 0; y < nsplit; ++y) {
+        uint64_t a[2 * NO];
+#pragma unroll
+        for (int o = 0; o < NO; ++o) {
+            const int e = lane + 32 * o;
+            a[o] = e < k ? part[(r * nsplit + y) * k + e] : kEmptyKey;
+            a[NO + o] = run[o];
+        }
+        sort_regs<2 * NO>(a);
+        warp_select_unique<2 * NO, NO>(a, k, run);
+    }
+    const int64_t q = list ? (int64_t)list[r] : r;
+#pragma unroll
+    for (int o = 0; o < NO; ++o)
+        if (lane + 32 * o < k) out[q * k + lane + 32 * o] = run[o];
 }
 
 __global__ void k_recall(const int32_t* __restrict__ ids, const float* __restrict__ d,
@@ -178,19 +240,33 @@ __global__ void k_check_finite(const float4* __restrict__ X4, int64_t n4, const 
 
 }  // namespace
 
-void launch_exact(const float* X, int64_t n, int D, int k, const int32_t* sample, int64_t s_rows, uint64_t* out,
+int exact_splits(int64_t n, int64_t s_rows) {
+    // one CTA fits an SM at D >= 128: two waves of CTAs, at least 8 column tiles each
+    const int64_t rt = (s_rows + kQR - 1) / kQR, tiles = (n + kCT - 1) / kCT;
+    return (int)std::max<int64_t>(1, std::min<int64_t>({(2 * 152 + rt - 1) / rt, tiles / 8, 32}));
+}
+
+void launch_exact(const float* X, int64_t n, int D, int k, const int32_t* sample, int64_t row0, int64_t s_rows,
+                  const int32_t* list, const int* list_count, int nsplit, uint64_t* part, uint64_t* out,
                   const int* status, cudaStream_t s) {
     int dch, stride;
     exact_chunk(D, &dch, &stride);
     const size_t smem = (size_t)(kQR + kCT) * stride * 4 + (size_t)kQR * (kCT + 1) * 4 + kQR * 8;
-    const int grid = (int)((s_rows + kQR - 1) / kQR);
-    LaunchScope ls("k7_exact", s, (double)grid * n * D * 4.0, (double)s_rows * n * 3.0 * D);
+    const dim3 grid((unsigned)((s_rows + kQR - 1) / kQR), (unsigned)nsplit);
+    // rows taken from a list: how many is known on the device only
+    LaunchScope ls("k7_exact", s, list ? 0.0 : (double)grid.x * n * D * 4.0, list ? 0.0 : (double)s_rows * n * 3.0 * D,
+                   nsplit > 1 ? 2 : 1);
+    const int mgrid = (int)((s_rows * 32 + 255) / 256);
     if (k > 32) {
         cudaFuncSetAttribute(k7_exact<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k7_exact<2><<<grid, kNT, smem, s>>>(X, n, D, k, sample, s_rows, out, status);
+        k7_exact<2><<<grid, kNT, smem, s>>>(X, n, D, k, sample, row0, s_rows, list, list_count, part, out, status);
+        if (nsplit > 1)
+            k7_merge<2><<<mgrid, 256, 0, s>>>(part, nsplit, k, s_rows, list, list_count, out, status);
     } else {
         cudaFuncSetAttribute(k7_exact<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k7_exact<1><<<grid, kNT, smem, s>>>(X, n, D, k, sample, s_rows, out, status);
+        k7_exact<1><<<grid, kNT, smem, s>>>(X, n, D, k, sample, row0, s_rows, list, list_count, part, out, status);
+        if (nsplit > 1)
+            k7_merge<1><<<mgrid, 256, 0, s>>>(part, nsplit, k, s_rows, list, list_count, out, status);
     }
 }
 

@@ -317,8 +317,35 @@ void launch_search(const float* X, int64_t n, int D, const int32_t* G, int k, co
                    int64_t q1, const int32_t* S, int s, int t0, int ks, int32_t* tab, int cap_log2, int32_t* out_ids,
                    float* out_d, cudaStream_t st);
 
-void launch_exact(const float* X, int64_t n, int D, int k, const int32_t* sample, int64_t s_rows,
-                  uint64_t* out, const int* status, cudaStream_t s);
+// The k nearest of rows sample[0 .. s_rows) (row0 + r without a sample), of
+// only the rows listed in list[0 .. *list_count) when a list is given, in
+// FP32 throughout; out: k keys per row.  nsplit > 1 (exact_splits) spreads the
+// columns over that many CTAs per row tile; part: s_rows * nsplit * k keys.
+int exact_splits(int64_t n, int64_t s_rows);
+void launch_exact(const float* X, int64_t n, int D, int k, const int32_t* sample, int64_t row0, int64_t s_rows,
+                  const int32_t* list, const int* list_count, int nsplit, uint64_t* part, uint64_t* out,
+                  const int* status, cudaStream_t s);
+
+// Tensor-core screening (screen.cu).  exact_screened: whether exact lists
+// over n points are screened; exact_batch: rows screened at once; the lists equal
+// launch_exact's bit for bit.  Checks X for non-finite values on the way.
+struct ScreenWork {
+    uint16_t *Xq, *Qq;      // BF16 copies of X and of a batch's rows
+    float *nrm, *err;       // [n]
+    float *qn, *qe;         // [batch]
+    float* cg;              // [batch][kScreenCap] candidates: product, id
+    int32_t* cid;
+    int32_t* cnt;           // [batch]
+    float *rowA, *rowR;     // [batch]
+    int* flags;             // [0] exactness flags, [1] rows in fb_list
+    int32_t *fb_list, *fb_flag;  // [batch]
+    uint64_t* part;         // [batch][exact_splits][k]
+};
+constexpr int kScreenCap = 4096;
+bool exact_screened(int64_t n);
+int64_t exact_batch(int64_t s_rows);
+bool launch_exact_screened(const float* X, int64_t n, int D, int k, const int32_t* sample, int64_t s_rows,
+                           const ScreenWork& w, uint64_t* out, int* status, cudaStream_t s);
 void launch_recall(const int32_t* ids, const float* d, const int32_t* gt_ids, const float* gt_d,
                    const int32_t* sample, int64_t s_rows, int k, unsigned long long* counts,
                    cudaStream_t s);

@@ -687,6 +687,14 @@ EncodeTiledFn encode_fn() {
 
 }  // namespace
 
+bool tensor_map_encode(CUtensorMap* m, CUtensorMapDataType type, const void* base, const cuuint64_t* gdim,
+                       const cuuint64_t* gstride, const cuuint32_t* box, const cuuint32_t* estride) {
+    EncodeTiledFn enc = encode_fn();
+    return enc && enc(m, type, 2, const_cast<void*>(base), gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 int lp_dim(int D) { return (D + kTcK - 1) / kTcK * kTcK; }
 
 int lp_row_bytes(int D, int qt) { return qt == 2 ? (D + kRowChunk - 1) / kRowChunk * kRowChunk : 2 * lp_dim(D); }

@@ -150,7 +150,7 @@ extern "C" KNNG_API int knng_exact_noalloc(const float* data, int64_t n, int D, 
     if (cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) return fail(KNNG_ECUDA, "status clear failed");
     launch_check_finite(data, n * (int64_t)D, status, st);
     launch_check_ids(sample, s, 0, n, status, st);
-    launch_exact(data, n, D, k, sample, s, keys, status, st);
+    launch_exact(data, n, D, k, sample, 0, s, nullptr, nullptr, 1, nullptr, keys, status, st);
     launch_unpack(keys, out_ids, out_dists, s * (int64_t)k, st);
     // a launch the runtime refused (for example the dynamic shared memory of
     // the exact kernel) leaves the outputs unwritten: report it before the

@@ -1,0 +1,994 @@
+// screen.cu -- exact nearest neighbours found by tensor-core screening: a
+// BF16 Gram matrix (tcgen05, TMA-fed, FP32 accumulators in tensor memory)
+// says which columns can matter to a row, and only those get their canonical
+// FP32 distance.  The error bound makes the result the plain FP32 form's, bit
+// for bit; a row the bound cannot serve goes to the FP32 kernel.
+//
+//   exact lists (Sec. 1)      rows = sampled points, columns = all points
+//   nearest word (Sec. 4.1)   rows = vectors, columns = up to 256 words
+//
+// Bound.  x^ is the BF16 copy, e = ||x - x^|| (rounded up), N = ||x^||^2, g the
+// computed x^_i . x^_j.  For the distance d of the FP32 points,
+//   |sqrt(d) - sqrt(d~)| <= e_i + e_j        (d~: exact distance of x^)
+//   |N_i + N_j - 2 g - d~| <= cD (||x^_i|| + ||x^_j||)^2 <= 2 cD (N_i + N_j)
+// with cD the leaf certificate's coefficient, and the canonical FP32 distance
+// is within a factor 1 +- gamma, gamma = (D + 8) 2^-23, of d.  A column whose
+// canonical distance is at most tau therefore has
+//   c_j - 2 g - 2 a_i e_j <= R_i,  c_j = N_j (1 - c) - e_j^2,
+//   a_i = sqrt(tau (1 + gamma)) + e_i,  R_i = a_i^2 + N_i (c - 1)
+// where c = 2 cD + 2^-19 also covers the test's own FP32 roundings.  When the
+// data are integers that BF16 holds exactly (the leaf stage's exactness
+// flag), every quantity is an exact integer and e, c and gamma are 0.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "common.cuh"
+#include "kernels.h"
+#include "tc.cuh"
+
+namespace knng {
+
+namespace {
+
+constexpr int kScM = 128;          // rows of a tile (tensor-memory lanes)
+constexpr int kScN = 256;          // columns of a tile
+constexpr int kScK = 64;           // BF16 elements per 128-byte swizzled row
+constexpr int kScStages = 4;
+constexpr int kScABytes = kScM * 128, kScBBytes = kScN * 128;
+constexpr int kScResident = 4;     // K chunks up to which a row tile stays in shared memory
+constexpr int kScEpi = 512;        // epilogue threads: 16 warps, four per tensor-memory quarter
+constexpr int kScPart = kScN / 4;  // columns per epilogue warp
+constexpr int kScThreads = 64 + kScEpi;  // + a TMA warp and an MMA warp
+constexpr int kScGrid = 152;       // one CTA per SM (512 tensor-memory columns, over half of shared memory)
+constexpr int kScCand = 2048;      // candidates buffered in shared memory (collect)
+constexpr int kScList = 8192;      // (row, word) pairs of one tile (nearest word)
+constexpr float kScTiny = 1e-17f;  // added to e: squares below FP32's range summed as zero
+
+enum ScreenMode { kScDump = 0, kScCollect = 1, kScArgmin = 2 };
+
+struct ScreenArgs {
+    int nk;                // K chunks
+    int64_t nrows, ncols;  // rows and columns of the product
+    int nrt, nct, nstripe;
+    // per row (original row of row r: rid ? rid[r] : rid0 + r)
+    const float* rnrm;     // [nrows]
+    const float* rerr;
+    // per column: column j is row j * cstride of these
+    const float* cnrm;
+    const float* cerr;
+    int64_t cstride;
+    float cD2, gamma;      // 2 cD + 2^-19; (D + 8) 2^-23
+    const int* flag_r;     // exactness flags of the two operands (may be equal)
+    const int* flag_c;
+    int* status;
+    // dump / collect
+    const int32_t* rid;
+    int64_t rid0;
+    int cap;               // candidates kept per row
+    float* cg;             // [nrows][cap] g
+    int32_t* cid;          // [nrows][cap] original row of the column (collect)
+    int32_t* cnt;          // [nrows]
+    const float* rowA;     // [nrows] a_i
+    const float* rowR;     // [nrows] R_i
+    // nearest word: vectors X (minus W1[c1]), words
+    const float* X;
+    const float* W1;
+    const int32_t* c1;
+    int c1_stride;
+    const float* words;
+    int D;
+    bool vec;
+    int32_t* out;
+    int out_stride;
+};
+
+// The flag bits of the copy (k0_quantize's) plus 8: some squared norm is too
+// large for the bound's arithmetic.
+__device__ __forceinline__ bool sc_exact(int f) { return (f & 9) == 0 && !((f & 2) && (f & 4)); }
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+// Barrier of the epilogue warps; true when every thread passed true.
+__device__ __forceinline__ bool epi_all(bool ok) {
+    uint32_t r;
+    asm volatile(
+        "{\n"
+        ".reg .pred p, q;\n"
+        "setp.ne.u32 p, %1, 0;\n"
+        "barrier.cta.red.and.pred q, 1, 512, p;\n"
+        "selp.u32 %0, 1, 0, q;\n"
+        "}\n"
+        : "=r"(r)
+        : "r"((uint32_t)ok)
+        : "memory");
+    return r != 0;
+}
+__device__ __forceinline__ void epi_sync() { asm volatile("barrier.cta.sync 1, 512;\n" ::: "memory"); }
+
+struct ScreenSmem {
+    size_t a_off, col_off, list_off, row_off, bar_off, total;
+    int stage_bytes;
+};
+__host__ __device__ inline ScreenSmem screen_smem(int nk, int mode) {
+    ScreenSmem L;
+    const bool res = nk <= kScResident;
+    L.stage_bytes = kScBBytes + (res ? 0 : kScABytes);
+    L.a_off = (size_t)kScStages * L.stage_bytes;
+    L.col_off = L.a_off + (res ? (size_t)nk * kScABytes : 0);
+    L.list_off = L.col_off + (mode == kScCollect ? kScEpi / 32 * kScPart : 2 * kScN) * 8;
+    L.row_off = L.list_off + (mode == kScCollect ? kScCand * 12 : mode == kScArgmin ? kScList * 2 : 0);
+    L.bar_off = L.row_off + (mode == kScArgmin ? kScM * (8 + 4 * 8 + 4 + 4) : 0);
+    L.total = L.bar_off + (2 * kScStages + 6) * 8 + 32;
+    return L;
+}
+
+// The canonical distance of one vector (x, minus w1 when given) to one word
+// (or to a point staged in shared memory).
+__device__ __forceinline__ float word_dist(const float* __restrict__ x, const float* __restrict__ w1,
+                                           const float* w, int D, bool vec) {
+    float acc = 0.f;
+    if (vec) {
+        for (int d = 0; d < D; d += 4) {
+            float4 a = __ldg(reinterpret_cast<const float4*>(x + d));
+            const float4 b = *reinterpret_cast<const float4*>(w + d);
+            if (w1) {
+                const float4 r = __ldg(reinterpret_cast<const float4*>(w1 + d));
+                a.x = __fsub_rn(a.x, r.x);
+                a.y = __fsub_rn(a.y, r.y);
+                a.z = __fsub_rn(a.z, r.z);
+                a.w = __fsub_rn(a.w, r.w);
+            }
+            float t = __fsub_rn(a.x, b.x);
+            acc = __fmaf_rn(t, t, acc);
+            t = __fsub_rn(a.y, b.y);
+            acc = __fmaf_rn(t, t, acc);
+            t = __fsub_rn(a.z, b.z);
+            acc = __fmaf_rn(t, t, acc);
+            t = __fsub_rn(a.w, b.w);
+            acc = __fmaf_rn(t, t, acc);
+        }
+        return acc;
+    }
+    for (int d = 0; d < D; ++d) {
+        float a = __ldg(x + d);
+        if (w1) a = __fsub_rn(a, __ldg(w1 + d));
+        const float t = __fsub_rn(a, w[d]);
+        acc = __fmaf_rn(t, t, acc);
+    }
+    return acc;
+}
+
+// c_j - 2 g_j - 2 a e_j of two columns (a2 = -2 a), with paired FP32 FMAs.
+__device__ __forceinline__ float2 screen_pair(float g0, float g1, float c0, float c1, float e0, float e1, float a2) {
+    float2 r;
+    asm("{\n"
+        ".reg .b64 g, c, e, m, a;\n"
+        "mov.b64 g, {%2, %3};\n"
+        "mov.b64 c, {%4, %5};\n"
+        "mov.b64 e, {%6, %7};\n"
+        "mov.b64 m, {%8, %8};\n"
+        "mov.b64 a, {%9, %9};\n"
+        "fma.rn.f32x2 c, m, g, c;\n"
+        "fma.rn.f32x2 c, a, e, c;\n"
+        "mov.b64 {%0, %1}, c;\n"
+        "}\n"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(g0), "f"(g1), "f"(c0), "f"(c1), "f"(e0), "f"(e1), "f"(-2.f), "f"(a2));
+    return r;
+}
+__device__ __forceinline__ float min_pair(float2 p, float m) {
+    float r;
+    asm("min.f32 %0, %1, %2, %3;\n" : "=f"(r) : "f"(p.x), "f"(p.y), "f"(m));
+    return r;
+}
+
+// An upper bound of the canonical distance of (i, j) from the copies.
+__device__ __forceinline__ float screen_ub(float ni, float nj, float g, float ei, float ej, float c, float gamma) {
+    const float s = __fadd_ru(ni, nj);
+    const float d = __fadd_ru(__fmaf_ru(-2.f, g, s), __fmul_ru(c, s));
+    const float r = __fadd_ru(__fsqrt_ru(fmaxf(d, 0.f)), __fadd_ru(ei, ej));
+    return __fmul_ru(__fmul_ru(r, r), __fadd_ru(1.f, gamma));
+}
+
+// a_i and R_i of a row whose candidates must have canonical distance <= tau.
+__device__ __forceinline__ void screen_row(float tau, float ni, float ei, float c, float gamma, bool exact, float& a,
+                                           float& R) {
+    if (exact) {
+        a = 0.f;
+        R = __fsub_rn(tau, ni);  // exact integers
+        return;
+    }
+    a = __fadd_ru(__fsqrt_ru(__fmul_ru(tau, __fadd_ru(1.f, gamma))), ei);
+    R = __fadd_ru(__fmaf_ru(__fmul_ru(a, a), 1.f + 1.9073486328125e-6f, 1e-30f), __fmul_ru(ni, c - 1.f));
+}
+
+// Persistent, warp-specialised screening product: warp 0 issues the TMA loads,
+// warp 1 the MMAs (128 x 256 tiles, two accumulators in tensor memory), warps
+// 2-17 read finished accumulators (64 columns of 32 rows each; fewer, wider
+// warps left the issue slots a third used).  A unit is one row tile against every
+// nstripe-th column tile, and units of consecutive row tiles run side by side,
+// so that a column tile is read from DRAM once and then from L2.  With up to
+// kScResident chunks of K the row tile stays in shared memory for the unit.
+template <int MODE>
+__global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant__ CUtensorMap tma,
+                                                          const __grid_constant__ CUtensorMap tmb,
+                                                          const ScreenArgs P) {
+    extern __shared__ uint8_t smem_raw[];
+    if (*P.status & kStatusStop) return;  // whole CTA, before any barrier or tensor memory
+    const ScreenSmem L = screen_smem(P.nk, MODE);
+    uint8_t* base = smem_raw + ((1024 - (tc::smem_addr(smem_raw) & 1023)) & 1023);
+    const bool res = P.nk <= kScResident;
+    float2* colc = reinterpret_cast<float2*>(base + L.col_off);  // (c_j, e_j): [2][kScN], or per warp
+    uint64_t* bars = reinterpret_cast<uint64_t*>(base + L.bar_off);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kScStages + 6);
+    int* ncand = reinterpret_cast<int*>(tmem_slot + 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t full0 = tc::smem_addr(bars), empty0 = full0 + 8 * kScStages;
+    const uint32_t afull = empty0 + 8 * kScStages, aempty = afull + 8, tfull0 = aempty + 8, tempty0 = tfull0 + 16;
+    const int nk = P.nk;
+    const int units = P.nrt * P.nstripe;
+
+    if (tid == 0) {
+        for (int s = 0; s < 2 * kScStages; ++s) tc::mbar_init(full0 + 8 * s, 1);
+        tc::mbar_init(afull, 1);
+        tc::mbar_init(aempty, 1);
+        for (int b = 0; b < 2; ++b) {
+            tc::mbar_init(tfull0 + 8 * b, 1);
+            tc::mbar_init(tempty0 + 8 * b, kScEpi / 32);
+        }
+        tc::mbar_fence_init();
+        ncand[0] = ncand[1] = 0;
+    }
+    if (warp == 1) {
+        tc::tmem_alloc(tc::smem_addr(tmem_slot), 2 * kScN);
+        tc::tmem_relinquish();
+    }
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            bool ok = true;
+            int it = 0, uu = 0;
+            for (int u = blockIdx.x; ok && u < units; u += gridDim.x, ++uu) {
+                const int rt = u % P.nrt;
+                if (res) {
+                    if (!(ok = tc::mbar_wait(aempty, (uint32_t)((uu & 1) ^ 1), P.status))) break;
+                    tc::mbar_expect_tx(afull, (uint32_t)(nk * kScABytes));
+                    for (int c = 0; c < nk; ++c)
+                        tc::tma_load_2d(tc::smem_addr(base + L.a_off + (size_t)c * kScABytes), &tma, c * kScK,
+                                        rt * kScM, afull);
+                }
+                for (int ct = u / P.nrt; ok && ct < P.nct; ct += P.nstripe)
+                    for (int c = 0; c < nk; ++c, ++it) {
+                        const int s = it % kScStages;
+                        if (!(ok = tc::mbar_wait(empty0 + 8 * s, (uint32_t)(((it / kScStages) & 1) ^ 1), P.status)))
+                            break;
+                        const uint32_t fb = full0 + 8 * s, st = tc::smem_addr(base + (size_t)s * L.stage_bytes);
+                        tc::mbar_expect_tx(fb, (uint32_t)L.stage_bytes);
+                        tc::tma_load_2d(st, &tmb, c * kScK, ct * kScN, fb);
+                        if (!res) tc::tma_load_2d(st + kScBBytes, &tma, c * kScK, rt * kScM, fb);
+                    }
+            }
+            if (!ok) {  // let the loads still in flight land before the CTA can exit
+                if (res && uu > 0) tc::mbar_wait(afull, (uint32_t)((uu - 1) & 1), P.status);
+                for (int j = std::max(0, it - kScStages); j < it; ++j)
+                    tc::mbar_wait(full0 + 8 * (j % kScStages), (uint32_t)((j / kScStages) & 1), P.status);
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            bool ok = true;
+            int it = 0, uu = 0, t = 0;
+            const uint32_t idesc = tc::idesc_f16(true, kScM, kScN);
+            for (int u = blockIdx.x; ok && u < units; u += gridDim.x, ++uu) {
+                if (res && !(ok = tc::mbar_wait(afull, (uint32_t)(uu & 1), P.status))) break;
+                for (int ct = u / P.nrt; ok && ct < P.nct; ct += P.nstripe, ++t) {
+                    const int buf = t & 1;
+                    if (!(ok = tc::mbar_wait(tempty0 + 8 * buf, (uint32_t)(((t >> 1) & 1) ^ 1), P.status))) break;
+                    tc::fence_after_sync();
+                    const uint32_t acc = tmem + (uint32_t)(buf * kScN);
+                    for (int c = 0; c < nk; ++c, ++it) {
+                        const int s = it % kScStages;
+                        if (!(ok = tc::mbar_wait(full0 + 8 * s, (uint32_t)((it / kScStages) & 1), P.status))) break;
+                        tc::fence_after_sync();
+                        const uint32_t st = tc::smem_addr(base + (size_t)s * L.stage_bytes);
+                        const uint64_t db = tc::sdesc_k128(st);
+                        const uint64_t da = tc::sdesc_k128(
+                            res ? tc::smem_addr(base + L.a_off + (size_t)c * kScABytes) : st + kScBBytes);
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk)
+                            tc::mma_f16(acc, da + 2 * kk, db + 2 * kk, idesc, (c | kk) != 0);
+                        tc::mma_commit(empty0 + 8 * s);
+                    }
+                    if (ok) tc::mma_commit(tfull0 + 8 * buf);
+                }
+                if (ok && res) tc::mma_commit(aempty);
+            }
+        }
+    } else {
+        const int et = tid - 64;                 // epilogue thread
+        const int qd = warp & 3;                 // tensor-memory quarter this warp may read
+        const int part = (warp - 2) >> 2;        // columns kScPart part .. of the tile
+        const int rl = qd * 32 + lane;           // row of the tile
+        const int fr = *P.flag_r, fc = *P.flag_c;
+        const bool exact = sc_exact(fr | fc), unsafe = ((fr | fc) & 8) != 0;
+        const float c2 = exact ? 0.f : P.cD2, gamma = exact ? 0.f : P.gamma;
+        // collect: candidates of the CTA, flushed to the rows' lists
+        int32_t* brow = reinterpret_cast<int32_t*>(base + L.list_off);
+        int32_t* bid = brow + kScCand;
+        float* bg = reinterpret_cast<float*>(bid + kScCand);
+        // nearest word
+        uint16_t* list = reinterpret_cast<uint16_t*>(base + L.list_off);
+        uint64_t* best = reinterpret_cast<uint64_t*>(base + L.row_off);  // [kScM]
+        float2* hmin = reinterpret_cast<float2*>(best + kScM);           // [4][kScM] (value, g)
+        int* rcount = reinterpret_cast<int*>(hmin + 4 * kScM);           // [kScM] candidates
+        int* rfull = rcount + kScM;                                      // [kScM] every word is one
+        int* nfull = ncand + 1;                                          // rows with rfull set
+        int t = 0;
+        auto col_const = [&](int64_t col) -> float2 {
+            if (col >= P.ncols) return make_float2(__int_as_float(0x7f800000), 0.f);
+            const float nj = __ldg(P.cnrm + col * P.cstride);
+            if (exact) return make_float2(nj, 0.f);
+            const float ej = __ldg(P.cerr + col * P.cstride);
+            return make_float2(__fsub_rd(__fmul_rd(nj, 1.f - c2), __fmul_ru(ej, ej)), ej);
+        };
+        float* wcol = reinterpret_cast<float*>(colc + (warp - 2) * kScPart);  // collect: this warp's c_j, then e_j
+        float2 next_col[2];
+        auto load_cols = [&](int ct) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                next_col[q] = col_const((int64_t)ct * kScN + part * kScPart + 32 * q + lane);
+        };
+        auto append = [&](int64_t row, int64_t own, int64_t id, float g) {
+            if (id == own) return;
+            const int at = atomicAdd(ncand, 1);
+            if (at < kScCand) {
+                brow[at] = (int32_t)row;
+                bid[at] = (int32_t)id;
+                bg[at] = g;
+                return;
+            }
+            // the buffer is full: straight to the row's list
+            const int pos = atomicAdd(P.cnt + row, 1);
+            if (pos < P.cap) {
+                P.cid[row * P.cap + pos] = (int32_t)id;
+                P.cg[row * P.cap + pos] = g;
+            }
+        };
+        auto flush = [&](int n) {  // every epilogue thread, uniform n
+            n = min(n, kScCand);
+            for (int e = et; e < n; e += kScEpi) {
+                const int64_t r = brow[e];
+                const int pos = atomicAdd(P.cnt + r, 1);
+                if (pos < P.cap) {
+                    P.cid[r * P.cap + pos] = bid[e];
+                    P.cg[r * P.cap + pos] = bg[e];
+                }
+            }
+            epi_sync();
+            if (et == 0) *ncand = 0;
+            epi_sync();
+        };
+        if (blockIdx.x < (unsigned)units && MODE == kScCollect) load_cols(blockIdx.x / P.nrt);
+        bool ok = true;
+        for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
+            const int rt = u % P.nrt;
+            const int64_t row = (int64_t)rt * kScM + rl;
+            const bool live = row < P.nrows;
+            float a2 = 0.f, R = __int_as_float(0xff800000), ni = 0.f, ei = 0.f;
+            int64_t own = -1;
+            if (live) {
+                ni = __ldg(P.rnrm + row);
+                ei = exact ? 0.f : __ldg(P.rerr + row);
+                if (MODE == kScCollect) {
+                    a2 = -2.f * P.rowA[row];
+                    R = P.rowR[row];
+                    own = P.rid ? (int64_t)P.rid[row] : P.rid0 + row;
+                }
+            }
+            for (int ct = u / P.nrt; ct < P.nct; ct += P.nstripe, ++t) {
+                const int buf = t & 1;
+                if (MODE == kScArgmin && et < kScN) colc[buf * kScN + et] = col_const((int64_t)ct * kScN + et);
+                if (MODE == kScCollect) {
+                    // the warp's own copy of its columns' constants: the
+                    // warps share nothing per tile, so one that appends
+                    // candidates holds no other back
+                    __syncwarp();
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        wcol[32 * q + lane] = next_col[q].x;
+                        wcol[kScPart + 32 * q + lane] = next_col[q].y;
+                    }
+                    __syncwarp();
+                    // the next tile's load while this one is read
+                    int nct = ct + P.nstripe;
+                    if (nct >= P.nct) nct = u + gridDim.x < units ? (int)(u + gridDim.x) / P.nrt : -1;
+                    if (nct >= 0) load_cols(nct);
+                }
+                ok = tc::mbar_wait(tfull0 + 8 * buf, (uint32_t)((t >> 1) & 1), P.status);
+                if (MODE == kScArgmin) ok = epi_all(ok);  // also: the column constants are in place
+                if (!ok) break;
+                tc::fence_after_sync();
+                const uint32_t taddr =
+                    tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(buf * kScN + part * kScPart);
+                const float2* cc = colc + buf * kScN + part * kScPart;
+                if (MODE == kScDump) {
+#pragma unroll 1
+                    for (int b = 0; b < kScPart / 32; ++b) {
+                        float v[32];
+                        tc::tmem_ld_32(taddr + b * 32, v);
+                        const int64_t col0 = (int64_t)ct * kScN + part * kScPart + b * 32;
+                        if (live) {
+#pragma unroll
+                            for (int q = 0; q < 8; ++q)
+                                if (col0 + 4 * q < P.ncols)  // cap is a multiple of 4 past the last column
+                                    *reinterpret_cast<float4*>(P.cg + row * P.cap + col0 + 4 * q) =
+                                        make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                        }
+                    }
+                } else if (MODE == kScCollect) {
+#pragma unroll 1  // one copy of the code: it stays within the instruction cache
+                    for (int b = 0; b < kScPart / 32; ++b) {
+                        float v[32];
+                        tc::tmem_ld_32(taddr + b * 32, v);
+                        if (b == kScPart / 32 - 1) {  // the last of it is in registers: hand the accumulator back
+                            tc::fence_before_sync();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(tempty0 + 8 * buf);
+                        }
+                        // two columns per instruction where there is one
+                        const float4* c4 = reinterpret_cast<const float4*>(wcol + b * 32);
+                        const float4* e4 = reinterpret_cast<const float4*>(wcol + kScPart + b * 32);
+                        float mn = __int_as_float(0x7f800000);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const float4 c = c4[q], e = e4[q];
+                            mn = min_pair(screen_pair(v[4 * q], v[4 * q + 1], c.x, c.y, e.x, e.y, a2), mn);
+                            mn = min_pair(screen_pair(v[4 * q + 2], v[4 * q + 3], c.z, c.w, e.z, e.w, a2), mn);
+                        }
+                        if (mn <= R) {  // few blocks hold a candidate
+                            unsigned hit = 0;
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) {
+                                const float4 c = c4[q], e = e4[q];
+                                const float2 x = screen_pair(v[4 * q], v[4 * q + 1], c.x, c.y, e.x, e.y, a2);
+                                const float2 y = screen_pair(v[4 * q + 2], v[4 * q + 3], c.z, c.w, e.z, e.w, a2);
+                                if (x.x <= R) hit |= 1u << (4 * q);
+                                if (x.y <= R) hit |= 2u << (4 * q);
+                                if (y.x <= R) hit |= 4u << (4 * q);
+                                if (y.y <= R) hit |= 8u << (4 * q);
+                            }
+                            for (; hit; hit &= hit - 1) {  // v[j] by a chain of selects
+                                const int j = __ffs(hit) - 1;
+                                float g = v[0];
+#pragma unroll
+                                for (int q = 1; q < 32; ++q) g = j == q ? v[q] : g;
+                                append(row, own, ((int64_t)ct * kScN + part * kScPart + b * 32 + j) * P.cstride, g);
+                            }
+                        }
+                        __syncwarp();
+                    }
+                } else {
+                    // nearest word: the tile's least approximate value gives an
+                    // upper bound tau of the row's least distance; every word
+                    // that could be within tau is a candidate
+                    float mv = __int_as_float(0x7f800000);
+                    int mc = 0;
+                    float mg = 0.f;
+#pragma unroll 1
+                    for (int b = 0; b < kScPart / 32; ++b) {
+                        float v[32];
+                        tc::tmem_ld_32(taddr + b * 32, v);
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) {
+                            const float x = __fmaf_rn(-2.f, v[j], cc[b * 32 + j].x);
+                            if (x < mv) {
+                                mv = x;
+                                mg = v[j];
+                                mc = part * kScPart + b * 32 + j;
+                            }
+                        }
+                    }
+                    hmin[part * kScM + rl] = make_float2(mv, mg);
+                    if (part == 0) {
+                        best[rl] = kEmptyKey;
+                        rcount[rl] = 0;
+                        rfull[rl] = 0;
+                    }
+                    if (et == 0) *ncand = *nfull = 0;
+                    // the column of each part's least value travels in the list's first words
+                    reinterpret_cast<uint8_t*>(list)[part * kScM + rl] = (uint8_t)mc;
+                    epi_sync();
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float2 o = hmin[q * kScM + rl];
+                        if (o.x < mv) {
+                            mv = o.x;
+                            mg = o.y;
+                            mc = reinterpret_cast<uint8_t*>(list)[q * kScM + rl];
+                        }
+                    }
+                    epi_sync();
+                    if (live) {
+                        const float nj = __ldg(P.cnrm + mc), ej = exact ? 0.f : __ldg(P.cerr + mc);
+                        const float tau = exact ? __fmaf_rn(-2.f, mg, __fadd_rn(ni, nj))
+                                                : screen_ub(ni, nj, mg, ei, ej, c2, gamma);
+                        float a;
+                        screen_row(tau, ni, ei, c2, gamma, exact, a, R);
+                        a2 = -2.f * a;
+                        if (unsafe) rfull[rl] = *nfull = 1;
+                    }
+#pragma unroll 1
+                    for (int b = 0; b < kScPart / 32; ++b) {
+                        float v[32];
+                        tc::tmem_ld_32(taddr + b * 32, v);
+                        unsigned hit = 0;
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) {
+                            const float2 c = cc[b * 32 + j];
+                            const bool in = __fmaf_rn(a2, c.y, __fmaf_rn(-2.f, v[j], c.x)) <= R;
+                            hit |= in ? 1u << j : 0u;
+                        }
+                        if (live && !unsafe && hit) {
+                            const int c = __popc(hit);
+                            atomicAdd(rcount + rl, c);
+                            int at = atomicAdd(ncand, c);
+                            if (at + c > kScList) {
+                                rfull[rl] = *nfull = 1;
+                                for (; hit && at < kScList; hit &= hit - 1) list[at++] = 0xFFFFu;
+                            }
+                            for (; hit; hit &= hit - 1)
+                                list[at++] = (uint16_t)((rl << 8) | (part * kScPart + b * 32 + __ffs(hit) - 1));
+                        }
+                    }
+                }
+                if (MODE != kScCollect) {  // the accumulator is read: hand it back
+                    tc::fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(tempty0 + 8 * buf);
+                }
+                if (MODE == kScArgmin) {
+                    epi_sync();
+                    const int nl = min(*(volatile int*)ncand, kScList);
+                    const int64_t row0 = (int64_t)rt * kScM;
+                    auto exact_key = [&](int r, int w) {
+                        const int64_t i = row0 + r;
+                        const float* w1 = P.W1 ? P.W1 + (int64_t)P.c1[i * P.c1_stride] * P.D : nullptr;
+                        return make_key(word_dist(P.X + i * P.D, w1, P.words + (int64_t)w * P.D, P.D, P.vec),
+                                        (uint32_t)w);
+                    };
+                    for (int e = et; e < nl; e += kScEpi) {
+                        const int v = list[e];
+                        const int r = v >> 8, w = v & 255;
+                        if (r >= kScM || rfull[r]) continue;  // a row taken whole below
+                        // the only candidate is the nearest word: no distance needed
+                        const uint64_t key = rcount[r] == 1 ? (uint64_t)w : exact_key(r, w);
+                        atomicMin(reinterpret_cast<unsigned long long*>(best + r), (unsigned long long)key);
+                    }
+                    for (int r = 0; *(volatile int*)nfull && r < kScM; ++r) {  // rows without a usable bound
+                        if (!rfull[r] || row0 + r >= P.nrows) continue;
+                        for (int w = et; w < (int)P.ncols; w += kScEpi)
+                            atomicMin(reinterpret_cast<unsigned long long*>(best + r),
+                                      (unsigned long long)exact_key(r, w));
+                    }
+                    epi_sync();
+                    if (et < kScM && row0 + et < P.nrows)
+                        P.out[(row0 + et) * P.out_stride] = (int32_t)key_id(best[et]);
+                }
+            }
+            if (MODE == kScCollect) {
+                ok = epi_all(ok);  // every warp comes here, done with the unit or out of time
+                if (!ok) break;
+                const int n = *(volatile int*)ncand;
+                epi_sync();
+                if (n > kScCand / 2 || (n > 0 && u + gridDim.x >= units)) flush(n);
+            }
+        }
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == 1) tc::tmem_dealloc(tmem, 2 * kScN);
+}
+
+// ---------------------------------------------------------------- copies
+// BF16 copy of N vectors (rows of X, gathered by perm when given, minus their
+// stage-1 word when W1 is given), zero-padded to Dp, with squared norms, error
+// bounds and the exactness flags of the leaf stage's k0_quantize plus 8: some
+// squared norm is not below 1e30 (the bound's arithmetic could overflow).
+// One warp takes 4 rows at once, so that 4 row pieces are in flight per lane.
+// status (may be NULL): kStatusNonFinite when a value is not finite.
+template <bool VEC>
+__global__ void __launch_bounds__(256) ks_copy(const float* __restrict__ X, int64_t N, int D, int Dp,
+                                              const float* __restrict__ W1, const int32_t* __restrict__ c1,
+                                              int c1_stride, uint16_t* __restrict__ Xq, float* __restrict__ nrm,
+                                              float* __restrict__ err, int* __restrict__ flags,
+                                              int* __restrict__ status) {
+    const int lane = threadIdx.x & 31;
+    const int64_t r0 = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * 4;
+    if (r0 >= N) return;
+    float red[8];  // squared norms of rows 0-3, then squared errors
+    float top = 0.f, low = 0.f;
+    bool ints = true;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) red[u] = 0.f;
+    for (int d0 = lane * 4; d0 < Dp; d0 += 128) {
+        float v[4][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[u][j] = 0.f;
+            if (r0 + u < N) {
+                const float* x = X + (r0 + u) * D + d0;
+                if (VEC) {
+                    if (d0 < D) {
+                        const float4 f = __ldg(reinterpret_cast<const float4*>(x));
+                        v[u][0] = f.x; v[u][1] = f.y; v[u][2] = f.z; v[u][3] = f.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (d0 + j < D) v[u][j] = __ldg(x + j);
+                }
+            }
+        }
+        if (W1) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (r0 + u < N) {
+                    const float* w = W1 + (int64_t)c1[(r0 + u) * c1_stride] * D + d0;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (d0 + j < D) v[u][j] = __fsub_rn(v[u][j], __ldg(w + j));
+                }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            uint32_t h[2];
+#pragma unroll
+            for (int j = 0; j < 4; j += 2) {
+                const float x = v[u][j], y = v[u][j + 1];
+                const __nv_bfloat162 q = __floats2bfloat162_rn(x, y);
+                h[j / 2] = *reinterpret_cast<const uint32_t*>(&q);
+                const float b = __uint_as_float(h[j / 2] << 16), c = __uint_as_float(h[j / 2] & 0xFFFF0000u);
+                red[u] = __fmaf_rn(b, b, red[u]);
+                red[u] = __fmaf_rn(c, c, red[u]);
+                const float s = __fsub_rn(x, b), t = __fsub_rn(y, c);  // exact: x and y rounded to fewer bits
+                red[4 + u] = __fmaf_rn(s, s, red[4 + u]);
+                red[4 + u] = __fmaf_rn(t, t, red[4 + u]);
+                // whether a value of magnitude <= 256 is an integer: adding
+                // 1.5 * 2^23 rounds it to one
+                ints &= __fsub_rn(__fadd_rn(x, 12582912.f), 12582912.f) == x;
+                ints &= __fsub_rn(__fadd_rn(y, 12582912.f), 12582912.f) == y;
+                top = fmaxf(top, fmaxf(fabsf(x), fabsf(y)));
+                low = fminf(low, fminf(x, y));
+            }
+            if (r0 + u < N) *reinterpret_cast<uint2*>(Xq + (r0 + u) * Dp + d0) = make_uint2(h[0], h[1]);
+        }
+    }
+    // lanes 4 e .. 4 e + 3 end with the warp's sum of red[e]: each exchange
+    // halves the sums a lane carries
+#pragma unroll
+    for (int st = 16, cnt = 4; st >= 4; st >>= 1, cnt >>= 1) {
+        const bool hi = (lane & st) != 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (u >= cnt) break;
+            const float send = hi ? red[u] : red[u + cnt], keep = hi ? red[u + cnt] : red[u];
+            red[u] = __fadd_rn(keep, __shfl_xor_sync(0xffffffffu, send, st));
+        }
+    }
+    float sum = red[0];
+    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+    const int e = lane >> 2;  // 0-3: squared norms, 4-7: squared errors
+    int f = 0;
+    if (e < 4) f = (sum >= 8388608.f ? 1 : 0) | (sum >= 4194304.f ? 4 : 0) | (!(sum < 1e30f) ? 8 : 0);
+    f |= ((!ints || !(top <= 256.f)) ? 1 : 0) | (low < 0.f ? 2 : 0);
+    f = __reduce_or_sync(0xffffffffu, f);
+    if ((lane & 3) == 0 && r0 + (e & 3) < N) {
+        if (e < 4)
+            nrm[r0 + e] = sum;
+        else  // rounded up as in k0_quantize, plus what squares below the FP32 range could hide
+            err[r0 + e - 4] = __fadd_ru(kScTiny, __fsqrt_ru(__fmul_ru(sum, 1.f + (float)(Dp + 8) * 5.9604645e-8f)));
+    }
+    if (lane == 0 && f) atomicOr(flags, f);
+    if (status && (f & 8)) {  // a value that is not finite, or only a large norm?
+        bool bad = false;
+        for (int u = 0; u < 4 && r0 + u < N; ++u)
+            for (int d = lane; d < D; d += 32) bad |= !isfinite(X[(r0 + u) * D + d]);
+        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(status, kStatusNonFinite);
+    }
+}
+
+// Rows perm[p] of a copy (q 16-byte pieces per row) with their norms and errors.
+__global__ void __launch_bounds__(256) ks_gather(const uint4* __restrict__ Xq, const float* __restrict__ nrm,
+                                                const float* __restrict__ err, int64_t n, int q,
+                                                const int32_t* __restrict__ perm, uint4* __restrict__ out,
+                                                float* __restrict__ onrm, float* __restrict__ oerr,
+                                                const int* __restrict__ status) {
+    if (*status & kStatusStop) return;  // a sampled id failed its check
+    const int64_t total = n * q;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t p = e / q;
+        const int c = (int)(e - p * q);
+        const int64_t i = perm[p];
+        out[e] = __ldg(Xq + i * q + c);
+        if (c == 0) {
+            onrm[p] = nrm[i];
+            oerr[p] = err[i];
+        }
+    }
+}
+
+// ---------------------------------------------------------------- thresholds and re-rank
+constexpr int kRrThreads = 256;
+
+// The value of rank `rank` (from 0) among u[0 .. c), by 8-bit digits from the
+// top.  Called by the whole CTA; u is read only; synchronised on return.
+__device__ uint32_t block_select32(const uint32_t* u, int c, int rank, int* hist, int* sh) {
+    uint32_t prefix = 0;
+    for (int sft = 24; sft >= 0; sft -= 8) {
+        hist[threadIdx.x] = 0;
+        __syncthreads();
+        for (int e = threadIdx.x; e < c; e += kRrThreads)
+            if (sft == 24 || (u[e] >> (sft + 8)) == (prefix >> (sft + 8))) atomicAdd(hist + ((u[e] >> sft) & 255), 1);
+        __syncthreads();
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, v = hist[threadIdx.x];
+        int x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) sh[w] = x;
+        __syncthreads();
+        int before = x - v;
+        for (int q = 0; q < w; ++q) before += sh[q];
+        if (before <= rank && rank < before + v) {
+            sh[8] = (int)threadIdx.x;
+            sh[9] = before;
+        }
+        __syncthreads();
+        prefix |= (uint32_t)sh[8] << sft;
+        rank -= sh[9];
+        __syncthreads();
+    }
+    return prefix;
+}
+
+// One CTA per row: the row's candidates (dump: every column of the last
+// product; else its collected list) give tau, an upper bound of its k-th least
+// canonical distance.  FINAL = false: stores a_i and R_i of tau for the next,
+// denser set of columns.  FINAL = true: the candidates that tau cannot exclude
+// get their canonical distance and the k least (distance, id) are written.  A
+// row whose list overflowed, or that the bound cannot serve, is listed for the
+// FP32 kernel (fb_list, fb_count) and takes no further part.
+template <bool FINAL>
+__global__ void __launch_bounds__(kRrThreads) k7_rank(ScreenArgs P, bool dump, int k, float* __restrict__ rowA,
+                                                     float* __restrict__ rowR, int* __restrict__ fb_flag,
+                                                     int32_t* __restrict__ fb_list, int* __restrict__ fb_count,
+                                                     uint64_t* __restrict__ out) {
+    extern __shared__ uint64_t rk_smem[];
+    __shared__ int hist[256], sh[10], ns_sh;
+    if (*P.status & kStatusStop) return;
+    const int64_t r = blockIdx.x;
+    if (fb_flag[r]) return;  // listed already (its R_i excludes every column)
+    uint32_t* u = reinterpret_cast<uint32_t*>(rk_smem);
+    const int f = *P.flag_r;
+    const bool exact = sc_exact(f);
+    const float c2 = exact ? 0.f : P.cD2, gamma = exact ? 0.f : P.gamma;
+    const int64_t own = P.rid ? (int64_t)P.rid[r] : P.rid0 + r;
+    const int found = dump ? (int)P.ncols : P.cnt[r];
+    const int c = min(found, P.cap);
+    const float ni = P.rnrm[r], ei = exact ? 0.f : P.rerr[r];
+    const float* cg = P.cg + r * P.cap;
+    const int32_t* cid = P.cid + r * P.cap;
+    const uint32_t kNone = 0xFFFFFFFFu;
+    for (int e = threadIdx.x; e < c; e += kRrThreads) {
+        const int64_t id = dump ? (int64_t)e * P.cstride : cid[e];
+        uint32_t v = kNone;
+        if (id != own) {
+            const float ub = screen_ub(ni, P.cnrm[id], cg[e], ei, exact ? 0.f : P.cerr[id], c2, gamma);
+            if (ub < __int_as_float(0x7f800000)) v = ord32(ub);
+        }
+        u[e] = v;
+    }
+    __syncthreads();
+    const uint32_t sel = c >= k ? block_select32(u, c, k - 1, hist, sh) : kNone;
+    if ((f & 8) || found > P.cap || sel == kNone) {
+        if (threadIdx.x == 0) {
+            fb_flag[r] = 1;
+            fb_list[atomicAdd(fb_count, 1)] = (int32_t)r;
+            rowA[r] = 0.f;
+            rowR[r] = __int_as_float(0xff800000);
+        }
+        return;
+    }
+    float a, R;
+    screen_row(unord32(sel), ni, ei, c2, gamma, exact, a, R);
+    if (!FINAL) {
+        if (threadIdx.x == 0) {
+            rowA[r] = a;
+            rowR[r] = R;
+        }
+        return;
+    }
+    uint64_t* keys = rk_smem;                                        // [cap] over u
+    int32_t* sid = reinterpret_cast<int32_t*>(rk_smem + P.cap);      // [cap]
+    float* q = reinterpret_cast<float*>(sid + P.cap);                // [D rounded up to 4]
+    if (threadIdx.x == 0) ns_sh = 0;
+    for (int d = threadIdx.x; d < P.D; d += kRrThreads) q[d] = P.X[own * P.D + d];
+    __syncthreads();
+    for (int e = threadIdx.x; e < c; e += kRrThreads) {
+        const int64_t id = dump ? (int64_t)e * P.cstride : cid[e];
+        const float nj = P.cnrm[id], ej = exact ? 0.f : P.cerr[id];
+        const float cj = exact ? nj : __fsub_rd(__fmul_rd(nj, 1.f - c2), __fmul_ru(ej, ej));
+        if (id != own && __fmaf_rn(-2.f * a, ej, __fmaf_rn(-2.f, cg[e], cj)) <= R) sid[atomicAdd(&ns_sh, 1)] = (int32_t)id;
+    }
+    __syncthreads();
+    const int ns = ns_sh;
+    int Pk = 2;
+    while (Pk < ns) Pk <<= 1;
+    for (int e = threadIdx.x; e < Pk; e += kRrThreads)
+        keys[e] = e < ns ? make_key(word_dist(P.X + (int64_t)sid[e] * P.D, nullptr, q, P.D, P.vec), (uint32_t)sid[e])
+                         : kEmptyKey;
+    __syncthreads();
+    for (int kk = 2; kk <= Pk; kk <<= 1)
+        for (int j = kk >> 1; j > 0; j >>= 1) {
+            for (int i = threadIdx.x; i < Pk; i += kRrThreads) {
+                const int l = i ^ j;
+                if (l > i) {
+                    const uint64_t x = keys[i], y = keys[l];
+                    if ((x > y) == ((i & kk) == 0)) {
+                        keys[i] = y;
+                        keys[l] = x;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    for (int e = threadIdx.x; e < k; e += kRrThreads) out[r * k + e] = e < Pk ? keys[e] : kEmptyKey;
+}
+
+// ---------------------------------------------------------------- host
+// 2 cD + 2^-19 for the BF16 copy.
+float screen_c(int D) { return 2.f * lp_cert_coeff(D, 1) + 1.9073486328125e-6f; }
+
+void launch_screen_copy(const float* X, int64_t N, int D, const float* W1, const int32_t* c1, int c1_stride,
+                        uint16_t* Xq, float* nrm, float* err, int* flags, int* status, cudaStream_t s) {
+    const int Dp = lp_dim(D);
+    LaunchScope ls("ks_copy", s, (double)N * (D * 4.0 + Dp * 2.0 + 8.0), 0);
+    const unsigned grid = (unsigned)((N + 31) / 32);
+    if (D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0)
+        ks_copy<true><<<grid, 256, 0, s>>>(X, N, D, Dp, W1, c1, c1_stride, Xq, nrm, err, flags, status);
+    else
+        ks_copy<false><<<grid, 256, 0, s>>>(X, N, D, Dp, W1, c1, c1_stride, Xq, nrm, err, flags, status);
+}
+
+bool screen_map(CUtensorMap* m, const uint16_t* p, int64_t rows, int Dp, int64_t stride, int box_rows) {
+    const cuuint64_t gdim[2] = {(cuuint64_t)Dp, (cuuint64_t)rows};
+    const cuuint64_t gstride[1] = {(cuuint64_t)Dp * 2 * (cuuint64_t)stride};
+    const cuuint32_t box[2] = {(cuuint32_t)kScK, (cuuint32_t)box_rows};
+    const cuuint32_t estride[2] = {1, 1};
+    return tensor_map_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p, gdim, gstride, box, estride);
+}
+
+template <int MODE>
+bool launch_screen(const uint16_t* A, const uint16_t* B, int Dp, ScreenArgs& P, const char* name, cudaStream_t s) {
+    CUtensorMap ta, tb;
+    if (!screen_map(&ta, A, P.nrows, Dp, 1, kScM) || !screen_map(&tb, B, P.ncols, Dp, P.cstride, kScN)) return false;
+    P.nk = Dp / kScK;
+    P.nrt = (int)((P.nrows + kScM - 1) / kScM);
+    P.nct = (int)((P.ncols + kScN - 1) / kScN);
+    // one unit per CTA, or, with many tiles, about four, so that the last wave
+    // is short
+    const bool many = (int64_t)P.nrt * P.nct >= 64 * kScGrid;
+    P.nstripe = std::max(1, std::min(P.nct, many ? (4 * kScGrid + P.nrt - 1) / P.nrt : kScGrid / P.nrt));
+    const size_t smem = screen_smem(P.nk, MODE).total + 1024;
+    const int64_t units = (int64_t)P.nrt * P.nstripe;
+    LaunchScope ls(name, s, (double)(P.nrows + P.ncols) * (Dp * 2.0 + 8.0), (double)P.nrows * P.ncols * 2.0 * Dp);
+    cudaFuncSetAttribute(ks_screen<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    ks_screen<MODE><<<(int)std::min<int64_t>(units, kScGrid), kScThreads, smem, s>>>(ta, tb, P);
+    return true;
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------- exact lists
+// The FP32 kernel spends two instructions per pair and dim and a long chain
+// per CTA, the screen one tensor-core product and about twelve short launches.
+// Measured (GB300): n = 500, D = 128, 15 rows 195 us against 95; n = 20,000,
+// D = 64, 7 rows 456 against 143; n = 1 M, D = 128, 1 row 5.7 ms against
+// 0.55, 2,000 rows 189 ms against 1.33 (0.94 of it the products).  Below one
+// column tile there is nothing to screen.
+bool exact_screened(int64_t n) { return n >= kScN; }
+
+int64_t exact_batch(int64_t s_rows) { return std::min<int64_t>(s_rows, 8192); }
+
+bool launch_exact_screened(const float* X, int64_t n, int D, int k, const int32_t* sample, int64_t s_rows,
+                           const ScreenWork& w, uint64_t* out, int* status, cudaStream_t s) {
+    const int Dp = lp_dim(D);
+    const bool vec = D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    cudaMemsetAsync(w.flags, 0, 2 * sizeof(int), s);
+    launch_screen_copy(X, n, D, nullptr, nullptr, 0, w.Xq, w.nrm, w.err, w.flags, status, s);
+    // column sets: every st0-th row (at most kScreenCap of them, all kept),
+    // then 4 times as many each time, up to every row.  A set's k-th least
+    // upper bound bounds the row's k-th distance, so about 4 k columns of the
+    // next one stay below it.
+    constexpr int64_t kGrow = 4;
+    int64_t st0 = 1;
+    while ((n + st0 - 1) / st0 > kScreenCap) st0 *= kGrow;
+    const int64_t batch = exact_batch(s_rows);
+    const int nsplit = exact_splits(n, batch);
+    const size_t rank_smem = (size_t)kScreenCap * 12 + ((size_t)D + 3) / 4 * 16;
+    cudaFuncSetAttribute(k7_rank<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rank_smem);
+    for (int64_t q0 = 0; q0 < s_rows; q0 += batch) {
+        const int64_t rows = std::min(batch, s_rows - q0);
+        ScreenArgs P{};
+        const uint16_t* A;
+        if (sample) {
+            LaunchScope ls("ks_gather", s, (double)rows * (Dp * 4.0 + 16.0), 0);
+            const int64_t pieces = rows * (Dp / 8);
+            ks_gather<<<(unsigned)std::min<int64_t>((pieces + 255) / 256, kScGrid * 16), 256, 0, s>>>(
+                reinterpret_cast<const uint4*>(w.Xq), w.nrm, w.err, rows, Dp / 8, sample + q0,
+                reinterpret_cast<uint4*>(w.Qq), w.qn, w.qe, status);
+            A = w.Qq;
+            P.rnrm = w.qn;
+            P.rerr = w.qe;
+            P.rid = sample + q0;
+        } else {
+            A = w.Xq + q0 * Dp;
+            P.rnrm = w.nrm + q0;
+            P.rerr = w.err + q0;
+            P.rid0 = q0;
+        }
+        P.nrows = rows;
+        P.cnrm = w.nrm;
+        P.cerr = w.err;
+        P.cD2 = screen_c(D);
+        P.gamma = (float)(D + 8) * 1.1920928955078125e-7f;
+        P.flag_r = P.flag_c = w.flags;
+        P.status = status;
+        P.cap = kScreenCap;
+        P.cg = w.cg;
+        P.cid = w.cid;
+        P.cnt = w.cnt;
+        P.rowA = w.rowA;
+        P.rowR = w.rowR;
+        P.X = X;
+        P.D = D;
+        P.vec = vec;
+        cudaMemsetAsync(w.fb_flag, 0, sizeof(int32_t) * rows, s);
+        cudaMemsetAsync(w.flags + 1, 0, sizeof(int), s);
+        for (int64_t st = st0;; st /= kGrow) {
+            P.cstride = st;
+            P.ncols = (n + st - 1) / st;
+            const bool dump = st == st0, last = st == 1;
+            if (dump) {
+                if (!launch_screen<kScDump>(A, w.Xq, Dp, P, "ks_screen", s)) return false;
+            } else {
+                cudaMemsetAsync(w.cnt, 0, sizeof(int32_t) * rows, s);
+                if (!launch_screen<kScCollect>(A, w.Xq, Dp, P, "ks_screen", s)) return false;
+            }
+            LaunchScope ls("k7_rank", s, 0, 0);
+            if (last) {
+                k7_rank<true><<<(unsigned)rows, kRrThreads, rank_smem, s>>>(P, dump, k, w.rowA, w.rowR, w.fb_flag,
+                                                                            w.fb_list, w.flags + 1, out + q0 * k);
+                break;
+            }
+            k7_rank<false><<<(unsigned)rows, kRrThreads, kScreenCap * 4, s>>>(P, dump, k, w.rowA, w.rowR, w.fb_flag,
+                                                                              w.fb_list, w.flags + 1, nullptr);
+        }
+        launch_exact(X, n, D, k, sample ? sample + q0 : nullptr, q0, rows, w.fb_list, w.flags + 1, nsplit, w.part,
+                     out + q0 * k, status, s);
+    }
+    return true;
+}
+
+}  // namespace knng
