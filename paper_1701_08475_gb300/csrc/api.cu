@@ -1199,25 +1199,48 @@ void validate_vocab(int W1, int W2, int D) {
     if (W1 < 1 || W1 > 256 || W2 < 1 || W2 > 256) fail(KNNG_EINVAL, "W1 = %d, W2 = %d outside [1, 256]", W1, W2);
 }
 
-// One stage of Lloyd's k-means on the device (Sec. 4.1): the vectors are the
-// points, or their residues against W1 (codes c1) when W1 is given.
-void rvq_lloyd(const float* X, int64_t N, int D, const float* W1, const int32_t* c1, int W, int iters,
-               uint64_t seed, int stage, float* words, int32_t* codes, int32_t* order, int32_t* hist, int32_t* gofs,
-               int32_t* scan_tmp, int64_t* dpos, std::vector<int64_t>& hpos, cudaStream_t s) {
+// One stage of Lloyd's k-means on the device (Sec. 4.1) over the N vectors V.
+// w (with aw->Xq set): the assignments are screened from its copy of V.
+struct RvqBuffers {
+    int32_t *codes, *order, *hist, *gofs, *scan_tmp;
+    int64_t* pos;
+    double* part;
+};
+void rvq_nearest(const float* V, int64_t N, int D, const float* W1, const int32_t* c1, int c1_stride,
+                 const float* words, int W, const AssignWork& aw, int32_t* out, int out_stride, int* status,
+                 cudaStream_t s) {
+    if (!aw.Xq ||
+        !launch_assign_screened(V, N, D, W1, c1, c1_stride, words, W, aw, out, out_stride, status, s))
+        launch_rvq_assign(V, N, D, W1, c1, c1_stride, words, W, out, out_stride, s);
+}
+void rvq_lloyd(const float* V, int64_t N, int D, int W, int iters, uint64_t seed, int stage, float* words,
+               const RvqBuffers& b, const AssignWork& aw, int* status, std::vector<int64_t>& hpos, cudaStream_t s) {
     const uint64_t h0 = splitmix64(seed ^ ((uint64_t)stage << 32));
     hpos.assign(W, 0);
     for (int c = 0; c < W; ++c) {
         const int64_t lo = (int64_t)c * N / W, hi = (int64_t)(c + 1) * N / W;
         hpos[c] = lo + (int64_t)(splitmix64(h0 ^ (uint64_t)c) % (uint64_t)(hi - lo));
     }
-    cuda_check(cudaMemcpyAsync(dpos, hpos.data(), sizeof(int64_t) * W, cudaMemcpyHostToDevice, s), "positions");
-    launch_rvq_init(X, D, W1, c1, 1, dpos, W, words, s);
+    cuda_check(cudaMemcpyAsync(b.pos, hpos.data(), sizeof(int64_t) * W, cudaMemcpyHostToDevice, s), "positions");
+    launch_rvq_init(V, D, b.pos, W, words, s);
     const int nb = digit_sort_blocks(N);
     for (int it = 0; it < iters; ++it) {
-        launch_rvq_assign(X, N, D, W1, c1, 1, words, W, codes, 1, s);
-        launch_digit_sort(nullptr, N, codes, 1, order, hist, gofs, scan_tmp, s);
-        launch_rvq_update(X, N, D, W1, c1, 1, order, gofs, nb, W, words, s);
+        rvq_nearest(V, N, D, nullptr, nullptr, 1, words, W, aw, b.codes, 1, status, s);
+        launch_digit_sort(nullptr, N, b.codes, 1, b.order, b.hist, b.gofs, b.scan_tmp, s);
+        launch_rvq_update(V, N, D, b.order, b.gofs, nb, W, b.part, words, s);
     }
+}
+// The screen's copies of N vectors and up to 256 words.
+void carve_assign(Workspace& ws, AssignWork& aw, int64_t N, int D) {
+    const size_t Dp = (size_t)lp_dim(D);
+    aw.Xq = ws.take<uint16_t>((size_t)N * Dp);
+    aw.nrm = ws.take<float>(N);
+    aw.err = ws.take<float>(N);
+    aw.Wq = ws.take<uint16_t>(256 * Dp);
+    aw.wnrm = ws.take<float>(256);
+    aw.werr = ws.take<float>(256);
+    aw.mask = ws.take<uint32_t>((size_t)N * 8);
+    aw.flags = ws.take<int>(2);
 }
 }  // namespace
 
@@ -1694,35 +1717,49 @@ int knng_rvq_train(const float* data, int64_t n, int D, int W1, int W2, int iter
         const size_t nh = digit_sort_hist_ints(n);
         Workspace ws;
         DevBuf<float> X, o1, o2;
-        int32_t *codes = nullptr, *c1 = nullptr, *order = nullptr, *hist = nullptr, *gofs = nullptr, *tmp = nullptr;
-        int64_t* pos = nullptr;
+        RvqBuffers b{};
+        AssignWork aw{};
+        int32_t* c1 = nullptr;
         float* R = nullptr;
         int* status = nullptr;
+        bool screen = true;  // with the updates' pieces; unless they do not fit
         for (int ps = 0; ps < 2; ++ps) {
             ws.used = 0;
             bind(ws, X, data, (size_t)n * D, ps);
             R = ws.take<float>((size_t)n * D);
             bind(ws, o1, (const float*)words1, (size_t)W1 * D, ps);
             bind(ws, o2, (const float*)words2, (size_t)W2 * D, ps);
-            codes = ws.take<int32_t>(n);
+            b.codes = ws.take<int32_t>(n);
             c1 = ws.take<int32_t>(n);
-            order = ws.take<int32_t>(n);
-            hist = ws.take<int32_t>(nh);
-            gofs = ws.take<int32_t>(nh + 1);
-            tmp = ws.take<int32_t>(scan_tmp_ints((int64_t)nh));
-            pos = ws.take<int64_t>(256);
+            b.order = ws.take<int32_t>(n);
+            b.hist = ws.take<int32_t>(nh);
+            b.gofs = ws.take<int32_t>(nh + 1);
+            b.scan_tmp = ws.take<int32_t>(scan_tmp_ints((int64_t)nh));
+            b.pos = ws.take<int64_t>(256);
             status = ws.take<int>(4);
-            if (ps == 0) ws.allocate(st);
+            aw = AssignWork{};
+            b.part = nullptr;
+            if (screen) {
+                carve_assign(ws, aw, n, D);
+                b.part = ws.take<double>(rvq_update_doubles(n, D));
+            }
+            if (ps == 0 && !ws.try_allocate(st, screen)) {
+                screen = false;
+                ps = -1;
+            }
         }
         cuda_check(cudaMemsetAsync(status, 0, 4 * sizeof(int), st), "status clear");
         upload(X, st);
-        launch_check_finite(X.dev, n * (int64_t)D, status, st);
-        std::vector<int64_t> hpos;
-        rvq_lloyd(X.dev, n, D, nullptr, nullptr, W1, iters, seed, 1, o1.dev, codes, order, hist, gofs, tmp, pos, hpos,
-                  st);
-        launch_rvq_assign(X.dev, n, D, nullptr, nullptr, 1, o1.dev, W1, c1, 1, st);
+        if (screen)
+            launch_screen_copy(X.dev, n, D, nullptr, nullptr, 0, aw, status, st);
+        else
+            launch_check_finite(X.dev, n * (int64_t)D, status, st);
+        std::vector<int64_t> hpos1, hpos2;
+        rvq_lloyd(X.dev, n, D, W1, iters, seed, 1, o1.dev, b, aw, status, hpos1, st);
+        rvq_nearest(X.dev, n, D, nullptr, nullptr, 1, o1.dev, W1, aw, c1, 1, status, st);
         launch_rvq_residues(X.dev, n, D, o1.dev, c1, R, st);   // stage 2 trains on the residues
-        rvq_lloyd(R, n, D, nullptr, nullptr, W2, iters, seed, 2, o2.dev, codes, order, hist, gofs, tmp, pos, hpos, st);
+        if (screen) launch_screen_copy(R, n, D, nullptr, nullptr, 0, aw, nullptr, st);
+        rvq_lloyd(R, n, D, W2, iters, seed, 2, o2.dev, b, aw, status, hpos2, st);
         download(o1, st);
         download(o2, st);
         cuda_check(launch_error(), "kernel launch");
@@ -1744,6 +1781,8 @@ int knng_rvq_index(const float* data, int64_t n, int D, const float* words1, int
         DevBuf<int32_t> cd, off, li;
         int32_t *order = nullptr, *hist = nullptr, *gofs = nullptr, *tmp = nullptr, *cnt = nullptr;
         int* status = nullptr;
+        AssignWork aw{};
+        bool screen = true;  // unless its copy does not fit
         for (int ps = 0; ps < 2; ++ps) {
             ws.used = 0;
             bind(ws, X, data, (size_t)n * D, ps);
@@ -1758,17 +1797,26 @@ int knng_rvq_index(const float* data, int64_t n, int D, const float* words1, int
             tmp = ws.take<int32_t>(std::max(scan_tmp_ints((int64_t)nh), scan_tmp_ints(nk)));
             cnt = ws.take<int32_t>(nk);
             status = ws.take<int>(4);
-            if (ps == 0) ws.allocate(st);
+            aw = AssignWork{};
+            if (screen) carve_assign(ws, aw, n, D);
+            if (ps == 0 && !ws.try_allocate(st, screen)) {
+                screen = false;
+                ps = -1;
+            }
         }
         cuda_check(cudaMemsetAsync(status, 0, 4 * sizeof(int), st), "status clear");
         upload(X, st);
         upload(w1, st);
         upload(w2, st);
-        launch_check_finite(X.dev, n * (int64_t)D, status, st);
         launch_check_finite(w1.dev, (int64_t)W1 * D, status, st);
         launch_check_finite(w2.dev, (int64_t)W2 * D, status, st);
-        launch_rvq_assign(X.dev, n, D, nullptr, nullptr, 2, w1.dev, W1, cd.dev, 2, st);
-        launch_rvq_assign(X.dev, n, D, w1.dev, cd.dev, 2, w2.dev, W2, cd.dev + 1, 2, st);
+        if (screen)
+            launch_screen_copy(X.dev, n, D, nullptr, nullptr, 2, aw, status, st);
+        else
+            launch_check_finite(X.dev, n * (int64_t)D, status, st);
+        rvq_nearest(X.dev, n, D, nullptr, nullptr, 2, w1.dev, W1, aw, cd.dev, 2, status, st);
+        if (screen) launch_screen_copy(X.dev, n, D, w1.dev, cd.dev, 2, aw, nullptr, st);
+        rvq_nearest(X.dev, n, D, w1.dev, cd.dev, 2, w2.dev, W2, aw, cd.dev + 1, 2, status, st);
         launch_digit_sort(nullptr, n, cd.dev + 1, 2, order, hist, gofs, tmp, st);   // by c2
         launch_digit_sort(order, n, cd.dev, 2, li.dev, hist, gofs, tmp, st);        // then by c1, stable
         cuda_check(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * nk, st), "count clear");

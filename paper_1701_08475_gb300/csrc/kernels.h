@@ -291,11 +291,12 @@ size_t digit_sort_hist_ints(int64_t n);
 void launch_digit_sort(const int32_t* in, int64_t n, const int32_t* key, int kstride, int32_t* out, int32_t* hist,
                        int32_t* gofs, int32_t* scan_tmp, cudaStream_t s);
 // words[c] = FP64 mean (ascending vector order) of the vectors of word c, in
-// FP32; words without members keep their value.
-void launch_rvq_update(const float* X, int64_t N, int D, const float* W1, const int32_t* c1, int c1_stride,
-                       const int32_t* order, const int32_t* gofs, int nb, int W, float* words, cudaStream_t s);
-void launch_rvq_init(const float* X, int D, const float* W1, const int32_t* c1, int c1_stride, const int64_t* pos,
-                     int W, float* words, cudaStream_t s);
+// FP32; words without members keep their value.  part:
+// rvq_update_doubles(N, D) doubles (NULL: slower, the same words).
+size_t rvq_update_doubles(int64_t N, int D);
+void launch_rvq_update(const float* X, int64_t N, int D, const int32_t* order, const int32_t* gofs, int nb, int W,
+                       double* part, float* words, cudaStream_t s);
+void launch_rvq_init(const float* X, int D, const int64_t* pos, int W, float* words, cudaStream_t s);
 // R = X - W1[c1] row by row (FP32): the stage-2 training vectors.
 void launch_rvq_residues(const float* X, int64_t N, int D, const float* W1, const int32_t* c1, float* R,
                          cudaStream_t s);
@@ -341,6 +342,24 @@ struct ScreenWork {
     int32_t *fb_list, *fb_flag;  // [batch]
     uint64_t* part;         // [batch][exact_splits][k]
 };
+// Nearest words by screening: the vectors' copy (launch_screen_copy, once per
+// set of vectors: rows of X, minus W1[c1] when given; checks for non-finite
+// values when status is given) and room for the words' copy.
+struct AssignWork {
+    uint16_t* Xq;      // [N][lp_dim(D)]
+    float *nrm, *err;  // [N]
+    uint16_t* Wq;      // [256][lp_dim(D)]
+    float *wnrm, *werr;
+    uint32_t* mask;    // [N][8] candidate words
+    int* flags;        // [2]
+};
+void launch_screen_copy(const float* X, int64_t N, int D, const float* W1, const int32_t* c1, int c1_stride,
+                        const AssignWork& w, int* status, cudaStream_t s);
+// launch_rvq_assign from the copies, the same codes; false when the tensor
+// maps cannot be made (nothing launched that matters).
+bool launch_assign_screened(const float* X, int64_t N, int D, const float* W1, const int32_t* c1, int c1_stride,
+                            const float* words, int W, const AssignWork& w, int32_t* out, int out_stride, int* status,
+                            cudaStream_t s);
 constexpr int kScreenCap = 4096;
 bool exact_screened(int64_t n);
 int64_t exact_batch(int64_t s_rows);

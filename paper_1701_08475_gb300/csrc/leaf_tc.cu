@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) k0_quantize(const float* __restrict__ X, 
         // the exact sum (Higham, Ch. 3), the square root rounds up
         qerr[p] = e2 > 0.f ? __fsqrt_ru(__fmul_ru(e2, 1.f + (float)(Dp + 8) * 5.9604645e-8f)) : 0.f;
         const int f = ((!exact || sq >= 8388608.f) ? 1 : 0) | (neg ? 2 : 0) | (sq >= 4194304.f ? 4 : 0);
-        if (f) atomicOr(notexact, f);
+        if (f & ~*(volatile int*)notexact) atomicOr(notexact, f);  // once set, a flag is only read
     }
 }
 

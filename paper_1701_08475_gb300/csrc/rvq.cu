@@ -215,52 +215,200 @@ __global__ void __launch_bounds__(kDsThreads) k9_digit_scatter(const int32_t* __
 }
 
 // ---------------------------------------------------------------- word update
-// One warp per (word, 32 dims): the FP64 sum of the members in ascending
-// vector order (the sorted run order[gofs[c * nb] .. gofs[(c + 1) * nb])),
-// divided by the count, rounded to FP32.  Loads run eight members ahead of
-// the additions; the additions keep their order.
-template <bool RES>
-__global__ void __launch_bounds__(128) k9_update(const float* __restrict__ X, int D, const float* __restrict__ W1,
-                                                const int32_t* __restrict__ c1, int c1_stride,
+// A word's mean is defined by the FP64 sum of its members in ascending vector
+// order.  Taken literally that is one chain of dependent additions per word
+// and dim, as long as the largest word.  But FP32 values that are all
+// multiples of a quantum q, with sums below 2^53 q, add without any rounding
+// in FP64, in any order; nearly every (word, dim) is such a case.  So the
+// members are summed in pieces (kUpRows consecutive positions of the sorted
+// order per warp, cut where the word changes), then the pieces of a word, with
+// the least and greatest magnitude on the way.  Where those do not prove the
+// sum exact, an error bound of both orders decides whether the rounded mean
+// can differ, and if it could, the word's chain runs as defined.
+constexpr int kUpRows = 32;
+constexpr int kUpDims = 128;  // dims per warp: 4 per lane
+
+// Piece slots: unit u (positions kUpRows u ..) and word c meet in slot u + c
+// (along the sorted order either the unit or the word moves on).  A slot holds
+// D sums, then D pairs: the exponent of the lowest last set bit (2^(lo - 150))
+// and A = sum |x| (rounded up).
+constexpr int kUpNone = 1 << 20;  // no nonzero value
+// e with 0 <= x < 2^e
+__device__ __forceinline__ int up_exp(float x) { return max((int)(__float_as_uint(x) >> 23), 1) - 126; }
+__device__ __forceinline__ double* up_slot(double* part, int64_t slot, int D) { return part + slot * 2 * D; }
+
+template <bool VEC>
+__global__ void __launch_bounds__(128) k9_pieces(const float* __restrict__ X, int64_t N, int D,
                                                 const int32_t* __restrict__ order, const int32_t* __restrict__ gofs,
-                                                int nb, int W, float* __restrict__ words) {
-    const int nch = (D + 31) / 32;
-    const int gw = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (gw >= W * nch) return;
-    const int c = gw / nch, j = (gw - c * nch) * 32 + lane;
-    const int a = __ldg(gofs + (int64_t)c * nb), b = __ldg(gofs + (int64_t)(c + 1) * nb);
-    if (b == a || j >= D) return;  // no members: the word keeps its value
-    auto value = [&](int t) {
-        const int32_t id = __ldg(order + t);
-        float v = __ldg(X + (int64_t)id * D + j);
-        if (RES) v = __fsub_rn(v, __ldg(W1 + (int64_t)__ldg(c1 + (int64_t)id * c1_stride) * D + j));
-        return v;
-    };
-    double acc = 0.0;
-    int t = a;
-    for (; t + 8 <= b; t += 8) {
-        float v[8];
+                                                int nb, int W, double* __restrict__ part) {
+    __shared__ int start[257];  // where each word's positions start
+    for (int c = threadIdx.x; c <= W; c += blockDim.x) start[c] = c < W ? gofs[(int64_t)c * nb] : (int)N;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, d0 = blockIdx.y * kUpDims;
+    const int64_t u = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int64_t p0 = u * kUpRows;
+    if (p0 >= N) return;
+    const int p1 = (int)min(N, p0 + kUpRows);
+    const int my_id = p0 + lane < p1 ? order[p0 + lane] : 0;
+    int c = 0;  // the last word that starts at or before p0 and is not empty there
+    for (int step = 128; step > 0; step >>= 1)
+        if (c + step < W && start[c + step] <= (int)p0) c += step;
+    for (int p = (int)p0; p < p1;) {
+        while (start[c + 1] <= p) ++c;
+        const int end = min(p1, start[c + 1]);
+        // FP32 sums h with the additions' rounding errors summed in l (Knuth's
+        // TwoSum): FP64 issues at a small fraction of the FP32 rate.  With
+        // A = sum |x| < 2^ea, each error is at most 2^(ea - 25) and l below
+        // 2^(ea - 20), exact up to 2^24 quanta of 2^(lo - 150).
+        float h[4], l[4], A[4];
+        int lo[4];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = value(t + u);
+        for (int j = 0; j < 4; ++j) {
+            h[j] = l[j] = A[j] = 0.f;
+            lo[j] = kUpNone;
+        }
+        auto load = [&](int id, bool in, float (&v)[4]) {
+            const float* x = X + (int64_t)id * D + d0;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) acc = __dadd_rn(acc, (double)v[u]);
+            for (int j = 0; j < 4; ++j) v[j] = 0.f;
+            if (!in) return;
+            if (VEC) {
+                if (d0 + 4 * lane < D) {
+                    const float4 f = __ldg(reinterpret_cast<const float4*>(x) + lane);
+                    v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (d0 + 4 * lane + j < D) v[j] = __ldg(x + 4 * lane + j);
+            }
+        };
+        for (int t = p; t < end; t += 8) {  // 8 rows in flight; rows past the end add +0
+            float v[8][4];
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                load(__shfl_sync(0xffffffffu, my_id, (t + q - (int)p0) & 31), t + q < end, v[q]);
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float x = v[q][j], sm = __fadd_rn(h[j], x), bp = __fsub_rn(sm, h[j]);
+                    l[j] = __fadd_rn(l[j], __fadd_rn(__fsub_rn(h[j], __fsub_rn(sm, bp)), __fsub_rn(x, bp)));
+                    h[j] = sm;
+                    const uint32_t m = __float_as_uint(x) & 0x7fffffffu;
+                    const uint32_t man = (m & 0x7fffffu) | (m >= 0x800000u ? 0x800000u : 0u);
+                    // exponent field (1 for subnormals) plus the zeros below
+                    // the last set bit
+                    const int last = max((int)(m >> 23), 1) + 31 - __clz((int)(man & (0u - man)));
+                    lo[j] = min(lo[j], m ? last : kUpNone);
+                    A[j] = __fadd_ru(A[j], fabsf(x));
+                }
+        }
+        double acc[4];
+        bool wide = false;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            acc[j] = __dadd_rn((double)h[j], (double)l[j]);
+            // (and no overflow of h: FP64 holds what FP32 does not)
+            wide |= up_exp(A[j]) - (lo[j] - 150) > 44 || !(A[j] < 1e38f);
+        }
+        if (__any_sync(0xffffffffu, wide)) {  // magnitudes too far apart: FP64 throughout
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[j] = 0.0;
+            for (int t = p; t < end; ++t) {
+                float v[4];
+                load(__shfl_sync(0xffffffffu, my_id, (t - (int)p0) & 31), true, v);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) acc[j] = __dadd_rn(acc[j], (double)v[j]);
+            }
+        }
+        p = end;
+        double* o = up_slot(part, u + c, D);
+        uint2* mags = reinterpret_cast<uint2*>(o + D);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int d = d0 + 4 * lane + j;
+            if (d < D) {
+                o[d] = acc[j];
+                mags[d] = make_uint2((uint32_t)lo[j], __float_as_uint(A[j]));
+            }
+        }
     }
-    for (; t < b; ++t) acc = __dadd_rn(acc, (double)value(t));
-    words[(int64_t)c * D + j] = __double2float_rn(__ddiv_rn(acc, (double)(b - a)));
+}
+
+// One CTA per word and 128 dims: the sum of its pieces, the proof that the
+// rounded mean is the defined one, and else the chain.
+constexpr int kCbGroups = 4;  // the pieces of a word are read by this many threads per dim
+__global__ void __launch_bounds__(128 * kCbGroups) k9_combine(const float* __restrict__ X, int64_t N, int D,
+                                                 const int32_t* __restrict__ order,
+                                                 const int32_t* __restrict__ gofs, int nb, int W,
+                                                 double* __restrict__ part, float* __restrict__ words) {
+    __shared__ double gsum[kCbGroups][128];
+    __shared__ float gabs[kCbGroups][128];
+    __shared__ int glo[kCbGroups][128];
+    const int dd = threadIdx.x & 127, g = threadIdx.x >> 7;
+    const int c = blockIdx.x, d = blockIdx.y * 128 + dd;
+    const int a = gofs[(int64_t)c * nb], b = c + 1 < W ? gofs[(int64_t)(c + 1) * nb] : (int)N;
+    if (b == a) return;  // no members: the word keeps its value
+    double sum = 0.0;
+    const int m = b - a;
+    auto chain = [&] {  // the defined order, the loads of 32 members ahead of their additions
+        double s = 0.0;
+        for (int t = a; t < b; t += 32) {
+            float v[32];
+#pragma unroll
+            for (int q = 0; q < 32; ++q) v[q] = t + q < b ? __ldg(X + (int64_t)order[t + q] * D + d) : 0.f;
+#pragma unroll
+            for (int q = 0; q < 32; ++q)
+                if (t + q < b) s = __dadd_rn(s, (double)v[q]);
+        }
+        return s;
+    };
+    if (part == nullptr) {  // no room for pieces
+        if (g == 0 && d < D) words[(int64_t)c * D + d] = __double2float_rn(__ddiv_rn(chain(), (double)m));
+        return;
+    }
+    int lo = kUpNone;
+    float A = 0.f;
+    if (d < D) {
+#pragma unroll 4
+        for (int64_t u = a / kUpRows + g; u <= (b - 1) / kUpRows; u += kCbGroups) {
+            const double* o = up_slot(part, u + c, D);
+            const uint2 mg = reinterpret_cast<const uint2*>(o + D)[d];
+            sum = __dadd_rn(sum, o[d]);
+            lo = min(lo, (int)mg.x);
+            A = __fadd_ru(A, __uint_as_float(mg.y));
+        }
+    }
+    gsum[g][dd] = sum;
+    gabs[g][dd] = A;
+    glo[g][dd] = lo;
+    __syncthreads();
+    if (g > 0 || d >= D) return;
+#pragma unroll
+    for (int q = 1; q < kCbGroups; ++q) {
+        sum = __dadd_rn(sum, gsum[q][dd]);
+        A = __fadd_ru(A, gabs[q][dd]);
+        lo = min(lo, glo[q][dd]);
+    }
+    // every value is a multiple of 2^(lo - 150) and no partial sum is above A
+    if (up_exp(A) > 53 + lo - 150) {
+        // either order is within (m - 1) 2^-53 A, and a little, of the true sum
+        const double e = ldexp((double)m * (double)A, -51);
+        const float x = __double2float_rn(__ddiv_rn(sum - e, (double)m));
+        const float y = __double2float_rn(__ddiv_rn(sum + e, (double)m));
+        if (x != y || x == 0.f) sum = chain();
+    }
+    words[(int64_t)c * D + d] = __double2float_rn(__ddiv_rn(sum, (double)m));
 }
 
 // words[c] = v_{pos[c]} (the initial words).
-template <bool RES>
-__global__ void k9_init_words(const float* __restrict__ X, int D, const float* __restrict__ W1,
-                              const int32_t* __restrict__ c1, int c1_stride, const int64_t* __restrict__ pos, int W,
+__global__ void k9_init_words(const float* __restrict__ X, int D, const int64_t* __restrict__ pos, int W,
                               float* __restrict__ words) {
     const int64_t total = (int64_t)W * D;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int c = (int)(e / D), j = (int)(e - (int64_t)c * D);
-        const int64_t id = pos[c];
-        float v = X[id * D + j];
-        if (RES) v = __fsub_rn(v, W1[(int64_t)c1[id * c1_stride] * D + j]);
-        words[e] = v;
+        words[e] = X[pos[c] * D + j];
     }
 }
 
@@ -503,24 +651,23 @@ void launch_digit_sort(const int32_t* in, int64_t n, const int32_t* key, int kst
     k9_digit_scatter<<<nb, kDsThreads, 0, s>>>(in, n, key, kstride, gofs, nb, out);
 }
 
-void launch_rvq_update(const float* X, int64_t N, int D, const float* W1, const int32_t* c1, int c1_stride,
-                       const int32_t* order, const int32_t* gofs, int nb, int W, float* words, cudaStream_t s) {
-    const int warps = W * ((D + 31) / 32);
-    LaunchScope ls(W1 ? "k9_update_res" : "k9_update", s, (double)N * D * (W1 ? 8.0 : 4.0) + N * 4.0, (double)N * D);
-    if (W1)
-        k9_update<true><<<(warps + 3) / 4, 128, 0, s>>>(X, D, W1, c1, c1_stride, order, gofs, nb, W, words);
-    else
-        k9_update<false><<<(warps + 3) / 4, 128, 0, s>>>(X, D, nullptr, nullptr, 0, order, gofs, nb, W, words);
+size_t rvq_update_doubles(int64_t N, int D) { return (size_t)((N + kUpRows - 1) / kUpRows + 256) * 2 * D; }
+
+void launch_rvq_update(const float* X, int64_t N, int D, const int32_t* order, const int32_t* gofs, int nb, int W,
+                       double* part, float* words, cudaStream_t s) {
+    LaunchScope ls("k9_update", s, (double)N * D * 4.0 + N * 4.0, (double)N * D, 2);
+    const int64_t units = (N + kUpRows - 1) / kUpRows;
+    const dim3 grid((unsigned)((units + 3) / 4), (unsigned)((D + kUpDims - 1) / kUpDims));
+    const bool vec = D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    if (part && vec) k9_pieces<true><<<grid, 128, 0, s>>>(X, N, D, order, gofs, nb, W, part);
+    if (part && !vec) k9_pieces<false><<<grid, 128, 0, s>>>(X, N, D, order, gofs, nb, W, part);
+    k9_combine<<<dim3((unsigned)W, (unsigned)((D + 127) / 128)), 128 * kCbGroups, 0, s>>>(X, N, D, order, gofs, nb, W, part,
+                                                                             words);
 }
 
-void launch_rvq_init(const float* X, int D, const float* W1, const int32_t* c1, int c1_stride, const int64_t* pos,
-                     int W, float* words, cudaStream_t s) {
+void launch_rvq_init(const float* X, int D, const int64_t* pos, int W, float* words, cudaStream_t s) {
     LaunchScope ls("k9_init_words", s, (double)W * D * 8.0, 0);
-    const int grid = grid_for_count((int64_t)W * D);
-    if (W1)
-        k9_init_words<true><<<grid, 256, 0, s>>>(X, D, W1, c1, c1_stride, pos, W, words);
-    else
-        k9_init_words<false><<<grid, 256, 0, s>>>(X, D, nullptr, nullptr, 0, pos, W, words);
+    k9_init_words<<<grid_for_count((int64_t)W * D), 256, 0, s>>>(X, D, pos, W, words);
 }
 
 void launch_rvq_residues(const float* X, int64_t N, int D, const float* W1, const int32_t* c1, float* R,

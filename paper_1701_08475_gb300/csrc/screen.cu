@@ -44,7 +44,6 @@ constexpr int kScPart = kScN / 4;  // columns per epilogue warp
 constexpr int kScThreads = 64 + kScEpi;  // + a TMA warp and an MMA warp
 constexpr int kScGrid = 152;       // one CTA per SM (512 tensor-memory columns, over half of shared memory)
 constexpr int kScCand = 2048;      // candidates buffered in shared memory (collect)
-constexpr int kScList = 8192;      // (row, word) pairs of one tile (nearest word)
 constexpr float kScTiny = 1e-17f;  // added to e: squares below FP32's range summed as zero
 
 enum ScreenMode { kScDump = 0, kScCollect = 1, kScArgmin = 2 };
@@ -73,16 +72,11 @@ struct ScreenArgs {
     int32_t* cnt;          // [nrows]
     const float* rowA;     // [nrows] a_i
     const float* rowR;     // [nrows] R_i
-    // nearest word: vectors X (minus W1[c1]), words
+    uint32_t* mask;        // nearest word: [nrows][8] the candidate words of each row
+    // re-rank
     const float* X;
-    const float* W1;
-    const int32_t* c1;
-    int c1_stride;
-    const float* words;
     int D;
     bool vec;
-    int32_t* out;
-    int out_stride;
 };
 
 // The flag bits of the copy (k0_quantize's) plus 8: some squared norm is too
@@ -120,8 +114,8 @@ __host__ __device__ inline ScreenSmem screen_smem(int nk, int mode) {
     L.a_off = (size_t)kScStages * L.stage_bytes;
     L.col_off = L.a_off + (res ? (size_t)nk * kScABytes : 0);
     L.list_off = L.col_off + (mode == kScCollect ? kScEpi / 32 * kScPart : 2 * kScN) * 8;
-    L.row_off = L.list_off + (mode == kScCollect ? kScCand * 12 : mode == kScArgmin ? kScList * 2 : 0);
-    L.bar_off = L.row_off + (mode == kScArgmin ? kScM * (8 + 4 * 8 + 4 + 4) : 0);
+    L.row_off = L.list_off + (mode == kScCollect ? kScCand * 12 : 0);
+    L.bar_off = L.row_off + (mode == kScArgmin ? 2 * 4 * kScM * 4 : 0);
     L.total = L.bar_off + (2 * kScStages + 6) * 8 + 32;
     return L;
 }
@@ -178,6 +172,21 @@ __device__ __forceinline__ float2 screen_pair(float g0, float g1, float c0, floa
         "}\n"
         : "=f"(r.x), "=f"(r.y)
         : "f"(g0), "f"(g1), "f"(c0), "f"(c1), "f"(e0), "f"(e1), "f"(-2.f), "f"(a2));
+    return r;
+}
+// c_j - 2 g_j of two columns.
+__device__ __forceinline__ float2 fma_pair(float g0, float g1, float c0, float c1) {
+    float2 r;
+    asm("{\n"
+        ".reg .b64 g, c, m;\n"
+        "mov.b64 g, {%2, %3};\n"
+        "mov.b64 c, {%4, %5};\n"
+        "mov.b64 m, {%6, %6};\n"
+        "fma.rn.f32x2 c, m, g, c;\n"
+        "mov.b64 {%0, %1}, c;\n"
+        "}\n"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(g0), "f"(g1), "f"(c0), "f"(c1), "f"(-2.f));
     return r;
 }
 __device__ __forceinline__ float min_pair(float2 p, float m) {
@@ -323,13 +332,11 @@ __global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant
         int32_t* brow = reinterpret_cast<int32_t*>(base + L.list_off);
         int32_t* bid = brow + kScCand;
         float* bg = reinterpret_cast<float*>(bid + kScCand);
-        // nearest word
-        uint16_t* list = reinterpret_cast<uint16_t*>(base + L.list_off);
-        uint64_t* best = reinterpret_cast<uint64_t*>(base + L.row_off);  // [kScM]
-        float2* hmin = reinterpret_cast<float2*>(best + kScM);           // [4][kScM] (value, g)
-        int* rcount = reinterpret_cast<int*>(hmin + 4 * kScM);           // [kScM] candidates
-        int* rfull = rcount + kScM;                                      // [kScM] every word is one
-        int* nfull = ncand + 1;                                          // rows with rfull set
+        // nearest word: the words' c_j, then e_j (one column tile, loaded
+        // once), the greatest N_j and e_j, and each part's least value of a row
+        float* colf = reinterpret_cast<float*>(colc);
+        uint32_t* cmax = reinterpret_cast<uint32_t*>(ncand);
+        float* hmin = reinterpret_cast<float*>(base + L.row_off);  // [2][4][kScM]
         int t = 0;
         auto col_const = [&](int64_t col) -> float2 {
             if (col >= P.ncols) return make_float2(__int_as_float(0x7f800000), 0.f);
@@ -376,6 +383,18 @@ __global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant
             epi_sync();
         };
         if (blockIdx.x < (unsigned)units && MODE == kScCollect) load_cols(blockIdx.x / P.nrt);
+        if (MODE == kScArgmin) {
+            if (et < kScN) {
+                const float2 c = col_const(et);
+                colf[et] = c.x;
+                colf[kScN + et] = c.y;
+                if (et < P.ncols) {  // both at least 0: their bits have their order
+                    atomicMax(cmax, __float_as_uint(__ldg(P.cnrm + et)));
+                    atomicMax(cmax + 1, __float_as_uint(c.y));
+                }
+            }
+            epi_sync();
+        }
         bool ok = true;
         for (int u = blockIdx.x; ok && u < units; u += gridDim.x) {
             const int rt = u % P.nrt;
@@ -394,7 +413,6 @@ __global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant
             }
             for (int ct = u / P.nrt; ct < P.nct; ct += P.nstripe, ++t) {
                 const int buf = t & 1;
-                if (MODE == kScArgmin && et < kScN) colc[buf * kScN + et] = col_const((int64_t)ct * kScN + et);
                 if (MODE == kScCollect) {
                     // the warp's own copy of its columns' constants: the
                     // warps share nothing per tile, so one that appends
@@ -412,12 +430,11 @@ __global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant
                     if (nct >= 0) load_cols(nct);
                 }
                 ok = tc::mbar_wait(tfull0 + 8 * buf, (uint32_t)((t >> 1) & 1), P.status);
-                if (MODE == kScArgmin) ok = epi_all(ok);  // also: the column constants are in place
+                if (MODE == kScArgmin) ok = epi_all(ok);  // the waits end for all warps or for none
                 if (!ok) break;
                 tc::fence_after_sync();
                 const uint32_t taddr =
                     tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(buf * kScN + part * kScPart);
-                const float2* cc = colc + buf * kScN + part * kScPart;
                 if (MODE == kScDump) {
 #pragma unroll 1
                     for (int b = 0; b < kScPart / 32; ++b) {
@@ -475,111 +492,67 @@ __global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant
                         __syncwarp();
                     }
                 } else {
-                    // nearest word: the tile's least approximate value gives an
-                    // upper bound tau of the row's least distance; every word
-                    // that could be within tau is a candidate
-                    float mv = __int_as_float(0x7f800000);
-                    int mc = 0;
-                    float mg = 0.f;
-#pragma unroll 1
-                    for (int b = 0; b < kScPart / 32; ++b) {
-                        float v[32];
-                        tc::tmem_ld_32(taddr + b * 32, v);
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const float x = __fmaf_rn(-2.f, v[j], cc[b * 32 + j].x);
-                            if (x < mv) {
-                                mv = x;
-                                mg = v[j];
-                                mc = part * kScPart + b * 32 + j;
-                            }
-                        }
-                    }
-                    hmin[part * kScM + rl] = make_float2(mv, mg);
-                    if (part == 0) {
-                        best[rl] = kEmptyKey;
-                        rcount[rl] = 0;
-                        rfull[rl] = 0;
-                    }
-                    if (et == 0) *ncand = *nfull = 0;
-                    // the column of each part's least value travels in the list's first words
-                    reinterpret_cast<uint8_t*>(list)[part * kScM + rl] = (uint8_t)mc;
-                    epi_sync();
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float2 o = hmin[q * kScM + rl];
-                        if (o.x < mv) {
-                            mv = o.x;
-                            mg = o.y;
-                            mc = reinterpret_cast<uint8_t*>(list)[q * kScM + rl];
-                        }
-                    }
-                    epi_sync();
-                    if (live) {
-                        const float nj = __ldg(P.cnrm + mc), ej = exact ? 0.f : __ldg(P.cerr + mc);
-                        const float tau = exact ? __fmaf_rn(-2.f, mg, __fadd_rn(ni, nj))
-                                                : screen_ub(ni, nj, mg, ei, ej, c2, gamma);
-                        float a;
-                        screen_row(tau, ni, ei, c2, gamma, exact, a, R);
-                        a2 = -2.f * a;
-                        if (unsafe) rfull[rl] = *nfull = 1;
-                    }
-#pragma unroll 1
-                    for (int b = 0; b < kScPart / 32; ++b) {
-                        float v[32];
-                        tc::tmem_ld_32(taddr + b * 32, v);
-                        unsigned hit = 0;
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const float2 c = cc[b * 32 + j];
-                            const bool in = __fmaf_rn(a2, c.y, __fmaf_rn(-2.f, v[j], c.x)) <= R;
-                            hit |= in ? 1u << j : 0u;
-                        }
-                        if (live && !unsafe && hit) {
-                            const int c = __popc(hit);
-                            atomicAdd(rcount + rl, c);
-                            int at = atomicAdd(ncand, c);
-                            if (at + c > kScList) {
-                                rfull[rl] = *nfull = 1;
-                                for (; hit && at < kScList; hit &= hit - 1) list[at++] = 0xFFFFu;
-                            }
-                            for (; hit; hit &= hit - 1)
-                                list[at++] = (uint16_t)((rl << 8) | (part * kScPart + b * 32 + __ffs(hit) - 1));
-                        }
-                    }
-                }
-                if (MODE != kScCollect) {  // the accumulator is read: hand it back
+                    // nearest word: the row's least approximate value gives an
+                    // upper bound tau of its least distance; every word that
+                    // could be within tau is a candidate
+                    float va[32], vb[32];
+                    tc::tmem_ld_issue(taddr, va);
+                    tc::tmem_ld_issue(taddr + 32, vb);
+                    tc::tmem_ld_wait(va);
+                    tc::tmem_ld_wait(vb);
                     tc::fence_before_sync();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tempty0 + 8 * buf);
-                }
-                if (MODE == kScArgmin) {
-                    epi_sync();
-                    const int nl = min(*(volatile int*)ncand, kScList);
-                    const int64_t row0 = (int64_t)rt * kScM;
-                    auto exact_key = [&](int r, int w) {
-                        const int64_t i = row0 + r;
-                        const float* w1 = P.W1 ? P.W1 + (int64_t)P.c1[i * P.c1_stride] * P.D : nullptr;
-                        return make_key(word_dist(P.X + i * P.D, w1, P.words + (int64_t)w * P.D, P.D, P.vec),
-                                        (uint32_t)w);
+                    const float4* c4 = reinterpret_cast<const float4*>(colf + part * kScPart);
+                    const float4* e4 = reinterpret_cast<const float4*>(colf + kScN + part * kScPart);
+                    float mn = __int_as_float(0x7f800000);
+                    auto least = [&](const float (&v)[32], int b) {
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const float4 c = c4[8 * b + q];
+                            mn = min_pair(fma_pair(v[4 * q], v[4 * q + 1], c.x, c.y), mn);
+                            mn = min_pair(fma_pair(v[4 * q + 2], v[4 * q + 3], c.z, c.w), mn);
+                        }
                     };
-                    for (int e = et; e < nl; e += kScEpi) {
-                        const int v = list[e];
-                        const int r = v >> 8, w = v & 255;
-                        if (r >= kScM || rfull[r]) continue;  // a row taken whole below
-                        // the only candidate is the nearest word: no distance needed
-                        const uint64_t key = rcount[r] == 1 ? (uint64_t)w : exact_key(r, w);
-                        atomicMin(reinterpret_cast<unsigned long long*>(best + r), (unsigned long long)key);
-                    }
-                    for (int r = 0; *(volatile int*)nfull && r < kScM; ++r) {  // rows without a usable bound
-                        if (!rfull[r] || row0 + r >= P.nrows) continue;
-                        for (int w = et; w < (int)P.ncols; w += kScEpi)
-                            atomicMin(reinterpret_cast<unsigned long long*>(best + r),
-                                      (unsigned long long)exact_key(r, w));
-                    }
+                    least(va, 0);
+                    least(vb, 1);
+                    hmin[(buf * 4 + part) * kScM + rl] = mn;
                     epi_sync();
-                    if (et < kScM && row0 + et < P.nrows)
-                        P.out[(row0 + et) * P.out_stride] = (int32_t)key_id(best[et]);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) mn = fminf(mn, hmin[(buf * 4 + q) * kScM + rl]);
+                    // N_j - 2 g <= mn + c N_j + e_j^2 for the word that has it
+                    const float ne = __uint_as_float(cmax[0]), ee = __uint_as_float(cmax[1]);
+                    float tau = __fadd_rn(ni, mn);
+                    if (!exact) {
+                        const float d = __fadd_ru(__fadd_ru(ni, mn), __fmaf_ru(c2, __fadd_ru(ni, __fmul_ru(2.f, ne)), __fmul_ru(ee, ee)));
+                        const float r = __fadd_ru(__fsqrt_ru(fmaxf(d, 0.f)), __fadd_ru(ei, ee));
+                        tau = __fmul_ru(__fmul_ru(r, r), __fadd_ru(1.f, gamma));
+                    }
+                    float a;
+                    screen_row(tau, ni, ei, c2, gamma, exact, a, R);
+                    a2 = -2.f * a;
+                    auto hits = [&](const float (&v)[32], int b) {
+                        unsigned hit = 0;
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const float4 c = c4[8 * b + q], e = e4[8 * b + q];
+                            const float2 x = screen_pair(v[4 * q], v[4 * q + 1], c.x, c.y, e.x, e.y, a2);
+                            const float2 y = screen_pair(v[4 * q + 2], v[4 * q + 3], c.z, c.w, e.z, e.w, a2);
+                            if (x.x <= R) hit |= 1u << (4 * q);
+                            if (x.y <= R) hit |= 2u << (4 * q);
+                            if (y.x <= R) hit |= 4u << (4 * q);
+                            if (y.y <= R) hit |= 8u << (4 * q);
+                        }
+                        return hit;
+                    };
+                    unsigned h0 = hits(va, 0), h1 = hits(vb, 1);
+                    if (unsafe) h0 = h1 = 0xFFFFFFFFu;  // ks_pick drops the columns past the last word
+                    if (live) *reinterpret_cast<uint2*>(P.mask + row * 8 + part * 2) = make_uint2(h0, h1);
+                }
+                if (MODE == kScDump) {  // the accumulator is read: hand it back
+                    tc::fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(tempty0 + 8 * buf);
                 }
             }
             if (MODE == kScCollect) {
@@ -615,6 +588,12 @@ __global__ void __launch_bounds__(256) ks_copy(const float* __restrict__ X, int6
     float red[8];  // squared norms of rows 0-3, then squared errors
     float top = 0.f, low = 0.f;
     bool ints = true;
+    int code[4] = {0, 0, 0, 0};
+    if (W1) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (r0 + u < N) code[u] = c1[(r0 + u) * c1_stride];
+    }
 #pragma unroll
     for (int u = 0; u < 8; ++u) red[u] = 0.f;
     for (int d0 = lane * 4; d0 < Dp; d0 += 128) {
@@ -641,10 +620,20 @@ __global__ void __launch_bounds__(256) ks_copy(const float* __restrict__ X, int6
 #pragma unroll
             for (int u = 0; u < 4; ++u)
                 if (r0 + u < N) {
-                    const float* w = W1 + (int64_t)c1[(r0 + u) * c1_stride] * D + d0;
+                    const float* w = W1 + (int64_t)code[u] * D + d0;
+                    if (VEC) {
+                        if (d0 < D) {
+                            const float4 f = __ldg(reinterpret_cast<const float4*>(w));
+                            v[u][0] = __fsub_rn(v[u][0], f.x);
+                            v[u][1] = __fsub_rn(v[u][1], f.y);
+                            v[u][2] = __fsub_rn(v[u][2], f.z);
+                            v[u][3] = __fsub_rn(v[u][3], f.w);
+                        }
+                    } else {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (d0 + j < D) v[u][j] = __fsub_rn(v[u][j], __ldg(w + j));
+                        for (int j = 0; j < 4; ++j)
+                            if (d0 + j < D) v[u][j] = __fsub_rn(v[u][j], __ldg(w + j));
+                    }
                 }
         }
 #pragma unroll
@@ -697,7 +686,9 @@ __global__ void __launch_bounds__(256) ks_copy(const float* __restrict__ X, int6
         else  // rounded up as in k0_quantize, plus what squares below the FP32 range could hide
             err[r0 + e - 4] = __fadd_ru(kScTiny, __fsqrt_ru(__fmul_ru(sum, 1.f + (float)(Dp + 8) * 5.9604645e-8f)));
     }
-    if (lane == 0 && f) atomicOr(flags, f);
+    // once set, a flag is only read: 250,000 warps' atomics on one word took
+    // longer than the copy
+    if (lane == 0 && (f & ~*(volatile int*)flags)) atomicOr(flags, f);
     if (status && (f & 8)) {  // a value that is not finite, or only a large norm?
         bool bad = false;
         for (int u = 0; u < 4 && r0 + u < N; ++u)
@@ -724,6 +715,72 @@ __global__ void __launch_bounds__(256) ks_gather(const uint4* __restrict__ Xq, c
             oerr[p] = err[i];
         }
     }
+}
+
+// ---------------------------------------------------------------- nearest words
+// One warp per 32 rows: a row with one candidate word takes it; the others'
+// (row, word) pairs are spread over the lanes, which compute canonical
+// distances; ties go to the smaller word.
+constexpr int kPickPairs = 512;  // pairs a warp lists at once
+__global__ void __launch_bounds__(128) ks_pick(const uint32_t* __restrict__ mask, int64_t N, int W,
+                                              const float* __restrict__ X, int D, bool vec,
+                                              const float* __restrict__ W1, const int32_t* __restrict__ c1,
+                                              int c1_stride, const float* __restrict__ words,
+                                              int32_t* __restrict__ out, int out_stride) {
+    __shared__ uint16_t pairs[4][kPickPairs];
+    __shared__ unsigned long long best[4][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t r0 = ((int64_t)blockIdx.x * 4 + w) * 32, row = r0 + lane;
+    if (r0 >= N) return;
+    uint32_t m[8];
+    int cnt = 0, first = 0;
+#pragma unroll
+    for (int q = 7; q >= 0; --q) {
+        m[q] = row < N && 32 * q < W ? mask[row * 8 + q] : 0;
+        if (W < 32 * q + 32 && W > 32 * q) m[q] &= (1u << (W - 32 * q)) - 1u;
+        cnt += __popc(m[q]);
+        if (m[q]) first = 32 * q + __ffs(m[q]) - 1;
+    }
+    best[w][lane] = cnt > 1 ? kEmptyKey : (unsigned long long)first;
+    __syncwarp();
+    int left = cnt > 1 ? cnt : 0;  // pairs still to list
+    int q = 0;
+    while (__any_sync(0xffffffffu, left > 0)) {
+        const int take = min(left, kPickPairs / 32);
+        int at = take;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, at, o);
+            if (lane >= o) at += y;
+        }
+        const int total = __shfl_sync(0xffffffffu, at, 31);
+        at -= take;
+        for (int t = 0; t < take; ++t) {
+            uint32_t cur = 0;
+            while (q < 8) {  // the next word of this row's mask
+#pragma unroll
+                for (int z = 0; z < 8; ++z) cur = z == q ? m[z] : cur;
+                if (cur) break;
+                ++q;
+            }
+            const int j = __ffs(cur) - 1;
+#pragma unroll
+            for (int z = 0; z < 8; ++z)
+                if (z == q) m[z] &= m[z] - 1;
+            pairs[w][at + t] = (uint16_t)((lane << 8) | (32 * q + j));
+        }
+        left -= take;
+        __syncwarp();
+        for (int e = lane; e < total; e += 32) {
+            const int r = pairs[w][e] >> 8, c = pairs[w][e] & 255;
+            const int64_t i = r0 + r;
+            const float* w1 = W1 ? W1 + (int64_t)c1[i * c1_stride] * D : nullptr;
+            const float d = word_dist(X + i * D, w1, words + (int64_t)c * D, D, vec);
+            atomicMin(&best[w][r], (unsigned long long)make_key(d, (uint32_t)c));
+        }
+        __syncwarp();
+    }
+    if (row < N) out[row * out_stride] = (int32_t)key_id(best[w][lane]);
 }
 
 // ---------------------------------------------------------------- thresholds and re-rank
@@ -865,7 +922,7 @@ void launch_screen_copy(const float* X, int64_t N, int D, const float* W1, const
     const int Dp = lp_dim(D);
     LaunchScope ls("ks_copy", s, (double)N * (D * 4.0 + Dp * 2.0 + 8.0), 0);
     const unsigned grid = (unsigned)((N + 31) / 32);
-    if (D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0)
+    if (D % 4 == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(W1)) & 15) == 0)
         ks_copy<true><<<grid, 256, 0, s>>>(X, N, D, Dp, W1, c1, c1_stride, Xq, nrm, err, flags, status);
     else
         ks_copy<false><<<grid, 256, 0, s>>>(X, N, D, Dp, W1, c1, c1_stride, Xq, nrm, err, flags, status);
@@ -899,6 +956,42 @@ bool launch_screen(const uint16_t* A, const uint16_t* B, int Dp, ScreenArgs& P, 
 }
 
 }  // namespace
+
+// ---------------------------------------------------------------- nearest words
+void launch_screen_copy(const float* X, int64_t N, int D, const float* W1, const int32_t* c1, int c1_stride,
+                        const AssignWork& w, int* status, cudaStream_t s) {
+    cudaMemsetAsync(w.flags, 0, sizeof(int), s);
+    launch_screen_copy(X, N, D, W1, c1, c1_stride, w.Xq, w.nrm, w.err, w.flags, status, s);
+}
+
+bool launch_assign_screened(const float* X, int64_t N, int D, const float* W1, const int32_t* c1, int c1_stride,
+                            const float* words, int W, const AssignWork& w, int32_t* out, int out_stride, int* status,
+                            cudaStream_t s) {
+    const int Dp = lp_dim(D);
+    cudaMemsetAsync(w.flags + 1, 0, sizeof(int), s);
+    launch_screen_copy(words, W, D, nullptr, nullptr, 0, w.Wq, w.wnrm, w.werr, w.flags + 1, nullptr, s);
+    ScreenArgs P{};
+    P.nrows = N;
+    P.ncols = W;
+    P.rnrm = w.nrm;
+    P.rerr = w.err;
+    P.cnrm = w.wnrm;
+    P.cerr = w.werr;
+    P.cstride = 1;
+    P.cD2 = screen_c(D);
+    P.gamma = (float)(D + 8) * 1.1920928955078125e-7f;
+    P.flag_r = w.flags;
+    P.flag_c = w.flags + 1;
+    P.status = status;
+    P.mask = w.mask;
+    if (!launch_screen<kScArgmin>(w.Xq, w.Wq, Dp, P, W1 ? "ks_assign_res" : "ks_assign", s)) return false;
+    const bool vec = D % 4 == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(words) |
+                                     reinterpret_cast<uintptr_t>(W1)) & 15) == 0;
+    LaunchScope ls("ks_pick", s, (double)N * 36.0, 0);
+    ks_pick<<<(unsigned)((N + 127) / 128), 128, 0, s>>>(w.mask, N, W, X, D, vec, W1, c1, c1_stride, words, out,
+                                                        out_stride);
+    return true;
+}
 
 // ---------------------------------------------------------------- exact lists
 // The FP32 kernel spends two instructions per pair and dim and a long chain

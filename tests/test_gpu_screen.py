@@ -64,3 +64,15 @@ def test_smallest(knng, n, D, k, s):
     ids, d = knng.knng_exact(X, k, rows)
     ref_ids, ref_d = knng.knng_exact_noalloc(X, k, rows)
     assert torch.equal(ids, ref_ids) and torch.equal(d, ref_d)
+
+
+@pytest.mark.parametrize("n,D,W,spread", [(3000, 130, 16, 20), (5000, 64, 3, 3), (2049, 300, 200, 0)])
+def test_word_means_in_the_defined_order(knng, n, D, W, spread):
+    """Sums whose magnitudes lie 2^(2 spread) apart round in FP64, so the words must come from the defined order."""
+    import oracle
+    rng = np.random.default_rng(11)
+    X = (rng.standard_normal((n, D)) * np.exp2(rng.uniform(-spread, spread, (n, D)))).astype(np.float32)
+    w1, w2 = knng.knng_rvq_train(torch.from_numpy(X).cuda(), W, W, 2, seed=3)
+    o1, o2 = oracle.rvq_train(X, W, W, 2, seed=3)
+    assert np.array_equal(w1.cpu().numpy().view(np.uint32), o1.view(np.uint32))
+    assert np.array_equal(w2.cpu().numpy().view(np.uint32), o2.view(np.uint32))
