@@ -838,7 +838,7 @@ int32_t* run_partition(const float* X, const Args& a, const TreePlan& tp, BuildL
         k_iota<<<grid_1d(a.n), 256, 0, s>>>(pin, a.n);
     }
     for (int l = 0; l < tp.L; ++l) {
-        run_split_level(X, a.D, tp.levels[l], a.p.twomeans_iters, ps, pin, pout, sb, s);
+        run_split_level(X, a.n, a.D, tp.levels[l], a.p.twomeans_iters, ps, pin, pout, sb, s);
         std::swap(pin, pout);
     }
     return pin;
@@ -937,6 +937,7 @@ void build_core(const float* X, const Args& a, BuildLayout& b, const TreePlan& t
     // slot q > 0 on helper stream q - 1, forked from the caller's stream); a
     // slot's next partition waits for the leaf stage that read its last one
     const int P = a.p.tree_passes, Q = b.nslots;
+    b.sb.share = std::max(1, std::min(P, Q));
     std::vector<int32_t*> perms((size_t)std::max(P, 0), nullptr);
     std::vector<cudaEvent_t> part_done((size_t)std::max(P, 0), nullptr), leaf_done((size_t)std::max(P, 0), nullptr);
     if (Q > 1 && P > 1) {

@@ -281,6 +281,27 @@ __device__ __forceinline__ float canon_dist(const float* __restrict__ xa, const 
     return acc;
 }
 
+// s / b rounded to nearest (FP64) from inv = RN(1 / b): the FMA residual
+// r = s - q0 b of q0 = RN(s inv) is exact, and q0 + r inv rounds to RN(s / b)
+// (Markstein's correction).  For integer s and b < 2^52 the quotient is never
+// within the correction's error of a rounding boundary, so the result equals
+// FP64 division bit for bit; it costs three FP64 operations, where GB300
+// issues FP64 at a small fraction of its FP32 rate.
+__device__ __forceinline__ double div_by(double s, double b, double inv) {
+    const double q0 = __dmul_rn(s, inv);
+    const double r = __fma_rn(-q0, b, s);
+    return __fma_rn(r, inv, q0);
+}
+
+// RN32(S / K) of an integer sum: FP32 division when S and K are exact in FP32
+// (no double rounding can separate it from RN32(RN64(S / K)) for K < 2^28:
+// the quotient is either an FP32 midpoint, which FP64 holds exactly, or
+// farther from one than FP64's rounding error), else FP64 division.
+__device__ __forceinline__ float mean_of_ints(long long S, int K) {
+    if (S > -16777216LL && S < 16777216LL && K < 16777216) return __fdiv_rn((float)S, (float)K);
+    return (float)((double)S / (double)K);
+}
+
 
 // Status word written by kernels that detect a bad input or an internal
 // limit; the host reads it once per call.

@@ -95,6 +95,7 @@ struct SplitBuffers {
     const int* bflag = nullptr;
     bool u8_host = false;   // the host's copy of that decision
     bool capture = false;   // recorded into a CUDA graph: the host knows nothing of the data
+    int share = 1;          // partitions that run side by side
 };
 
 constexpr int kTile = 2048;         // positions per select/partition tile
@@ -103,9 +104,13 @@ constexpr int kSmallMax = 8192;     // segments up to this size select in one CT
 constexpr int kSortSelectMax = 2048; // segments up to this size select by a sort in registers
 constexpr int kRadixBits = 11;
 
+// The level in one launch (level.cu), a cluster per segment with its rows in
+// shared memory; false (nothing launched) when the largest segment does not fit.
+bool launch_level(const float* X, int64_t n, int D, const LevelPlan& lp, int iters, uint64_t pass_seed,
+                  const int32_t* perm_in, int32_t* perm_out, const SplitBuffers& b, cudaStream_t s);
 // One level of the balanced two-means tree: T Lloyd iterations, then the
 // final cut that writes perm_out.
-void run_split_level(const float* X, int D, const LevelPlan& lp, int iters, uint64_t pass_seed,
+void run_split_level(const float* X, int64_t n_rows, int D, const LevelPlan& lp, int iters, uint64_t pass_seed,
                      const int32_t* perm_in, int32_t* perm_out, const SplitBuffers& b,
                      cudaStream_t s);
 

@@ -1372,27 +1372,6 @@ __global__ void __launch_bounds__(kSuThreads) k1_sums_async(const float* __restr
                            su_smem);
 }
 
-// s / b rounded to nearest (FP64) from inv = RN(1 / b): the FMA residual
-// r = s - q0 b of q0 = RN(s inv) is exact, and q0 + r inv rounds to RN(s / b)
-// (Markstein's correction).  For integer s and b < 2^52 the quotient is never
-// within the correction's error of a rounding boundary, so the result equals
-// FP64 division bit for bit; it costs three FP64 operations, where GB300
-// issues FP64 at a small fraction of its FP32 rate.
-__device__ __forceinline__ double div_by(double s, double b, double inv) {
-    const double q0 = __dmul_rn(s, inv);
-    const double r = __fma_rn(-q0, b, s);
-    return __fma_rn(r, inv, q0);
-}
-
-// RN32(S / K) of an integer sum: FP32 division when S and K are exact in FP32
-// (no double rounding can separate it from RN32(RN64(S / K)) for K < 2^28:
-// the quotient is either an FP32 midpoint, which FP64 holds exactly, or
-// farther from one than FP64's rounding error), else FP64 division.
-__device__ __forceinline__ float mean_of_ints(long long S, int K) {
-    if (S > -16777216LL && S < 16777216LL && K < 16777216) return __fdiv_rn((float)S, (float)K);
-    return (float)((double)S / (double)K);
-}
-
 // c1 - c0 of one dim from integer sums (int64 in segsum and segleft).  Full
 // sweep: s0, s1 are the left and right sums; the segment's total and left sum
 // are kept.  Delta sweep: s0, s1 are the sums of the points that moved left
@@ -1622,7 +1601,7 @@ __global__ void __launch_bounds__(256) k1_part_scatter(const float* __restrict__
 
 }  // namespace
 
-void run_split_level(const float* X, int D, const LevelPlan& lp, int iters, uint64_t pass_seed,
+void run_split_level(const float* X, int64_t n_rows, int D, const LevelPlan& lp, int iters, uint64_t pass_seed,
                      const int32_t* perm_in, int32_t* perm_out, const SplitBuffers& b, cudaStream_t s) {
     // algorithmic bytes: a sweep reads every row once plus its id and key
     const double n = lp.n, rows = n * (b.u8_host ? b.Db * 1.0 : b.q16_host ? b.Dq * 2.0 : D * 4.0);
@@ -1634,6 +1613,7 @@ void run_split_level(const float* X, int D, const LevelPlan& lp, int iters, uint
     // finished trees' leaves keep their place: the cut below writes only the
     // segments that split
     if (lp.frozen) cudaMemcpyAsync(perm_out, perm_in, sizeof(int32_t) * (size_t)lp.n, cudaMemcpyDeviceToDevice, s);
+    if (launch_level(X, n_rows, D, lp, iters, pass_seed, perm_in, perm_out, b, s)) return;
     {
         LaunchScope ls("k1_init", s, (double)lp.nseg * 3 * D * 4, 0);
         k1_init<<<lp.nseg, 128, 0, s>>>(X, D, perm_in, lp.seg_off, lp.seg_tile0, lp.seg_local, lp.level, pass_seed,
