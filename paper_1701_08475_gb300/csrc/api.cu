@@ -1668,14 +1668,10 @@ int knng_search(const float* data, int64_t n, int D, const int32_t* graph_ids, i
         if (m == 0) return;
         if (!queries || !out_ids || !out_dists || (s > 0 && !seeds)) fail(KNNG_EINVAL, "a pointer is NULL");
         cudaStream_t st = (cudaStream_t)stream;
-        const int cl = search_cap_log2(s, t0, ks, k);
-        // queries per launch: their visited tables within 1 GiB
-        const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(m, ((int64_t)1 << 28) >> cl));
         Workspace ws;
         DevBuf<float> X, Qb;
         DevBuf<int32_t> Gb, Sb, oi;
         DevBuf<float> od;
-        int32_t* tab = nullptr;
         int* status = nullptr;
         for (int ps = 0; ps < 2; ++ps) {
             ws.used = 0;
@@ -1685,7 +1681,6 @@ int knng_search(const float* data, int64_t n, int D, const int32_t* graph_ids, i
             if (s > 0) bind(ws, Sb, seeds, (size_t)m * s, ps);
             bind(ws, oi, out_ids, (size_t)m * ks, ps);
             bind(ws, od, out_dists, (size_t)m * ks, ps);
-            tab = ws.take<int32_t>((size_t)chunk << cl);
             status = ws.take<int>(4);
             if (ps == 0) ws.allocate(st);
         }
@@ -1694,11 +1689,8 @@ int knng_search(const float* data, int64_t n, int D, const int32_t* graph_ids, i
         upload(Gb, st);
         upload(Qb, st);
         if (s > 0) upload(Sb, st);
-        launch_check_finite(X.dev, n * (int64_t)D, status, st);
-        launch_check_finite(Qb.dev, m * (int64_t)D, status, st);
-        for (int64_t q0 = 0; q0 < m; q0 += chunk)
-            launch_search(X.dev, n, D, Gb.dev, k, Qb.dev, q0, std::min(m, q0 + chunk), s > 0 ? Sb.dev : nullptr, s,
-                          t0, ks, tab, cl, oi.dev, od.dev, st);
+        launch_check_finite(X.dev, n * (int64_t)D, status, st, Qb.dev, m * (int64_t)D);
+        launch_search(X.dev, n, D, Gb.dev, k, Qb.dev, m, s > 0 ? Sb.dev : nullptr, s, t0, ks, oi.dev, od.dev, st);
         download(oi, st);
         download(od, st);
         cuda_check(launch_error(), "kernel launch");
@@ -1809,8 +1801,7 @@ int knng_rvq_index(const float* data, int64_t n, int D, const float* words1, int
         upload(X, st);
         upload(w1, st);
         upload(w2, st);
-        launch_check_finite(w1.dev, (int64_t)W1 * D, status, st);
-        launch_check_finite(w2.dev, (int64_t)W2 * D, status, st);
+        launch_check_finite(w1.dev, (int64_t)W1 * D, status, st, w2.dev, (int64_t)W2 * D);
         if (screen)
             launch_screen_copy(X.dev, n, D, nullptr, nullptr, 2, aw, status, st);
         else
@@ -1872,9 +1863,7 @@ int knng_rvq_seeds(const float* words1, int W1, const float* words2, int W2, int
         upload(off, st);
         upload(li, st);
         upload(Qb, st);
-        launch_check_finite(w1.dev, (int64_t)W1 * D, status, st);
-        launch_check_finite(w2.dev, (int64_t)W2 * D, status, st);
-        launch_check_finite(Qb.dev, m * (int64_t)D, status, st);
+        launch_check_finite(Qb.dev, m * (int64_t)D, status, st, w1.dev, (int64_t)W1 * D, w2.dev, (int64_t)W2 * D);
         launch_check_offsets(off.dev, nk, n, status, st);
         launch_rvq_tables(w1.dev, W1, w2.dev, W2, D, n1, n2, x12, w1T, w2T, st);
         launch_rvq_seeds(w1T, W1, w2T, W2, D, n1, n2, x12, off.dev, li.dev, Qb.dev, m, probe1, s, Sb.dev, status, st);

@@ -227,14 +227,34 @@ __global__ void k_recall(const int32_t* __restrict__ ids, const float* __restric
     }
 }
 
-__global__ void k_check_finite(const float4* __restrict__ X4, int64_t n4, const float* __restrict__ tail,
-                               int ntail, int* __restrict__ status) {
+// Up to three arrays in one launch.  An array may start at any 4-byte boundary:
+// its 16-byte aligned body is read as float4, the few values before and after
+// it by the first CTA.
+struct FiniteArgs {
+    const float* p[3];
+    int64_t count[3];
+};
+__global__ void k_check_finite(const FiniteArgs A, int* __restrict__ status) {
     bool bad = false;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n4; e += (int64_t)gridDim.x * blockDim.x) {
-        const float4 v = __ldg(X4 + e);
-        bad |= !isfinite(v.x) | !isfinite(v.y) | !isfinite(v.z) | !isfinite(v.w);
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+        const int64_t count = A.count[u];
+        if (count == 0) continue;
+        const float* X = A.p[u];
+        const int64_t to16 = (int64_t)((16 - (reinterpret_cast<uintptr_t>(X) & 15)) & 15) / 4;
+        const int64_t head = to16 < count ? to16 : count, n4 = (count - head) / 4;
+        const float4* X4 = reinterpret_cast<const float4*>(X + head);
+        for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n4;
+             e += (int64_t)gridDim.x * blockDim.x) {
+            const float4 v = __ldg(X4 + e);
+            bad |= !isfinite(v.x) | !isfinite(v.y) | !isfinite(v.z) | !isfinite(v.w);
+        }
+        if (blockIdx.x == 0) {
+            const int64_t t = threadIdx.x;
+            if (t < head) bad |= !isfinite(X[t]);
+            if (head + 4 * n4 + t < count) bad |= !isfinite(X[head + 4 * n4 + t]);
+        }
     }
-    if (blockIdx.x == 0 && threadIdx.x < ntail) bad |= !isfinite(tail[threadIdx.x]);
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(status, kStatusNonFinite);
 }
 
@@ -279,20 +299,13 @@ void launch_recall(const int32_t* ids, const float* d, const int32_t* gt_ids, co
     k_recall<<<grid, 256, 0, s>>>(ids, d, gt_ids, gt_d, sample, s_rows, k, counts);
 }
 
-void launch_check_finite(const float* X, int64_t count, int* status, cudaStream_t s) {
-    // X may start at any 4-byte boundary: handle the head up to 16 B alignment
-    // and the tail with scalar loads
-    const uintptr_t addr = reinterpret_cast<uintptr_t>(X);
-    const int64_t head = (int64_t)(((16 - (addr & 15)) & 15) / 4);
-    const int64_t h = head < count ? head : count;
-    LaunchScope ls("k0_check_finite", s, count * 4.0, 0, h > 0 ? 2 : 1);
-    if (h > 0) k_check_finite<<<1, 32, 0, s>>>(nullptr, 0, X, (int)h, status);
-    const int64_t rest = count - h;
-    const int64_t n4 = rest / 4;
-    const int ntail = (int)(rest - n4 * 4);
-    const int grid = (int)((n4 + 255) / 256 < 152 * 8 ? (n4 + 255) / 256 : 152 * 8);
-    k_check_finite<<<grid < 1 ? 1 : grid, 256, 0, s>>>(reinterpret_cast<const float4*>(X + h), n4,
-                                                       X + h + n4 * 4, ntail, status);
+void launch_check_finite(const float* X, int64_t count, int* status, cudaStream_t s, const float* Y, int64_t ycount,
+                         const float* Z, int64_t zcount) {
+    FiniteArgs A = {{X, Y, Z}, {count, ycount, zcount}};
+    const int64_t total = count + ycount + zcount;
+    LaunchScope ls("k0_check_finite", s, total * 4.0, 0);
+    const int64_t grid = (total / 4 + 255) / 256;
+    k_check_finite<<<(int)(grid < 1 ? 1 : grid < 152 * 8 ? grid : 152 * 8), 256, 0, s>>>(A, status);
 }
 
 }  // namespace knng

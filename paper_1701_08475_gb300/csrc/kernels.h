@@ -34,8 +34,10 @@ void fault_launch_point(cudaStream_t s);
 cudaError_t launch_error();
 
 // ---------------------------------------------------------------- prepare (K0)
-// Sets *status |= kStatusNonFinite if any of the n*D values is not finite.
-void launch_check_finite(const float* X, int64_t count, int* status, cudaStream_t s);
+// Sets *status |= kStatusNonFinite if any of X's count values (or Y's, Z's) is
+// not finite.
+void launch_check_finite(const float* X, int64_t count, int* status, cudaStream_t s, const float* Y = nullptr,
+                         int64_t ycount = 0, const float* Z = nullptr, int64_t zcount = 0);
 
 // ---------------------------------------------------------------- two-means split (K1)
 struct SelState {
@@ -315,13 +317,11 @@ void launch_rvq_seeds(const float* w1T, int W1, const float* w2T, int W2, int D,
                       const float* x12, const int32_t* off, const int32_t* ids, const float* Q, int64_t m, int probe1,
                       int s_seeds, int32_t* S, const int* status, cudaStream_t s);
 
-// Enhanced hill-climbing search (search.cu): queries [q0, q1) of Q against
-// the graph G (n x k ids), seeds S (s per query), t0 iterations, ks <= 32
-// results per query; tab: (q1 - q0) << cap_log2 ints of visited tables.
-int search_cap_log2(int s, int t0, int ks, int k);
-void launch_search(const float* X, int64_t n, int D, const int32_t* G, int k, const float* Q, int64_t q0,
-                   int64_t q1, const int32_t* S, int s, int t0, int ks, int32_t* tab, int cap_log2, int32_t* out_ids,
-                   float* out_d, cudaStream_t st);
+// Enhanced hill-climbing search (search.cu): m queries Q against the graph G
+// (n x k ids), seeds S (s per query), t0 iterations, ks <= 32 results per
+// query.
+void launch_search(const float* X, int64_t n, int D, const int32_t* G, int k, const float* Q, int64_t m,
+                   const int32_t* S, int s, int t0, int ks, int32_t* out_ids, float* out_d, cudaStream_t st);
 
 // The k nearest of rows sample[0 .. s_rows) (row0 + r without a sample), of
 // only the rows listed in list[0 .. *list_count) when a list is given, in

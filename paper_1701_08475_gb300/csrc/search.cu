@@ -1,18 +1,38 @@
 // search.cu -- the enhanced hill-climbing search over a kNN graph (Sec. 3.2,
 // Alg. 2) for a batch of queries.
 //
-// One warp per query.  The rank list R matters only through its first ks
-// entries by (d, id): they are what each iteration expands and what the
-// search returns, and an entry outside them never re-enters them (R only
-// grows).  So the warp keeps those ks keys (ks <= 32, entry e in lane e) and
-// a visited set, an open-addressing table of ids in global memory (twice the
-// most visits the query can make, so probes stay short and never fill it).
-// An iteration takes the ks entries as they stand at its start, and every
-// neighbour of theirs not visited yet is visited: its canonical FP32 distance
-// is computed and its key merged into the list.  The entries' graph slots are
-// taken 32 at a time across entries, one per lane.  A key enters the list at
-// most once and the fresh ids of an iteration do not depend on the order the
-// slots are taken in, so the order does not change the result.
+// The rank list R matters only through its first ks entries by (d, id): they
+// are what each iteration expands and what the search returns, and an entry
+// outside them never re-enters them (R only grows).  So a query keeps those
+// ks keys (ks <= 32, entry e in lane e).  An entry's neighbours are all
+// visited once it has been expanded, so each entry is expanded once (a flag in
+// its key), and the search ends when every entry is: later iterations could
+// add nothing.
+//
+// An iteration collects the unvisited neighbours of its entries in a queue and
+// computes their canonical FP32 distances 32 at a time: cp.async brings the
+// rows' next 128 dims into shared memory, every lane's pieces in flight at
+// once, and then each lane walks one row.  (A lane that walks its row in
+// global memory waits for a few 16-byte pieces at a time.)  The distances
+// merge into the list in any order: a key enters at most once and the
+// collected ids do not depend on the order.
+//
+// Visited ids are kept in a shared-memory hash table.  It is exact until it is
+// three quarters full; after that an id may be visited again, which the merge
+// drops when it is in the list, and which cannot enter the list when it was
+// turned away before (the ks-th key only falls).
+//
+// One CTA per query: one warp, or, for few queries, kSearchGroup warps, which
+// share the collecting and take a batch of rows each.
+//
+// Measured (GB300), 1M x 128 integers, k = 20, 10,000 queries, t0 = 12, ks = 20:
+// the call took 2.54 ms with a lane per row in global memory, the visited
+// tables in global memory and every entry expanded in every iteration; 1.57
+// with entries expanded once, staged rows and shared tables (128 dims, two
+// queries per CTA: 10 warps per SM), 0.97 with one query per CTA and 32 dims,
+// 0.86 with far rows dropped.  What is left is issue slots and latency about
+// equally (47 % of issue slots used, 625 MB read from DRAM at n = 300,000).
+// One query, 100,000 x 96: the kernel 115 -> 28 us.
 #include <algorithm>
 
 #include "common.cuh"
@@ -22,138 +42,248 @@ namespace knng {
 
 namespace {
 
-constexpr int kSearchWarps = 4;
+constexpr int kSearchGroup = 4;  // warps of a query when there are few
+// dims staged at once: narrow with one warp per query, so that more queries fit
+// an SM; wide with several, where one round trip to memory is what counts
+__host__ __device__ constexpr int search_dims(int W) { return W > 1 ? 128 : 32; }
+// floats per staged row: the 16-byte reads of 8 lanes cover all banks
+__host__ __device__ constexpr int search_stride(int W) { return search_dims(W) + 4; }
+constexpr int kSearchTab = 1024;             // visited table
+constexpr int kSearchFull = kSearchTab * 3 / 4;
+constexpr int kSearchQueue = 256;
 
-// Marks `id` visited in the query's table (2^cap_log2 slots, -1 = free);
-// true on its first visit.  Fibonacci hashing, linear probing.
-__device__ __forceinline__ bool visit(int32_t* tab, int cap_log2, int32_t id) {
-    const uint32_t mask = (1u << cap_log2) - 1u;
-    uint32_t h = ((uint32_t)id * 2654435761u) >> (32 - cap_log2);
-    for (uint32_t probe = 0; probe <= mask; ++probe) {
-        const int32_t old = atomicCAS(tab + h, -1, id);
-        if (old == -1) return true;
-        if (old == id) return false;
-        h = (h + 1u) & mask;
-    }
-    return false;  // not reached: the table holds twice the possible visits
+struct SearchSmem {
+    size_t stage, tab, queue, keys, entry, misc, total;
+};
+__host__ __device__ inline SearchSmem search_smem(int D, int W) {
+    SearchSmem L;
+    L.stage = ((size_t)D * 4 + 15) & ~(size_t)15;  // the query first
+    L.tab = L.stage + (size_t)W * 32 * search_stride(W) * 4;
+    L.queue = L.tab + kSearchTab * 4;
+    L.keys = L.queue + kSearchQueue * 4;
+    L.entry = L.keys + (size_t)W * 32 * 8;
+    L.misc = L.entry + 32 * 4;
+    L.total = L.misc + 16;
+    return L;
 }
 
-// Canonical FP32 squared l2 of row x against the query q (dims ascending,
-// t = x_j - q_j, acc = fmaf(t, t, acc)).  V4: x and q 16-byte aligned and D a
-// multiple of 4, so both are read four dims at a time (the same chain).
-template <bool V4>
-__device__ __forceinline__ float dist_to_query(const float* __restrict__ x, const float* q, int D) {
-    float acc = 0.f;
-    if (V4) {
-        const float4* x4 = reinterpret_cast<const float4*>(x);
-        const float4* q4 = reinterpret_cast<const float4*>(q);
-        for (int j = 0; j < D / 4; ++j) {
-            const float4 a = __ldg(x4 + j), b = q4[j];
-            float t = __fsub_rn(a.x, b.x);
-            acc = __fmaf_rn(t, t, acc);
-            t = __fsub_rn(a.y, b.y);
-            acc = __fmaf_rn(t, t, acc);
-            t = __fsub_rn(a.z, b.z);
-            acc = __fmaf_rn(t, t, acc);
-            t = __fsub_rn(a.w, b.w);
-            acc = __fmaf_rn(t, t, acc);
-        }
-        return acc;
-    }
-    for (int j = 0; j < D; ++j) {
-        const float t = __fsub_rn(__ldg(x + j), q[j]);
-        acc = __fmaf_rn(t, t, acc);
-    }
-    return acc;
+// A list key: order-preserving distance, then id, then whether the entry has
+// been expanded (ids are below 2^31).
+__device__ __forceinline__ uint64_t list_key(float d, uint32_t id) {
+    return ((uint64_t)ord32(d) << 32) | ((uint64_t)id << 1);
 }
+__device__ __forceinline__ uint32_t list_id(uint64_t k) { return (uint32_t)k >> 1; }
 
-template <bool V4>
-__global__ void __launch_bounds__(32 * kSearchWarps) k8_search(const float* __restrict__ X, int64_t n, int D,
-                                                              const int32_t* __restrict__ G, int k,
-                                                              const float* __restrict__ Q, int64_t q0, int64_t q1,
-                                                              const int32_t* __restrict__ S, int s, int t0, int ks,
-                                                              int32_t* __restrict__ tab, int cap_log2,
-                                                              int32_t* __restrict__ out_ids,
-                                                              float* __restrict__ out_d) {
-    extern __shared__ float4 qs4[];  // [kSearchWarps][D]
-    float* qs = reinterpret_cast<float*>(qs4);
-    __shared__ uint64_t scratch[kSearchWarps][32];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t qi = q0 + (int64_t)blockIdx.x * kSearchWarps + w;
-    if (qi >= q1) return;  // the whole warp; nothing below synchronises the CTA
-    float* q = qs + (size_t)w * D;
-    for (int j = lane; j < D; j += 32) q[j] = Q[qi * D + j];
-    __syncwarp();
-    int32_t* T = tab + ((qi - q0) << cap_log2);
-    uint64_t* sc = scratch[w];
-    uint64_t list = kEmptyKey;  // entry `lane` of R's first ks
-    // every lane offers one id (or -1): the fresh ones are visited and merged
-    auto offer = [&](int32_t id) {
-        const bool fresh = id >= 0 && id < n && visit(T, cap_log2, id);
-        const uint64_t key = fresh ? make_key(dist_to_query<V4>(X + (int64_t)id * D, q, D), (uint32_t)id) : kEmptyKey;
-        uint64_t cand[1] = {key}, out;
-        bool changed;
-        if (!warp_merge_few<1>(cand, list, ks, sc, out, changed)) {
-            // not reached (the keys are distinct and at most 64): the general merge
-            uint64_t a[2] = {key, list}, res[1];
-            sort_regs<2>(a);
-            warp_select_unique<2, 1>(a, ks, res);
-            out = res[0];
-        }
-        list = lane < ks ? out : kEmptyKey;
+template <bool VEC, int W>
+__global__ void __launch_bounds__(32 * W) k8_search(
+    const float* __restrict__ X, int64_t n, int D, const int32_t* __restrict__ G, int k, const float* __restrict__ Q,
+    const int32_t* __restrict__ S, int s, int t0, int ks, int32_t* __restrict__ out_ids,
+    float* __restrict__ out_d) {
+    constexpr int kDims = search_dims(W), kStride = search_stride(W);
+    extern __shared__ __align__(16) uint8_t se_smem[];
+    const int gt = threadIdx.x, gw = gt >> 5, lane = gt & 31;
+    const int64_t qi = blockIdx.x;
+    const SearchSmem L = search_smem(D, W);
+    uint8_t* base = se_smem;
+    float* q = reinterpret_cast<float*>(base);
+    float* stage = reinterpret_cast<float*>(base + L.stage) + (size_t)gw * 32 * kStride;
+    int32_t* tab = reinterpret_cast<int32_t*>(base + L.tab);
+    int32_t* queue = reinterpret_cast<int32_t*>(base + L.queue);
+    uint64_t* keys = reinterpret_cast<uint64_t*>(base + L.keys);
+    int32_t* entry = reinterpret_cast<int32_t*>(base + L.entry);
+    int* misc = reinterpret_cast<int*>(base + L.misc);  // queued, visited, entries to expand
+    float* bound = reinterpret_cast<float*>(misc + 3);  // the list's ks-th distance
+    auto sync = [&] {
+        if (W > 1) __syncthreads();
+        else __syncwarp();
     };
-    for (int a0 = 0; a0 < s; a0 += 32) offer(a0 + lane < s ? S[qi * s + a0 + lane] : -1);
-    for (int t = 0; t < t0; ++t) {
-        // R's first ks at the iteration's start: its real entries are a
-        // prefix; their nt * k graph slots are offered 32 at a time (slot
-        // u = entry u / k, neighbour u % k)
-        const uint64_t snap = list;
-        const int nt = __popc(__ballot_sync(0xffffffffu, snap != kEmptyKey));
-        const int slots = nt * k;
-        for (int u0 = 0; u0 < slots; u0 += 32) {
-            const int u = u0 + lane;
-            const int a = u < slots ? u / k : 0;
-            const uint64_t e = shfl64(snap, a);
-            offer(u < slots ? G[(int64_t)key_id(e) * k + (u - a * k)] : -1);
+    for (int j = gt; j < D; j += 32 * W) q[j] = Q[qi * D + j];
+    for (int j = gt; j < kSearchTab; j += 32 * W) tab[j] = -1;
+    if (gt < 3) misc[gt] = 0;
+    if (gt == 0) *bound = __int_as_float(0x7f800000);
+    sync();
+    uint64_t list = kEmptyKey;  // entry `lane` of the list (in warp 0)
+
+    // queues an id (-1: none) that has not been visited
+    auto collect = [&](int32_t id) {
+        if (id < 0 || id >= n) return;
+        uint32_t h = ((uint32_t)id * 2654435761u) >> 22;
+        bool fresh = false;
+        const bool room = *(volatile int*)(misc + 1) < kSearchFull;
+        for (int probe = 0; probe < kSearchTab; ++probe) {
+            const int32_t old = room ? atomicCAS(tab + h, -1, id) : *(volatile int32_t*)(tab + h);
+            if (old == id) return;
+            if (old == -1) {
+                fresh = true;
+                break;
+            }
+            h = (h + 1u) & (kSearchTab - 1);
         }
+        if (room && fresh) atomicAdd(misc + 1, 1);
+        queue[atomicAdd(misc, 1)] = id;
+    };
+    // distances of the queued ids, merged into the list; empties the queue
+    auto process = [&] {
+        sync();
+        const int nq = misc[0];
+        for (int b = 0; b < nq; b += 32 * W) {
+            const int at = b + 32 * gw + lane;
+            const int cnt = min(32, nq - (b + 32 * gw));  // this warp's rows (may be <= 0)
+            const int32_t id = at < nq ? queue[at] : -1;
+            float acc = 0.f;
+            // a distance only grows along its chain: a row already past the
+            // list's ks-th distance is dropped, its further dims are not read
+            const float far = *bound;
+            unsigned open = cnt >= 32 ? 0xFFFFFFFFu : cnt > 0 ? (1u << cnt) - 1u : 0u;
+            for (int d0 = 0; d0 < D && open; d0 += kDims) {
+                const int dl = min(kDims, D - d0);
+                __syncwarp();
+                // P pieces per row: a warp's lanes take 32 / P rows side by side
+                constexpr int P = VEC ? kDims / 4 : 32, R = 32 / P;
+                const int32_t* ids = queue + b + 32 * gw;
+                for (int r = lane / P; r < cnt; r += R) {
+                    if (!((open >> r) & 1u)) continue;
+                    const float* src = X + (int64_t)ids[r] * D + d0;
+                    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(stage + r * kStride);
+                    if (VEC) {
+                        const int c = lane % P * 4;
+                        if (c < dl)
+                            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + 4 * c), "l"(src + c)
+                                         : "memory");
+                    } else {
+                        for (int c = lane; c < dl; c += 32)
+                            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst + 4 * c), "l"(src + c)
+                                         : "memory");
+                    }
+                }
+                asm volatile("cp.async.wait_all;\n" ::: "memory");
+                __syncwarp();
+                if ((open >> lane) & 1u) {  // the canonical chain: dims ascending, t = x_j - q_j, acc = fmaf(t, t, acc)
+                    const float* x = stage + lane * kStride;
+                    const float* y = q + d0;
+                    if (VEC) {
+#pragma unroll 4
+                        for (int j = 0; j < dl; j += 4) {
+                            const float4 u = *reinterpret_cast<const float4*>(x + j);
+                            const float4 v = *reinterpret_cast<const float4*>(y + j);
+                            float t = __fsub_rn(u.x, v.x);
+                            acc = __fmaf_rn(t, t, acc);
+                            t = __fsub_rn(u.y, v.y);
+                            acc = __fmaf_rn(t, t, acc);
+                            t = __fsub_rn(u.z, v.z);
+                            acc = __fmaf_rn(t, t, acc);
+                            t = __fsub_rn(u.w, v.w);
+                            acc = __fmaf_rn(t, t, acc);
+                        }
+                    } else {
+                        for (int j = 0; j < dl; ++j) {
+                            const float t = __fsub_rn(x[j], y[j]);
+                            acc = __fmaf_rn(t, t, acc);
+                        }
+                    }
+                }
+                open = __ballot_sync(0xffffffffu, ((open >> lane) & 1u) && acc <= far);
+            }
+            keys[32 * gw + lane] = ((open >> lane) & 1u) ? list_key(acc, (uint32_t)id) : kEmptyKey;
+            sync();
+            if (gw == 0) {
+                for (int v = 0; v < W && b + 32 * v < nq; ++v) {
+                    uint64_t cand[1] = {keys[32 * v + lane]}, out;
+                    if (misc[1] >= kSearchFull) {
+                        // the table is no longer exact: drop ids the list
+                        // holds, and repeats
+                        const uint32_t cid = cand[0] == kEmptyKey ? 0xFFFFFFFFu : list_id(cand[0]);
+                        bool drop = (__match_any_sync(0xffffffffu, cid) & ((1u << lane) - 1u)) != 0;
+                        for (int e = 0; e < ks; ++e) {
+                            const uint64_t o = shfl64(list, e);
+                            drop |= o != kEmptyKey && list_id(o) == cid;
+                        }
+                        if (drop) cand[0] = kEmptyKey;
+                    }
+                    __syncwarp();
+                    bool changed;
+                    // the keys are distinct and at most 64, so this never declines
+                    if (warp_merge_few<1>(cand, list, ks, keys + 32 * v, out, changed))
+                        list = lane < ks ? out : kEmptyKey;
+                    __syncwarp();
+                }
+                if (lane == ks - 1 && list != kEmptyKey) *bound = key_dist(list);
+            }
+            sync();
+        }
+        if (gt == 0) misc[0] = 0;
+        sync();
+    };
+    // the queue takes one more round of every thread's id
+    auto make_room = [&] {
+        sync();
+        const bool full = *(volatile int*)misc > kSearchQueue - 32 * W;
+        sync();  // every thread has read it before one appends
+        if (full) process();
+    };
+    for (int a0 = 0; a0 < s; a0 += 32 * W) {
+        make_room();
+        collect(a0 + gt < s ? S[qi * s + a0 + gt] : -1);
     }
-    if (lane < ks) {
+    process();
+    for (int t = 0; t < t0; ++t) {
+        if (gw == 0) {  // the entries not expanded yet
+            const bool open = list != kEmptyKey && (list & 1) == 0;
+            const unsigned bal = __ballot_sync(0xffffffffu, open);
+            if (open) {
+                entry[__popc(bal & ((1u << lane) - 1u))] = (int32_t)list_id(list);
+                list |= 1;
+            }
+            if (lane == 0) misc[2] = __popc(bal);
+        }
+        sync();
+        const int slots = misc[2] * k;
+        if (slots == 0) break;  // every entry's neighbours are visited: nothing can change any more
+        for (int u0 = 0; u0 < slots; u0 += 32 * W) {
+            make_room();
+            const int u = u0 + gt, e = u / k;
+            collect(u < slots ? G[(int64_t)entry[e] * k + (u - e * k)] : -1);
+        }
+        process();
+    }
+    if (gw == 0 && lane < ks) {
         const bool real = list != kEmptyKey;
-        out_ids[qi * ks + lane] = real ? (int32_t)key_id(list) : -1;
+        out_ids[qi * ks + lane] = real ? (int32_t)list_id(list) : -1;
         out_d[qi * ks + lane] = real ? key_dist(list) : __int_as_float(0x7f800000);
     }
 }
 
-}  // namespace
-
-int search_cap_log2(int s, int t0, int ks, int k) {
-    const double visits = (double)s + (double)t0 * ks * k;
-    int c = 6;
-    while (c < 30 && (double)(1ll << c) < 2.0 * visits) ++c;
-    return c;
+template <bool VEC, int W>
+void launch_search_t(const float* X, int64_t n, int D, const int32_t* G, int k, const float* Q, int64_t m,
+                     const int32_t* S, int s, int t0, int ks, int32_t* out_ids, float* out_d, cudaStream_t st) {
+    const size_t smem = search_smem(D, W).total;
+    cudaFuncSetAttribute(k8_search<VEC, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    k8_search<VEC, W><<<(unsigned)m, 32 * W, smem, st>>>(X, n, D, G, k, Q, S, s, t0, ks, out_ids, out_d);
 }
 
-void launch_search(const float* X, int64_t n, int D, const int32_t* G, int k, const float* Q, int64_t q0,
-                   int64_t q1, const int32_t* S, int s, int t0, int ks, int32_t* tab, int cap_log2, int32_t* out_ids,
-                   float* out_d, cudaStream_t st) {
-    if (q1 <= q0) return;
-    const int64_t m = q1 - q0;
-    cudaMemsetAsync(tab, 0xFF, (size_t)(m << cap_log2) * sizeof(int32_t), st);
+}  // namespace
+
+void launch_search(const float* X, int64_t n, int D, const int32_t* G, int k, const float* Q, int64_t m,
+                   const int32_t* S, int s, int t0, int ks, int32_t* out_ids, float* out_d, cudaStream_t st) {
+    if (m <= 0) return;
     // algorithmic bytes: every possible visit reads a row and every expansion a
     // list (an upper bound; the visits actually made are fewer)
     const double visits = (double)s + (double)t0 * ks * k;
     LaunchScope ls("k8_search", st, (double)m * (visits * (D * 4.0 + 8.0) + (double)t0 * ks * k * 4.0 + D * 4.0),
                    (double)m * visits * 3.0 * D);
-    const size_t smem = (size_t)kSearchWarps * D * sizeof(float);
-    const int64_t grid = (m + kSearchWarps - 1) / kSearchWarps;
-    if (D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0) {
-        cudaFuncSetAttribute(k8_search<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k8_search<true><<<(unsigned)grid, 32 * kSearchWarps, smem, st>>>(X, n, D, G, k, Q, q0, q1, S, s, t0, ks, tab,
-                                                                         cap_log2, out_ids, out_d);
-    } else {
-        cudaFuncSetAttribute(k8_search<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k8_search<false><<<(unsigned)grid, 32 * kSearchWarps, smem, st>>>(X, n, D, G, k, Q, q0, q1, S, s, t0, ks,
-                                                                          tab, cap_log2, out_ids, out_d);
+    const bool vec = D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    // with less than two queries per SM the chip is idle anyway: four warps on each
+    const bool few = m <= 2 * 152;
+    for (int64_t q0 = 0; q0 < m; q0 += (int64_t)1 << 30) {  // one CTA per query
+        const int64_t c = std::min(m - q0, (int64_t)1 << 30);
+        const float* Qc = Q + q0 * D;
+        const int32_t* Sc = S ? S + q0 * s : nullptr;
+        int32_t* ic = out_ids + q0 * ks;
+        float* dc = out_d + q0 * ks;
+        if (few && vec) launch_search_t<true, kSearchGroup>(X, n, D, G, k, Qc, c, Sc, s, t0, ks, ic, dc, st);
+        else if (few) launch_search_t<false, kSearchGroup>(X, n, D, G, k, Qc, c, Sc, s, t0, ks, ic, dc, st);
+        else if (vec) launch_search_t<true, 1>(X, n, D, G, k, Qc, c, Sc, s, t0, ks, ic, dc, st);
+        else launch_search_t<false, 1>(X, n, D, G, k, Qc, c, Sc, s, t0, ks, ic, dc, st);
     }
 }
 
