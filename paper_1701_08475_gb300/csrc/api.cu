@@ -1840,7 +1840,9 @@ int knng_rvq_seeds(const float* words1, int W1, const float* words2, int W2, int
         DevBuf<float> w1, w2, Qb;
         DevBuf<int32_t> off, li, Sb;
         float *n1 = nullptr, *n2 = nullptr, *x12 = nullptr, *w1T = nullptr, *w2T = nullptr;
+        SeedWork sw{};
         int* status = nullptr;
+        bool few = rvq_few_seeds(s);  // unless its products do not fit
         for (int ps = 0; ps < 2; ++ps) {
             ws.used = 0;
             bind(ws, w1, words1, (size_t)W1 * D, ps);
@@ -1849,13 +1851,26 @@ int knng_rvq_seeds(const float* words1, int W1, const float* words2, int W2, int
             bind(ws, li, list_ids, (size_t)n, ps);
             bind(ws, Qb, queries, (size_t)m * D, ps);
             bind(ws, Sb, (const int32_t*)seeds, (size_t)m * s, ps);
-            n1 = ws.take<float>(W1);
-            n2 = ws.take<float>(W2);
-            x12 = ws.take<float>((size_t)nk);
-            w1T = ws.take<float>((size_t)W1 * D);
-            w2T = ws.take<float>((size_t)W2 * D);
+            if (few) {
+                const size_t W = (size_t)W1 + W2, batch = (size_t)rvq_seed_batch(m);
+                sw.words = ws.take<float>(W * D);
+                sw.table = ws.take<float>(W * W);
+                sw.self = ws.take<float>(W);
+                sw.part = ws.take<float>((size_t)nk);
+                sw.dots = ws.take<float>(batch * W);
+                sw.qq = ws.take<float>(batch);
+            } else {
+                n1 = ws.take<float>(W1);
+                n2 = ws.take<float>(W2);
+                x12 = ws.take<float>((size_t)nk);
+                w1T = ws.take<float>((size_t)W1 * D);
+                w2T = ws.take<float>((size_t)W2 * D);
+            }
             status = ws.take<int>(4);
-            if (ps == 0) ws.allocate(st);
+            if (ps == 0 && !ws.try_allocate(st, few)) {
+                few = false;
+                ps = -1;
+            }
         }
         cuda_check(cudaMemsetAsync(status, 0, 4 * sizeof(int), st), "status clear");
         upload(w1, st);
@@ -1865,8 +1880,14 @@ int knng_rvq_seeds(const float* words1, int W1, const float* words2, int W2, int
         upload(Qb, st);
         launch_check_finite(Qb.dev, m * (int64_t)D, status, st, w1.dev, (int64_t)W1 * D, w2.dev, (int64_t)W2 * D);
         launch_check_offsets(off.dev, nk, n, status, st);
-        launch_rvq_tables(w1.dev, W1, w2.dev, W2, D, n1, n2, x12, w1T, w2T, st);
-        launch_rvq_seeds(w1T, W1, w2T, W2, D, n1, n2, x12, off.dev, li.dev, Qb.dev, m, probe1, s, Sb.dev, status, st);
+        if (few) {
+            launch_rvq_few_seeds(w1.dev, W1, w2.dev, W2, D, off.dev, li.dev, Qb.dev, m, probe1, s, sw, Sb.dev, status,
+                                 st);
+        } else {
+            launch_rvq_tables(w1.dev, W1, w2.dev, W2, D, n1, n2, x12, w1T, w2T, st);
+            launch_rvq_seeds(w1T, W1, w2T, W2, D, n1, n2, x12, off.dev, li.dev, Qb.dev, m, probe1, s, Sb.dev, status,
+                             st);
+        }
         download(Sb, st);
         cuda_check(launch_error(), "kernel launch");
         check_status(status, st);

@@ -311,6 +311,20 @@ void launch_rvq_key_count(const int32_t* codes, int64_t n, int W2, int32_t* cnt,
 void launch_check_offsets(const int32_t* off, int64_t nk, int64_t n, int* status, cudaStream_t s);
 void launch_rvq_tables(const float* w1, int W1, const float* w2, int W2, int D, float* n1, float* n2, float* x12,
                        float* w1T, float* w2T, cudaStream_t s);
+// Up to 32 seeds per query (rvq_few_seeds) by another route, the same seeds.
+struct SeedWork {
+    float* words;  // [W1 + W2][D]
+    float* table;  // [W1 + W2][W1 + W2]
+    float* self;   // [W1 + W2]
+    float* part;   // [W1 W2]
+    float* dots;   // [rvq_seed_batch(m)][W1 + W2]
+    float* qq;     // [rvq_seed_batch(m)]
+};
+bool rvq_few_seeds(int s_seeds);
+int64_t rvq_seed_batch(int64_t m);
+void launch_rvq_few_seeds(const float* w1, int W1, const float* w2, int W2, int D, const int32_t* off,
+                          const int32_t* ids, const float* Q, int64_t m, int probe1, int s_seeds,
+                          const SeedWork& w, int32_t* S, const int* status, cudaStream_t s);
 int rvq_seed_keys(int probe1, int W2);
 size_t rvq_seeds_smem(int probe1, int W2, int D);
 void launch_rvq_seeds(const float* w1T, int W1, const float* w2T, int W2, int D, const float* n1, const float* n2,

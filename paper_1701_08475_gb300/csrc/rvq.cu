@@ -610,6 +610,326 @@ __global__ void __launch_bounds__(kSdT) k9_seeds(const float* __restrict__ w1T, 
     for (int p = min(total, s) + tid; p < s; p += kSdT) S[qi * s + p] = -1;
 }
 
+// ---------------------------------------------------------------- few seeds
+// For up to 32 seeds per query (kSeedFew): the products of all queries and
+// words as one blocked FP32 product (k9_dots), the query-independent part of
+// every key's distance once (k9_keys), and then one CTA per query picks the
+// kept words and the seeds (k9_few_seeds).  Every float operation is
+// k9_seeds's own.
+constexpr int kSeedFew = 32;
+constexpr int kDotRows = 64, kDotCols = 128, kDotDims = 64, kDotStride = kDotDims + 4;
+constexpr uint32_t kNoList = 0x7FFFDEADu;  // in place of a key's part of the distance: its list is empty
+
+// out[r][c] = a_r . b_c (canonical: dims ascending, fmaf), self[r] = a_r . a_r.
+// 256 threads: 16 row groups x 16 column groups, 4 x 8 products each.
+template <bool VEC>
+__global__ void __launch_bounds__(256) k9_dots(const float* __restrict__ A, int64_t M, const float* __restrict__ B,
+                                              int W, int D, float* __restrict__ out, float* __restrict__ self) {
+    extern __shared__ __align__(16) float dt_smem[];
+    float* as = dt_smem;                          // [kDotRows][kDotStride]
+    float* bs = as + kDotRows * kDotStride;       // [kDotCols][kDotStride]
+    const int tid = threadIdx.x, rg = tid % 16, cg = tid / 16;
+    const int64_t r0 = (int64_t)blockIdx.x * kDotRows;
+    const int c0 = blockIdx.y * kDotCols;
+    float acc[4][8], own = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+    auto stage = [&](float* dst, const float* src, int rows, int64_t first, int64_t count, int d0) {
+        if (VEC) {
+            for (int e = tid; e < rows * (kDotDims / 4); e += 256) {
+                const int r = e / (kDotDims / 4), c = e % (kDotDims / 4) * 4;
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (first + r < count && d0 + c < D)
+                    v = __ldg(reinterpret_cast<const float4*>(src + (first + r) * D + d0 + c));
+                *reinterpret_cast<float4*>(dst + r * kDotStride + c) = v;
+            }
+        } else {
+            for (int e = tid; e < rows * kDotDims; e += 256) {
+                const int r = e / kDotDims, c = e % kDotDims;
+                dst[r * kDotStride + c] = first + r < count && d0 + c < D ? __ldg(src + (first + r) * D + d0 + c) : 0.f;
+            }
+        }
+    };
+    for (int d0 = 0; d0 < D; d0 += kDotDims) {
+        __syncthreads();
+        stage(as, A, kDotRows, r0, M, d0);
+        stage(bs, B, kDotCols, c0, W, d0);
+        __syncthreads();
+        const int dl = (min(kDotDims, D - d0) + 3) & ~3;  // dims past D are zeros: they change no sum
+        for (int dq = 0; dq < dl; dq += 4) {
+            float4 av[4], bv[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                av[i] = *reinterpret_cast<const float4*>(as + (rg + 16 * i) * kDotStride + dq);
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                bv[j] = *reinterpret_cast<const float4*>(bs + (cg + 16 * j) * kDotStride + dq);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    acc[i][j] = __fmaf_rn(av[i].x, bv[j].x, acc[i][j]);
+                    acc[i][j] = __fmaf_rn(av[i].y, bv[j].y, acc[i][j]);
+                    acc[i][j] = __fmaf_rn(av[i].z, bv[j].z, acc[i][j]);
+                    acc[i][j] = __fmaf_rn(av[i].w, bv[j].w, acc[i][j]);
+                }
+        }
+        if (blockIdx.y == 0 && tid < kDotRows) {
+            const float* x = as + tid * kDotStride;
+            for (int d = 0; d < dl; ++d) own = __fmaf_rn(x[d], x[d], own);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int64_t r = r0 + rg + 16 * i;
+            const int c = c0 + cg + 16 * j;
+            if (r < M && c < W) out[r * W + c] = acc[i][j];
+        }
+    if (blockIdx.y == 0 && tid < kDotRows && r0 + tid < M) self[r0 + tid] = own;
+}
+
+// part[a * W2 + b] = fmaf(2, w1_a . w2_b, |w2_b|^2), or kNoList when the key's
+// list is empty.  T, self: products of the stacked words with themselves.
+__global__ void k9_keys(const float* __restrict__ T, const float* __restrict__ self, int W1, int W2,
+                        const int32_t* __restrict__ off, float* __restrict__ part, const int* __restrict__ status) {
+    if (*status & kStatusStop) return;  // the caller's offsets failed their check
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < W1 * W2; e += gridDim.x * blockDim.x) {
+        const int a = e / W2, b = e - a * W2;
+        part[e] = off[e + 1] > off[e] ? __fmaf_rn(2.f, T[(int64_t)a * (W1 + W2) + W1 + b], self[W1 + b])
+                                      : __uint_as_float(kNoList);
+    }
+}
+
+// One CTA per query; its first warp ranks the words and the seeds, all four
+// form and sift the candidates (one warp per query waited for memory most of
+// the time: 344 us for 10,000 queries).  Shared memory: 256 keys, the kept
+// words, the products with the second words, 256 counters, the threads' least
+// distances, the candidate distances (probe1 W2).
+constexpr int kFewKeys = 256, kFewT = 128;
+size_t few_seeds_smem(int p1, int W2) {
+    return (size_t)kFewKeys * 8 + 256 * 8 + 256 * 4 + 260 * 4 + kFewT * 4 + (size_t)p1 * W2 * 4;
+}
+
+// VEC: W2 is a multiple of 4.
+template <bool VEC>
+__global__ void __launch_bounds__(kFewT) k9_few_seeds(const float* __restrict__ dots, const float* __restrict__ qq,
+                                                     const float* __restrict__ self, int W1, int W2, int p1,
+                                                     const float* __restrict__ part, const int32_t* __restrict__ off,
+                                                     const int32_t* __restrict__ ids, int s,
+                                                     int32_t* __restrict__ S, const int* __restrict__ status) {
+    if (*status & kStatusStop) return;
+    extern __shared__ __align__(16) uint64_t fs_smem[];
+    uint64_t* keys = fs_smem;                                        // [kFewKeys]
+    uint64_t* kept = keys + kFewKeys;                                // [256] (term 1, word), the first p1 kept
+    float* qw2 = reinterpret_cast<float*>(kept + 256);               // [256]
+    int* hist = reinterpret_cast<int*>(qw2 + 256);                   // [256]
+    int* count = hist + 256;                                         // keys taken
+    uint32_t* slim = reinterpret_cast<uint32_t*>(count + 1);         // the bound, the least distance
+    uint32_t* lmin = reinterpret_cast<uint32_t*>(hist + 260);        // [kFewT]
+    uint32_t* cand = lmin + kFewT;                                   // [p1 W2] distances (ord32), ~0: no list
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t qi = blockIdx.x;
+    const float* dq = dots + qi * (W1 + W2);
+    uint64_t v[8];
+    if (warp == 0) {
+        // Eqn. 3's term 1 of every stage-1 word; the p1 least are kept
+        const float q2 = qq[qi];
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            const int a = 32 * r + lane;
+            v[r] = a < W1 ? make_key(__fadd_rn(__fadd_rn(__fmaf_rn(-2.f, dq[a], q2), self[a]), 0.f), (uint32_t)a)
+                          : kEmptyKey;
+        }
+        if (p1 <= 32) {
+            uint64_t first[1];
+            sort_regs<8>(v);
+            warp_select_unique<8, 1>(v, p1, first);  // the keys are distinct
+            kept[lane] = first[0];
+        } else {
+            bitonic_sort_keys<8, 1>(v, nullptr);
+#pragma unroll
+            for (int r = 0; r < 8; ++r) kept[8 * lane + r] = v[r];
+        }
+    } else {
+        for (int b = tid - 32; b < W2; b += kFewT - 32) qw2[b] = dq[W1 + b];
+        for (int e = tid - 32; e < 256; e += kFewT - 32) hist[e] = 0;
+        if (tid == 32) *count = 0;
+    }
+    __syncthreads();
+    // d(q, I) of the kept words' keys; each thread's least on the way
+    uint32_t least = 0xFFFFFFFFu;
+    auto distance = [&](float t1, float qw, float c) -> uint32_t {
+        if (__float_as_uint(c) == kNoList) return 0xFFFFFFFFu;
+        return min(0xFFFFFFFEu, ord32(__fadd_rn(__fadd_rn(t1, __fmaf_rn(-2.f, qw, c)), 0.f)));
+    };
+    for (int r = warp; r < p1; r += kFewT / 32) {
+        const uint64_t kk = kept[r];
+        const float t1 = key_dist(kk);
+        const float* pr = part + (int64_t)key_id(kk) * W2;
+        if (VEC) {
+            for (int b = 4 * lane; b < W2; b += 128) {
+                const float4 c = __ldg(reinterpret_cast<const float4*>(pr + b));
+                const float4 w = *reinterpret_cast<const float4*>(qw2 + b);
+                const uint4 u = make_uint4(distance(t1, w.x, c.x), distance(t1, w.y, c.y), distance(t1, w.z, c.z),
+                                           distance(t1, w.w, c.w));
+                *reinterpret_cast<uint4*>(cand + r * W2 + b) = u;
+                least = min(least, min(min(u.x, u.y), min(u.z, u.w)));
+            }
+        } else {
+            for (int b = lane; b < W2; b += 32) {
+                const uint32_t u = distance(t1, qw2[b], __ldg(pr + b));
+                cand[r * W2 + b] = u;
+                least = min(least, u);
+            }
+        }
+    }
+    lmin[tid] = least;
+    __syncthreads();
+    // The s-th least of the threads' least distances bounds the s-th least of
+    // all: only keys up to it can be among the first s (every list gives at
+    // least one seed).  The near words of the second stage crowd into few
+    // threads, so the bound can be loose: the keys up to it are counted in 256
+    // even steps, and the bound becomes the end of the step with the s-th.
+    int below = 0;
+    uint32_t mn = 0xFFFFFFFFu;
+    for (int j = 0; j < kFewT; j += 4) {
+        const uint4 o = *reinterpret_cast<const uint4*>(lmin + j);
+        mn = min(mn, min(min(o.x, o.y), min(o.z, o.w)));
+        below += (o.x < least || (o.x == least && j < tid)) + (o.y < least || (o.y == least && j + 1 < tid)) +
+                 (o.z < least || (o.z == least && j + 2 < tid)) + (o.w < least || (o.w == least && j + 3 < tid));
+    }
+    if (below == s - 1) *slim = min(least, 0xFFFFFFFEu);
+    __syncthreads();
+    uint32_t lim = *slim;
+    const int nc = p1 * W2;
+    if (mn <= lim) {  // the same for every thread
+        const int sft = max(0, 24 - __clz((int)(lim - mn)));
+        auto tally = [&](uint32_t u) {
+            if (u <= lim) atomicAdd(hist + ((u - mn) >> sft), 1);
+        };
+        for (int e = (VEC ? 4 : 1) * tid; e < nc; e += (VEC ? 4 : 1) * kFewT) {
+            if (VEC) {
+                const uint4 u = *reinterpret_cast<const uint4*>(cand + e);
+                tally(u.x);
+                tally(u.y);
+                tally(u.z);
+                tally(u.w);
+            } else {
+                tally(cand[e]);
+            }
+        }
+        __syncthreads();
+        if (warp == 0) {
+            int c[8], sum = 0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                c[j] = hist[8 * lane + j];
+                sum += c[j];
+            }
+            int run = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, run, o);
+                if (lane >= o) run += y;
+            }
+            const unsigned got = __ballot_sync(0xffffffffu, run >= s);
+            run -= sum;
+            int step = 8 * lane;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (run + c[j] >= s) break;
+                run += c[j];
+                ++step;
+            }
+            if (got && lane == __ffs(got) - 1)  // else fewer than s keys
+                *slim = min(lim, mn + (uint32_t)((((uint64_t)step + 1) << sft) - 1));
+        }
+        __syncthreads();
+        lim = *slim;
+    }
+    auto take = [&](uint32_t u, int e) {
+        if (u > lim) return;
+        const int at = atomicAdd(count, 1);
+        const int r = e / W2;
+        if (at < kFewKeys) keys[at] = ((uint64_t)u << 32) | (key_id(kept[r]) * (uint32_t)W2 + (e - r * W2));
+    };
+    for (int e = (VEC ? 4 : 1) * tid; e < nc; e += (VEC ? 4 : 1) * kFewT) {
+        if (VEC) {
+            const uint4 u = *reinterpret_cast<const uint4*>(cand + e);
+            if (min(min(u.x, u.y), min(u.z, u.w)) > lim) continue;
+            take(u.x, e);
+            take(u.y, e + 1);
+            take(u.z, e + 2);
+            take(u.w, e + 3);
+        } else {
+            take(cand[e], e);
+        }
+    }
+    __syncthreads();
+    if (warp > 0) return;
+    const int total = *count;
+    if (total <= 32) {
+        const uint64_t one = warp_sort32(lane < total ? keys[lane] : kEmptyKey);
+        __syncwarp();
+        keys[lane] = one;
+    } else if (total <= 64) {
+        uint64_t two[2] = {keys[lane], lane + 32 < total ? keys[lane + 32] : kEmptyKey};
+        __syncwarp();
+        bitonic_sort_keys<2, 1>(two, nullptr);
+        if (lane < 16) {
+            keys[2 * lane] = two[0];
+            keys[2 * lane + 1] = two[1];
+        }
+    } else if (total <= kFewKeys) {
+#pragma unroll
+        for (int r = 0; r < 8; ++r) v[r] = 32 * r + lane < total ? keys[32 * r + lane] : kEmptyKey;
+        __syncwarp();
+        bitonic_sort_keys<8, 1>(v, nullptr);
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+            if (8 * lane + r < 32) keys[8 * lane + r] = v[r];
+    } else {  // crowded: the least key above the last one, s times
+        uint64_t last = 0;
+        for (int t = 0; t < 32; ++t) {
+            uint64_t m = kEmptyKey;
+            for (int e = lane; e < nc; e += 32) {
+                const int r = e / W2;
+                const uint64_t key = ((uint64_t)cand[e] << 32) | (key_id(kept[r]) * (uint32_t)W2 + (e - r * W2));
+                if (cand[e] != 0xFFFFFFFFu && (t == 0 || key > last)) m = min(m, key);
+            }
+            m = warp_min64(m);
+            if (lane == 0) keys[t] = m;
+            last = m;
+            if (m == kEmptyKey) {
+                for (int q = t + lane; q < 32; q += 32) keys[q] = kEmptyKey;
+                break;
+            }
+        }
+    }
+    __syncwarp();
+    // the lists in that order
+    const uint64_t key = keys[lane];
+    int a0 = 0, len = 0;
+    if (key != kEmptyKey) {
+        a0 = off[key_id(key)];
+        len = min(off[key_id(key) + 1] - a0, s);
+    }
+    int end = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, end, o);
+        if (lane >= o) end += y;
+    }
+    int32_t* out = S + qi * s;
+    for (int t = 0, p = end - len; t < len && p < s; ++t, ++p) out[p] = ids[a0 + t];
+    const int all = __shfl_sync(0xffffffffu, end, 31);
+    for (int p = all + lane; p < s; p += 32) out[p] = -1;
+}
+
 int grid_for_count(int64_t count) {
     const int64_t g = (count + 255) / 256;
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, 152 * 16));
@@ -693,6 +1013,49 @@ void launch_rvq_tables(const float* w1, int W1, const float* w2, int W2, int D, 
     LaunchScope ls("k9_tables", s, (double)(W1 + W2) * D * 12.0 + (double)W1 * W2 * 4.0,
                    (double)(W1 + 1) * (W2 + 1) * D * 2.0);
     k9_tables<<<grid_for_count((int64_t)W1 * W2), 256, 0, s>>>(w1, W1, w2, W2, D, n1, n2, x12, w1T, w2T);
+}
+
+bool rvq_few_seeds(int s_seeds) { return s_seeds <= kSeedFew; }
+
+int64_t rvq_seed_batch(int64_t m) { return std::min<int64_t>(m, 65536); }
+
+namespace {
+void launch_dots(const float* A, int64_t M, const float* B, int W, int D, float* out, float* self, cudaStream_t s) {
+    LaunchScope ls("k9_dots", s, ((double)M + W) * D * 4.0 + (double)M * W * 4.0, (double)M * W * D * 2.0);
+    const dim3 grid((unsigned)((M + kDotRows - 1) / kDotRows), (unsigned)((W + kDotCols - 1) / kDotCols));
+    const size_t smem = (size_t)(kDotRows + kDotCols) * kDotStride * 4;
+    if (D % 4 == 0 && ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0) {
+        cudaFuncSetAttribute(k9_dots<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k9_dots<true><<<grid, 256, smem, s>>>(A, M, B, W, D, out, self);
+    } else {
+        cudaFuncSetAttribute(k9_dots<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k9_dots<false><<<grid, 256, smem, s>>>(A, M, B, W, D, out, self);
+    }
+}
+}  // namespace
+
+void launch_rvq_few_seeds(const float* w1, int W1, const float* w2, int W2, int D, const int32_t* off,
+                          const int32_t* ids, const float* Q, int64_t m, int probe1, int s_seeds,
+                          const SeedWork& w, int32_t* S, const int* status, cudaStream_t s) {
+    const int W = W1 + W2;
+    cudaMemcpyAsync(w.words, w1, sizeof(float) * W1 * D, cudaMemcpyDeviceToDevice, s);
+    cudaMemcpyAsync(w.words + (size_t)W1 * D, w2, sizeof(float) * W2 * D, cudaMemcpyDeviceToDevice, s);
+    launch_dots(w.words, W, w.words, W, D, w.table, w.self, s);
+    {
+        LaunchScope ls("k9_keys", s, (double)W1 * W2 * 16.0, 0);
+        k9_keys<<<grid_for_count((int64_t)W1 * W2), 256, 0, s>>>(w.table, w.self, W1, W2, off, w.part, status);
+    }
+    const size_t smem = few_seeds_smem(probe1, W2);
+    auto kernel = W2 % 4 == 0 ? k9_few_seeds<true> : k9_few_seeds<false>;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int64_t batch = rvq_seed_batch(m);
+    for (int64_t q0 = 0; q0 < m; q0 += batch) {
+        const int64_t c = std::min(batch, m - q0);
+        launch_dots(Q + q0 * D, c, w.words, W, D, w.dots, w.qq, s);
+        LaunchScope ls("k9_seeds", s, (double)c * (W * 4.0 + (double)probe1 * W2 * 4.0 + s_seeds * 8.0), 0);
+        kernel<<<(unsigned)c, kFewT, smem, s>>>(w.dots, w.qq, w.self, W1, W2, probe1, w.part, off, ids, s_seeds,
+                                                  S + q0 * s_seeds, status);
+    }
 }
 
 int rvq_seed_keys(int probe1, int W2) {

@@ -597,61 +597,6 @@ __global__ void __launch_bounds__(1024) k1_select_small(const float* __restrict_
     }
 }
 
-__host__ __device__ constexpr int ilog2c(int x) { return x <= 1 ? 0 : 1 + ilog2c(x / 2); }
-
-// Ascending bitonic sort of 32 R NW keys held by NW warps (R per lane;
-// element e = 32 R warp + R lane + r): exchanges within a lane for distances
-// below R, across lanes by shuffles up to 32 R, across warps through shared
-// memory (xch: 32 R NW keys) above.
-template <int R, int NW>
-__device__ __forceinline__ void bitonic_sort_keys(uint64_t (&v)[R], uint64_t* xch) {
-    const int lane = threadIdx.x & 31, warp = NW > 1 ? (int)(threadIdx.x >> 5) : 0;
-    constexpr int LOG = ilog2c(32 * R * NW);
-    static_assert((32 * R * NW) == (1 << LOG), "R and NW are powers of two");
-    const int e0 = 32 * R * warp + R * lane;  // element of v[0]
-#pragma unroll
-    for (int lk = 1; lk <= LOG; ++lk) {
-#pragma unroll
-        for (int lj = LOG - 1; lj >= 0; --lj) {  // constant trip count: unrolls fully
-            const int k = 1 << lk, j = 1 << lj;
-            if (lj < lk && j >= 32 * R) {
-                const int wj = j / (32 * R);
-                // the direction bit and the pair are warp bits
-                const bool keep_min = ((warp & wj) == 0) == ((e0 & k) == 0);
-#pragma unroll
-                for (int r = 0; r < R; ++r) xch[r * 32 * NW + threadIdx.x] = v[r];
-                __syncthreads();
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const uint64_t o = xch[r * 32 * NW + (threadIdx.x ^ (32 * wj))];
-                    v[r] = keep_min ? (o < v[r] ? o : v[r]) : (o > v[r] ? o : v[r]);
-                }
-                __syncthreads();
-            } else if (lj < lk && j >= R) {
-                const int lj2 = j / R;
-                // k > j >= R: the direction bit of the pair is a lane or warp bit
-                const bool keep_min = ((lane & lj2) == 0) == ((e0 & k) == 0);
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const uint64_t o = shfl_xor64(v[r], lj2);
-                    v[r] = keep_min ? (o < v[r] ? o : v[r]) : (o > v[r] ? o : v[r]);
-                }
-            } else if (lj < lk) {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    if ((r & j) == 0) {
-                        const bool up = ((e0 + r) & k) == 0;
-                        const uint64_t x = v[r], y = v[r | j];
-                        const bool sw = (x > y) == up;
-                        v[r] = sw ? y : x;
-                        v[r | j] = sw ? x : y;
-                    }
-                }
-            }
-        }
-    }
-}
-
 // Segments of up to 32 R NW points: NW warps hold a segment's keys in
 // registers, sort them and take the floor(m/2)-th smallest.  NW = 1: four
 // segments per CTA, one per warp; NW > 1: one segment per CTA.  On the final
