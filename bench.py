@@ -482,8 +482,7 @@ OTHER_CONFIGS = [
 def measure_config(knng, name, forms, cpu_n, steps, dev, stream, recall_rows=2000):
     """One workload: for each form, `steps` direct builds timed with CUDA
     events after one warm-up, a further build with events around every launch
-    (per-kernel times, the dominant kernel's roofline, the certificate's
-    fallback rows), recall@k against exact lists on sampled rows and the
+    (per-kernel times, the dominant kernel's roofline), recall@k against exact lists on sampled rows and the
     distance error against FP64; the graphs of the forms compared; the oracle
     timed single-threaded on a bounded draw of the same recipe."""
     import torch
@@ -527,7 +526,6 @@ def measure_config(knng, name, forms, cpu_n, steps, dev, stream, recall_rows=200
         st = knng.stats()
         roof = roofline(st, None, name, 1)
         roof["share_of_step"] = round(st[roof["kernel"]]["ms"] / ms_k, 4)
-        leaf = [v for key, v in st.items() if key.startswith("k2_leaf_") and key != "k2_leaf_fp32"]
         r_ids, r_tie = knng.knng_recall(ids, dists, gi, gd, smp_d)
         form = {"value": round(n * steps / (ms * 1e-3), 1), "unit": "points/s", "ms_per_step": round(ms / steps, 3),
                 "timed": "CUDA-graph replays of the recorded build", "replay_equals_direct": replay_same,
@@ -537,9 +535,6 @@ def measure_config(knng, name, forms, cpu_n, steps, dev, stream, recall_rows=200
                 "roofline": roof,
                 "whole_build_roofline": whole_build_roofline(st, None, 1, ms / steps),
                 "kernels_ms": {key: round(v["ms"], 3) for key, v in sorted(st.items(), key=lambda kv: -kv[1]["ms"])[:6]}}
-        if leaf:
-            form["certificate_fallback_rows"] = {"rows": int(leaf[0]["items"]), "of": n * cfg["tree_passes"],
-                                                 "rate": round(leaf[0]["items"] / (n * cfg["tree_passes"]), 4)}
         out["forms"][prec] = form
         if first is None:
             first = (ids, dists)

@@ -64,12 +64,13 @@ enum knng_join_mode {
 
 enum knng_precision {
     KNNG_FP32 = 0,         /* canonical FP32 everywhere */
-    KNNG_BF16 = 1,         /* leaf Gram on tensor cores from a BF16 copy, certified FP32 re-rank */
+    KNNG_BF16 = 1,         /* leaf and join Grams on tensor cores from a BF16 copy where it is exact */
     KNNG_FP16 = 2,         /* the same from an FP16 copy */
-    KNNG_FP8 = 3           /* the same from an FP8 E4M3 copy, each row scaled by max|x| / 448 */
-    /* With BF16/FP16 the graph is identical to the FP32 one: every row whose
-     * low-precision selection cannot be certified by the error bound is
-     * recomputed in FP32.  Leaves above 128 points use the FP32 leaf kernel. */
+    KNNG_FP8 = 3           /* E4M3 rows scaled by max|x| / 448 (never exact; see knng_leaf_dhat) */
+    /* The graph is identical to the FP32 one: a 16-bit copy is used where
+     * every product and sum of it is an exact integer in FP32; other data, and
+     * FP8 builds, take the FP32 leaf, which measured faster than tensor-core
+     * distances with an exact FP32 re-rank at every size. */
 };
 
 typedef struct knng_params {

@@ -573,15 +573,15 @@ struct BuildLayout {
     JoinBuffers jb{};
     int32_t *perm_a = nullptr, *perm_b = nullptr, *plan_dev = nullptr;
     uint64_t *G = nullptr, *G2 = nullptr;
-    int* status = nullptr;  // [0] status bits, [1] rows re-ranked exactly after a failed certificate
+    int* status = nullptr;  // status bits
     int64_t nodes_per_chunk = 0;
     // low-precision leaf stage
     uint16_t* Xl = nullptr;
-    float *lp_nrm = nullptr, *lp_err = nullptr, *lp_scale = nullptr;
+    float* lp_nrm = nullptr;
     int* notexact = nullptr;
     // tensor-core join
     uint16_t* Xq = nullptr;
-    float *q_nrm = nullptr, *q_err = nullptr, *q_scale = nullptr;
+    float *q_nrm = nullptr, *q_err = nullptr;
     // byte copy for the tree sweeps
     uint8_t* Xb = nullptr;
     int* bflag = nullptr;
@@ -622,17 +622,17 @@ void make_bytes(const float* X, const Args& a, BuildLayout& b, cudaStream_t s) {
 }
 
 // Quantisation type of the low-precision copy for a precision (0 FP16, 1
-// BF16, 2 FP8 E4M3) and the name of its leaf kernel.
+// BF16, 2 FP8 E4M3).
 int qtype(int precision) { return precision == KNNG_BF16 ? 1 : precision == KNNG_FP16 ? 0 : 2; }
-const char* leaf_kernel_name(int precision) {
-    return precision == KNNG_BF16 ? "k2_leaf_bf16" : precision == KNNG_FP16 ? "k2_leaf_fp16" : "k2_leaf_fp8";
-}
+// Whether a build keeps the copy: the leaf, the join and the sweeps read it
+// when it is exact, which an FP8 copy never is.
+bool lp_copy(int precision) { return precision == KNNG_BF16 || precision == KNNG_FP16; }
 
 // Original-order 16-bit copy for the tensor-core stages (also sets the
 // exactness flag); nothing in FP32.
 void quantize_for_join(const float* X, const Args& a, BuildLayout& b, cudaStream_t s) {
     if (!b.Xq) return;
-    launch_quantize(X, a.n, a.D, nullptr, qtype(a.p.precision), b.Xq, b.q_nrm, b.q_err, b.q_scale, b.notexact, s);
+    launch_quantize(X, a.n, a.D, nullptr, qtype(a.p.precision), b.Xq, b.q_nrm, b.q_err, nullptr, b.notexact, s);
     if (b.jb.capture) return;  // a graph records no host reads
     // the kernels pick their path from the device flag; the host copy only
     // sizes the statistics' algorithmic bytes
@@ -643,7 +643,7 @@ void quantize_for_join(const float* X, const Args& a, BuildLayout& b, cudaStream
 }
 
 bool lp_leaf(const Args& a, const TreePlan& tp) {
-    return a.p.precision != KNNG_FP32 && a.p.tree_passes > 0 && tp.max_leaf <= 256;
+    return lp_copy(a.p.precision) && a.p.tree_passes > 0 && tp.max_leaf <= 256;
 }
 
 void carve(Workspace& ws, BuildLayout& b, const Args& a, const TreePlan& tp, bool tree, bool join) {
@@ -651,25 +651,18 @@ void carve(Workspace& ws, BuildLayout& b, const Args& a, const TreePlan& tp, boo
     const int k = a.p.k, D = a.D;
     b.status = ws.take<int>(4);
     b.G = ws.take<uint64_t>((size_t)n * k);
-    bool lp_any = a.p.precision != KNNG_FP32;
+    const bool lp_any = lp_copy(a.p.precision);
     if (lp_any) b.notexact = ws.take<int>(4);
-    const int qt = qtype(a.p.precision);
-    const size_t row_halves = (size_t)lp_row_bytes(D, qt) / 2;
+    const size_t row_halves = (size_t)lp_dim(D);
     if (tree && lp_leaf(a, tp)) {
         b.Xl = ws.take<uint16_t>((size_t)n * row_halves);
         b.lp_nrm = ws.take<float>(n);
-        b.lp_err = ws.take<float>(n);
-        if (qt == 2) b.lp_scale = ws.take<float>(n);
     }
     if (lp_any && (join || tree)) {  // original-order low-precision copy
         b.Xq = ws.take<uint16_t>((size_t)n * row_halves);
         b.q_nrm = ws.take<float>(n);
         b.q_err = ws.take<float>(n);
-        if (qt == 2) b.q_scale = ws.take<float>(n);
     }
-    // the tensor-core join and the tree sweeps read a 16-bit copy when it is
-    // exact; an FP8 copy never is
-    lp_any = lp_any && qt != 2;
     if (join && lp_any) {  // the tensor-core join reads the original-order copy
         b.jb.lp = true;
         b.jb.bf16 = a.p.precision == KNNG_BF16;
@@ -782,13 +775,11 @@ int grid_1d(int64_t count) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, 152 * 16));
 }
 
-void check_status(const int* dstatus, cudaStream_t s, const char* fallback_kernel = nullptr) {
-    int hs[2] = {0, 0};
-    cuda_check(cudaMemcpyAsync(hs, dstatus, sizeof hs, cudaMemcpyDeviceToHost, s), "status read");
+void check_status(const int* dstatus, cudaStream_t s) {
+    int st = 0;
+    cuda_check(cudaMemcpyAsync(&st, dstatus, sizeof st, cudaMemcpyDeviceToHost, s), "status read");
     cuda_check(cudaStreamSynchronize(s), "stream synchronize");
     reg().flush();
-    if (fallback_kernel) record_items(fallback_kernel, (double)hs[1]);
-    const int st = hs[0];
     if (st & kStatusTimeout) fail(KNNG_ETIMEOUT, "a bounded device wait ran out");
     if (st & kStatusNonFinite) fail(KNNG_EINVAL, "data holds a non-finite value");
     if (st & kStatusBadInput) fail(KNNG_EINVAL, "an id or offset given by the caller is out of range");
@@ -875,7 +866,7 @@ void prepare_rows(const float* X, int64_t r0, int64_t rows, const Args& a, Build
         const int qt = qtype(a.p.precision);
         launch_quantize(X + r0 * D, rows, D, nullptr, qt,
                         reinterpret_cast<uint8_t*>(b.Xq) + r0 * (int64_t)lp_row_bytes(D, qt), b.q_nrm + r0,
-                        b.q_err + r0, b.q_scale ? b.q_scale + r0 : nullptr, b.notexact, s);
+                        b.q_err + r0, nullptr, b.notexact, s);
     }
     if (b.Xb) launch_bytes(X + r0 * D, rows, D, byte_dim(D), b.Xb + r0 * byte_dim(D), b.bflag, s);
 }
@@ -895,8 +886,6 @@ void build_core(const float* X, const Args& a, BuildLayout& b, const TreePlan& t
                    "plan upload");
     const bool lp = lp_leaf(a, tp);
     const int qt = qtype(a.p.precision);
-    // re-ranked candidates per row: k plus a margin, at most 63
-    const int kp = std::min(63, k + std::max(k / 2, 8));
     if (b.notexact) cuda_check(cudaMemsetAsync(b.notexact, 0, sizeof(int), s), "flag clear");
     if (b.Xb) cuda_check(cudaMemsetAsync(b.bflag, 0, sizeof(int), s), "flag clear");
     SideStreams side_local;
@@ -964,14 +953,18 @@ void build_core(const float* X, const Args& a, BuildLayout& b, const TreePlan& t
         int32_t* perm = perms[pass];
         const int32_t* leaf_off = b.plan_dev + tp.leaf_off_at;
         const int nleaf = (int)(tp.off[tp.L].size() - 1);
-        bool done = false;
-        if (lp) {
-            launch_permute16(b.Xq, b.q_nrm, b.q_err, b.q_scale, n, lp_row_bytes(a.D, qt), perm, b.Xl, b.lp_nrm,
-                             b.lp_err, b.lp_scale, s);
-            done = launch_leaf_tc(b.Xl, n, X, a.D, perm, leaf_off, nleaf, tp.max_leaf, b.lp_nrm, b.lp_err,
-                                  b.lp_scale, k, kp, qt, b.G, b.status, b.notexact, s);
+        // the tensor-core leaf when the 16-bit copy is exact, else the FP32
+        // leaf; in a capture both are launched and the device flag decides
+        const bool tc = lp && (b.jb.capture || b.sb.q16_host);
+        bool tc_on = false;
+        if (tc) {
+            launch_permute16(b.Xq, b.q_nrm, n, lp_row_bytes(a.D, qt), perm, b.Xl, b.lp_nrm, b.notexact, s);
+            tc_on = launch_leaf_tc(b.Xl, n, a.D, perm, leaf_off, nleaf, tp.max_leaf, b.lp_nrm, nullptr, k, qt, b.G,
+                                   b.status, b.notexact, s);
         }
-        if (!done) launch_leaf_fp32(X, a.D, perm, leaf_off, nleaf, tp.max_leaf, k, b.G, b.status, s);
+        if (!tc_on || b.jb.capture)
+            launch_leaf_fp32(X, a.D, perm, leaf_off, nleaf, tp.max_leaf, k, b.G, b.status, s,
+                             tc_on ? b.notexact : nullptr);
         const int slot = pass - (a.p.tree_passes - b.jb.npass);
         if (b.lid && slot >= 0) launch_leaf_ids(perm, leaf_off, nleaf, n, slot, b.lid, s);
         // the next partition on this pass's slot may reuse its permutations
@@ -1053,8 +1046,7 @@ int knng_build_ex(const float* data, int64_t n, int D, const knng_params* p, int
         download(oi, s);
         download(od, s);
         cuda_check(launch_error(), "kernel launch");
-        check_status(b.status, s,
-                     lp_leaf(a, tp) ? leaf_kernel_name(p->precision) : nullptr);
+        check_status(b.status, s);
         offers_end(b);
     });
 }
@@ -1176,7 +1168,7 @@ int knng_build_batched(int n_inst, const knng_instance* inst, const knng_params*
             offers_begin(g.b, s);
             run_group(g, inst, s);
             cuda_check(launch_error(), "kernel launch");
-            check_status(g.b.status, s, lp_leaf(g.a, g.tp) ? leaf_kernel_name(p->precision) : nullptr);
+            check_status(g.b.status, s);
             offers_end(g.b);
         }
     });
@@ -1581,8 +1573,8 @@ int knng_leaf_dhat(const float* data, int64_t m, int D, int precision, float* ou
         // scales: FP8 writes them; 16-bit copies have none (1)
         if (qt != 2) launch_fill_value(sc.dev, m, 1.f, s);
         launch_quantize(X.dev, m, D, nullptr, qt, Xq, nr.dev, er.dev, qt == 2 ? sc.dev : nullptr, notexact, s);
-        if (!launch_leaf_tc(Xq, m, X.dev, D, perm, off, 1, (int)m, nr.dev, er.dev, qt == 2 ? sc.dev : nullptr, 1, 1,
-                            qt, G, status, notexact, s, dh.dev))
+        if (!launch_leaf_tc(Xq, m, D, perm, off, 1, (int)m, nr.dev, qt == 2 ? sc.dev : nullptr, 1, qt, G, status,
+                            notexact, s, dh.dev))
             fail(KNNG_ECUDA, "the tensor-core leaf kernel cannot run for D = %d", D);
         launch_lp_to_float(Xq, m, D, qt, q.dev, s);
         download(dh, s);

@@ -119,8 +119,10 @@ void run_split_level(const float* X, int64_t n_rows, int D, const LevelPlan& lp,
 // ---------------------------------------------------------------- leaf stage (K2)
 // For every leaf l (perm[leaf_off[l] .. leaf_off[l+1]), 2..256 points): all
 // pairs, canonical FP32 distances, merged into the key graph G (n x k).
+// skip_if_exact: return at once when this flag says the 16-bit copy is exact.
 void launch_leaf_fp32(const float* X, int D, const int32_t* perm, const int32_t* leaf_off,
-                      int nleaf, int max_leaf, int k, uint64_t* G, const int* status, cudaStream_t s);
+                      int nleaf, int max_leaf, int k, uint64_t* G, const int* status, cudaStream_t s,
+                      const int* skip_if_exact = nullptr);
 
 // ---------------------------------------------------------------- low precision (K0, K2 tensor cores, K3)
 int lp_dim(int D);  // D rounded up to the 64-element rows of the swizzled tiles
@@ -138,22 +140,20 @@ void launch_bytes(const float* X, int64_t n, int D, int Db, uint8_t* Xb, int* bf
 // the low-precision arithmetic is not exact for this input (always for FP8).
 void launch_quantize(const float* X, int64_t n, int D, const int32_t* perm, int qt, void* Xq, float* nrm,
                      float* qerr, float* scale, int* notexact, cudaStream_t s);
-// Leaf-order gather of a low-precision copy (with its norms, errors and
-// scales; scale may be NULL).
-void launch_permute16(const void* Xq, const float* nrm, const float* qerr, const float* scale, int64_t n,
-                      int row_bytes, const int32_t* perm, void* Xl, float* lnrm, float* lerr, float* lscale,
-                      cudaStream_t s);
-// Leaf stage on tcgen05 from the leaf-order copy; false when it cannot run
-// (leaf above 256 points, no tensor-map encoder) and nothing was launched.
-// status[1] counts the rows whose first batch of exact evaluations did not
-// settle them.  dump (a parity hook, one leaf of m points): the m x m
-// approximate distances are written there and nothing is selected.
+// Leaf-order gather of a 16-bit copy with its norms; nothing on the device
+// unless the copy is exact.
+void launch_permute16(const void* Xq, const float* nrm, int64_t n, int row_bytes, const int32_t* perm, void* Xl,
+                      float* lnrm, const int* notexact, cudaStream_t s);
 // The values of a low-precision copy as FP32 (m x D; FP8: the unscaled q).
 void launch_lp_to_float(const void* Xq, int64_t m, int D, int qt, float* out, cudaStream_t s);
-bool launch_leaf_tc(const void* Xl, int64_t n, const float* X, int D, const int32_t* perm,
-                    const int32_t* leaf_off, int nleaf, int max_leaf, const float* nrm, const float* qerr,
-                    const float* scale, int k, int kp, int qt, uint64_t* G, int* status, const int* notexact,
-                    cudaStream_t s, float* dump = nullptr);
+// Leaf stage on tcgen05 from the leaf-order copy, on the device only when the
+// copy is exact; false when it cannot run (leaf above 256 points, no
+// tensor-map encoder) and nothing was launched.  dump (a parity hook, one leaf
+// of m points): the m x m approximate distances are written there, exact or
+// not, and nothing is selected.
+bool launch_leaf_tc(const void* Xl, int64_t n, int D, const int32_t* perm, const int32_t* leaf_off, int nleaf,
+                    int max_leaf, const float* nrm, const float* scale, int k, int qt, uint64_t* G, int* status,
+                    const int* notexact, cudaStream_t s, float* dump = nullptr);
 
 // ---------------------------------------------------------------- refinement (K4-K6)
 struct JoinBuffers {

@@ -50,9 +50,14 @@ __global__ void __launch_bounds__(LeafCfg<MC>::NT, NB) k2_leaf_fp32(const float*
                                                                  const int32_t* __restrict__ perm,
                                                                  const int32_t* __restrict__ leaf_off, int k,
                                                                  uint64_t* __restrict__ G,
-                                                                 const int* __restrict__ status) {
+                                                                 const int* __restrict__ status,
+                                                                 const int* __restrict__ skip_if_exact) {
     using C = LeafCfg<MC>;
     if (*status & kStatusStop) return;  // ids or offsets failed their check
+    if (skip_if_exact) {  // the tensor-core leaf did this pass
+        const int f = *skip_if_exact;
+        if ((f & 1) == 0 && !((f & 2) && (f & 4))) return;
+    }
     constexpr int NS = MC / 32 + NSG;
     extern __shared__ float4 smem4[];
     int dch, nch, stride;
@@ -211,19 +216,19 @@ __global__ void __launch_bounds__(LeafCfg<MC>::NT, NB) k2_leaf_fp32(const float*
 
 template <int MC, int NSG, int NB>
 void launch_leaf_t(const float* X, int D, const int32_t* perm, const int32_t* leaf_off, int nleaf, int k,
-                   uint64_t* G, const int* status, cudaStream_t s) {
+                   uint64_t* G, const int* status, cudaStream_t s, const int* skip) {
     using C = LeafCfg<MC>;
     int dch, nch, stride;
     leaf_chunk(D, MC, &dch, &nch, &stride);
     const size_t smem = (size_t)(nch > 1 ? 2 : 1) * MC * stride * 4 + (size_t)C::RB * (MC + 1) * 4 + MC * 4 + (C::NT / 32) * 32 * 8;
     cudaFuncSetAttribute(k2_leaf_fp32<MC, NSG, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k2_leaf_fp32<MC, NSG, NB><<<nleaf, C::NT, smem, s>>>(X, D, perm, leaf_off, k, G, status);
+    k2_leaf_fp32<MC, NSG, NB><<<nleaf, C::NT, smem, s>>>(X, D, perm, leaf_off, k, G, status, skip);
 }
 
 }  // namespace
 
 void launch_leaf_fp32(const float* X, int D, const int32_t* perm, const int32_t* leaf_off, int nleaf,
-                      int max_leaf, int k, uint64_t* G, const int* status, cudaStream_t s) {
+                      int max_leaf, int k, uint64_t* G, const int* status, cudaStream_t s, const int* skip_if_exact) {
     // algorithmic work: every leaf row once, every ordered pair once
     const double mm = (double)max_leaf;
     LaunchScope ls("k2_leaf_fp32", s, (double)nleaf * mm * (D * 4.0 + 2 * 8.0 * k),
@@ -234,17 +239,17 @@ void launch_leaf_fp32(const float* X, int D, const int32_t* perm, const int32_t*
         // of 122): 400,000 x 64 1.35 -> 1.20 ms for three passes; from 128 dims
         // on shared memory allows fewer and the registers are worth more (1.73
         // against 1.83 ms)
-        if (two) launch_leaf_t<64, 2, 6>(X, D, perm, leaf_off, nleaf, k, G, status, s);
-        else launch_leaf_t<64, 1, 6>(X, D, perm, leaf_off, nleaf, k, G, status, s);
+        if (two) launch_leaf_t<64, 2, 6>(X, D, perm, leaf_off, nleaf, k, G, status, s, skip_if_exact);
+        else launch_leaf_t<64, 1, 6>(X, D, perm, leaf_off, nleaf, k, G, status, s, skip_if_exact);
     } else if (max_leaf <= 64) {
-        if (two) launch_leaf_t<64, 2, 1>(X, D, perm, leaf_off, nleaf, k, G, status, s);
-        else launch_leaf_t<64, 1, 1>(X, D, perm, leaf_off, nleaf, k, G, status, s);
+        if (two) launch_leaf_t<64, 2, 1>(X, D, perm, leaf_off, nleaf, k, G, status, s, skip_if_exact);
+        else launch_leaf_t<64, 1, 1>(X, D, perm, leaf_off, nleaf, k, G, status, s, skip_if_exact);
     } else if (max_leaf <= 128) {
-        if (two) launch_leaf_t<128, 2, 1>(X, D, perm, leaf_off, nleaf, k, G, status, s);
-        else launch_leaf_t<128, 1, 1>(X, D, perm, leaf_off, nleaf, k, G, status, s);
+        if (two) launch_leaf_t<128, 2, 1>(X, D, perm, leaf_off, nleaf, k, G, status, s, skip_if_exact);
+        else launch_leaf_t<128, 1, 1>(X, D, perm, leaf_off, nleaf, k, G, status, s, skip_if_exact);
     } else {
-        if (two) launch_leaf_t<256, 2, 1>(X, D, perm, leaf_off, nleaf, k, G, status, s);
-        else launch_leaf_t<256, 1, 1>(X, D, perm, leaf_off, nleaf, k, G, status, s);
+        if (two) launch_leaf_t<256, 2, 1>(X, D, perm, leaf_off, nleaf, k, G, status, s, skip_if_exact);
+        else launch_leaf_t<256, 1, 1>(X, D, perm, leaf_off, nleaf, k, G, status, s, skip_if_exact);
     }
 }
 

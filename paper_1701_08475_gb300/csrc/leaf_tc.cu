@@ -1,44 +1,42 @@
-// leaf_tc.cu -- the low-precision leaf stage on tcgen05 tensor cores.
+// leaf_tc.cu -- the low-precision copies and the leaf stage on tcgen05 tensor
+// cores for data whose 16-bit copy is exact.
 //
-//   K0 quantize   a BF16 or FP16 copy x^ of every point in leaf order, its
-//                 squared norm ||x^||^2 (FP32) and its quantisation error
-//                 e = ||x - x^|| (rounded up), plus one flag saying whether
-//                 the low-precision arithmetic is exact for this input
-//   K2 leaf       per leaf (m <= 128 points): the Gram matrix x^_i . x^_j on
+//   K0 quantize   a BF16 or FP16 copy x^ of every point, its squared norm
+//                 ||x^||^2 (FP32) and its quantisation error e = ||x - x^||
+//                 (rounded up), plus one flag saying whether the
+//                 low-precision arithmetic is exact for this input
+//   K2 leaf       per leaf (up to 256 points): the Gram matrix x^_i . x^_j on
 //                 the tensor cores (TMA loads of the leaf's rows into 128-byte
 //                 swizzled shared memory, tcgen05.mma with the FP32
-//                 accumulator in tensor memory), approximate distances
-//                 d^ = ||x^_i||^2 + ||x^_j||^2 - 2 x^_i . x^_j, and per row:
-//   K3 re-rank    the k' best approximate candidates get their canonical FP32
-//                 distance; the row is certified when no excluded candidate
-//                 can beat the row's k-th exact entry by the error bound below,
-//                 else it is recomputed exactly over the whole leaf.
+//                 accumulator in tensor memory), distances
+//                 d^ = ||x^_i||^2 + ||x^_j||^2 - 2 x^_i . x^_j, and per row a
+//                 warp's merge into the row's list
 //
-// With the certificate the graph is identical to the FP32 path's.  When all
-// values are integers that the 16-bit type holds exactly and every norm is
-// below 2^23, products and sums are exact integers in FP32, d^ is the
-// canonical distance itself and no re-rank is needed.
+// When all values are integers that the 16-bit type holds exactly and every
+// norm is below 2^23, products and sums are exact integers in FP32 and d^ is
+// the canonical distance itself.  For any other data the distances would have
+// to be computed again in FP32 near each row's k-th entry, and the plain FP32
+// leaf (leaf.cu) is the faster way to the same graph: with an exact re-rank of
+// the candidates that an error bound left, three leaf passes over 400,000
+// unit vectors of 96 dims took 4.5 ms (BF16), 4.3 (FP16) and 7.7 (FP8) at leaves
+// of up to 128 points, against 3.5 in FP32; over 104,000 GIST-like rows of 960
+// dims at 256 points 14.2, 11.9 and 48 ms against 8.1; no size from 32 to 960
+// dims was faster.  (On 1M exact rows of 128 dims a pass takes 1.0 ms here and
+// about 3 in FP32.)  An FP8 copy is never exact.
 //
-// FP8 E4M3 form: each row is scaled first, x~ = s q with s = max|x| / 448 and
-// q the E4M3 rounding (nearest even, saturating) of x / s; the tensor cores
-// form q_i . q_j (kind::f8f6f4, FP32 accumulation), and
-// d^ = ||x~_i||^2 + ||x~_j||^2 - 2 s_i s_j (q_i . q_j).  The bound below then
-// holds with x~ in place of x^ and the FP8 accumulation term c8 added to c_D:
-// the PTX ISA does not state how many bits the FP8 path keeps while it sums,
-// so the certificate assumes at least a 14-bit significand with truncation,
-// c8 = D 2^-13 (a previous generation's FP8 path was reported to keep about
-// 14 bits); the Gram error the hardware actually makes is measured against
-// this assumption by the tests.
+// FP8 E4M3 form (of knng_leaf_dhat): each row is scaled first, x~ = s q with
+// s = max|x| / 448 and q the E4M3 rounding (nearest even, saturating) of
+// x / s; the tensor cores form q_i . q_j (kind::f8f6f4, FP32 accumulation), and
+// d^ = ||x~_i||^2 + ||x~_j||^2 - 2 s_i s_j (q_i . q_j).
 //
-// Error bound of d^ against the exact distance d of the FP32 points (per row
-// i, against every candidate j of the leaf):
+// Error bound of d^ against the exact distance d of the FP32 points:
 //   |sqrt(d) - sqrt(d~)| <= e_i + e_j            (d~: exact distance of x^)
 //   |d^ - d~| <= c_D (||x^_i|| + ||x^_j||)^2 + 2^-23 |d^|
 // with c_D = (16 D + 8) 2^-24: four times the textbook bound for the FP32
 // sums (Higham, Ch. 3) because the tensor cores' summation order and internal
-// rounding are not specified.  A candidate excluded with approximate value
-// a >= a* can only beat the k-th exact entry t if
-//   (sqrt(max(0, a* - eps)) - e_i - e_max)^2 <= t.
+// rounding are not specified.  For FP8 the accumulation term c8 = D 2^-13 is
+// added (at least a 14-bit significand with truncation is assumed).  The
+// screens of screen.cu and join_tc.cu rest on it.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -163,28 +161,24 @@ __global__ void __launch_bounds__(256) k0_quantize_e4m3(const float* __restrict_
 __device__ __forceinline__ bool lp_exact(int f) { return (f & 1) == 0 && !((f & 2) && (f & 4)); }
 
 // Leaf-order copy gathered from the original-order one: row p of the output
-// is row perm[p] of the input (16-byte pieces), with its norm, error and
-// (FP8 only) scale.
+// is row perm[p] of the input (16-byte pieces), with its norm.  Returns at once
+// when the copy is not exact (the FP32 leaf reads X).
 __global__ void __launch_bounds__(256) k0_permute16(const uint4* __restrict__ Xq, const float* __restrict__ nrm,
-                                                    const float* __restrict__ qerr, const float* __restrict__ scale,
                                                     int64_t n, int q_per_row, const int32_t* __restrict__ perm,
                                                     uint4* __restrict__ Xl, float* __restrict__ lnrm,
-                                                    float* __restrict__ lerr, float* __restrict__ lscale) {
+                                                    const int* __restrict__ notexact) {
+    if (!lp_exact(*notexact)) return;
     const int64_t total = n * q_per_row;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t p = e / q_per_row;
         const int q = (int)(e - p * q_per_row);
         const int64_t i = perm[p];
         Xl[e] = __ldg(Xq + i * q_per_row + q);
-        if (q == 0) {
-            lnrm[p] = nrm[i];
-            lerr[p] = qerr[i];
-            if (scale) lscale[p] = scale[i];
-        }
+        if (q == 0) lnrm[p] = nrm[i];
     }
 }
 
-// ---------------------------------------------------------------- K2/K3
+// ---------------------------------------------------------------- K2
 constexpr int kTcRows = 128;             // M = N = 128 tile: leaves up to 128 points
 constexpr int kTcK = 64;                 // 16-bit elements per 128-byte swizzled row
 constexpr int kRowChunk = 128;           // bytes of a row per K chunk (one swizzle span)
@@ -197,9 +191,8 @@ struct TcSmem {
 };
 
 // MT row tiles of 128 (leaves up to 128 MT points): stages of MT boxes, the
-// d^ rows of one tile, barriers, then misc: tmem address, abort flag,
-// ids / norms / errors / rounded-up sqrt norms / scales [128 MT] each, two
-// maxima; then 32 keys of merge scratch per warp.  Dpb: bytes per row.
+// d^ rows of one tile, barriers, then misc: tmem address, abort flag, ids,
+// norms and scales [128 MT] each; then 32 keys of merge scratch per warp.  Dpb: bytes per row.
 __host__ __device__ inline TcSmem tc_smem(int Dpb, int MT) {
     TcSmem L;
     const int nk = Dpb / kRowChunk;
@@ -213,36 +206,22 @@ __host__ __device__ inline TcSmem tc_smem(int Dpb, int MT) {
     const size_t dt = (size_t)(kTcRows / 2) * (kTcRows * MT + 1) * 4;
     L.bar_off = ((stages > dt ? stages : dt) + 15) & ~(size_t)15;
     L.misc_off = L.bar_off + (size_t)(2 * L.stages + 1) * 8;
-    L.scratch_off = L.misc_off + 16 + 5 * (size_t)kTcRows * MT * 4 + 16;
+    L.scratch_off = (L.misc_off + 16 + 3 * (size_t)kTcRows * MT * 4 + 15) & ~(size_t)15;
     L.total = L.scratch_off + (kTcThreads / 32) * 32 * 8;
     return L;
 }
 
-// the key that lane `src` holds
-__device__ __forceinline__ uint64_t lane_key(uint64_t v, int src) { return shfl64(v, src); }
-
-// entry r of a list held lane-major in NO slots (r < 32 * NO)
-template <int NO>
-__device__ __forceinline__ uint64_t list_at(const uint64_t (&v)[NO], int r) {
-    uint64_t mine = v[0];
-#pragma unroll
-    for (int o = 1; o < NO; ++o)
-        if (o == (r >> 5)) mine = v[o];
-    return shfl64(mine, r & 31);
-}
-
 // QT: 0 FP16, 1 BF16 (kind::f16), 2 FP8 E4M3 (kind::f8f6f4, scaled rows).
-// Dpb: bytes per row of the copy; cD: the certificate's coefficient of
-// (||x^_i|| + ||x^_j||)^2.  dump (a parity hook; one leaf): the d^ rows are
-// written to dump (m x m) and nothing is selected.
+// Dpb: bytes per row of the copy.  Without dump the kernel returns at once when
+// the copy is not exact (the FP32 leaf then does the work).  dump (a parity
+// hook; one leaf): the d^ rows are written to dump (m x m) and nothing is
+// selected.
 template <int QT, int NSG, int MT>
 __global__ void __launch_bounds__(kTcThreads, 1) k2_leaf_tc(const __grid_constant__ CUtensorMap tmap, int Dpb,
-                                                           float cD, const float* __restrict__ X, int D,
                                                            const int32_t* __restrict__ perm,
                                                            const int32_t* __restrict__ leaf_off,
                                                            const float* __restrict__ nrm,
-                                                           const float* __restrict__ qerr,
-                                                           const float* __restrict__ scale, int k, int kp,
+                                                           const float* __restrict__ scale, int k,
                                                            uint64_t* __restrict__ G, int* __restrict__ status,
                                                            const int* __restrict__ notexact,
                                                            float* __restrict__ dump) {
@@ -250,7 +229,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k2_leaf_tc(const __grid_constan
     constexpr int DTS = RW + 1;           // d^ row stride
     constexpr int SB = kStageBytes * MT;  // one K chunk of all rows
     extern __shared__ uint8_t smem_raw[];
-    if (*status & kStatusStop) return;  // whole CTA, before any barrier or tensor memory
+    // whole CTA, before any barrier or tensor memory
+    if (*status & kStatusStop) return;
+    if (!dump && !lp_exact(*notexact)) return;
     const TcSmem L = tc_smem(Dpb, MT);
     uint8_t* base = smem_raw + ((1024 - (tc::smem_addr(smem_raw) & 1023)) & 1023);
     float* dt = reinterpret_cast<float*>(base + L.dt_off);
@@ -259,10 +240,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k2_leaf_tc(const __grid_constan
     int* abort_flag = reinterpret_cast<int*>(base + L.misc_off + 4);
     int32_t* sid = reinterpret_cast<int32_t*>(base + L.misc_off + 16);
     float* snrm = reinterpret_cast<float*>(sid + RW);
-    float* serr = snrm + RW;
-    float* srt = serr + RW;   // ||x^|| rounded up
-    float* sscl = srt + RW;   // row scales (FP8; 1 otherwise)
-    float* smax = sscl + RW;  // [0] max ||x^||, [1] max e
+    float* sscl = snrm + RW;  // row scales (FP8; 1 otherwise)
 
     const int S = L.stages, nk = Dpb / kRowChunk;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -292,7 +270,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k2_leaf_tc(const __grid_constan
         const bool in = r < m;
         sid[r] = in ? perm[a + r] : 0;
         snrm[r] = in ? nrm[a + r] : 0.f;
-        serr[r] = in ? qerr[a + r] : 0.f;
         sscl[r] = (in && QT == 2) ? scale[a + r] : 1.f;
     }
     __syncthreads();
@@ -361,27 +338,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k2_leaf_tc(const __grid_constan
         return;
     }
 
-    // leaf maxima of ||x^|| and e for the certificate; every ||x^|| rounded up
-    for (int r = tid; r < RW; r += kTcThreads) srt[r] = r < m ? __fsqrt_ru(snrm[r]) : 0.f;
-    if (warp == 0) {
-        float mn = 0.f, me = 0.f;
-        for (int r = lane; r < m; r += 32) {
-            mn = fmaxf(mn, sqrtf(snrm[r]));
-            me = fmaxf(me, serr[r]);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            mn = fmaxf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-            me = fmaxf(me, __shfl_xor_sync(0xffffffffu, me, o));
-        }
-        if (lane == 0) {
-            smax[0] = mn * (1.f + 1e-6f);
-            smax[1] = me;
-        }
-    }
-
-    const bool exact = lp_exact(*notexact);
-    const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
     constexpr int NC = RW / 32;
     uint64_t* wscratch = reinterpret_cast<uint64_t*>(base + L.scratch_off) + warp * 32;
     // Two phases: the two halves of the CTA's row tile; dt holds the phase's
@@ -437,207 +393,36 @@ __global__ void __launch_bounds__(kTcThreads, 1) k2_leaf_tc(const __grid_constan
 #pragma unroll
         for (int s = 0; s < NSG; ++s) old[s] = lane + 32 * s < k ? grow[lane + 32 * s] : kEmptyKey;
         uint64_t res[NSG];
-        bool done_row = false;
-        if (exact) {
-            // d^ is the canonical distance itself
-            uint64_t cand[NC + NSG];
+        // d^ is the canonical distance itself
+        uint64_t cand[NC + NSG];
 #pragma unroll
-            for (int s = 0; s < NC; ++s) {
-                const int c = lane + 32 * s;
-                cand[s] = (c < m && c != R) ? make_key(__fadd_rn(dt[rd * DTS + c], 0.f), (uint32_t)sid[c])
-                                            : kEmptyKey;
-            }
-            if (NSG == 1) {
-                // few candidates beat the row's k-th entry after the first pass
-                uint64_t few[NC];
+        for (int s = 0; s < NC; ++s) {
+            const int c = lane + 32 * s;
+            cand[s] = (c < m && c != R) ? make_key(__fadd_rn(dt[rd * DTS + c], 0.f), (uint32_t)sid[c]) : kEmptyKey;
+        }
+        if (NSG == 1) {
+            // few candidates beat the row's k-th entry after the first pass
+            uint64_t few[NC];
 #pragma unroll
-                for (int s = 0; s < NC; ++s) few[s] = cand[s];
-                uint64_t out;
-                bool changed;
-                if (warp_merge_few<NC>(few, old[0], k, wscratch, out, changed)) {
-                    if (changed && lane < k) grow[lane] = out;
-                    continue;
-                }
-                // many survive (the first pass): the lanes' smallest first
-#pragma unroll
-                for (int s = 0; s < NC; ++s) few[s] = cand[s];
-                if (warp_merge_many<NC>(few, old[0], k, wscratch, out, changed)) {
-                    if (changed && lane < k) grow[lane] = out;
-                    continue;
-                }
-            }
-#pragma unroll
-            for (int s = 0; s < NSG; ++s) cand[NC + s] = old[s];
-            sort_regs<NC + NSG>(cand);
-            warp_select_unique<NC + NSG, NSG>(cand, k, res);
-            done_row = true;
-        } else if (m - 1 > 0) {
-            if (NSG == 1) {
-                // Pruned exact re-rank (k <= 32).  With the bound above,
-                // evaluated per candidate and rounded so that it stays a lower
-                // bound, lb_c = (sqrt(a_c - eps_c) - e_i - e_c)^2 <= d_c; a
-                // candidate with lb_c above the row's k-th exact key tau
-                // cannot enter.  Batches of the 32 live candidates of least
-                // approximate value get canonical distances and merge into the
-                // row, which lowers tau; the rest are pruned against it; when
-                // at most 32 remain they are evaluated at once.  The row ends
-                // as the k best of its list and every candidate, the FP32
-                // form's result.
-                const uint64_t kth0 = lane_key(old[0], k - 1);
-                float tau = kth0 == kEmptyKey ? __int_as_float(0x7f800000) : key_dist(kth0);
-                float lbv[NC];
-                uint64_t apx[NC];
-                bool alive[NC];
-#pragma unroll
-                for (int s = 0; s < NC; ++s) {
-                    const int c = lane + 32 * s;
-                    const bool valid = c < m && c != R;
-                    apx[s] = kEmptyKey;
-                    lbv[s] = __int_as_float(0x7f800000);
-                    if (valid) {
-                        const float av = dt[rd * DTS + c];
-                        apx[s] = make_key(__fadd_rn(av, 0.f), (uint32_t)sid[c]);
-                        const float sn = __fadd_ru(srt[R], srt[c]);
-                        const float eps =
-                            __fadd_ru(__fmul_ru(cD, __fmul_ru(sn, sn)), __fmul_ru(1.1920928955078125e-7f, fabsf(av)));
-                        const float lo = __fsub_rd(av, eps);
-                        float lb = 0.f;
-                        if (lo > 0.f) {
-                            const float root = __fsub_rd(__fsub_rd(__fsqrt_rd(lo), serr[R]), serr[c]);
-                            if (root > 0.f) lb = __fmul_rd(root, root);
-                        }
-                        lbv[s] = lb;
-                    }
-                    alive[s] = valid && lbv[s] <= tau;
-                }
-                uint64_t list = old[0];
-                int batches = 0;
-                for (int it = 0; it <= NC; ++it) {
-                    unsigned bal[NC];
-                    int total = 0;
-#pragma unroll
-                    for (int s = 0; s < NC; ++s) {
-                        bal[s] = __ballot_sync(0xffffffffu, alive[s]);
-                        total += __popc(bal[s]);
-                    }
-                    if (total == 0) break;
-                    // into an empty list the first batch is k wide (its k-th
-                    // exact key is the first finite tau); later batches 32
-                    const int B = (it == 0 && kth0 == kEmptyKey) ? k : 32;
-                    uint64_t pick = kEmptyKey;  // this lane's candidate of the batch
-                    if (total <= B) {
-                        int at = 0;
-#pragma unroll
-                        for (int s = 0; s < NC; ++s) {
-                            if (alive[s]) wscratch[at + __popc(bal[s] & ((1u << lane) - 1u))] = apx[s];
-                            at += __popc(bal[s]);
-                        }
-                        __syncwarp();
-                        pick = lane < total ? wscratch[lane] : kEmptyKey;
-                        __syncwarp();
-                    } else {
-                        uint64_t tmp[NC], top[1];
-#pragma unroll
-                        for (int s = 0; s < NC; ++s) tmp[s] = alive[s] ? apx[s] : kEmptyKey;
-                        sort_regs<NC>(tmp);
-                        warp_select_unique<NC, 1>(tmp, B, top);
-                        pick = top[0];
-                    }
-                    const uint64_t last = lane_key(pick, B - 1);  // the batch's largest key (lanes below B hold one)
-                    uint64_t one[1] = {kEmptyKey};
-                    if (pick != kEmptyKey) {
-                        const uint32_t cid = key_id(pick);
-                        one[0] = make_key(canon_dist(X + (int64_t)gi * D, X + (int64_t)cid * D, D, vec), cid);
-                    }
-                    uint64_t out;
-                    bool changed;
-                    if (!warp_merge_few<1>(one, list, k, wscratch, out, changed)) {
-                        uint64_t both[2] = {one[0], list};
-                        uint64_t res1[1];
-                        sort_regs<2>(both);
-                        warp_select_unique<2, 1>(both, k, res1);
-                        out = res1[0];
-                    }
-                    list = lane < k ? out : kEmptyKey;
-                    ++batches;
-                    if (total <= B) break;
-                    const uint64_t kth = lane_key(list, k - 1);
-                    if (kth != kEmptyKey) tau = key_dist(kth);
-#pragma unroll
-                    for (int s = 0; s < NC; ++s) alive[s] = alive[s] && apx[s] > last && lbv[s] <= tau;
-                }
-                if (batches > (kth0 == kEmptyKey ? 2 : 1) && lane == 0)
-                    atomicAdd(status + 1, 1);  // rows the approximate order did not settle at once
-                if (__any_sync(0xffffffffu, list != old[0]) && lane < k) grow[lane] = list;
+            for (int s = 0; s < NC; ++s) few[s] = cand[s];
+            uint64_t out;
+            bool changed;
+            if (warp_merge_few<NC>(few, old[0], k, wscratch, out, changed)) {
+                if (changed && lane < k) grow[lane] = out;
                 continue;
             }
-            // the kp + 1 best approximate candidates (keys unique: distinct ids)
-            uint64_t apx[NC];
+            // many survive (the first pass): the lanes' smallest first
 #pragma unroll
-            for (int s = 0; s < NC; ++s) {
-                const int c = lane + 32 * s;
-                apx[s] = (c < m && c != R) ? make_key(__fadd_rn(dt[rd * DTS + c], 0.f), (uint32_t)sid[c])
-                                           : kEmptyKey;
-            }
-            sort_regs<NC>(apx);
-            uint64_t top[2];
-            const int want = kp + 1 < m - 1 ? kp + 1 : m - 1;
-            warp_select_unique<NC, 2>(apx, want, top);
-            const int nre = want < kp ? want : kp;  // re-ranked candidates
-            // canonical distances of the re-ranked ones; excluded: from rank kp on
-            uint64_t ex[2];
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                const int j = lane + 32 * s;
-                ex[s] = kEmptyKey;
-                if (j < nre) {
-                    const uint32_t cid = key_id(top[s]);
-                    const float d = canon_dist(X + (int64_t)gi * D, X + (int64_t)cid * D, D, vec);
-                    ex[s] = make_key(d, cid);
-                }
-            }
-            uint64_t merged[2 + NSG];
-            merged[0] = ex[0];
-            merged[1] = ex[1];
-#pragma unroll
-            for (int s = 0; s < NSG; ++s) merged[2 + s] = old[s];
-            sort_regs<2 + NSG>(merged);
-            warp_select_unique<2 + NSG, NSG>(merged, k, res);
-            if (want <= kp) {
-                done_row = true;  // nothing excluded
-            } else {
-                const uint64_t astar_key = list_at<2>(top, kp);
-                const uint64_t tau_key = list_at<NSG>(res, k - 1);
-                if (tau_key != kEmptyKey) {
-                    const double astar = (double)key_dist(astar_key);
-                    const double tau = (double)key_dist(tau_key);
-                    const double ni = sqrt((double)snrm[R]);
-                    const double eps = (double)cD * (ni + smax[0]) * (ni + smax[0]) + 1.1920928955078125e-7 * fabs(astar);
-                    const double lo = astar - eps;
-                    double root = lo > 0.0 ? sqrt(lo) : 0.0;
-                    root -= (double)serr[R] + (double)smax[1];
-                    const double lower = root > 0.0 ? root * root : 0.0;
-                    done_row = lower * (1.0 - 1e-12) > tau;
-                }
+            for (int s = 0; s < NC; ++s) few[s] = cand[s];
+            if (warp_merge_many<NC>(few, old[0], k, wscratch, out, changed)) {
+                if (changed && lane < k) grow[lane] = out;
+                continue;
             }
         }
-        if (!done_row) {
-            // not certified: exact distances to the whole leaf
-            uint64_t cand[NC + NSG];
 #pragma unroll
-            for (int s = 0; s < NC; ++s) {
-                const int c = lane + 32 * s;
-                cand[s] = kEmptyKey;
-                if (c < m && c != R)
-                    cand[s] = make_key(canon_dist(X + (int64_t)gi * D, X + (int64_t)sid[c] * D, D, vec),
-                                       (uint32_t)sid[c]);
-            }
-#pragma unroll
-            for (int s = 0; s < NSG; ++s) cand[NC + s] = old[s];
-            sort_regs<NC + NSG>(cand);
-            warp_select_unique<NC + NSG, NSG>(cand, k, res);
-            if (lane == 0) atomicAdd(status + 1, 1);  // fallback counter (statistics)
-        }
+        for (int s = 0; s < NSG; ++s) cand[NC + s] = old[s];
+        sort_regs<NC + NSG>(cand);
+        warp_select_unique<NC + NSG, NSG>(cand, k, res);
 #pragma unroll
         for (int s = 0; s < NSG; ++s)
             if (lane + 32 * s < k) grow[lane + 32 * s] = res[s];
@@ -724,15 +509,14 @@ void launch_quantize(const float* X, int64_t n, int D, const int32_t* perm, int 
         k0_quantize<false><<<grid, 256, 0, s>>>(X, n, D, Dp, perm, static_cast<uint16_t*>(Xq), nrm, qerr, notexact);
 }
 
-void launch_permute16(const void* Xq, const float* nrm, const float* qerr, const float* scale, int64_t n,
-                      int row_bytes, const int32_t* perm, void* Xl, float* lnrm, float* lerr, float* lscale,
-                      cudaStream_t s) {
+void launch_permute16(const void* Xq, const float* nrm, int64_t n, int row_bytes, const int32_t* perm, void* Xl,
+                      float* lnrm, const int* notexact, cudaStream_t s) {
     const int q = row_bytes / 16;
-    LaunchScope ls("k0_permute16", s, (double)n * (row_bytes * 2.0 + (scale ? 24.0 : 16.0)), 0);
+    LaunchScope ls("k0_permute16", s, (double)n * (row_bytes * 2.0 + 12.0), 0);
     int64_t g = (n * q + 255) / 256;
     if (g > 152 * 32) g = 152 * 32;
-    k0_permute16<<<(int)g, 256, 0, s>>>(static_cast<const uint4*>(Xq), nrm, qerr, scale, n, q, perm,
-                                        static_cast<uint4*>(Xl), lnrm, lerr, lscale);
+    k0_permute16<<<(int)g, 256, 0, s>>>(static_cast<const uint4*>(Xq), nrm, n, q, perm, static_cast<uint4*>(Xl), lnrm,
+                                        notexact);
 }
 
 void launch_lp_to_float(const void* Xq, int64_t m, int D, int qt, float* out, cudaStream_t s) {
@@ -743,10 +527,9 @@ void launch_lp_to_float(const void* Xq, int64_t m, int D, int qt, float* out, cu
                                                        out);
 }
 
-bool launch_leaf_tc(const void* Xl, int64_t n, const float* X, int D, const int32_t* perm,
-                    const int32_t* leaf_off, int nleaf, int max_leaf, const float* nrm, const float* qerr,
-                    const float* scale, int k, int kp, int qt, uint64_t* G, int* status, const int* notexact,
-                    cudaStream_t s, float* dump) {
+bool launch_leaf_tc(const void* Xl, int64_t n, int D, const int32_t* perm, const int32_t* leaf_off, int nleaf,
+                    int max_leaf, const float* nrm, const float* scale, int k, int qt, uint64_t* G, int* status,
+                    const int* notexact, cudaStream_t s, float* dump) {
     if (max_leaf > 2 * kTcRows) return false;
     const int MT = max_leaf > kTcRows ? 2 : 1;
     EncodeTiledFn enc = encode_fn();
@@ -767,7 +550,6 @@ bool launch_leaf_tc(const void* Xl, int64_t n, const float* X, int D, const int3
     const TcSmem L = tc_smem(Dpb, MT);
     const size_t smem = L.total + 1024;
     if (smem > 227 * 1024) return false;
-    const float cD = lp_cert_coeff(D, qt);
     const double mm = (double)max_leaf, rw = 128.0 * MT;
     const double elems = qt == 2 ? Dpb : Dpb / 2;
     static const char* names[3] = {"k2_leaf_fp16", "k2_leaf_bf16", "k2_leaf_fp8"};
@@ -775,8 +557,8 @@ bool launch_leaf_tc(const void* Xl, int64_t n, const float* X, int D, const int3
 #define KNNG_LEAF_TC(Q, NS, T)                                                                                  \
     do {                                                                                                        \
         cudaFuncSetAttribute(k2_leaf_tc<Q, NS, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);     \
-        k2_leaf_tc<Q, NS, T><<<nleaf * T, kTcThreads, smem, s>>>(tmap, Dpb, cD, X, D, perm, leaf_off, nrm,   \
-                                                             qerr, scale, k, kp, G, status, notexact, dump);    \
+        k2_leaf_tc<Q, NS, T><<<nleaf * T, kTcThreads, smem, s>>>(tmap, Dpb, perm, leaf_off, nrm, scale, k, G,  \
+                                                             status, notexact, dump);                           \
     } while (0)
 #define KNNG_LEAF_TC_K(Q, T)               \
     do {                                   \
