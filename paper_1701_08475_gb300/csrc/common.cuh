@@ -309,6 +309,28 @@ __device__ __forceinline__ bool warp_merge_many(uint64_t (&cand)[NC], uint64_t l
     return true;
 }
 
+// Two FP32 values in one register pair: acc + (r - c)^2 of both (fmaf), and
+// the pair the other way round.
+__device__ __forceinline__ uint64_t add_square(uint64_t r, uint64_t c, uint64_t acc) {
+    asm("{\n"
+        ".reg .b64 t;\n"
+        "sub.rn.f32x2 t, %1, %2;\n"
+        "fma.rn.f32x2 %0, t, t, %0;\n"
+        "}\n"
+        : "+l"(acc)
+        : "l"(r), "l"(c));
+    return acc;
+}
+__device__ __forceinline__ uint64_t swap_pair(uint64_t c) { return (c << 32) | (c >> 32); }
+// Four dims of two members, interleaved dim by dim, to 32 bytes of shared
+// memory (`alt`: which half first; alternate it between groups of four lanes
+// that write consecutive 32-byte pieces, and no bank is hit twice).
+__device__ __forceinline__ void store_pairs(float* dst, const float4& u, const float4& v, bool alt) {
+    const float4 lo = make_float4(u.x, v.x, u.y, v.y), hi = make_float4(u.z, v.z, u.w, v.w);
+    reinterpret_cast<float4*>(dst)[alt ? 1 : 0] = alt ? hi : lo;
+    reinterpret_cast<float4*>(dst)[alt ? 0 : 1] = alt ? lo : hi;
+}
+
 // canonical FP32 squared distance between rows xa and xb (dims ascending,
 // fmaf); vec: D % 4 == 0 and 16-byte aligned rows
 __device__ __forceinline__ float canon_dist(const float* __restrict__ xa, const float* __restrict__ xb, int D,

@@ -390,8 +390,9 @@ __global__ void __launch_bounds__(256) k6_active(const int32_t* __restrict__ ord
 constexpr int kJoinWarps = 4;
 
 // Dims per shared-memory chunk (about 12 KB of member rows per warp, equal
-// chunks) and the row stride (stride / 4 odd: consecutive rows in different
-// banks for float4 reads).
+// chunks) and the stride of a pair row, which holds members 2 p and 2 p + 1
+// interleaved dim by dim for paired FP32 instructions (stride / 4 odd:
+// consecutive pair rows in different banks for 16-byte reads).
 __host__ __device__ inline void join_chunk(int D, int mcap, int* dch, int* stride) {
     const int d4 = (D + 3) & ~3;
     int cap = (12 * 1024 / (mcap * 4) - 4) & ~3;
@@ -399,7 +400,13 @@ __host__ __device__ inline void join_chunk(int D, int mcap, int* dch, int* strid
     const int nch = (d4 + cap - 1) / cap;
     const int c = ((d4 + nch - 1) / nch + 3) & ~3;
     *dch = c;
-    *stride = ((c / 4) & 1) ? c : c + 4;
+    *stride = 2 * c + 4;
+}
+
+// A warp's shared memory: the members' pair rows, thresholds and ids (mcap is
+// a multiple of 4).
+__host__ __device__ inline size_t join_warp_bytes(int mcap, int stride) {
+    return ((size_t)(mcap / 2) * stride * 4 + (size_t)mcap * 12 + 31) & ~(size_t)15;
 }
 
 // Whether entry (a, b) of block row ia, column ib is a pair to evaluate:
@@ -492,69 +499,91 @@ __device__ __forceinline__ void join_node(const float* __restrict__ X, int D, in
             }
         }
     }
-    float acc[BPL][4][4];
+    // sums of members (2 h, 2 w), (2 h + 1, 2 w + 1) of the block, and of
+    // (2 h, 2 w + 1), (2 h + 1, 2 w)
+    uint64_t same[BPL][2][2], cross[BPL][2][2];
 #pragma unroll
     for (int q = 0; q < BPL; ++q)
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int b = 0; b < 4; ++b) acc[q][a][b] = 0.f;
+            for (int w = 0; w < 2; ++w) same[q][h][w] = cross[q][h][w] = 0ull;
     const bool vec = (D % 4 == 0);
     for (int d0 = 0; d0 < D; d0 += dch) {
         const int dl = min(dch, D - d0);
-        // gather the members' dims [d0, d0 + dch)
+        // gather the members' dims [d0, d0 + dch); members M .. 4 RGN - 1
+        // read as zeros
         if (vec) {
             const int q4 = dch >> 2;
-            for (int e = lane; e < M * q4; e += 32) {
-                const int r = e / q4, c4 = e - r * q4;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (c4 * 4 < dl) v = __ldg(reinterpret_cast<const float4*>(X + (int64_t)mem[r] * D + d0) + c4);
-                *reinterpret_cast<float4*>(xs + r * stride + c4 * 4) = v;
+            for (int e = lane; e < RGN * 2 * q4; e += 32) {
+                const int p = e / q4, c4 = e - p * q4;
+                float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
+                if (c4 * 4 < dl) {
+                    if (2 * p < M) u = __ldg(reinterpret_cast<const float4*>(X + (int64_t)mem[2 * p] * D + d0) + c4);
+                    if (2 * p + 1 < M)
+                        v = __ldg(reinterpret_cast<const float4*>(X + (int64_t)mem[2 * p + 1] * D + d0) + c4);
+                }
+                store_pairs(xs + p * stride + c4 * 8, u, v, (c4 >> 2) & 1);
             }
         } else {
-            for (int e = lane; e < M * dch; e += 32) {
-                const int r = e / dch, c = e - r * dch;
-                xs[r * stride + c] = c < dl ? __ldg(X + (int64_t)mem[r] * D + d0 + c) : 0.f;
+            for (int e = lane; e < RGN * 2 * dch; e += 32) {
+                const int p = e / dch, c = e - p * dch;
+                const bool in = c < dl;
+                *reinterpret_cast<float2*>(xs + p * stride + 2 * c) =
+                    make_float2(in && 2 * p < M ? __ldg(X + (int64_t)mem[2 * p] * D + d0 + c) : 0.f,
+                                in && 2 * p + 1 < M ? __ldg(X + (int64_t)mem[2 * p + 1] * D + d0 + c) : 0.f);
             }
         }
-        // rows M .. 4*RGN-1 read as zeros
-        for (int e = lane; e < (RGN * 4 - M) * dch; e += 32) {
-            const int r = M + e / dch, c = e % dch;
-            xs[r * stride + c] = 0.f;
-        }
         __syncwarp();
-        // block (rg, cg) holds members {rg + a * RGN} x {cg + b * RGN}: lanes
-        // then read consecutive rows, which the odd stride / 4 puts in
-        // different banks
+        // block (rg, cg) holds the members of pair rows {rg, rg + RSTEP} x
+        // {cg, cg + RGN}: lanes then read consecutive pair rows
 #pragma unroll
         for (int q = 0; q < BPL; ++q) {
             if (brg[q] < 0) continue;
             const float* rp = xs + brg[q] * stride;
             const float* cp = xs + bcg[q] * stride;
             const int rstep = RSTEP * stride, cstep = RGN * stride;
-            for (int dq = 0; dq < dch; dq += 4) {
-                float4 rv[4], cv[4];
+            for (int dq = 0; dq < 2 * dch; dq += 8) {  // 4 dims
+                ulonglong2 r[2][2], c[2][2];
 #pragma unroll
-                for (int a = 0; a < 4; ++a) rv[a] = *reinterpret_cast<const float4*>(rp + a * rstep + dq);
+                for (int h = 0; h < 2; ++h)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) cv[b] = *reinterpret_cast<const float4*>(cp + b * cstep + dq);
+                    for (int p = 0; p < 2; ++p) {
+                        r[h][p] = *reinterpret_cast<const ulonglong2*>(rp + h * rstep + dq + 4 * p);
+                        c[h][p] = *reinterpret_cast<const ulonglong2*>(cp + h * cstep + dq + 4 * p);
+                    }
 #pragma unroll
-                for (int a = 0; a < 4; ++a)
+                for (int p = 0; p < 2; ++p)
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        float t = __fsub_rn(rv[a].x, cv[b].x);
-                        acc[q][a][b] = __fmaf_rn(t, t, acc[q][a][b]);
-                        t = __fsub_rn(rv[a].y, cv[b].y);
-                        acc[q][a][b] = __fmaf_rn(t, t, acc[q][a][b]);
-                        t = __fsub_rn(rv[a].z, cv[b].z);
-                        acc[q][a][b] = __fmaf_rn(t, t, acc[q][a][b]);
-                        t = __fsub_rn(rv[a].w, cv[b].w);
-                        acc[q][a][b] = __fmaf_rn(t, t, acc[q][a][b]);
+                    for (int w = 0; w < 2; ++w) {
+                        const uint64_t c0 = c[w][p].x, c1 = c[w][p].y, x0 = swap_pair(c0), x1 = swap_pair(c1);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            same[q][h][w] = add_square(r[h][p].x, c0, same[q][h][w]);
+                            cross[q][h][w] = add_square(r[h][p].x, x0, cross[q][h][w]);
+                            same[q][h][w] = add_square(r[h][p].y, c1, same[q][h][w]);
+                            cross[q][h][w] = add_square(r[h][p].y, x1, cross[q][h][w]);
+                        }
                     }
             }
         }
         __syncwarp();
     }
+    float acc[BPL][4][4];
+#pragma unroll
+    for (int q = 0; q < BPL; ++q)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+                acc[q][2 * h][2 * w] = __uint_as_float((uint32_t)same[q][h][w]);
+                acc[q][2 * h + 1][2 * w + 1] = __uint_as_float((uint32_t)(same[q][h][w] >> 32));
+                acc[q][2 * h][2 * w + 1] = __uint_as_float((uint32_t)cross[q][h][w]);
+                acc[q][2 * h + 1][2 * w] = __uint_as_float((uint32_t)(cross[q][h][w] >> 32));
+            }
+    // entry (a, b) of a block: member a % 2 of pair row a / 2 of the rows, the same for the columns
+    auto row_of = [&](int q, int a) { return 2 * (brg[q] + (a >> 1) * RSTEP) + (a & 1); };
+    auto col_of = [&](int q, int b) { return 2 * (bcg[q] + (b >> 1) * RGN) + (b & 1); };
     // offers: count, reserve, write.  In the triangle every unordered member
     // pair lies in exactly one block once diagonal blocks keep only a < b;
     // pairs of two old members are dropped.
@@ -566,7 +595,7 @@ __device__ __forceinline__ void join_node(const float* __restrict__ X, int D, in
         for (int a = 0; a < 4; ++a)
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
-                const int ia = brg[q] + a * RSTEP, ib = bcg[q] + b * RGN;
+                const int ia = row_of(q, a), ib = col_of(q, b);
                 if (pair_live(rect, ia, ib, M, nn, brg[q] < bcg[q] || a < b)) {
                     const uint32_t u = (uint32_t)mem[ia], v = (uint32_t)mem[ib];
                     if (u != v) {
@@ -594,7 +623,7 @@ __device__ __forceinline__ void join_node(const float* __restrict__ X, int D, in
         for (int a = 0; a < 4; ++a)
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
-                const int ia = brg[q] + a * RSTEP, ib = bcg[q] + b * RGN;
+                const int ia = row_of(q, a), ib = col_of(q, b);
                 if (pair_live(rect, ia, ib, M, nn, brg[q] < bcg[q] || a < b)) {
                     const uint32_t u = (uint32_t)mem[ia], v = (uint32_t)mem[ib];
                     if (u != v) {
@@ -643,9 +672,9 @@ __global__ void __launch_bounds__(32 * kJoinWarps) k5_join(const float* __restri
     int dch, stride;
     join_chunk(D, mcap, &dch, &stride);
     const int warp = threadIdx.x >> 5;
-    char* base = reinterpret_cast<char*>(smem4) + (size_t)warp * ((size_t)mcap * (stride * 4 + 12) + 16);
-    float* xs = reinterpret_cast<float*>(base);                                   // [mcap][stride]
-    uint64_t* thr = reinterpret_cast<uint64_t*>(xs + (size_t)mcap * stride);      // [mcap]
+    char* base = reinterpret_cast<char*>(smem4) + (size_t)warp * join_warp_bytes(mcap, stride);
+    float* xs = reinterpret_cast<float*>(base);                                   // [mcap / 2][stride]
+    uint64_t* thr = reinterpret_cast<uint64_t*>(xs + (size_t)(mcap / 2) * stride);  // [mcap]
     int32_t* mem = reinterpret_cast<int32_t*>(thr + mcap);                        // [mcap]
     for (int64_t pos = node0 + (int64_t)blockIdx.x * kJoinWarps + warp; pos < node1;
          pos += (int64_t)gridDim.x * kJoinWarps)
@@ -660,13 +689,20 @@ __global__ void __launch_bounds__(32 * kJoinWarps) k5_join(const float* __restri
 // mcap / 4; a CTA of 256 threads takes G = 256 / NB nodes at a time and
 // thread t computes block t % NB of node t / NB, so a warp's lanes stay busy
 // whatever NB is (one node per warp leaves lanes idle when NB is not a
-// multiple of 32).  Block (rg, cg) holds members {4 rg + a} x {4 cg + b};
-// member m of a node sits in shared-memory row (m % 4) RGN + m / 4, so lanes
-// of consecutive cg read consecutive rows (an odd float4 stride puts them in
-// different banks) and lanes of one rg read the same row.  Members are new
-// first, so blocks whose two groups hold only old members are skipped whole.
-// Offers as in k5_join; a pair of members that shared a leaf in one of the
-// build's last tree passes makes none (the leaf stage offered it already).
+// multiple of 32).  Block (rg, cg) holds members {4 rg + a} x {4 cg + b}.
+// Members are new first, so blocks whose two groups hold only old members are
+// skipped whole.  Offers as in k5_join; a pair of members that shared a leaf in
+// one of the build's last tree passes makes none (the leaf stage offered it
+// already).
+//
+// Bound by issue slots.  So the differences and sums are paired FP32
+// instructions, two pairs of members each: members 4 g + 2 h and 4 g + 2 h + 1
+// are staged interleaved dim by dim in row h RGN + g, (r0, r1) - (c0, c1) and
+// (r0, r1) - (c1, c0) give all four differences of two such rows, and every
+// sum keeps its chain.  Lanes of consecutive cg read consecutive rows (an odd
+// number of 16-byte pieces apart: different banks), lanes of one rg the same.
+// First round on 1M x 96, k = 16: 6.5 ms with scalar instructions (70 % of issue
+// slots used), 5.3 paired (59 %; the FMA pipe 48 %).
 constexpr int kJ2Threads = 256;
 
 struct J2Layout {
@@ -685,11 +721,11 @@ __host__ __device__ inline J2Layout j2_layout(int D, int mcap, bool leafids) {
     if (cap < 4) cap = 4;
     const int nch = (d4 + cap - 1) / cap;
     L.dch = ((d4 + nch - 1) / nch + 3) & ~3;
-    L.stride = ((L.dch / 4) & 1) ? L.dch : L.dch + 4;
+    L.stride = 2 * L.dch + 4;  // an odd number of 16-byte pieces
     L.thr = 0;
     L.lid = L.thr + (size_t)slots * 8;
     L.rows = L.lid + (leafids ? (size_t)slots * 16 : 0);
-    L.mem = L.rows + (size_t)slots * L.stride * 4;
+    L.mem = L.rows + (size_t)(slots / 2) * L.stride * 4;
     L.cnt = L.mem + (size_t)slots * 4;
     L.total = L.cnt + (size_t)L.G * 2 * 4;
     return L;
@@ -723,7 +759,7 @@ __global__ void __launch_bounds__(kJ2Threads, 4) k5_join_cta(const float* __rest
     char* base = reinterpret_cast<char*>(smem4);
     uint64_t* thr = reinterpret_cast<uint64_t*>(base + L.thr);  // [G][mcap] by slot
     int4* slid = reinterpret_cast<int4*>(base + L.lid);         // [G][mcap] by slot
-    float* rows = reinterpret_cast<float*>(base + L.rows);      // [G][mcap][stride] by slot
+    float* rows = reinterpret_cast<float*>(base + L.rows);      // [G][mcap / 2][stride] by pair row
     int32_t* mem = reinterpret_cast<int32_t*>(base + L.mem);    // [G][mcap] by member index
     int* cnt = reinterpret_cast<int*>(base + L.cnt);            // [G] members, then [G] new members
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -806,63 +842,82 @@ __global__ void __launch_bounds__(kJ2Threads, 4) k5_join_cta(const float* __rest
         const int Mj = jn < G ? cnt[jn] : 0, nnj = jn < G ? cnt[G + jn] : 0;
         // a block with a live pair: both groups hold members, one holds a new one
         const bool live = jn < G && 4 * rg < Mj && 4 * cg < Mj && (4 * rg < nnj || 4 * cg < nnj);
-        float acc[4][4];
+        // sums of (2 h, 2 w), (2 h + 1, 2 w + 1) and of (2 h, 2 w + 1), (2 h + 1, 2 w)
+        uint64_t same[2][2], cross[2][2];
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-        const int q4 = dch >> 2;
+            for (int w = 0; w < 2; ++w) same[h][w] = cross[h][w] = 0ull;
+        const int q4 = dch >> 2, half = mcap / 2;
         for (int d0 = 0; d0 < D; d0 += dch) {
             const int dl = min(dch, D - d0);
-            // gather dims [d0, d0 + dch) of every member slot (zeros past
-            // the members and past D)
+            // gather dims [d0, d0 + dch) of every member (zeros past the
+            // members and past D), two members interleaved
             if (vec) {
-                for (int e = tid; e < G * mcap * q4; e += kJ2Threads) {
-                    const int sl = e / q4, c4 = e - sl * q4;
-                    const int j = sl / mcap, s = sl - j * mcap;
-                    const int m = (s % RGN) * 4 + s / RGN;  // the member stored in slot s
-                    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (m < cnt[j] && c4 * 4 < dl)
-                        v = __ldg(reinterpret_cast<const float4*>(X + (int64_t)mem[j * mcap + m] * D + d0) + c4);
-                    *reinterpret_cast<float4*>(rows + (size_t)sl * stride + c4 * 4) = v;
+                for (int e = tid; e < G * half * q4; e += kJ2Threads) {
+                    const int pr = e / q4, c4 = e - pr * q4;
+                    const int j = pr / half, s = pr - j * half;
+                    const int m = s < RGN ? 4 * s : 4 * (s - RGN) + 2, M = cnt[j];  // members m, m + 1
+                    float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
+                    if (c4 * 4 < dl) {
+                        if (m < M) u = __ldg(reinterpret_cast<const float4*>(X + (int64_t)mem[j * mcap + m] * D + d0) + c4);
+                        if (m + 1 < M)
+                            v = __ldg(reinterpret_cast<const float4*>(X + (int64_t)mem[j * mcap + m + 1] * D + d0) + c4);
+                    }
+                    store_pairs(rows + (size_t)pr * stride + c4 * 8, u, v, (c4 >> 2) & 1);
                 }
             } else {
-                for (int e = tid; e < G * mcap * dch; e += kJ2Threads) {
-                    const int sl = e / dch, c = e - sl * dch;
-                    const int j = sl / mcap, s = sl - j * mcap;
-                    const int m = (s % RGN) * 4 + s / RGN;
-                    rows[(size_t)sl * stride + c] =
-                        (m < cnt[j] && c < dl) ? __ldg(X + (int64_t)mem[j * mcap + m] * D + d0 + c) : 0.f;
+                for (int e = tid; e < G * half * dch; e += kJ2Threads) {
+                    const int pr = e / dch, c = e - pr * dch;
+                    const int j = pr / half, s = pr - j * half;
+                    const int m = s < RGN ? 4 * s : 4 * (s - RGN) + 2, M = cnt[j];
+                    const bool in = c < dl;
+                    *reinterpret_cast<float2*>(rows + (size_t)pr * stride + 2 * c) =
+                        make_float2(in && m < M ? __ldg(X + (int64_t)mem[j * mcap + m] * D + d0 + c) : 0.f,
+                                    in && m + 1 < M ? __ldg(X + (int64_t)mem[j * mcap + m + 1] * D + d0 + c) : 0.f);
                 }
             }
             __syncthreads();
             if (live) {
-                const float* rp = rows + (size_t)(jn * mcap + rg) * stride;
-                const float* cp = rows + (size_t)(jn * mcap + cg) * stride;
-                const int step = RGN * stride;  // member 4 g + a sits a RGN rows below member 4 g
-                for (int dq = 0; dq < dch; dq += 4) {
-                    float4 rv[4], cv[4];
+                const float* rp = rows + (size_t)(jn * half + rg) * stride;
+                const float* cp = rows + (size_t)(jn * half + cg) * stride;
+                const int step = RGN * stride;  // members 4 g + 2, 4 g + 3 sit RGN rows below 4 g, 4 g + 1
+                for (int dq = 0; dq < 2 * dch; dq += 8) {  // 4 dims
+                    ulonglong2 r[2][2], c[2][2];
 #pragma unroll
-                    for (int a = 0; a < 4; ++a) rv[a] = *reinterpret_cast<const float4*>(rp + a * step + dq);
+                    for (int h = 0; h < 2; ++h)
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) cv[b] = *reinterpret_cast<const float4*>(cp + b * step + dq);
+                        for (int p = 0; p < 2; ++p) {
+                            r[h][p] = *reinterpret_cast<const ulonglong2*>(rp + h * step + dq + 4 * p);
+                            c[h][p] = *reinterpret_cast<const ulonglong2*>(cp + h * step + dq + 4 * p);
+                        }
 #pragma unroll
-                    for (int a = 0; a < 4; ++a)
+                    for (int p = 0; p < 2; ++p)
 #pragma unroll
-                        for (int b = 0; b < 4; ++b) {
-                            float t = __fsub_rn(rv[a].x, cv[b].x);
-                            acc[a][b] = __fmaf_rn(t, t, acc[a][b]);
-                            t = __fsub_rn(rv[a].y, cv[b].y);
-                            acc[a][b] = __fmaf_rn(t, t, acc[a][b]);
-                            t = __fsub_rn(rv[a].z, cv[b].z);
-                            acc[a][b] = __fmaf_rn(t, t, acc[a][b]);
-                            t = __fsub_rn(rv[a].w, cv[b].w);
-                            acc[a][b] = __fmaf_rn(t, t, acc[a][b]);
+                        for (int w = 0; w < 2; ++w) {
+                            const uint64_t c0 = c[w][p].x, c1 = c[w][p].y, x0 = swap_pair(c0), x1 = swap_pair(c1);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                same[h][w] = add_square(r[h][p].x, c0, same[h][w]);
+                                cross[h][w] = add_square(r[h][p].x, x0, cross[h][w]);
+                                same[h][w] = add_square(r[h][p].y, c1, same[h][w]);
+                                cross[h][w] = add_square(r[h][p].y, x1, cross[h][w]);
+                            }
                         }
                 }
             }
             __syncthreads();  // the next chunk overwrites the rows
         }
+        float acc[4][4];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+                acc[2 * h][2 * w] = __uint_as_float((uint32_t)same[h][w]);
+                acc[2 * h + 1][2 * w + 1] = __uint_as_float((uint32_t)(same[h][w] >> 32));
+                acc[2 * h][2 * w + 1] = __uint_as_float((uint32_t)cross[h][w]);
+                acc[2 * h + 1][2 * w] = __uint_as_float((uint32_t)(cross[h][w] >> 32));
+            }
         // offers: count, reserve (one atomic per warp), write
         int c = 0;
         if (live) {
@@ -1173,7 +1228,7 @@ int join_blocks_per_lane(int mcap) {
 size_t join_smem_bytes(int D, int mcap) {
     int dch, stride;
     join_chunk(D, mcap, &dch, &stride);
-    return (size_t)kJoinWarps * ((size_t)mcap * (stride * 4 + 12) + 16);
+    return (size_t)kJoinWarps * join_warp_bytes(mcap, stride);
 }
 
 namespace {
