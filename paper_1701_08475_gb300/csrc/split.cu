@@ -858,65 +858,88 @@ __global__ void __launch_bounds__(256) k1_select_pos(const float* __restrict__ S
 // per warp ascending positions, then warps 0..15, then tiles.
 constexpr int kSumsWarps = 16;
 
-// Adds the n rows listed in rows[] (one side of the cut) to the per-lane
-// compensated sums (h, l), with the loads of up to U rows in flight.  Q = 0
-// reads the FP32 rows of X (VEC: lane l owns dims 4l .. 4l+3, else l, l+32,
-// ...), Q = 1 / 2 the BF16 / FP16 copy (dims 4l .. 4l+3).
+// Adds the rows listed in rows[0 .. n0) to the per-lane compensated sums
+// (hL, lL) and rows[n0 .. n) to (hR, lR), in order; the next U rows load while
+// U are added.  Q = 0 reads the FP32 rows of X (VEC: lane l owns dims 4l ..
+// 4l+3, else l, l+32, ...), Q = 1 / 2 the BF16 / FP16 copy (dims 4l .. 4l+3).
 template <bool VEC, int Q>
-__device__ __forceinline__ void sums_side(const float* __restrict__ X, int D, const uint16_t* __restrict__ Xq, int Dq,
-                                          const int* rows, int n, int dbase, float* h, float* l) {
+__device__ __forceinline__ void sums_rows(const float* __restrict__ X, int D, const uint16_t* __restrict__ Xq, int Dq,
+                                          const int* rows, int n0, int n, int dbase, float* hL, float* lL, float* hR,
+                                          float* lR) {
     const int lane = threadIdx.x & 31;
-    constexpr int U = Q != 0 ? 16 : 8;  // 4 KB per warp in flight
-    for (int q0 = 0; q0 < n; q0 += U) {
+    // 4 rows in flight and 4 being added fit 64 registers, so that two CTAs
+    // share an SM (at 94 registers one did, 24 % of the warps active): a full
+    // sweep of 2M x 96 464 -> 370 us, a later one 63 -> 47; 2 and 6 rows were slower
+    constexpr int U = 4;
+    struct Batch {
         float v[U][4];
-        uint2 hq[U];  // Q != 0: four raw 16-bit values
+        uint2 q[U];  // Q != 0: four raw 16-bit values
+    };
+    auto load = [&](int q0, Batch& b) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
+            if (Q != 0) b.q[u] = make_uint2(0u, 0u);
+            else
 #pragma unroll
-            for (int j = 0; j < 4; ++j) v[u][j] = 0.f;
-            hq[u] = make_uint2(0u, 0u);
+                for (int j = 0; j < 4; ++j) b.v[u][j] = 0.f;
             if (q0 + u < n) {
                 const int row = rows[q0 + u];
                 const float* x = X + (int64_t)row * D + dbase;
                 if (Q != 0) {  // rows padded to Dq: the four values are in bounds
                     if (dbase + lane * 4 < D)
-                        hq[u] = __ldg(reinterpret_cast<const uint2*>(Xq + (int64_t)row * Dq + dbase + 4 * lane));
+                        b.q[u] = __ldg(reinterpret_cast<const uint2*>(Xq + (int64_t)row * Dq + dbase + 4 * lane));
                 } else if (VEC) {
                     if (dbase + lane * 4 < D) {
                         const float4 f = __ldg(reinterpret_cast<const float4*>(x) + lane);
-                        v[u][0] = f.x; v[u][1] = f.y; v[u][2] = f.z; v[u][3] = f.w;
+                        b.v[u][0] = f.x; b.v[u][1] = f.y; b.v[u][2] = f.z; b.v[u][3] = f.w;
                     }
                 } else {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) v[u][j] = (dbase + lane + 32 * j < D) ? __ldg(x + lane + 32 * j) : 0.f;
+                    for (int j = 0; j < 4; ++j)
+                        b.v[u][j] = (dbase + lane + 32 * j < D) ? __ldg(x + lane + 32 * j) : 0.f;
                 }
             }
         }
+    };
+    auto add = [&](float (&v)[4], float* h, float* l) {
+        if (Q != 0) {
+            // exact-mode values are integers of magnitude <= 2048 and a
+            // lane adds at most 128 of them per tile: FP32 sums are exact
+#pragma unroll
+            for (int j = 0; j < 4; ++j) h[j] = __fadd_rn(h[j], v[j]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {  // TwoSum: s + err == h + v exactly
+                const float s = __fadd_rn(h[j], v[j]);
+                const float bp = __fsub_rn(s, h[j]);
+                const float err = __fadd_rn(__fsub_rn(h[j], __fsub_rn(s, bp)), __fsub_rn(v[j], bp));
+                h[j] = s;
+                l[j] = __fadd_rn(l[j], err);
+            }
+        }
+    };
+    Batch cur;
+    load(0, cur);
+    for (int q0 = 0; q0 < n; q0 += U) {
+        Batch next;
+        load(q0 + U, next);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (q0 + u >= n) break;
+            float v[4];
             if (Q != 0) {
-                v[u][0] = q16_to_float<Q>(hq[u].x & 0xFFFFu);
-                v[u][1] = q16_to_float<Q>(hq[u].x >> 16);
-                v[u][2] = q16_to_float<Q>(hq[u].y & 0xFFFFu);
-                v[u][3] = q16_to_float<Q>(hq[u].y >> 16);
-            }
-            if (Q != 0) {
-                // exact-mode values are integers of magnitude <= 2048 and a
-                // lane adds at most 128 of them per tile: FP32 sums are exact
-#pragma unroll
-                for (int j = 0; j < 4; ++j) h[j] = __fadd_rn(h[j], v[u][j]);
+                v[0] = q16_to_float<Q>(cur.q[u].x & 0xFFFFu);
+                v[1] = q16_to_float<Q>(cur.q[u].x >> 16);
+                v[2] = q16_to_float<Q>(cur.q[u].y & 0xFFFFu);
+                v[3] = q16_to_float<Q>(cur.q[u].y >> 16);
             } else {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {  // TwoSum: s + err == h + v exactly
-                    const float s = __fadd_rn(h[j], v[u][j]);
-                    const float bp = __fsub_rn(s, h[j]);
-                    const float err = __fadd_rn(__fsub_rn(h[j], __fsub_rn(s, bp)), __fsub_rn(v[u][j], bp));
-                    h[j] = s;
-                    l[j] = __fadd_rn(l[j], err);
-                }
+                for (int j = 0; j < 4; ++j) v[j] = cur.v[u][j];
             }
+            if (q0 + u < n0) add(v, hL, lL);
+            else add(v, hR, lR);
         }
+        cur = next;
     }
 }
 
@@ -969,13 +992,12 @@ __device__ __forceinline__ void sums_run(const float* __restrict__ X, int D, con
         else if (c1)
             rows[n0 + __popc(b1 & lt)] = my_row;
         __syncwarp();
-        sums_side<VEC, Q>(X, D, Xq, Dq, rows, n0, dbase, hL, lL);
-        sums_side<VEC, Q>(X, D, Xq, Dq, rows + n0, __popc(b1), dbase, hR, lR);
+        sums_rows<VEC, Q>(X, D, Xq, Dq, rows, n0, n0 + __popc(b1), dbase, hL, lL, hR, lR);
     }
 }
 
 template <bool VEC>
-__global__ void __launch_bounds__(32 * kSumsWarps) k1_sums(const float* __restrict__ X, int D,
+__global__ void __launch_bounds__(32 * kSumsWarps, 2) k1_sums(const float* __restrict__ X, int D,
                                                           const int32_t* __restrict__ perm,
                                                           const int4* __restrict__ tiles,
                                                           const float* __restrict__ S,
