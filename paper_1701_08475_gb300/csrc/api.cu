@@ -478,7 +478,7 @@ struct TreePlan {
             lp.nsweep = (int)sweep.size() / 4;
             lp.max_m = max_m;
             lp.pos_bits = bits_for(max_m - 1);
-            lp.small = max_m <= kSmallMax;
+            lp.small = max_m <= kClusterSelectMax;
             lp.frozen = frozen;
             nseg_max = std::max(nseg_max, nseg);
             ntiles_max = std::max(ntiles_max, lp.ntiles);

@@ -53,7 +53,7 @@ struct LevelPlan {
     int ntiles;
     int max_m;        // largest segment size at this level
     int pos_bits;     // bits of a position inside a segment
-    bool small;       // one CTA per segment selects and partitions
+    bool small;       // one launch selects (kClusterSelectMax)
     int nsweep;       // sweep tiles (project, sums)
     const int32_t* seg_off;    // device [nseg + 1]
     const int4* tiles;         // device [ntiles] select tiles {seg, begin, end, first_of_seg}
@@ -102,7 +102,7 @@ struct SplitBuffers {
 
 constexpr int kTile = 2048;         // positions per select/partition tile
 constexpr int kSweepTile = 512;     // positions per project/sums tile
-constexpr int kSmallMax = 8192;     // segments up to this size select in one CTA
+constexpr int kClusterSelectMax = 131072;  // segments up to this size select and partition in one launch
 constexpr int kSortSelectMax = 2048; // segments up to this size select by a sort in registers
 constexpr int kRadixBits = 11;
 
@@ -110,6 +110,10 @@ constexpr int kRadixBits = 11;
 // shared memory; false (nothing launched) when the largest segment does not fit.
 bool launch_level(const float* X, int64_t n, int D, const LevelPlan& lp, int iters, uint64_t pass_seed,
                   const int32_t* perm_in, int32_t* perm_out, const SplitBuffers& b, cudaStream_t s);
+// The cut of segments of kSortSelectMax + 1 to 131,072 points (select.cu): the
+// selected key of every segment into thr, or, with perm_out, the partition.
+bool launch_select_cluster(const LevelPlan& lp, const float* S, uint64_t* thr, const int32_t* perm_in,
+                           int32_t* perm_out, int* status, cudaStream_t s);
 // One level of the balanced two-means tree: T Lloyd iterations, then the
 // final cut that writes perm_out.
 void run_split_level(const float* X, int64_t n_rows, int D, const LevelPlan& lp, int iters, uint64_t pass_seed,

@@ -62,7 +62,6 @@ __device__ __forceinline__ int block_sum(int v, int* warp_tot) {
     return total;
 }
 
-// Warp 0: digit b with below(b) <= krem < below(b) + hist[b].
 // Radix digits of a selection key (ord32(s) << pos_bits | position), from the
 // top: the 32 value bits in digits of 11, 11 and 10 bits, then the position
 // bits 11 at a time.  `hi` is a digit's upper bound; returns its lower one.
@@ -74,35 +73,9 @@ __host__ __device__ inline int digit_lo(int hi, int pos_bits) {
                          : (hi - kRadixBits > 0 ? hi - kRadixBits : 0);
 }
 
-__device__ __forceinline__ void find_digit(const uint32_t* hist, int nb, uint32_t krem, int* out_digit,
-                                           uint32_t* out_below) {
-    const int lane = threadIdx.x & 31;
-    const int per = nb >= 32 ? nb / 32 : 1;
-    const int b0 = lane * per;
-    uint32_t sum = 0;
-    for (int b = b0; b < b0 + per && b < nb; ++b) sum += hist[b];
-    uint32_t incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const uint32_t excl = incl - sum;
-    if (excl <= krem && krem < incl) {
-        uint32_t run = excl;
-        for (int b = b0; b < b0 + per && b < nb; ++b) {
-            if (krem < run + hist[b]) {
-                *out_digit = b;
-                *out_below = run;
-                break;
-            }
-            run += hist[b];
-        }
-    }
-}
-
-// find_digit with the whole CTA: thread t sums bins [t per, (t + 1) per), one
-// block scan, and the thread whose range holds rank krem walks its bins.
+// Digit b with below(b) <= krem < below(b) + hist[b]: thread t sums bins [t per,
+// (t + 1) per), one block scan, and the thread whose range holds rank krem walks
+// its bins.
 // Called by every thread of the CTA (it synchronises).
 __device__ __forceinline__ void block_find_digit(const uint32_t* hist, int nb, uint32_t krem, int* warp_tot,
                                                  int* out_digit, uint32_t* out_below) {
@@ -536,65 +509,6 @@ int sm_count() {
         return v > 0 ? v : 1;
     }();
     return n;
-}
-
-// Small segments: one CTA per segment keeps all keys in shared memory,
-// selects the floor(m/2)-th key, and either records it (thr) or, on the
-// final cut, partitions the segment stably into perm_out.
-__global__ void __launch_bounds__(1024) k1_select_small(const float* __restrict__ S,
-                                                        const int32_t* __restrict__ seg_off,
-                                                        const int32_t* __restrict__ seg_tile0, int pos_bits,
-                                                        uint64_t* __restrict__ thr,
-                                                        const int32_t* __restrict__ perm_in,
-                                                        int32_t* __restrict__ perm_out, int* __restrict__ status) {
-    extern __shared__ uint64_t keys[];
-    __shared__ uint32_t hist[1 << kRadixBits];
-    __shared__ int sh_digit;
-    __shared__ uint32_t sh_below;
-    __shared__ int warp_tot[32];
-    if (seg_tile0[blockIdx.x + 1] == seg_tile0[blockIdx.x]) return;  // a finished tree's leaf
-    const int seg = blockIdx.x, a = seg_off[seg], m = seg_off[seg + 1] - a;
-    for (int p = threadIdx.x; p < m; p += blockDim.x) keys[p] = sel_key(S[a + p], p, pos_bits);
-    uint64_t prefix = 0;
-    uint32_t krem = (uint32_t)(m / 2);
-    for (int hi = 32 + pos_bits, lo; hi > 0 && !(hi == pos_bits && krem == 0); hi = lo) {
-        lo = digit_lo(hi, pos_bits);
-        const int width = hi - lo;
-        const uint32_t mask = (1u << width) - 1u;
-        for (int b = threadIdx.x; b < (1 << width); b += blockDim.x) hist[b] = 0;
-        __syncthreads();
-        for (int p = threadIdx.x; p < m; p += blockDim.x) {
-            const uint64_t kk = keys[p];
-            if ((kk >> hi) == (prefix >> hi)) atomicAdd(&hist[(uint32_t)(kk >> lo) & mask], 1u);
-        }
-        __syncthreads();
-        if (threadIdx.x < 32) find_digit(hist, 1 << width, krem, &sh_digit, &sh_below);
-        __syncthreads();
-        prefix |= (uint64_t)sh_digit << lo;
-        krem -= sh_below;
-        __syncthreads();
-    }
-    if (perm_out == nullptr) {
-        if (threadIdx.x == 0) thr[seg] = prefix;
-        return;
-    }
-    const int K = m / 2;
-    int left_before = 0;
-    for (int base = 0; base < m; base += blockDim.x) {
-        const int p = base + threadIdx.x;
-        const int isl = (p < m) && keys[p] < prefix;
-        int tot;
-        const int ex = block_excl_scan(isl, warp_tot, &tot);
-        if (p < m) {
-            const int lb = left_before + ex;
-            const int np = isl ? lb : K + (p - lb);
-            if ((isl ? np < K : np < m) && np >= 0)
-                perm_out[a + np] = perm_in[a + p];
-            else
-                atomicOr(status, kStatusInternal);
-        }
-        left_before += tot;
-    }
 }
 
 // Segments of up to 32 R NW points: NW warps hold a segment's keys in
@@ -1613,7 +1527,7 @@ void run_split_level(const float* X, int64_t n_rows, int D, const LevelPlan& lp,
                 k1_project<false><<<lp.nsweep, 256, 0, s>>>(X, D, perm_in, lp.sweep, lp.seg_off, b.W, bi.S, st,
                                                             b.status, b.Xq, b.Dq, b.qtype, b.qflag);
         }
-        if (lp.small && lp.max_m <= kSortSelectMax) {
+        if (lp.max_m <= kSortSelectMax) {
             LaunchScope ls("k1_select_sort", s, n * 4 + (last ? n * 8 : 0), 0);
             int32_t* out = last ? perm_out : nullptr;
             if (lp.max_m <= 32)
@@ -1632,13 +1546,7 @@ void run_split_level(const float* X, int64_t n_rows, int D, const LevelPlan& lp,
                 launch_select_sort<8, 8>(lp, bi, perm_in, out, s);
             if (last) break;
         } else if (lp.small) {
-            const size_t smem = (size_t)lp.max_m * sizeof(uint64_t);
-            // one thread per point up to 1024, at least 4 warps
-            const int nt = std::min(1024, std::max(128, (lp.max_m + 31) & ~31));
-            LaunchScope ls("k1_select_small", s, n * 4 + (last ? n * 8 : 0), 0);
-            cudaFuncSetAttribute(k1_select_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            k1_select_small<<<lp.nseg, nt, smem, s>>>(bi.S, lp.seg_off, lp.seg_tile0, lp.pos_bits, bi.thr, perm_in,
-                                                      last ? perm_out : nullptr, b.status);
+            launch_select_cluster(lp, bi.S, bi.thr, perm_in, last ? perm_out : nullptr, b.status, s);
             if (last) break;
         } else {
             // every value digit is launched, then the position pass; a

@@ -65,3 +65,25 @@ def test_forest_of_uneven_depths(knng):
     for x, (ids, d) in zip(datas, knng.knng_build_batched(datas, p)):
         one, od = knng.knng_build_ex(x, p)
         assert torch.equal(ids, one) and torch.equal(d, od)
+
+
+@pytest.mark.parametrize("kind", ["signed", "few"])
+@pytest.mark.parametrize("n,D,levels", [(2049, 960, 1), (4100, 960, 2), (16384, 200, 1), (16385, 200, 1), (32769, 100, 2),
+                                        (65537, 64, 1), (131072, 64, 1), (131073, 64, 2)])
+def test_one_launch_cuts_of_larger_segments(knng, kind, n, D, levels):
+    """Rows too many for a cluster's shared memory: sweeps, with the cut of up to 131,072 points in one launch
+    (1, 2, 4 and 8 CTAs, one point more than each holds, hundreds of equal projections across CTAs)."""
+    X = _points(kind, n, D)
+    leaf = -(-n // 2 ** levels)
+    perm, off = knng.knng_partition(torch.from_numpy(X).cuda(), leaf, twomeans_iters=2, seed=3)
+    o_perm, o_off = oracle.partition(X, leaf, iters=2, seed=3)
+    assert np.array_equal(perm.cpu().numpy(), o_perm) and np.array_equal(off.cpu().numpy(), o_off)
+
+
+def test_cut_of_uneven_forest(knng):
+    """A level whose largest segment takes eight CTAs and whose smallest has fewer points than one warp."""
+    datas = [torch.from_numpy(_points("signed", n, 200)).cuda() for n in (40000, 30, 5000)]
+    p = knng.default_params(k=4, leaf_max=20, tree_passes=1, twomeans_iters=1, seed=6)
+    for x, (ids, d) in zip(datas, knng.knng_build_batched(datas, p)):
+        one, od = knng.knng_build_ex(x, p)
+        assert torch.equal(ids, one) and torch.equal(d, od)
