@@ -10,12 +10,15 @@
 // distance matrix reaches HBM; G is updated in place (a point lives in one
 // leaf per pass).
 //
-// Bound by its FP32 instructions and the selection's.  The rows come by
-// cp.async; with more dims than fit at once, equal chunks alternate between
-// two buffers.  Before that (a division and a 4-byte load per value, one
-// buffer, the last chunk padded to the first one's size) three passes over
-// 104,000 x 960 took 23.3 ms at leaves of up to 256 and 7.6 at 128, now 8.0 and
-// 3.9; 400,000 x 96 at 256 9.0, now 4.2, and at 128 3.7, now 3.5.
+// Bound by its FP32 instructions and the selection's.  Leaves whose dims fit
+// at once are held as interleaved pairs of points and computed with paired
+// instructions (400,000 points in three passes: 64 dims at leaves of up to 64
+// 1.38 -> 1.09 ms, 96 at 64 1.58 -> 1.33, 128 at 128 3.63 -> 3.30, 64 at 256
+// 3.04 -> 2.92).  With more dims, equal chunks come by cp.async and alternate
+// between two buffers.  Before that (a division and a 4-byte load per value,
+// one buffer, the last chunk padded to the first one's size) three passes over
+// 104,000 x 960 took 23.3 ms at leaves of up to 256 and 7.6 at 128, now 7.8 and
+// 3.9; 400,000 x 96 at 256 9.0, now 4.1, and at 128 3.7, now 3.3.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -32,20 +35,24 @@ struct LeafCfg {
 };
 
 // Dims per chunk, chunks (of equal size: the last one computes no more zeros
-// than it must) and padded stride (stride / 4 odd: conflict-free float4 rows).
-// Several chunks alternate between two buffers: the next one's copies are in
-// flight while one is used.
+// than it must) and padded stride.  One chunk: pair rows, which hold points 2 p
+// and 2 p + 1 of the leaf interleaved dim by dim for paired FP32 instructions.
+// Several chunks alternate between two buffers of plain rows: the next one's
+// 16-byte copies are in flight while one is used (copies that interleave move 4
+// bytes each, and cost more than the pairing saves: 104,000 x 960 at leaves of
+// 256 points 8.0 against 10.0 ms for three passes).  stride / 4 is odd: 16-byte
+// reads of consecutive rows are free of conflicts.
 __host__ __device__ inline void leaf_chunk(int D, int MC, int* dch, int* nch, int* stride) {
     const int d4 = (D + 3) & ~3;
     const int cap = (72 * 1024 / (MC * 4) - 4) & ~3, half = (36 * 1024 / (MC * 4) - 4) & ~3;
     *nch = d4 <= cap ? 1 : (d4 + half - 1) / half;
     const int c = ((d4 + *nch - 1) / *nch + 3) & ~3;
     *dch = c;
-    *stride = ((c / 4) & 1) ? c : c + 4;
+    *stride = *nch == 1 ? 2 * c + 4 : ((c / 4) & 1) ? c : c + 4;
 }
 
-// NB: CTAs per SM the registers must allow.
-template <int MC, int NSG, int NB>
+// NB: CTAs per SM the registers must allow.  PAIR: one chunk.
+template <int MC, int NSG, int NB, bool PAIR>
 __global__ void __launch_bounds__(LeafCfg<MC>::NT, NB) k2_leaf_fp32(const float* __restrict__ X, int D,
                                                                  const int32_t* __restrict__ perm,
                                                                  const int32_t* __restrict__ leaf_off, int k,
@@ -62,8 +69,8 @@ __global__ void __launch_bounds__(LeafCfg<MC>::NT, NB) k2_leaf_fp32(const float*
     extern __shared__ float4 smem4[];
     int dch, nch, stride;
     leaf_chunk(D, MC, &dch, &nch, &stride);
-    float* xs = reinterpret_cast<float*>(smem4);          // [1 or 2][MC][stride]
-    float* dt = xs + (nch > 1 ? 2 : 1) * MC * stride;      // [RB][MC + 1]
+    float* xs = reinterpret_cast<float*>(smem4);           // [MC / 2][stride], or [2][MC][stride]
+    float* dt = xs + (PAIR ? MC / 2 : 2 * MC) * stride;     // [RB][MC + 1]
     int32_t* ids = reinterpret_cast<int32_t*>(dt + C::RB * (MC + 1));  // [MC]
     uint64_t* wscratch = reinterpret_cast<uint64_t*>(ids + MC) + (threadIdx.x >> 5) * 32;  // 32 keys per warp
 
@@ -75,13 +82,23 @@ __global__ void __launch_bounds__(LeafCfg<MC>::NT, NB) k2_leaf_fp32(const float*
     for (int r = tid; r < MC; r += C::NT) ids[r] = r < m ? perm[a + r] : 0;
     __syncthreads();
 
-    // copies of chunk c's dims of every row into buffer c & 1 (zeros past the
-    // leaf and past D)
+    // chunk c's dims of every row (zeros past the leaf and past D)
     const bool vec = D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
     auto load_chunk = [&](int c) {
         const int d0 = c * dch, dl = min(dch, D - d0);
-        float* buf = xs + (c & 1) * MC * stride;
-        if (vec) {
+        float* buf = xs + (c & 1) * MC * stride;  // one chunk: xs
+        if (PAIR && vec) {
+            const int q4 = dch / 4;
+            for (int e = tid; e < (MC / 2) * q4; e += C::NT) {
+                const int p = e / q4, c4 = e - p * q4;
+                float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
+                if (4 * c4 < dl) {
+                    if (2 * p < m) u = __ldg(reinterpret_cast<const float4*>(X + (int64_t)ids[2 * p] * D) + c4);
+                    if (2 * p + 1 < m) v = __ldg(reinterpret_cast<const float4*>(X + (int64_t)ids[2 * p + 1] * D) + c4);
+                }
+                store_pairs(buf + p * stride + 8 * c4, u, v, (c4 >> 2) & 1);
+            }
+        } else if (vec) {
             const int q4 = dch / 4;
             // consecutive threads take a row's 16-byte pieces; the row moves on
             // by C::NT / q4 rows and a remainder, without a division per piece
@@ -108,26 +125,33 @@ __global__ void __launch_bounds__(LeafCfg<MC>::NT, NB) k2_leaf_fp32(const float*
                 const int r = e / dch, dd = e - r * dch;
                 float v = 0.f;
                 if (r < m && dd < dl) v = __ldg(X + (int64_t)ids[r] * D + d0 + dd);
-                buf[r * stride + dd] = v;
+                buf[PAIR ? (r >> 1) * stride + 2 * dd + (r & 1) : r * stride + dd] = v;
             }
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
-    if (nch == 1) {
+    if (PAIR) {
         load_chunk(0);
-        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         __syncthreads();
     }
 
     for (int rb = 0; rb * C::RB < m; ++rb) {
+        // the thread's 4 x 8 distances.  PAIR: rows 2 (rg + h RG) + {0, 1} and
+        // columns 2 (cg + w CG) + {0, 1}, as the sums of (0, 0), (1, 1) and of
+        // (1, 0), (0, 1).  Else rows rg + i RG and columns cg + j CG.
+        uint64_t same[2][4], cross[2][4];
         float acc[4][8];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int w = 0; w < 4; ++w) same[h][w] = cross[h][w] = 0ull;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
             for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
-        if (nch > 1) load_chunk(0);
-        for (int c = 0; c < nch; ++c) {
-            if (nch > 1) {
+        if (!PAIR) load_chunk(0);
+        for (int c = 0; c < (PAIR ? 1 : nch); ++c) {
+            if (!PAIR) {
                 if (c + 1 < nch) {
                     load_chunk(c + 1);
                     asm volatile("cp.async.wait_group 1;\n" ::: "memory");
@@ -136,35 +160,77 @@ __global__ void __launch_bounds__(LeafCfg<MC>::NT, NB) k2_leaf_fp32(const float*
                 }
                 __syncthreads();
             }
-            const float* rp = xs + (c & 1) * MC * stride + (rb * C::RB + rg) * stride;
-            const float* cp = xs + (c & 1) * MC * stride + cg * stride;
-            for (int dq = 0; dq < dch; dq += 4) {
-                float4 rv[4], cv[8];
+            if constexpr (PAIR) {
+                const float* rp = xs + (rb * (C::RB / 2) + rg) * stride;
+                const float* cp = xs + cg * stride;
+                for (int dq = 0; dq < 2 * dch; dq += 8) {  // 4 dims
+                    ulonglong2 r[2][2], x[2][2];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) rv[i] = *reinterpret_cast<const float4*>(rp + i * C::RG * stride + dq);
+                    for (int h = 0; h < 2; ++h)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) cv[j] = *reinterpret_cast<const float4*>(cp + j * C::CG * stride + dq);
+                        for (int p = 0; p < 2; ++p) {
+                            r[h][p] = *reinterpret_cast<const ulonglong2*>(rp + h * C::RG * stride + dq + 4 * p);
+                            x[h][p].x = swap_pair(r[h][p].x);
+                            x[h][p].y = swap_pair(r[h][p].y);
+                        }
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                    for (int w = 0; w < 4; ++w)
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        float t = __fsub_rn(rv[i].x, cv[j].x);
-                        acc[i][j] = __fmaf_rn(t, t, acc[i][j]);
-                        t = __fsub_rn(rv[i].y, cv[j].y);
-                        acc[i][j] = __fmaf_rn(t, t, acc[i][j]);
-                        t = __fsub_rn(rv[i].z, cv[j].z);
-                        acc[i][j] = __fmaf_rn(t, t, acc[i][j]);
-                        t = __fsub_rn(rv[i].w, cv[j].w);
-                        acc[i][j] = __fmaf_rn(t, t, acc[i][j]);
-                    }
+                        for (int p = 0; p < 2; ++p) {
+                            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(cp + w * C::CG * stride + dq + 4 * p);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                same[h][w] = add_square(r[h][p].x, v.x, same[h][w]);
+                                cross[h][w] = add_square(x[h][p].x, v.x, cross[h][w]);
+                                same[h][w] = add_square(r[h][p].y, v.y, same[h][w]);
+                                cross[h][w] = add_square(x[h][p].y, v.y, cross[h][w]);
+                            }
+                        }
+                }
+            } else {
+                const float* rp = xs + (c & 1) * MC * stride + (rb * C::RB + rg) * stride;
+                const float* cp = xs + (c & 1) * MC * stride + cg * stride;
+                for (int dq = 0; dq < dch; dq += 4) {
+                    float4 rv[4], cv[8];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) rv[i] = *reinterpret_cast<const float4*>(rp + i * C::RG * stride + dq);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) cv[j] = *reinterpret_cast<const float4*>(cp + j * C::CG * stride + dq);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            float t = __fsub_rn(rv[i].x, cv[j].x);
+                            acc[i][j] = __fmaf_rn(t, t, acc[i][j]);
+                            t = __fsub_rn(rv[i].y, cv[j].y);
+                            acc[i][j] = __fmaf_rn(t, t, acc[i][j]);
+                            t = __fsub_rn(rv[i].z, cv[j].z);
+                            acc[i][j] = __fmaf_rn(t, t, acc[i][j]);
+                            t = __fsub_rn(rv[i].w, cv[j].w);
+                            acc[i][j] = __fmaf_rn(t, t, acc[i][j]);
+                        }
+                }
             }
-            if (nch > 1) __syncthreads();  // the buffer is refilled
+            if (!PAIR) __syncthreads();  // the buffer is refilled
         }
         __syncthreads();  // previous selection done with dt
+        if constexpr (PAIR) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+            for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int j = 0; j < 8; ++j) dt[(rg + i * C::RG) * (MC + 1) + cg + j * C::CG] = acc[i][j];
+                for (int w = 0; w < 4; ++w) {
+                    float* at = dt + 2 * (rg + h * C::RG) * (MC + 1) + 2 * (cg + w * C::CG);
+                    at[0] = __uint_as_float((uint32_t)same[h][w]);
+                    at[MC + 2] = __uint_as_float((uint32_t)(same[h][w] >> 32));
+                    at[MC + 1] = __uint_as_float((uint32_t)cross[h][w]);
+                    at[1] = __uint_as_float((uint32_t)(cross[h][w] >> 32));
+                }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 8; ++j) dt[(rg + i * C::RG) * (MC + 1) + cg + j * C::CG] = acc[i][j];
+        }
         __syncthreads();
         // one warp per row: k best of G[i] + leaf candidates
         for (int r = warp; r < C::RB; r += C::NT / 32) {
@@ -220,9 +286,10 @@ void launch_leaf_t(const float* X, int D, const int32_t* perm, const int32_t* le
     using C = LeafCfg<MC>;
     int dch, nch, stride;
     leaf_chunk(D, MC, &dch, &nch, &stride);
-    const size_t smem = (size_t)(nch > 1 ? 2 : 1) * MC * stride * 4 + (size_t)C::RB * (MC + 1) * 4 + MC * 4 + (C::NT / 32) * 32 * 8;
-    cudaFuncSetAttribute(k2_leaf_fp32<MC, NSG, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k2_leaf_fp32<MC, NSG, NB><<<nleaf, C::NT, smem, s>>>(X, D, perm, leaf_off, k, G, status, skip);
+    const size_t smem = (size_t)(nch > 1 ? 2 * MC : MC / 2) * stride * 4 + (size_t)C::RB * (MC + 1) * 4 + MC * 4 + (C::NT / 32) * 32 * 8;
+    auto kernel = nch == 1 ? k2_leaf_fp32<MC, NSG, NB, true> : k2_leaf_fp32<MC, NSG, NB, false>;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kernel<<<nleaf, C::NT, smem, s>>>(X, D, perm, leaf_off, k, G, status, skip);
 }
 
 }  // namespace
