@@ -19,9 +19,6 @@
 
 namespace knng {
 
-size_t join_smem_bytes(int D, int mcap);
-int join_blocks_per_lane(int mcap);
-
 // ---------------------------------------------------------------- errors
 namespace {
 thread_local std::string g_last_error;

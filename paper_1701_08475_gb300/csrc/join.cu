@@ -383,341 +383,58 @@ __global__ void __launch_bounds__(256) k6_active(const int32_t* __restrict__ ord
 }
 
 // ---------------------------------------------------------------- K5
-// One warp per node i.  Members N_i in shared memory; the upper triangle of
-// member pairs is cut into 4 x 4 blocks, BPL blocks per lane; distances are
-// canonical (dims ascending, fmaf); surviving offers are appended to the
-// chunk's buffer.
-constexpr int kJoinWarps = 4;
-
-// Dims per shared-memory chunk (about 12 KB of member rows per warp, equal
-// chunks) and the stride of a pair row, which holds members 2 p and 2 p + 1
-// interleaved dim by dim for paired FP32 instructions (stride / 4 odd:
-// consecutive pair rows in different banks for 16-byte reads).
-__host__ __device__ inline void join_chunk(int D, int mcap, int* dch, int* stride) {
-    const int d4 = (D + 3) & ~3;
-    int cap = (12 * 1024 / (mcap * 4) - 4) & ~3;
-    if (cap < 4) cap = 4;
-    const int nch = (d4 + cap - 1) / cap;
-    const int c = ((d4 + nch - 1) / nch + 3) & ~3;
-    *dch = c;
-    *stride = 2 * c + 4;
-}
-
-// A warp's shared memory: the members' pair rows, thresholds and ids (mcap is
-// a multiple of 4).
-__host__ __device__ inline size_t join_warp_bytes(int mcap, int stride) {
-    return ((size_t)(mcap / 2) * stride * 4 + (size_t)mcap * 12 + 31) & ~(size_t)15;
-}
-
-// Whether entry (a, b) of block row ia, column ib is a pair to evaluate:
-// in the rectangle ia is a new member and ib any later member or an old one;
-// in the triangle `upper` says the entry is above the diagonal.  Pairs of
-// two old members (indices >= nn) are skipped.
-__device__ __forceinline__ bool pair_live(bool rect, int ia, int ib, int M, int nn, bool upper) {
-    if (rect) return ia < nn && ib < M && (ib >= nn || ib > ia);
-    return ia < M && ib < M && upper && (ia < nn || ib < nn);
-}
-
-// The local join of node i by one warp (members, distances, offers).
-template <int BPL>
-__device__ __forceinline__ void join_node(const float* __restrict__ X, int D, int k, int rev, int mcap,
-                                          const uint64_t* __restrict__ Gold, const uint64_t* __restrict__ R,
-                                          const uint64_t* __restrict__ fnew, const uint64_t* __restrict__ rnew,
-                                          int64_t i, uint32_t* __restrict__ counter, int64_t cap,
-                                          uint32_t* __restrict__ ptgt, uint64_t* __restrict__ pkey,
-                                          int32_t* __restrict__ pcnt, int* __restrict__ status, float* xs,
-                                          uint64_t* thr, int32_t* mem, int dch, int stride) {
-    const int lane = threadIdx.x & 31;
-    __syncwarp();  // the warp's previous node is done with xs, thr and mem
-    // members: the new ones first (flags from the previous round; none =
-    // all new), then the old ones; each takes ids of G_old[i], then of R[i]
-    int M = 0, nn = 0;
-    const uint64_t fbits = fnew ? fnew[i] : ~0ull, rbits = rnew ? rnew[i] : ~0ull;
-    auto take_member = [&](uint64_t key, bool take) {
-        const unsigned bal = __ballot_sync(0xffffffffu, take);
-        if (take) {
-            const int at = M + __popc(bal & ((1u << lane) - 1u));
-            const uint32_t u = key_id(key);
-            mem[at] = (int32_t)u;
-            thr[at] = Gold[(int64_t)u * k + k - 1];
-        }
-        M += __popc(bal);
-    };
-    if (!(rev && k > 32)) {
-        // at most 64 entries, a mutual neighbour once
-        uint64_t key0, key1;
-        bool new0, new1;
-        member_keys(Gold, R, i, k, rev != 0, fbits, rbits, key0, key1, new0, new1);
-        for (int want = 1; want >= 0; --want) {
-            take_member(key0, key0 != kEmptyKey && new0 == (want == 1));
-            take_member(key1, key1 != kEmptyKey && new1 == (want == 1));
-            if (want == 1) nn = M;
-        }
-    } else {
-        for (int want = 1; want >= 0; --want) {
-            for (int src = 0; src < 2; ++src) {
-                const uint64_t* row = (src == 0 ? Gold : R) + i * k;
-                const uint64_t bits = src == 0 ? fbits : rbits;
-                for (int e0 = 0; e0 < k; e0 += 32) {
-                    const int e = e0 + lane;
-                    const uint64_t key = e < k ? row[e] : kEmptyKey;
-                    take_member(key, key != kEmptyKey && (int)((bits >> e) & 1ull) == want);
-                }
-            }
-            if (want == 1) nn = M;
-        }
-    }
-    __syncwarp();
-    if (M < 2 || nn == 0) return;
-    // Pairs with a new member: the upper triangle of all members cut into
-    // 4 x 4 blocks, or, when fewer blocks do, the rectangle new x all (rows
-    // 0 .. nn-1 against every member, each new x new pair kept once).
-    const int RGN = (M + 3) >> 2;
-    const int nb_tri = RGN * (RGN + 1) / 2;
-    const int RBN = (nn + 3) >> 2;
-    const bool rect = RBN * RGN < nb_tri;
-    const int nb = rect ? RBN * RGN : nb_tri;
-    const int RSTEP = rect ? RBN : RGN;  // member index step between a block's rows
-    int brg[BPL], bcg[BPL];
-#pragma unroll
-    for (int q = 0; q < BPL; ++q) {
-        int b = lane + 32 * q;
-        brg[q] = -1;
-        bcg[q] = 0;
-        if (b < nb) {
-            if (rect) {
-                brg[q] = b / RGN;
-                bcg[q] = b - brg[q] * RGN;
-            } else {
-                int rg = 0;
-                while (b >= RGN - rg) {
-                    b -= RGN - rg;
-                    ++rg;
-                }
-                brg[q] = rg;
-                bcg[q] = rg + b;
-            }
-        }
-    }
-    // sums of members (2 h, 2 w), (2 h + 1, 2 w + 1) of the block, and of
-    // (2 h, 2 w + 1), (2 h + 1, 2 w)
-    uint64_t same[BPL][2][2], cross[BPL][2][2];
-#pragma unroll
-    for (int q = 0; q < BPL; ++q)
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int w = 0; w < 2; ++w) same[q][h][w] = cross[q][h][w] = 0ull;
-    const bool vec = (D % 4 == 0);
-    for (int d0 = 0; d0 < D; d0 += dch) {
-        const int dl = min(dch, D - d0);
-        // gather the members' dims [d0, d0 + dch); members M .. 4 RGN - 1
-        // read as zeros
-        if (vec) {
-            const int q4 = dch >> 2;
-            for (int e = lane; e < RGN * 2 * q4; e += 32) {
-                const int p = e / q4, c4 = e - p * q4;
-                float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
-                if (c4 * 4 < dl) {
-                    if (2 * p < M) u = __ldg(reinterpret_cast<const float4*>(X + (int64_t)mem[2 * p] * D + d0) + c4);
-                    if (2 * p + 1 < M)
-                        v = __ldg(reinterpret_cast<const float4*>(X + (int64_t)mem[2 * p + 1] * D + d0) + c4);
-                }
-                store_pairs(xs + p * stride + c4 * 8, u, v, (c4 >> 2) & 1);
-            }
-        } else {
-            for (int e = lane; e < RGN * 2 * dch; e += 32) {
-                const int p = e / dch, c = e - p * dch;
-                const bool in = c < dl;
-                *reinterpret_cast<float2*>(xs + p * stride + 2 * c) =
-                    make_float2(in && 2 * p < M ? __ldg(X + (int64_t)mem[2 * p] * D + d0 + c) : 0.f,
-                                in && 2 * p + 1 < M ? __ldg(X + (int64_t)mem[2 * p + 1] * D + d0 + c) : 0.f);
-            }
-        }
-        __syncwarp();
-        // block (rg, cg) holds the members of pair rows {rg, rg + RSTEP} x
-        // {cg, cg + RGN}: lanes then read consecutive pair rows
-#pragma unroll
-        for (int q = 0; q < BPL; ++q) {
-            if (brg[q] < 0) continue;
-            const float* rp = xs + brg[q] * stride;
-            const float* cp = xs + bcg[q] * stride;
-            const int rstep = RSTEP * stride, cstep = RGN * stride;
-            for (int dq = 0; dq < 2 * dch; dq += 8) {  // 4 dims
-                ulonglong2 r[2][2], c[2][2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-#pragma unroll
-                    for (int p = 0; p < 2; ++p) {
-                        r[h][p] = *reinterpret_cast<const ulonglong2*>(rp + h * rstep + dq + 4 * p);
-                        c[h][p] = *reinterpret_cast<const ulonglong2*>(cp + h * cstep + dq + 4 * p);
-                    }
-#pragma unroll
-                for (int p = 0; p < 2; ++p)
-#pragma unroll
-                    for (int w = 0; w < 2; ++w) {
-                        const uint64_t c0 = c[w][p].x, c1 = c[w][p].y, x0 = swap_pair(c0), x1 = swap_pair(c1);
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            same[q][h][w] = add_square(r[h][p].x, c0, same[q][h][w]);
-                            cross[q][h][w] = add_square(r[h][p].x, x0, cross[q][h][w]);
-                            same[q][h][w] = add_square(r[h][p].y, c1, same[q][h][w]);
-                            cross[q][h][w] = add_square(r[h][p].y, x1, cross[q][h][w]);
-                        }
-                    }
-            }
-        }
-        __syncwarp();
-    }
-    float acc[BPL][4][4];
-#pragma unroll
-    for (int q = 0; q < BPL; ++q)
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int w = 0; w < 2; ++w) {
-                acc[q][2 * h][2 * w] = __uint_as_float((uint32_t)same[q][h][w]);
-                acc[q][2 * h + 1][2 * w + 1] = __uint_as_float((uint32_t)(same[q][h][w] >> 32));
-                acc[q][2 * h][2 * w + 1] = __uint_as_float((uint32_t)cross[q][h][w]);
-                acc[q][2 * h + 1][2 * w] = __uint_as_float((uint32_t)(cross[q][h][w] >> 32));
-            }
-    // entry (a, b) of a block: member a % 2 of pair row a / 2 of the rows, the same for the columns
-    auto row_of = [&](int q, int a) { return 2 * (brg[q] + (a >> 1) * RSTEP) + (a & 1); };
-    auto col_of = [&](int q, int b) { return 2 * (bcg[q] + (b >> 1) * RGN) + (b & 1); };
-    // offers: count, reserve, write.  In the triangle every unordered member
-    // pair lies in exactly one block once diagonal blocks keep only a < b;
-    // pairs of two old members are dropped.
-    int cnt = 0;
-#pragma unroll
-    for (int q = 0; q < BPL; ++q) {
-        if (brg[q] < 0) continue;
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const int ia = row_of(q, a), ib = col_of(q, b);
-                if (pair_live(rect, ia, ib, M, nn, brg[q] < bcg[q] || a < b)) {
-                    const uint32_t u = (uint32_t)mem[ia], v = (uint32_t)mem[ib];
-                    if (u != v) {
-                        cnt += make_key(acc[q][a][b], v) < thr[ia];
-                        cnt += make_key(acc[q][a][b], u) < thr[ib];
-                    }
-                }
-            }
-    }
-    const int incl = warp_incl_scan(cnt);
-    const int total = __shfl_sync(0xffffffffu, incl, 31);
-    if (total == 0) return;
-    uint32_t at = 0;
-    if (lane == 31) at = atomicAdd(counter, (uint32_t)total);
-    at = __shfl_sync(0xffffffffu, at, 31);
-    if ((int64_t)at + total > cap) {
-        if (lane == 0) atomicOr(status, kStatusOverflow);
-        return;
-    }
-    uint32_t w = at + incl - cnt;
-#pragma unroll
-    for (int q = 0; q < BPL; ++q) {
-        if (brg[q] < 0) continue;
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const int ia = row_of(q, a), ib = col_of(q, b);
-                if (pair_live(rect, ia, ib, M, nn, brg[q] < bcg[q] || a < b)) {
-                    const uint32_t u = (uint32_t)mem[ia], v = (uint32_t)mem[ib];
-                    if (u != v) {
-                        const uint64_t ku = make_key(acc[q][a][b], v);
-                        if (ku < thr[ia]) {
-                            ptgt[w] = u;
-                            pkey[w] = ku;
-                            ++w;
-                            atomicAdd(&pcnt[u], 1);
-                        }
-                        const uint64_t kv = make_key(acc[q][a][b], u);
-                        if (kv < thr[ib]) {
-                            ptgt[w] = v;
-                            pkey[w] = kv;
-                            ++w;
-                            atomicAdd(&pcnt[v], 1);
-                        }
-                    }
-                }
-            }
-    }
-}
-
-// Warps stride over the node positions [node0, node1) (of `list` when given).
-template <int BPL>
-__global__ void __launch_bounds__(32 * kJoinWarps) k5_join(const float* __restrict__ X, int D, int k, int rev,
-                                                          int mcap, const uint64_t* __restrict__ Gold,
-                                                          const uint64_t* __restrict__ R,
-                                                          const int32_t* __restrict__ list,
-                                                          const uint64_t* __restrict__ fnew,
-                                                          const uint64_t* __restrict__ rnew, int64_t node0,
-                                                          int64_t node1, uint32_t* __restrict__ counter,
-                                                          int64_t cap, uint32_t* __restrict__ ptgt,
-                                                          uint64_t* __restrict__ pkey,
-                                                          int32_t* __restrict__ pcnt, int* __restrict__ status,
-                                                          const int* __restrict__ skip_if_exact,
-                                                          const int32_t* __restrict__ count_dev) {
-    extern __shared__ float4 smem4[];
-    if (*status & kStatusStop) return;
-    if (count_dev && (int64_t)*count_dev < node1) node1 = *count_dev;
-    // the tensor-core join does this round when the 16-bit copy is exact
-    if (skip_if_exact) {
-        const int f = *skip_if_exact;
-        if ((f & 1) == 0 && !((f & 2) && (f & 4))) return;
-    }
-    int dch, stride;
-    join_chunk(D, mcap, &dch, &stride);
-    const int warp = threadIdx.x >> 5;
-    char* base = reinterpret_cast<char*>(smem4) + (size_t)warp * join_warp_bytes(mcap, stride);
-    float* xs = reinterpret_cast<float*>(base);                                   // [mcap / 2][stride]
-    uint64_t* thr = reinterpret_cast<uint64_t*>(xs + (size_t)(mcap / 2) * stride);  // [mcap]
-    int32_t* mem = reinterpret_cast<int32_t*>(thr + mcap);                        // [mcap]
-    for (int64_t pos = node0 + (int64_t)blockIdx.x * kJoinWarps + warp; pos < node1;
-         pos += (int64_t)gridDim.x * kJoinWarps)
-        join_node<BPL>(X, D, k, rev, mcap, Gold, R, fnew, rnew, list ? (int64_t)list[pos] : pos, counter, cap, ptgt,
-                       pkey, pcnt, status, xs, thr, mem, dch, stride);
-}
-
-// ---------------------------------------------------------------- K5, CTA-wide
 // The FP32 local join with the pairs of several nodes spread over one CTA.
 // A node's member pairs are cut into the 4 x 4 blocks of the upper triangle
 // of its (mcap / 4)-group member grid: NB = RGN (RGN + 1) / 2 blocks, RGN =
-// mcap / 4; a CTA of 256 threads takes G = 256 / NB nodes at a time and
-// thread t computes block t % NB of node t / NB, so a warp's lanes stay busy
-// whatever NB is (one node per warp leaves lanes idle when NB is not a
-// multiple of 32).  Block (rg, cg) holds members {4 rg + a} x {4 cg + b}.
-// Members are new first, so blocks whose two groups hold only old members are
-// skipped whole.  Offers as in k5_join; a pair of members that shared a leaf in
-// one of the build's last tree passes makes none (the leaf stage offered it
-// already).
+// mcap / 4; a CTA of 256 threads takes G = 256 / NB nodes at a time.  Block
+// (rg, cg) holds members {4 rg + a} x {4 cg + b}.  Distances are canonical
+// (dims ascending, fmaf); surviving offers are appended to the chunk's buffer.
+// A pair of members that shared a leaf in one of the build's last tree passes
+// makes none (the leaf stage offered it already).
 //
-// Bound by issue slots.  So the differences and sums are paired FP32
-// instructions, two pairs of members each: members 4 g + 2 h and 4 g + 2 h + 1
-// are staged interleaved dim by dim in row h RGN + g, (r0, r1) - (c0, c1) and
-// (r0, r1) - (c1, c0) give all four differences of two such rows, and every
-// sum keeps its chain.  Lanes of consecutive cg read consecutive rows (an odd
-// number of 16-byte pieces apart: different banks), lanes of one rg the same.
-// First round on 1M x 96, k = 16: 6.5 ms with scalar instructions (70 % of issue
-// slots used), 5.3 paired (59 %; the FMA pipe 48 %).
+// Only blocks that can make an offer are computed: both groups hold members,
+// one holds a new one (members are new first), and, in the first round, some
+// pair shared no leaf (there the members come in the order of the leaf they
+// share with the node, which makes whole blocks of leaf-mates).  1M x 96,
+// k = 16: 8.7 of the 21 blocks in the first round, then 11.1, 8.2 and 5.7.
+// They are listed in shared memory and dealt one per thread, so full warps
+// compute and the others go on to wait; co-resident CTAs start at different
+// warps.
+//
+// Bound by issue slots and the barriers between gather and sums.  So the
+// differences and sums are paired FP32 instructions, two pairs of members
+// each: members 4 g + 2 h and 4 g + 2 h + 1 are staged interleaved dim by dim
+// in row h RGN + g, (r0, r1) - (c0, c1) and (r0, r1) - (c1, c0) give all four
+// differences of two such rows, and every sum keeps its chain.  Lanes of
+// consecutive cg read consecutive rows (an odd number of 16-byte pieces apart:
+// different banks), lanes of one rg the same.  The gather's indices are
+// stepped without divisions and two pieces are in flight per thread (one or
+// three: 16.7 and 16.3 ms against 15.9 below); offers are a bit mask per
+// thread, so that only the pairs that make one are visited again.  128 threads
+// a CTA: 20.5.
+// Four rounds on 1M x 96, k = 16: 31.8 ms with every block and scalar
+// instructions, 27.1 paired, 21.3 with the live blocks dealt densely, 19.8
+// with the stepped gather, 15.9 with the mask.  A form with one node per warp
+// is gone: with the same gains it would idle the lanes past a node's blocks
+// (100,000 x 960, k = 20: 17.8 against 11.6 ms; 300,000 x 96, k = 32: 24.0
+// against 12.7; forward lists of 64: 40.6 against 23.8; none was faster).
 constexpr int kJ2Threads = 256;
+constexpr int kJ2Dist = 20;  // floats of a thread's 16 distances in shared memory (16 plus padding)
+constexpr int kJ2Ahead = 2;  // pieces of the gather in flight per thread
 
 struct J2Layout {
     int RGN, NB, G, dch, stride;
-    size_t thr, lid, rows, mem, cnt, total;
+    size_t thr, lid, rows, mem, cnt, live, total;
 };
 
 __host__ __device__ inline J2Layout j2_layout(int D, int mcap, bool leafids) {
     J2Layout L;
     L.RGN = mcap / 4;
     L.NB = L.RGN * (L.RGN + 1) / 2;
-    L.G = L.NB > kJ2Threads ? 1 : kJ2Threads / L.NB;
+    L.G = kJ2Threads / L.NB;  // mcap <= 64: NB <= 136
     const int slots = L.G * mcap;
     const int d4 = (D + 3) & ~3;
-    int cap = (44 * 1024 / (slots * 4) - 4) & ~3;
+    int cap = (kJ2Threads * 176 / (slots * 4) - 4) & ~3;
     if (cap < 4) cap = 4;
     const int nch = (d4 + cap - 1) / cap;
     L.dch = ((d4 + nch - 1) / nch + 3) & ~3;
@@ -725,15 +442,19 @@ __host__ __device__ inline J2Layout j2_layout(int D, int mcap, bool leafids) {
     L.thr = 0;
     L.lid = L.thr + (size_t)slots * 8;
     L.rows = L.lid + (leafids ? (size_t)slots * 16 : 0);
-    L.mem = L.rows + (size_t)(slots / 2) * L.stride * 4;
+    const size_t rows = (size_t)(slots / 2) * L.stride * 4, dist = (size_t)kJ2Threads * kJ2Dist * 4;
+    L.mem = L.rows + (rows > dist ? rows : dist);
     L.cnt = L.mem + (size_t)slots * 4;
-    L.total = L.cnt + (size_t)L.G * 2 * 4;
+    L.live = L.cnt + (size_t)L.G * 2 * 4;
+    L.total = L.live + (size_t)(1 + kJ2Threads) * 4;
     return L;
 }
 
 __device__ __forceinline__ int j2_slot(int m, int RGN) { return (m & 3) * RGN + (m >> 2); }
+// Where member m's id lies: pair row p's two ids are neighbours.
+__device__ __forceinline__ int j2_mem(int m, int RGN) { return 2 * ((m & 2) / 2 * RGN + (m >> 2)) + (m & 1); }
 
-__global__ void __launch_bounds__(kJ2Threads, 4) k5_join_cta(const float* __restrict__ X, int D, int k, int rev,
+__global__ void __launch_bounds__(kJ2Threads, 1024 / kJ2Threads) k5_join_cta(const float* __restrict__ X, int D, int k, int rev,
                                                          int mcap, const uint64_t* __restrict__ Gold,
                                                          const uint64_t* __restrict__ R,
                                                          const int32_t* __restrict__ list,
@@ -760,28 +481,37 @@ __global__ void __launch_bounds__(kJ2Threads, 4) k5_join_cta(const float* __rest
     uint64_t* thr = reinterpret_cast<uint64_t*>(base + L.thr);  // [G][mcap] by slot
     int4* slid = reinterpret_cast<int4*>(base + L.lid);         // [G][mcap] by slot
     float* rows = reinterpret_cast<float*>(base + L.rows);      // [G][mcap / 2][stride] by pair row
-    int32_t* mem = reinterpret_cast<int32_t*>(base + L.mem);    // [G][mcap] by member index
+    int32_t* mem = reinterpret_cast<int32_t*>(base + L.mem);    // [G][mcap / 2][2] by pair row, -1: none
     int* cnt = reinterpret_cast<int*>(base + L.cnt);            // [G] members, then [G] new members
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int RGN = L.RGN, NB = L.NB, G = L.G, dch = L.dch, stride = L.stride;
-    // this thread's block, fixed for the launch
-    const int jn = tid / NB, bk = tid - jn * NB;
-    int rg = 0, cg = 0;
-    {
-        int b = bk;
-        while (b >= RGN - rg) {
-            b -= RGN - rg;
-            ++rg;
+    int* nlive = reinterpret_cast<int*>(base + L.live);  // blocks to compute, then the blocks
+    uint32_t* items = reinterpret_cast<uint32_t*>(nlive + 1);  // node | rg << 8 | cg << 16
+    // the block this thread lists, fixed for the launch
+    uint32_t own = 0u;
+    if (tid < G * NB) {
+        const int j = tid / NB;
+        int b = tid - j * NB, g = 0;
+        while (b >= RGN - g) {
+            b -= RGN - g;
+            ++g;
         }
-        cg = rg + b;
+        own = (uint32_t)(j | g << 8 | (g + b) << 16);
     }
-    const bool vec = (D % 4 == 0);
+    // every member is new in a build's first round: then most pairs are leaf-mates
+    const bool by_leaf = lids && fnew == nullptr && rnew == nullptr;
+    const bool vec = D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    // the gather's pieces: piece c4 of pair row pr, stepped without divisions
+    const int q4 = dch >> 2, half = mcap / 2;
+    const int pr0 = tid / q4, c40 = tid - pr0 * q4, dpr = kJ2Threads / q4, dc = kJ2Threads - dpr * q4;
     const int64_t ngroups = (node1 - node0 + G - 1) / G;
     for (int64_t grp = blockIdx.x; grp < ngroups; grp += gridDim.x) {
         const int64_t first = node0 + grp * G;
+        if (tid == 0) *nlive = 0;
         // members of the group's nodes (warp w collects nodes w, w + 8, ...):
         // the new ones first, then the old ones; each takes ids of G_old[i],
-        // then of R[i]
+        // then of R[i] (by_leaf: in the order of the first pass in which they
+        // share i's leaf)
         for (int j = warp; j < G; j += kJ2Threads / 32) {
             const int64_t pos = first + j;
             int M = 0, nn = 0;
@@ -794,90 +524,134 @@ __global__ void __launch_bounds__(kJ2Threads, 4) k5_join_cta(const float* __rest
                         const int m = M + __popc(bal & ((1u << lane) - 1u));
                         const uint32_t u = key_id(key);
                         const int sl = j * mcap + j2_slot(m, RGN);
-                        mem[j * mcap + m] = (int32_t)u;
+                        mem[j * mcap + j2_mem(m, RGN)] = (int32_t)u;
                         thr[sl] = Gold[(int64_t)u * k + k - 1];
                         if (lids) slid[sl] = __ldg(reinterpret_cast<const int4*>(leafid) + u);
                     }
                     M += __popc(bal);
                 };
-                if (!(rev && k > 32)) {
-                    // at most 64 entries, a mutual neighbour once
-                    uint64_t key0, key1;
-                    bool new0, new1;
-                    member_keys(Gold, R, i, k, rev != 0, fbits, rbits, key0, key1, new0, new1);
-                    // more members than the slot holds (slots smaller than 2k):
-                    // the node goes to the overflow list, for the full-slot launch
-                    const int all = __popc(__ballot_sync(0xffffffffu, key0 != kEmptyKey)) +
-                                    __popc(__ballot_sync(0xffffffffu, key1 != kEmptyKey));
-                    if (all > mcap) {
-                        if (lane == 0) ovf_list[atomicAdd(ovf_count, 1)] = (int32_t)i;
-                        key0 = key1 = kEmptyKey;
+                // at most 64 entries, a mutual neighbour once
+                uint64_t key0, key1;
+                bool new0, new1;
+                member_keys(Gold, R, i, k, rev != 0, fbits, rbits, key0, key1, new0, new1);
+                // more members than the slot holds (slots smaller than 2k):
+                // the node goes to the overflow list, for the full-slot launch
+                const int all = __popc(__ballot_sync(0xffffffffu, key0 != kEmptyKey)) +
+                                __popc(__ballot_sync(0xffffffffu, key1 != kEmptyKey));
+                if (all > mcap) {
+                    if (lane == 0) ovf_list[atomicAdd(ovf_count, 1)] = (int32_t)i;
+                    key0 = key1 = kEmptyKey;
+                }
+                if (by_leaf) {
+                    const int4* lp = reinterpret_cast<const int4*>(leafid);
+                    const int4 li = __ldg(lp + i);
+                    const int q0 = key0 == kEmptyKey ? -1 : leaf_shared(li, __ldg(lp + key_id(key0)), npass);
+                    const int q1 = key1 == kEmptyKey ? -1 : leaf_shared(li, __ldg(lp + key_id(key1)), npass);
+                    for (int q = 0; q <= npass; ++q) {
+                        take_member(key0, q0 == q);
+                        take_member(key1, q1 == q);
                     }
+                    nn = M;
+                } else {
                     for (int want = 1; want >= 0; --want) {
                         take_member(key0, key0 != kEmptyKey && new0 == (want == 1));
                         take_member(key1, key1 != kEmptyKey && new1 == (want == 1));
                         if (want == 1) nn = M;
                     }
-                } else {
-                    for (int want = 1; want >= 0; --want) {
-                        for (int src = 0; src < 2; ++src) {
-                            const uint64_t* row = (src == 0 ? Gold : R) + i * k;
-                            const uint64_t bits = src == 0 ? fbits : rbits;
-                            for (int e0 = 0; e0 < k; e0 += 32) {
-                                const int e = e0 + lane;
-                                const uint64_t key = e < k ? row[e] : kEmptyKey;
-                                take_member(key, key != kEmptyKey && (int)((bits >> e) & 1ull) == want);
-                            }
-                        }
-                        if (want == 1) nn = M;
-                    }
                 }
             }
+            for (int m = M + lane; m < mcap; m += 32) mem[j * mcap + j2_mem(m, RGN)] = -1;
             if (lane == 0) {
                 cnt[j] = M;
                 cnt[G + j] = nn;
             }
         }
         __syncthreads();
-        const int Mj = jn < G ? cnt[jn] : 0, nnj = jn < G ? cnt[G + jn] : 0;
-        // a block with a live pair: both groups hold members, one holds a new one
-        const bool live = jn < G && 4 * rg < Mj && 4 * cg < Mj && (4 * rg < nnj || 4 * cg < nnj);
+        // list the blocks that can make an offer: both groups hold members, one
+        // holds a new one, and not every pair of theirs shared a leaf
+        {
+            bool on = false;
+            if (tid < G * NB) {
+                const int j = own & 255, rg = own >> 8 & 255, cg = own >> 16, M = cnt[j], nn = cnt[G + j];
+                on = 4 * cg < M && (4 * rg < nn || 4 * cg < nn);
+                if (on && by_leaf) {
+                    on = false;
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        const int4 lb = slid[j * mcap + b * RGN + cg];
+#pragma unroll
+                        for (int a = 0; a < 4; ++a)
+                            on |= 4 * rg + a < M && 4 * cg + b < M && (rg < cg || a < b) &&
+                                  !leaf_mates(slid[j * mcap + a * RGN + rg], lb, npass);
+                    }
+                }
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, on);
+            int at = 0;
+            if (lane == 0 && bal) at = atomicAdd(nlive, __popc(bal));
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (on) items[at + __popc(bal & ((1u << lane) - 1u))] = own;
+        }
+        bool live = false;
+        int jn = 0, rg = 0, cg = 0, Mj = 0, nnj = 0;
         // sums of (2 h, 2 w), (2 h + 1, 2 w + 1) and of (2 h, 2 w + 1), (2 h + 1, 2 w)
         uint64_t same[2][2], cross[2][2];
 #pragma unroll
         for (int h = 0; h < 2; ++h)
 #pragma unroll
             for (int w = 0; w < 2; ++w) same[h][w] = cross[h][w] = 0ull;
-        const int q4 = dch >> 2, half = mcap / 2;
         for (int d0 = 0; d0 < D; d0 += dch) {
             const int dl = min(dch, D - d0);
-            // gather dims [d0, d0 + dch) of every member (zeros past the
-            // members and past D), two members interleaved
+            // gather dims [d0, d0 + dch) of every member, two members
+            // interleaved (zeros past D and for a pair row's missing second
+            // member; a pair row without members is not written, and nothing
+            // reads the sums it enters)
             if (vec) {
-                for (int e = tid; e < G * half * q4; e += kJ2Threads) {
-                    const int pr = e / q4, c4 = e - pr * q4;
-                    const int j = pr / half, s = pr - j * half;
-                    const int m = s < RGN ? 4 * s : 4 * (s - RGN) + 2, M = cnt[j];  // members m, m + 1
-                    float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
-                    if (c4 * 4 < dl) {
-                        if (m < M) u = __ldg(reinterpret_cast<const float4*>(X + (int64_t)mem[j * mcap + m] * D + d0) + c4);
-                        if (m + 1 < M)
-                            v = __ldg(reinterpret_cast<const float4*>(X + (int64_t)mem[j * mcap + m + 1] * D + d0) + c4);
+                int pr = pr0, c4 = c40;
+                while (pr < G * half) {
+                    int2 id[kJ2Ahead];
+                    float4 u[kJ2Ahead], v[kJ2Ahead];
+                    int at[kJ2Ahead], c[kJ2Ahead];
+#pragma unroll
+                    for (int q = 0; q < kJ2Ahead; ++q) {
+                        id[q] = pr < G * half ? *reinterpret_cast<const int2*>(mem + 2 * pr) : make_int2(-1, -1);
+                        at[q] = pr * stride;
+                        c[q] = c4;
+                        const bool in = c4 * 4 < dl;
+                        u[q] = v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (in && id[q].x >= 0) u[q] = __ldg(reinterpret_cast<const float4*>(X + (int64_t)id[q].x * D + d0) + c4);
+                        if (in && id[q].y >= 0) v[q] = __ldg(reinterpret_cast<const float4*>(X + (int64_t)id[q].y * D + d0) + c4);
+                        pr += dpr;
+                        c4 += dc;
+                        if (c4 >= q4) {
+                            c4 -= q4;
+                            ++pr;
+                        }
                     }
-                    store_pairs(rows + (size_t)pr * stride + c4 * 8, u, v, (c4 >> 2) & 1);
+#pragma unroll
+                    for (int q = 0; q < kJ2Ahead; ++q)
+                        if (id[q].x >= 0) store_pairs(rows + at[q] + c[q] * 8, u[q], v[q], (c[q] >> 2) & 1);
                 }
             } else {
                 for (int e = tid; e < G * half * dch; e += kJ2Threads) {
                     const int pr = e / dch, c = e - pr * dch;
-                    const int j = pr / half, s = pr - j * half;
-                    const int m = s < RGN ? 4 * s : 4 * (s - RGN) + 2, M = cnt[j];
+                    const int2 id = *reinterpret_cast<const int2*>(mem + 2 * pr);
                     const bool in = c < dl;
                     *reinterpret_cast<float2*>(rows + (size_t)pr * stride + 2 * c) =
-                        make_float2(in && m < M ? __ldg(X + (int64_t)mem[j * mcap + m] * D + d0 + c) : 0.f,
-                                    in && m + 1 < M ? __ldg(X + (int64_t)mem[j * mcap + m + 1] * D + d0 + c) : 0.f);
+                        make_float2(in && id.x >= 0 ? __ldg(X + (int64_t)id.x * D + d0 + c) : 0.f,
+                                    in && id.y >= 0 ? __ldg(X + (int64_t)id.y * D + d0 + c) : 0.f);
                 }
             }
             __syncthreads();
+            if (d0 == 0) {  // the blocks go densely to the warps, from another one for each CTA of an SM
+                const int it = (tid + 32 * (int)(grp / 152)) & (kJ2Threads - 1);
+                live = it < *nlive;
+                if (live) {
+                    const uint32_t e = items[it];
+                    jn = e & 255, rg = e >> 8 & 255, cg = e >> 16;
+                    Mj = cnt[jn], nnj = cnt[G + jn];
+                }
+            }
             if (live) {
                 const float* rp = rows + (size_t)(jn * half + rg) * stride;
                 const float* cp = rows + (size_t)(jn * half + cg) * stride;
@@ -908,36 +682,43 @@ __global__ void __launch_bounds__(kJ2Threads, 4) k5_join_cta(const float* __rest
             }
             __syncthreads();  // the next chunk overwrites the rows
         }
-        float acc[4][4];
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int w = 0; w < 2; ++w) {
-                acc[2 * h][2 * w] = __uint_as_float((uint32_t)same[h][w]);
-                acc[2 * h + 1][2 * w + 1] = __uint_as_float((uint32_t)(same[h][w] >> 32));
-                acc[2 * h][2 * w + 1] = __uint_as_float((uint32_t)cross[h][w]);
-                acc[2 * h + 1][2 * w] = __uint_as_float((uint32_t)(cross[h][w] >> 32));
-            }
-        // offers: count, reserve (one atomic per warp), write
-        int c = 0;
+        // offers: a bit per direction of the block's 16 pairs (2 (4 a + b): b
+        // offered to a; plus 1: a to b), their distances in shared memory (the
+        // rows are done with), then one slot range per warp
+        uint32_t hits = 0;
+        float* dist = rows + tid * kJ2Dist;
+        const int2* id2 = reinterpret_cast<const int2*>(mem) + jn * half;  // the node's ids by pair row
         if (live) {
+            const int2 u0 = id2[rg], u1 = id2[RGN + rg], v0 = id2[cg], v1 = id2[RGN + cg];
+            const uint32_t u[4] = {(uint32_t)u0.x, (uint32_t)u0.y, (uint32_t)u1.x, (uint32_t)u1.y};
+            const uint32_t v[4] = {(uint32_t)v0.x, (uint32_t)v0.y, (uint32_t)v1.x, (uint32_t)v1.y};
+            uint64_t tv[4];
 #pragma unroll
-            for (int a = 0; a < 4; ++a)
+            for (int b = 0; b < 4; ++b) tv[b] = thr[jn * mcap + b * RGN + cg];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const uint64_t tu = thr[jn * mcap + a * RGN + rg];
+                float d[4];
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
+                    const uint64_t sum = (a ^ b) & 1 ? cross[a >> 1][b >> 1] : same[a >> 1][b >> 1];
+                    d[b] = __uint_as_float((uint32_t)(a & 1 ? sum >> 32 : sum));
                     const int ia = 4 * rg + a, ib = 4 * cg + b;
-                    if (ia < Mj && ib < Mj && (ia < nnj || ib < nnj) && (rg < cg || a < b)) {
-                        const uint32_t u = (uint32_t)mem[jn * mcap + ia], v = (uint32_t)mem[jn * mcap + ib];
-                        if (u != v) {
-                            const int sa = jn * mcap + a * RGN + rg, sb = jn * mcap + b * RGN + cg;
-                            const bool ou = make_key(acc[a][b], v) < thr[sa];
-                            const bool ov = make_key(acc[a][b], u) < thr[sb];
-                            if ((ou || ov) && !(lids && leaf_mates(slid[sa], slid[sb], npass))) c += ou + ov;
-                        }
-                    }
+                    const bool pair = ia < Mj && ib < Mj && (ia < nnj || ib < nnj) && (rg < cg || a < b) && u[a] != v[b];
+                    hits |= (uint32_t)(pair && make_key(d[b], v[b]) < tu) << (2 * (4 * a + b));
+                    hits |= (uint32_t)(pair && make_key(d[b], u[a]) < tv[b]) << (2 * (4 * a + b) + 1);
                 }
+                *reinterpret_cast<float4*>(dist + 4 * a) = make_float4(d[0], d[1], d[2], d[3]);
+            }
         }
-        const int incl = warp_incl_scan(c);
+        if (lids) {
+            for (uint32_t rest = (hits | hits >> 1) & 0x55555555u; rest; rest &= rest - 1) {
+                const int bit = __ffs(rest) - 1, a = bit >> 3, b = bit >> 1 & 3;
+                if (leaf_mates(slid[jn * mcap + a * RGN + rg], slid[jn * mcap + b * RGN + cg], npass))
+                    hits &= ~(3u << bit);
+            }
+        }
+        const int c = __popc(hits), incl = warp_incl_scan(c);
         const int total = __shfl_sync(0xffffffffu, incl, 31);
         if (total > 0) {
             uint32_t at = 0;
@@ -945,36 +726,19 @@ __global__ void __launch_bounds__(kJ2Threads, 4) k5_join_cta(const float* __rest
             at = __shfl_sync(0xffffffffu, at, 31);
             if ((int64_t)at + total > cap) {
                 if (lane == 0) atomicOr(status, kStatusOverflow);
-            } else if (c > 0) {
+            } else {
                 uint32_t w = at + incl - c;
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        const int ia = 4 * rg + a, ib = 4 * cg + b;
-                        if (ia < Mj && ib < Mj && (ia < nnj || ib < nnj) && (rg < cg || a < b)) {
-                            const uint32_t u = (uint32_t)mem[jn * mcap + ia], v = (uint32_t)mem[jn * mcap + ib];
-                            if (u != v) {
-                                const int sa = jn * mcap + a * RGN + rg, sb = jn * mcap + b * RGN + cg;
-                                const uint64_t ku = make_key(acc[a][b], v), kv = make_key(acc[a][b], u);
-                                const bool ou = ku < thr[sa], ov = kv < thr[sb];
-                                if ((ou || ov) && !(lids && leaf_mates(slid[sa], slid[sb], npass))) {
-                                    if (ou) {
-                                        ptgt[w] = u;
-                                        pkey[w] = ku;
-                                        ++w;
-                                        atomicAdd(&pcnt[u], 1);
-                                    }
-                                    if (ov) {
-                                        ptgt[w] = v;
-                                        pkey[w] = kv;
-                                        ++w;
-                                        atomicAdd(&pcnt[v], 1);
-                                    }
-                                }
-                            }
-                        }
-                    }
+                const int* ids = mem + jn * mcap;
+                for (; hits; hits &= hits - 1) {
+                    const int bit = __ffs(hits) - 1, a = bit >> 3, b = bit >> 1 & 3;
+                    const uint32_t u = (uint32_t)ids[2 * ((a >> 1) * RGN + rg) + (a & 1)],
+                                   v = (uint32_t)ids[2 * ((b >> 1) * RGN + cg) + (b & 1)];
+                    const uint32_t to = bit & 1 ? v : u;
+                    ptgt[w] = to;
+                    pkey[w] = make_key(dist[bit >> 1], bit & 1 ? u : v);
+                    ++w;
+                    atomicAdd(&pcnt[to], 1);
+                }
             }
         }
         __syncthreads();  // the next group overwrites members, thresholds and counts
@@ -1217,26 +981,12 @@ void launch_reverse_lists(const uint64_t* G, int64_t n, int k, const JoinBuffers
         k6_select<1><<<grid, 256, 0, s>>>(b.rbuf, b.roff, n, k, b.R);
 }
 
-int join_blocks_per_lane(int mcap) {
-    const int rgn = (mcap + 3) / 4;
-    const int nb = rgn * (rgn + 1) / 2;
-    return (nb + 31) / 32;
-}
-
-// shared memory of one join CTA: per warp the member rows (mcap, a multiple
-// of 4, rows of one dim chunk), their thresholds and their ids
-size_t join_smem_bytes(int D, int mcap) {
-    int dch, stride;
-    join_chunk(D, mcap, &dch, &stride);
-    return (size_t)kJoinWarps * join_warp_bytes(mcap, stride);
-}
-
 namespace {
 
 // One refinement round over the nodes at positions [0, count) of b.list
 // (all nodes when b.list is NULL): reads Gold (and b.R), writes Gnew.
 const char* launch_join_chunk(const float* X, int64_t n, int D, int k, bool rev, const uint64_t* Gold,
-                              const JoinBuffers& b, bool tc, int64_t c0, int64_t c1, int mcap, int bpl, size_t smem,
+                              const JoinBuffers& b, bool tc, int64_t c0, int64_t c1, int mcap,
                               int* status, cudaStream_t s);
 void finish_chunk(int64_t n, int k, uint64_t* Gnew, const JoinBuffers& b, double offers, int* status,
                   cudaStream_t s);
@@ -1268,15 +1018,13 @@ void join_round(const float* X, int64_t n, int D, int k, bool rev, const uint64_
                 cudaStream_t s, const uint64_t* Gbase = nullptr) {
     cudaMemcpyAsync(Gnew, Gbase ? Gbase : Gold, sizeof(uint64_t) * n * k, cudaMemcpyDeviceToDevice, s);
     const int mcap = ((rev ? 2 * k : k) + 3) & ~3;
-    const int bpl = join_blocks_per_lane(mcap);
-    const size_t smem = join_smem_bytes(D, mcap);
     const double m_max = rev ? 2.0 * k : (double)k;
     // the 32-bit offer counter must not wrap, even in the worst case
     const int64_t wrap_nodes = (int64_t)(4294967295.0 / std::max(1.0, m_max * (m_max - 1)));
     if (b.capture) {  // no host reads: worst-case chunks over every position
         for (int64_t c0 = 0; c0 < count; c0 += nodes_per_chunk) {
             const int64_t c1 = std::min(count, c0 + nodes_per_chunk);
-            launch_join_chunk(X, n, D, k, rev, Gold, b, tc, c0, c1, mcap, bpl, smem, status, s);
+            launch_join_chunk(X, n, D, k, rev, Gold, b, tc, c0, c1, mcap, status, s);
             finish_chunk(n, k, Gnew, b, 0.0, status, s);
         }
         return;
@@ -1287,7 +1035,7 @@ void join_round(const float* X, int64_t n, int D, int k, bool rev, const uint64_
         c1 = std::min(count, c0 + want);
         uint32_t offers = 0;
         for (;;) {
-            const char* who = launch_join_chunk(X, n, D, k, rev, Gold, b, tc, c0, c1, mcap, bpl, smem, status, s);
+            const char* who = launch_join_chunk(X, n, D, k, rev, Gold, b, tc, c0, c1, mcap, status, s);
             int st = 0;
             cudaMemcpyAsync(&offers, b.counter, sizeof offers, cudaMemcpyDeviceToHost, s);
             cudaMemcpyAsync(&st, status, sizeof st, cudaMemcpyDeviceToHost, s);
@@ -1311,7 +1059,7 @@ void join_round(const float* X, int64_t n, int D, int k, bool rev, const uint64_
 
 // The join of the chunk [c0, c1); returns the name of the kernel that ran.
 const char* launch_join_chunk(const float* X, int64_t n, int D, int k, bool rev, const uint64_t* Gold,
-                              const JoinBuffers& b, bool tc, int64_t c0, int64_t c1, int mcap, int bpl, size_t smem,
+                              const JoinBuffers& b, bool tc, int64_t c0, int64_t c1, int mcap,
                               int* status, cudaStream_t s) {
     {
         cudaMemsetAsync(b.pcnt, 0, sizeof(int32_t) * (n + 1), s);
@@ -1335,61 +1083,34 @@ const char* launch_join_chunk(const float* X, int64_t n, int D, int k, bool rev,
             const double m = rev ? 2.0 * k : (double)k;
             const bool lids = b.leafid != nullptr && b.npass > 0;
             const J2Layout L2 = j2_layout(D, mcap, lids);
-            // the CTA-wide kernel when it keeps clearly more lanes busy than
-            // one node per warp (whose lanes idle when the block count is not
-            // a multiple of 32)
-            const double warp_eff = (double)L2.NB / (32.0 * ((L2.NB + 31) / 32));
-            const double cta_eff = (double)(L2.G * L2.NB) / kJ2Threads;
-            const bool cta = cta_eff >= warp_eff + 0.1;
             // With reverse lists a mutual neighbour is one member: slots of
             // three quarters of 2k when that packs more nodes into a CTA, the
             // nodes that overflow joined after them with full slots (their
             // count read on the device)
             const int small = (mcap * 3 / 4 + 3) & ~3;
-            const bool packed = cta && rev && k <= 32 && b.ovf_list && b.ovf_count && small >= 4 &&
+            const bool packed = rev && b.ovf_list && b.ovf_count && small >= 4 &&
                                 j2_layout(D, small, lids).G > L2.G;
             LaunchScope ls("k5_join", s, (double)(c1 - c0) * (m * D * 4.0 + 2 * k * 8.0 + m * 8.0),
                            (double)(c1 - c0) * m * (m - 1) / 2 * 3.0 * D, packed ? 2 : 1);
-            if (cta) {
-                auto cta_launch = [&](int mc, const int32_t* lst, const int32_t* cnt_dev, int64_t n0, int64_t n1,
-                                      bool ovf) {
-                    const J2Layout Lc = j2_layout(D, mc, lids);
-                    cudaFuncSetAttribute(k5_join_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lc.total);
-                    int per_sm = 0;
-                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k5_join_cta, kJ2Threads, Lc.total);
-                    if (per_sm < 1) per_sm = 1;
-                    const int64_t groups = (n1 - n0 + Lc.G - 1) / Lc.G;
-                    const int grid2 = (int)std::max<int64_t>(1, std::min<int64_t>(groups, (int64_t)152 * per_sm));
-                    k5_join_cta<<<grid2, kJ2Threads, Lc.total, s>>>(
-                        X, D, k, rev ? 1 : 0, mc, Gold, b.R, lst, b.fnew, b.rnew, n0, n1, b.counter, b.cap, b.ptgt,
-                        b.pkey, b.pcnt, status, tc_dev ? b.notexact : nullptr, cnt_dev, lids ? b.leafid : nullptr,
-                        b.npass, ovf ? b.ovf_list : nullptr, ovf ? b.ovf_count : nullptr);
-                };
-                if (packed) {
-                    cudaMemsetAsync(b.ovf_count, 0, sizeof(int32_t), s);
-                    cta_launch(small, b.list, b.count_dev, c0, c1, true);
-                    cta_launch(mcap, b.ovf_list, b.ovf_count, 0, c1 - c0, false);
-                } else {
-                    cta_launch(mcap, b.list, b.count_dev, c0, c1, false);
-                }
-                return "k5_join";
+            auto cta_launch = [&](int mc, const int32_t* lst, const int32_t* cnt_dev, int64_t n0, int64_t n1,
+                                  bool ovf) {
+                const J2Layout Lc = j2_layout(D, mc, lids);
+                cudaFuncSetAttribute(k5_join_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lc.total);
+                const int per_sm = (int)std::min<size_t>(1024 / kJ2Threads, (227 * 1024) / (Lc.total + 1024));
+                const int64_t groups = (n1 - n0 + Lc.G - 1) / Lc.G;
+                const int grid2 = (int)std::max<int64_t>(1, std::min<int64_t>(groups, (int64_t)152 * per_sm));
+                k5_join_cta<<<grid2, kJ2Threads, Lc.total, s>>>(
+                    X, D, k, rev ? 1 : 0, mc, Gold, b.R, lst, b.fnew, b.rnew, n0, n1, b.counter, b.cap, b.ptgt,
+                    b.pkey, b.pcnt, status, tc_dev ? b.notexact : nullptr, cnt_dev, lids ? b.leafid : nullptr,
+                    b.npass, ovf ? b.ovf_list : nullptr, ovf ? b.ovf_count : nullptr);
+            };
+            if (packed) {
+                cudaMemsetAsync(b.ovf_count, 0, sizeof(int32_t), s);
+                cta_launch(small, b.list, b.count_dev, c0, c1, true);
+                cta_launch(mcap, b.ovf_list, b.ovf_count, 0, c1 - c0, false);
+            } else {
+                cta_launch(mcap, b.list, b.count_dev, c0, c1, false);
             }
-            const int grid = (int)std::min<int64_t>((c1 - c0 + kJoinWarps - 1) / kJoinWarps, 152 * 32);
-#define KNNG_JOIN(BPL)                                                                                     \
-    do {                                                                                                   \
-        cudaFuncSetAttribute(k5_join<BPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);        \
-        k5_join<BPL><<<grid, 32 * kJoinWarps, smem, s>>>(X, D, k, rev ? 1 : 0, mcap, Gold, b.R, b.list,     \
-                                                         b.fnew, b.rnew, c0, c1, b.counter, b.cap, b.ptgt,  \
-                                                         b.pkey, b.pcnt, status,                            \
-                                                         tc_dev ? b.notexact : nullptr,                     \
-                                                         b.count_dev);                                      \
-    } while (0)
-            if (bpl <= 1) KNNG_JOIN(1);
-            else if (bpl <= 2) KNNG_JOIN(2);
-            else if (bpl <= 3) KNNG_JOIN(3);
-            else if (bpl <= 4) KNNG_JOIN(4);
-            else KNNG_JOIN(5);
-#undef KNNG_JOIN
         }
     }
     return "k5_join";

@@ -232,6 +232,11 @@ __device__ __forceinline__ bool leaf_mates(const int4& a, const int4& b, int npa
     return (npass > 0 && a.x == b.x) || (npass > 1 && a.y == b.y) || (npass > 2 && a.z == b.z) ||
            (npass > 3 && a.w == b.w);
 }
+// The first slot in which they share a leaf; npass when there is none.
+__device__ __forceinline__ int leaf_shared(const int4& a, const int4& b, int npass) {
+    const int q = a.x == b.x ? 0 : a.y == b.y ? 1 : a.z == b.z ? 2 : a.w == b.w ? 3 : 4;
+    return q < npass ? q : npass;
+}
 
 // lid[perm[p] * kMaxLeafPasses + slot] = the leaf of position p (leaf_off:
 // nleaf + 1 offsets).
