@@ -787,80 +787,110 @@ __device__ __forceinline__ bool offer_useful(uint64_t key, const uint64_t* row, 
     return row[lo] != key;
 }
 
-// Inserts id into a warp's open-addressing set of kSeenSlots ids (linear
-// probing); true when it was not there.  The callers insert fewer ids than
-// there are slots, so a probe always ends.
-constexpr int kSeenSlots = 256;
-constexpr int kSeenOffers = 160;  // offers per node taken through the set (with at most 32 list ids)
-__device__ __forceinline__ bool seen_insert(uint32_t* tab, uint32_t id) {
-    for (uint32_t h = (id * 2654435761u) >> 24, t = 0; t < kSeenSlots; ++t, h = (h + 1) & (kSeenSlots - 1)) {
-        const uint32_t old = atomicCAS(&tab[h], 0xFFFFFFFFu, id);
-        if (old == 0xFFFFFFFFu) return true;
-        if (old == id) return false;
+// Merges up to kFewOffers offers into a list of k <= 32 distinct keys held one
+// per lane (`run`, ascending; lanes past k hold empty keys), 32 at a time.  An
+// offer enters when it is below the k-th key and its id is neither in the list
+// nor in a lower lane (a pair always has the same canonical distance, and a
+// repeat of an offer that did not make the list cannot make it later: the k-th
+// key only falls).  Every list entry and every offer that enters then counts
+// what lies below it: that is its place.  `key`: the lane's first offer.
+// Returns whether the list changed.
+constexpr int kFewOffers = 160;
+__device__ __forceinline__ bool merge_few_offers(const uint64_t* __restrict__ grouped, int beg, int end, int k,
+                                                 uint64_t key, uint64_t& run, uint64_t* scratch) {
+    const int lane = threadIdx.x & 31;
+    bool changed = false;
+    for (int c = beg; c < end; c += 32) {
+        if (c > beg) key = c + lane < end ? grouped[c + lane] : kEmptyKey;
+        bool in = key < shfl64(run, k - 1);
+        if (!__any_sync(0xffffffffu, in)) continue;
+        // lanes without an offer match themselves only: ids are below 2^31
+        const uint32_t id = in ? key_id(key) : 0x80000000u | (uint32_t)lane;
+        const unsigned same = __match_any_sync(0xffffffffu, id);
+        in &= (same & ((1u << lane) - 1u)) == 0;
+        const uint32_t have = run == kEmptyKey ? 0xFFFFFFFFu : key_id(run);
+        for (int e = 0; e < k; ++e) {
+            const uint32_t other = __shfl_sync(0xffffffffu, have, e);
+            in &= other != id;
+        }
+        const unsigned ins = __ballot_sync(0xffffffffu, in);
+        if (!ins) continue;
+        int at = 0, to = lane;  // places of the lane's offer and of its list entry
+        for (unsigned m = ins; m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            const uint64_t o = shfl64(key, src);
+            const int below = __popc(__ballot_sync(0xffffffffu, run < o));
+            at += lane == src ? below : (o < key ? 1 : 0);
+            to += o < run ? 1 : 0;
+        }
+        if (to < k) scratch[to] = run;
+        __syncwarp();
+        if (in && at < k) scratch[at] = key;
+        __syncwarp();
+        run = lane < k ? scratch[lane] : kEmptyKey;
+        __syncwarp();
+        changed = true;
     }
-    return false;
+    return changed;
 }
 
-// Merges one node's offers into its list: the list sits in shared memory;
-// every lane drops the offers that cannot change it, and only the rest go
-// through the warp selection.  For k <= 32 and at most kSeenOffers offers the
-// drop is by id in the warp's set `seen` (a pair always has the same canonical
-// distance): the list's ids first, then each offer below the k-th key enters
-// once, so the survivors are distinct and new and usually one bitonic merge
-// takes them; a repeat of an offer that did not make the list cannot make it
-// later either (the k-th key only falls).
+// A node's list and its first 32 offers, one per lane, as loaded.
+template <int NO>
+struct MergeLoad {
+    int64_t u;
+    int beg, end;
+    uint64_t run[NO], key;
+    __device__ __forceinline__ void load(const uint64_t* Gnew, const uint64_t* __restrict__ grouped, int64_t u_,
+                                         int beg_, int end_, int k) {
+        const int lane = threadIdx.x & 31;
+        u = u_;
+        beg = beg_;
+        end = end_;
+#pragma unroll
+        for (int o = 0; o < NO; ++o) run[o] = lane + 32 * o < k ? Gnew[u * k + lane + 32 * o] : kEmptyKey;
+        key = beg + lane < end ? grouped[beg + lane] : kEmptyKey;
+    }
+};
+
+// Merges one node's offers into its list.  Usually by merge_few_offers; else
+// (k > 32, more offers, or a given list that holds a key twice) the list sits
+// in shared memory, every lane drops the offers that cannot change it, and
+// the rest go through the warp selection.  Bound by instructions and the latency
+// of its loads: four rounds on 10M x 96, k = 16 took 48.7 ms when the ids went
+// through a hash set in shared memory and the survivors through a bitonic sort
+// and merge, 35.1 by counting places and with the next node's loads in flight;
+// 1M x 128, k = 20 1.55 -> 1.23.
 template <int NO>
 __device__ __forceinline__ void merge_node(uint64_t* __restrict__ Gnew, const uint64_t* __restrict__ grouped,
-                                           int64_t u, int beg, int end, int k, uint64_t* srow, uint64_t* scratch,
-                                           uint32_t* seen) {
-    const int lane = threadIdx.x & 31;
-    uint64_t* row = Gnew + u * k;
+                                           const MergeLoad<NO>& in, int k, uint64_t* srow, uint64_t* scratch) {
+    const int lane = threadIdx.x & 31, beg = in.beg, end = in.end;
+    uint64_t* row = Gnew + in.u * k;
     uint64_t run[NO];
 #pragma unroll
-    for (int o = 0; o < NO; ++o) {
-        run[o] = lane + 32 * o < k ? row[lane + 32 * o] : kEmptyKey;
-        srow[lane + 32 * o] = run[o];
+    for (int o = 0; o < NO; ++o) run[o] = in.run[o];
+    if (NO == 1 && end - beg <= kFewOffers) {
+        const uint64_t next = shfl64(run[0], (lane + 1) & 31);
+        if (!__any_sync(0xffffffffu, lane < 31 && run[0] != kEmptyKey && run[0] == next)) {
+            if (merge_few_offers(grouped, beg, end, k, in.key, run[0], scratch) && lane < k) row[lane] = run[0];
+            return;
+        }
     }
+#pragma unroll
+    for (int o = 0; o < NO; ++o) srow[lane + 32 * o] = run[o];
     __syncwarp();
     constexpr int NC = 4;
     bool changed = false;
-    const bool hashed = NO == 1 && end - beg <= kSeenOffers;
-    if (hashed) {
-        for (int t = lane; t < kSeenSlots; t += 32) seen[t] = 0xFFFFFFFFu;
-        __syncwarp();
-        if (run[0] != kEmptyKey) seen_insert(seen, key_id(run[0]));
-        __syncwarp();
-    }
     for (int c = beg; c < end; c += 32 * NC) {
         uint64_t a[NC + NO];
         bool any = false;
-        const uint64_t kth = hashed ? shfl64(run[0], k - 1) : kEmptyKey;
 #pragma unroll
         for (int s = 0; s < NC; ++s) {
             const int e = c + lane + 32 * s;
             a[s] = (e < end) ? grouped[e] : kEmptyKey;
-            if (a[s] != kEmptyKey &&
-                !(hashed ? (a[s] < kth && seen_insert(seen, key_id(a[s]))) : offer_useful(a[s], srow, k)))
-                a[s] = kEmptyKey;
+            if (a[s] != kEmptyKey && !offer_useful(a[s], srow, k)) a[s] = kEmptyKey;
             any |= a[s] != kEmptyKey;
         }
         if (!__any_sync(0xffffffffu, any)) continue;
-        if (NO == 1) {  // usually few offers survive: one bitonic merge
-            uint64_t few[NC], out;
-            bool ch;
-#pragma unroll
-            for (int s = 0; s < NC; ++s) few[s] = a[s];
-            if (warp_merge_few<NC>(few, run[0], k, scratch, out, ch)) {
-                if (ch) {
-                    run[0] = lane < k ? out : kEmptyKey;
-                    __syncwarp();
-                    srow[lane] = run[0];
-                    __syncwarp();
-                    changed = true;
-                }
-                continue;
-            }
-        }
 #pragma unroll
         for (int o = 0; o < NO; ++o) a[NC + o] = run[o];
         sort_regs<NC + NO>(a);
@@ -887,7 +917,6 @@ __global__ void __launch_bounds__(256) k4_merge(uint64_t* __restrict__ Gnew, con
                                                 const int* __restrict__ status) {
     __shared__ uint64_t rows[8][32 * NO];
     __shared__ uint64_t scratch[8][32];
-    __shared__ uint32_t seen[8][NO == 1 ? kSeenSlots : 1];
     if (*status & kStatusStop) return;
     const int lane = threadIdx.x & 31;
     uint64_t* srow = rows[threadIdx.x >> 5];
@@ -896,12 +925,20 @@ __global__ void __launch_bounds__(256) k4_merge(uint64_t* __restrict__ Gnew, con
         const int64_t u = g0 + lane;
         const int beg = u < n ? poff[u] : 0, end = u < n ? poff[u + 1] : 0;
         unsigned todo = __ballot_sync(0xffffffffu, end > beg);
-        while (todo) {
+        // the next node's loads are in flight while one is merged
+        MergeLoad<NO> now, next;
+        auto load = [&](MergeLoad<NO>& to) {
             const int src = __ffs(todo) - 1;
             todo &= todo - 1;
-            merge_node<NO>(Gnew, grouped, g0 + src, __shfl_sync(0xffffffffu, beg, src),
-                           __shfl_sync(0xffffffffu, end, src), k, srow, scratch[threadIdx.x >> 5],
-                           seen[threadIdx.x >> 5]);
+            to.load(Gnew, grouped, g0 + src, __shfl_sync(0xffffffffu, beg, src), __shfl_sync(0xffffffffu, end, src), k);
+        };
+        if (todo) load(next);
+        else continue;
+        for (bool more = true; more;) {
+            now = next;
+            more = todo != 0;
+            if (more) load(next);
+            merge_node<NO>(Gnew, grouped, now, k, srow, scratch[threadIdx.x >> 5]);
         }
     }
 }

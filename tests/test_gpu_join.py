@@ -41,3 +41,27 @@ def test_build_equals_oracle(knng, k, mode, D, leaf, passes, shift):
     o_ids, o_d = oracle.build_graph(X, k, leaf, passes=passes, rounds=3, seed=11, mode=mode)
     np.testing.assert_array_equal(ids.cpu().numpy(), o_ids)
     np.testing.assert_array_equal(d.cpu().numpy(), o_d)
+
+
+@pytest.mark.parametrize("k", [3, 8, 32, 40])
+@pytest.mark.parametrize("hubs", [1, 12])
+def test_offers_to_a_few_nodes_match_oracle(knng, k, hubs):
+    # every list holds the hubs, so these get from a few to hundreds of offers,
+    # most of them repeats, and the others a handful
+    n, D = 400, 9
+    rng = np.random.default_rng(k + hubs)
+    X = rng.integers(-50, 51, size=(n, D)).astype(np.float32)
+    ids, d = oracle.new_graph(n, k)
+    for i in range(n):
+        first = [j for j in range(hubs) if j != i][:k]
+        rest = rng.permutation(np.setdiff1d(np.arange(n), first + [i]))[:k - len(first)]
+        for j in first + rest.tolist():
+            oracle.list_insert(ids[i], d[i], oracle.dist_f32(X[i], X[j]), j)
+    mode = oracle.FWD_REV if k <= 32 else oracle.FWD
+    o = (ids.copy(), d.copy())
+    for _ in range(2):
+        o = oracle.refine_round(X, *o, mode=mode)
+    p = knng.default_params(k=k, refine_rounds=2, join_mode=mode)
+    g_ids, g_d = knng.knng_refine(*[torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (X, ids, d)], p)
+    np.testing.assert_array_equal(g_ids.cpu().numpy(), o[0])
+    np.testing.assert_array_equal(g_d.cpu().numpy(), o[1])
