@@ -126,9 +126,10 @@ def measured_peaks():
 # the sources whose change makes a kernel's committed counters stale: its own
 # file, and for the tensor-core join also join.cu, which sets the order in
 # which it takes the nodes (and so its DRAM traffic)
-KERNEL_SOURCES = {"k1_": ("split.cu",), "k2_leaf_fp32": ("leaf.cu",), "k2_": ("leaf_tc.cu",), "k4_": ("join.cu",),
+KERNEL_SOURCES = {"k1_level": ("level.cu",), "k1_select": ("split.cu", "select.cu"), "k1_": ("split.cu",),
+                  "k2_leaf_fp32": ("leaf.cu",), "k2_": ("leaf_tc.cu",), "k4_": ("join.cu",),
                   "k5_join_tc": ("join_tc.cu", "join.cu"), "k5_": ("join.cu",), "k6_": ("join.cu",),
-                  "k7_": ("exact.cu",), "k0_": ("leaf_tc.cu",)}
+                  "ks_": ("screen.cu",), "k7_rank": ("screen.cu",), "k7_": ("exact.cu",), "k0_": ("leaf_tc.cu",)}
 ALU_KERNELS = ("k5_join", "k2_leaf_fp32", "k7_exact")
 TENSOR_KERNELS = ("k2_leaf_bf16", "k2_leaf_fp16", "k2_leaf_fp8")
 

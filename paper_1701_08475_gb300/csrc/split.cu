@@ -516,7 +516,7 @@ int sm_count() {
 // segments per CTA, one per warp; NW > 1: one segment per CTA.  On the final
 // cut each thread takes R consecutive positions, and an exclusive scan of
 // the left counts gives every position its place in perm_out (left positions
-// first, each side in position order), as k1_select_small does.
+// first, each side in position order), as k1_select_cluster does.
 template <int R, int NW>
 __global__ void __launch_bounds__(NW > 1 ? 32 * NW : 128) k1_select_sort(const float* __restrict__ S,
                                                                         const int32_t* __restrict__ seg_off,
