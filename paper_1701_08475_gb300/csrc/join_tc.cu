@@ -154,7 +154,8 @@ __global__ void __launch_bounds__(kThreads, 4) k5_join_tc(const uint16_t* __rest
     extern __shared__ uint8_t smem_raw[];
     // the exact form runs when the 16-bit copy is exact, the screening form
     // (CERT) when it is not; each returns at once otherwise
-    if ((*status & kStatusStop) || (CERT == lp_exact_flag(*notexact))) return;
+    if (CERT == lp_exact_flag(*notexact)) return;
+    if (tc::stopped(status)) return;  // whole CTA, before any other barrier or tensor memory
     if (count_dev && (int64_t)*count_dev < node1) node1 = *count_dev;
     const JtSmem L = jt_smem(Dp, mcap, CERT);
     uint8_t* base = smem_raw + ((1024 - (tc::smem_addr(smem_raw) & 1023)) & 1023);

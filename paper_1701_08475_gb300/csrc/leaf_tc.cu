@@ -229,9 +229,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k2_leaf_tc(const __grid_constan
     constexpr int DTS = RW + 1;           // d^ row stride
     constexpr int SB = kStageBytes * MT;  // one K chunk of all rows
     extern __shared__ uint8_t smem_raw[];
-    // whole CTA, before any barrier or tensor memory
-    if (*status & kStatusStop) return;
+    // whole CTA, before any other barrier or tensor memory
     if (!dump && !lp_exact(*notexact)) return;
+    if (tc::stopped(status)) return;
     const TcSmem L = tc_smem(Dpb, MT);
     uint8_t* base = smem_raw + ((1024 - (tc::smem_addr(smem_raw) & 1023)) & 1023);
     float* dt = reinterpret_cast<float*>(base + L.dt_off);

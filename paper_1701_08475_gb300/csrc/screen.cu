@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant
                                                           const __grid_constant__ CUtensorMap tmb,
                                                           const ScreenArgs P) {
     extern __shared__ uint8_t smem_raw[];
-    if (*P.status & kStatusStop) return;  // whole CTA, before any barrier or tensor memory
+    if (tc::stopped(P.status)) return;  // whole CTA, before any other barrier or tensor memory
     const ScreenSmem L = screen_smem(P.nk, MODE);
     uint8_t* base = smem_raw + ((1024 - (tc::smem_addr(smem_raw) & 1023)) & 1023);
     const bool res = P.nk <= kScResident;
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant
                     if (nct >= P.nct) nct = u + gridDim.x < units ? (int)(u + gridDim.x) / P.nrt : -1;
                     if (nct >= 0) load_cols(nct);
                 }
-                ok = tc::mbar_wait(tfull0 + 8 * buf, (uint32_t)((t >> 1) & 1), P.status);
+                ok = tc::mbar_wait_warp(tfull0 + 8 * buf, (uint32_t)((t >> 1) & 1), P.status);
                 if (MODE == kScArgmin) ok = epi_all(ok);  // the waits end for all warps or for none
                 if (!ok) break;
                 tc::fence_after_sync();

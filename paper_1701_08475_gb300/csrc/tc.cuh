@@ -63,6 +63,20 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* st
     }
     return true;
 }
+// The same wait by all 32 lanes, with one answer for the warp: a lane's own
+// clock may run out while another lane still sees the phase complete, and
+// lanes that part before a warp-collective instruction (tcgen05.ld, __syncwarp,
+// a counted barrier) never meet again.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, int* status) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, status));
+}
+
+// Whether an earlier stage (or another CTA of this launch, whose wait ran out)
+// has stopped the work: read once and shared, so that all threads of the CTA
+// return or none.  Called by every thread.
+__device__ __forceinline__ bool stopped(const int* status) {
+    return __syncthreads_or(threadIdx.x == 0 && (*(const volatile int*)status & kStatusStop)) != 0;
+}
 
 // ---------------------------------------------------------------- TMA
 // 2-D tile load of the tensor map's box at element coordinates (x, y) into
