@@ -35,12 +35,24 @@ namespace {
 
 constexpr int kLvDims = 128;  // dims of one sums chunk: 4 per lane
 constexpr int kLvSms = 152;
+// Dynamic shared memory of a CTA: the block limit (227 KB), and what two CTAs
+// may take of an SM's 228 KB, of which each CTA also costs 1 KB.  The kernel
+// declares no static shared memory, so these are all of it.
+constexpr size_t kLvOne = 227 * 1024, kLvTwo = 113 * 1024;
 
 struct LvLayout {
     int C, q, nt;      // CTAs, rows per CTA, threads
     int stride;        // bytes per staged row
     int dcap;          // dims owned per CTA
-    size_t S, ids, side, W, red, part, tot, total;
+    size_t S, ids, side, W, red, part, tot, misc, total;
+};
+
+// What a segment's cut needs besides: keys to rank by counting, the means'
+// reciprocals, warps' scan totals, and values one thread gives to all.
+struct LvMisc {
+    uint64_t few[32];
+    double inv[2];
+    int warp_tot[16], sh[4];
 };
 
 // Bytes of a staged row: whole 16-byte pieces, an odd number of them (the
@@ -66,7 +78,8 @@ __host__ __device__ inline LvLayout lv_layout(int D, int m, int row_bytes, int C
     L.red = L.W + up((size_t)((D + 15) & ~15) * 4);
     L.part = L.red + (size_t)(L.nt / 32) * 2 * kLvDims * 8;  // also the selection's histogram
     L.tot = L.part + (size_t)C * 2 * L.dcap * 8;
-    L.total = L.tot + (size_t)2 * L.dcap * 8;
+    L.misc = L.tot + (size_t)2 * L.dcap * 8;
+    L.total = L.misc + sizeof(LvMisc);
     return L;
 }
 
@@ -151,9 +164,10 @@ __device__ __forceinline__ int lv_excl_scan(int v, int* warp_tot, int* total) {
 
 template <int Q, int C>
 __device__ __forceinline__ void level_segment(const LvArgs& P, const LvLayout& L, uint8_t* smem, int seg, int rank) {
-    __shared__ int warp_tot[16], sh[4];
-    __shared__ double inv[2];
-    __shared__ uint64_t few[32];
+    LvMisc& misc = *reinterpret_cast<LvMisc*>(smem + L.misc);
+    uint64_t* few = misc.few;
+    double* inv = misc.inv;
+    int *warp_tot = misc.warp_tot, *sh = misc.sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = (int)blockDim.x >> 5;
     const int a = P.seg_off[seg], m = P.seg_off[seg + 1] - a, K = m / 2, D = P.D;
     const int p0 = min(m, rank * L.q), ql = min(m, p0 + L.q) - p0;  // this CTA's positions p0 .. p0 + ql - 1
@@ -503,7 +517,7 @@ __global__ void __launch_bounds__(512, 2) k1_level(const LvArgs P) {
 }
 
 template <int C>
-cudaError_t launch_level_c(const LvArgs& P, int nseg, int nt, size_t smem, cudaStream_t s) {
+void launch_level_c(const LvArgs& P, int nseg, int nt, size_t smem, cudaStream_t s) {
     cudaFuncSetAttribute(k1_level<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)nseg * C);
@@ -517,7 +531,7 @@ cudaError_t launch_level_c(const LvArgs& P, int nseg, int nt, size_t smem, cudaS
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = C > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k1_level<C>, P);
+    cudaLaunchKernelEx(&cfg, k1_level<C>, P);  // an error is the call's (LaunchScope)
 }
 
 }  // namespace
@@ -529,12 +543,11 @@ bool launch_level(const float* X, int64_t n, int D, const LevelPlan& lp, int ite
     const int row_bytes = b.u8_host ? (D + 15) / 16 * 16 : b.q16_host ? (D + 7) / 8 * 16 : (D + 3) / 4 * 16;
     // the fewest CTAs whose segments leave room for two per SM, else eight
     // with one per SM; more of them while that still fills no more than the chip
-    constexpr size_t kTwo = 113 * 1024, kOne = 226 * 1024;
     int C = 1;
-    while (C < 8 && lv_layout(D, lp.max_m, row_bytes, C).total > kTwo) C *= 2;
+    while (C < 8 && lv_layout(D, lp.max_m, row_bytes, C).total > kLvTwo) C *= 2;
     while (C < 8 && lp.max_m / C >= 512 && (int64_t)lp.nseg * 2 * C <= kLvSms) C *= 2;
     const LvLayout L = lv_layout(D, lp.max_m, row_bytes, C);
-    if (L.total > kOne) return false;
+    if (L.total > kLvOne) return false;
     // A level in one launch costs 40-70 us per wave of CTAs, where the sweeps
     // cost about 20 launches of at least 5 us and then the rows' passes over
     // memory; and other partitions want the chip as well.  Three passes,
@@ -569,12 +582,11 @@ bool launch_level(const float* X, int64_t n, int D, const LevelPlan& lp, int ite
     P.row_bytes = row_bytes;
     // every row read once, with its id; the ids written
     LaunchScope ls("k1_level", s, (double)lp.n * (row_bytes + 8.0), (double)lp.n * D * (2.0 * (iters + 1) + 1.0));
-    cudaError_t e;
-    if (C == 1) e = launch_level_c<1>(P, lp.nseg, L.nt, L.total, s);
-    else if (C == 2) e = launch_level_c<2>(P, lp.nseg, L.nt, L.total, s);
-    else if (C == 4) e = launch_level_c<4>(P, lp.nseg, L.nt, L.total, s);
-    else e = launch_level_c<8>(P, lp.nseg, L.nt, L.total, s);
-    return e == cudaSuccess;
+    if (C == 1) launch_level_c<1>(P, lp.nseg, L.nt, L.total, s);
+    else if (C == 2) launch_level_c<2>(P, lp.nseg, L.nt, L.total, s);
+    else if (C == 4) launch_level_c<4>(P, lp.nseg, L.nt, L.total, s);
+    else launch_level_c<8>(P, lp.nseg, L.nt, L.total, s);
+    return true;
 }
 
 }  // namespace knng
