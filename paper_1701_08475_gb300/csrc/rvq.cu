@@ -845,8 +845,11 @@ __global__ void __launch_bounds__(kFewT) k9_few_seeds(const float* __restrict__ 
                 run += c[j];
                 ++step;
             }
-            if (got && lane == __ffs(got) - 1)  // else fewer than s keys
-                *slim = min(lim, mn + (uint32_t)((((uint64_t)step + 1) << sft) - 1));
+            if (got && lane == __ffs(got) - 1) {  // else fewer than s keys
+                // the step's end may lie past the last 32-bit key
+                const uint64_t end = mn + (((uint64_t)step + 1) << sft) - 1;
+                *slim = end < lim ? (uint32_t)end : lim;
+            }
         }
         __syncthreads();
         lim = *slim;
