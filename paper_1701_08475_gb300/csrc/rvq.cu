@@ -391,8 +391,9 @@ __global__ void __launch_bounds__(128 * kCbGroups) k9_combine(const float* __res
         A = __fadd_ru(A, gabs[q][dd]);
         lo = min(lo, glo[q][dd]);
     }
-    // every value is a multiple of 2^(lo - 150) and no partial sum is above A
-    if (up_exp(A) > 53 + lo - 150) {
+    // every value is a multiple of 2^(lo - 150) and no partial sum is above A,
+    // which past FP32's range is no bound at all (then x and y below differ)
+    if (up_exp(A) > 53 + lo - 150 || isinf(A)) {
         // either order is within (m - 1) 2^-53 A, and a little, of the true sum
         const double e = ldexp((double)m * (double)A, -51);
         const float x = __double2float_rn(__ddiv_rn(sum - e, (double)m));
