@@ -218,6 +218,34 @@ LaunchScope::~LaunchScope() {
     if (slot_ >= 0 && slot_ < (int)r.pending.size()) cudaEventRecord(r.pending[slot_].b, s_);
 }
 
+// ---------------------------------------------------------------- shared memory
+void allow_smem_of(const void* kernel) {
+    // what a kernel's own static shared memory leaves of the block's 227 KB;
+    // a property of the code, so it is asked for once (no heap: knng_exact_noalloc)
+    constexpr int kBlock = 227 * 1024;
+    struct Entry {
+        const void* kernel;
+        int bytes;
+    };
+    static std::mutex mu;
+    static Entry known[64];
+    static int count = 0;
+    int bytes = -1;
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        for (int i = 0; i < count && bytes < 0; ++i)
+            if (known[i].kernel == kernel) bytes = known[i].bytes;
+    }
+    if (bytes < 0) {
+        cudaFuncAttributes at;
+        if (cudaFuncGetAttributes(&at, kernel) != cudaSuccess) return;  // the launch reports it
+        bytes = kBlock - (int)at.sharedSizeBytes;
+        std::lock_guard<std::mutex> lk(mu);
+        if (count < 64) known[count++] = {kernel, bytes};
+    }
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
 // ---------------------------------------------------------------- memory
 namespace {
 std::mutex g_pool_mu;

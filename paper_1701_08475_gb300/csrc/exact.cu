@@ -278,12 +278,12 @@ void launch_exact(const float* X, int64_t n, int D, int k, const int32_t* sample
                    nsplit > 1 ? 2 : 1);
     const int mgrid = (int)((s_rows * 32 + 255) / 256);
     if (k > 32) {
-        cudaFuncSetAttribute(k7_exact<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k7_exact<2>);
         k7_exact<2><<<grid, kNT, smem, s>>>(X, n, D, k, sample, row0, s_rows, list, list_count, part, out, status);
         if (nsplit > 1)
             k7_merge<2><<<mgrid, 256, 0, s>>>(part, nsplit, k, s_rows, list, list_count, out, status);
     } else {
-        cudaFuncSetAttribute(k7_exact<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k7_exact<1>);
         k7_exact<1><<<grid, kNT, smem, s>>>(X, n, D, k, sample, row0, s_rows, list, list_count, part, out, status);
         if (nsplit > 1)
             k7_merge<1><<<mgrid, 256, 0, s>>>(part, nsplit, k, s_rows, list, list_count, out, status);

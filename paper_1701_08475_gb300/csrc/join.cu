@@ -1141,7 +1141,7 @@ const char* launch_join_chunk(const float* X, int64_t n, int D, int k, bool rev,
             auto cta_launch = [&](int mc, const int32_t* lst, const int32_t* cnt_dev, int64_t n0, int64_t n1,
                                   bool ovf) {
                 const J2Layout Lc = j2_layout(D, mc, lids);
-                cudaFuncSetAttribute(k5_join_cta, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Lc.total);
+                allow_smem(k5_join_cta);
                 const int per_sm = (int)std::min<size_t>(1024 / kJ2Threads, (227 * 1024) / (Lc.total + 1024));
                 const int64_t groups = (n1 - n0 + Lc.G - 1) / Lc.G;
                 const int grid2 = (int)std::max<int64_t>(1, std::min<int64_t>(groups, (int64_t)152 * per_sm));

@@ -599,13 +599,13 @@ void join_tc_once(const uint16_t* Xq, int Dp, const float* nrm, int k, bool rev,
     int32_t* ol = ovf ? b.ovf_list : nullptr;
     int32_t* oc = ovf ? b.ovf_count : nullptr;
     if (cert) {
-        cudaFuncSetAttribute(k5_join_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k5_join_tc<true>);
         k5_join_tc<true><<<grid, kThreads, smem, s>>>(Xq, Dp, nrm, k, rev ? 1 : 0, mcap, npc, Gold, R, b.list, b.fnew,
                                                       b.rnew, node0, node1, b.counter, b.cap, b.ptgt, b.pkey, b.pcnt,
                                                       status, notexact, bf16, X, D, b.qerr, b.count_dev, b.leafid,
                                                       b.npass, ol, oc);
     } else {
-        cudaFuncSetAttribute(k5_join_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k5_join_tc<false>);
         k5_join_tc<false><<<grid, kThreads, smem, s>>>(Xq, Dp, nrm, k, rev ? 1 : 0, mcap, npc, Gold, R, b.list,
                                                        b.fnew, b.rnew, node0, node1, b.counter, b.cap, b.ptgt, b.pkey,
                                                        b.pcnt, status, notexact, bf16, nullptr, 0, nullptr,

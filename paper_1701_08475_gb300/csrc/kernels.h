@@ -33,6 +33,17 @@ void fault_launch_point(cudaStream_t s);
 // after each launch), else the runtime's last error; both are cleared.
 cudaError_t launch_error();
 
+// Lets a kernel take as much dynamic shared memory as a block may have: the
+// same value before every launch, because the attribute is the process's (a
+// launch's own size would be lowered by another thread's smaller one before the
+// launch: six threads building trees of two sizes had 15 % of their builds
+// refused).  How much a launch asks for does not depend on it.
+void allow_smem_of(const void* kernel);
+template <class... Args>
+void allow_smem(void (*kernel)(Args...)) {
+    allow_smem_of(reinterpret_cast<const void*>(kernel));
+}
+
 // ---------------------------------------------------------------- prepare (K0)
 // Sets *status |= kStatusNonFinite if any of X's count values (or Y's, Z's) is
 // not finite.

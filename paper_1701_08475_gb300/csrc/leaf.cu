@@ -288,7 +288,7 @@ void launch_leaf_t(const float* X, int D, const int32_t* perm, const int32_t* le
     leaf_chunk(D, MC, &dch, &nch, &stride);
     const size_t smem = (size_t)(nch > 1 ? 2 * MC : MC / 2) * stride * 4 + (size_t)C::RB * (MC + 1) * 4 + MC * 4 + (C::NT / 32) * 32 * 8;
     auto kernel = nch == 1 ? k2_leaf_fp32<MC, NSG, NB, true> : k2_leaf_fp32<MC, NSG, NB, false>;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(kernel);
     kernel<<<nleaf, C::NT, smem, s>>>(X, D, perm, leaf_off, k, G, status, skip);
 }
 

@@ -556,7 +556,7 @@ bool launch_leaf_tc(const void* Xl, int64_t n, int D, const int32_t* perm, const
     LaunchScope ls(names[qt], s, (double)nleaf * mm * (Dpb + 2 * 8.0 * k), (double)nleaf * rw * rw * 2.0 * elems);
 #define KNNG_LEAF_TC(Q, NS, T)                                                                                  \
     do {                                                                                                        \
-        cudaFuncSetAttribute(k2_leaf_tc<Q, NS, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);     \
+        allow_smem(k2_leaf_tc<Q, NS, T>);                                                                       \
         k2_leaf_tc<Q, NS, T><<<nleaf * T, kTcThreads, smem, s>>>(tmap, Dpb, perm, leaf_off, nrm, scale, k, G,  \
                                                              status, notexact, dump);                           \
     } while (0)

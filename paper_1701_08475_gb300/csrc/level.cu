@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(512, 2) k1_level(const LvArgs P) {
 
 template <int C>
 void launch_level_c(const LvArgs& P, int nseg, int nt, size_t smem, cudaStream_t s) {
-    cudaFuncSetAttribute(k1_level<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k1_level<C>);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)nseg * C);
     cfg.blockDim = dim3((unsigned)nt);

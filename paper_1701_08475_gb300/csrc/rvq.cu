@@ -951,10 +951,10 @@ void launch_rvq_assign(const float* X, int64_t N, int D, const float* W1, const 
     LaunchScope ls(res ? "k9_assign_res" : "k9_assign", s, (double)N * D * (res ? 8.0 : 4.0) + N * 4.0,
                    (double)N * W * D * 3.0);
     if (res) {
-        cudaFuncSetAttribute(k9_assign<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k9_assign<true>);
         k9_assign<true><<<(unsigned)grid, kAT, smem, s>>>(X, N, D, W1, c1, c1_stride, words, W, out, out_stride);
     } else {
-        cudaFuncSetAttribute(k9_assign<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k9_assign<false>);
         k9_assign<false><<<(unsigned)grid, kAT, smem, s>>>(X, N, D, nullptr, nullptr, 0, words, W, out, out_stride);
     }
 }
@@ -1029,10 +1029,10 @@ void launch_dots(const float* A, int64_t M, const float* B, int W, int D, float*
     const dim3 grid((unsigned)((M + kDotRows - 1) / kDotRows), (unsigned)((W + kDotCols - 1) / kDotCols));
     const size_t smem = (size_t)(kDotRows + kDotCols) * kDotStride * 4;
     if (D % 4 == 0 && ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15) == 0) {
-        cudaFuncSetAttribute(k9_dots<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k9_dots<true>);
         k9_dots<true><<<grid, 256, smem, s>>>(A, M, B, W, D, out, self);
     } else {
-        cudaFuncSetAttribute(k9_dots<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(k9_dots<false>);
         k9_dots<false><<<grid, 256, smem, s>>>(A, M, B, W, D, out, self);
     }
 }
@@ -1051,7 +1051,7 @@ void launch_rvq_few_seeds(const float* w1, int W1, const float* w2, int W2, int 
     }
     const size_t smem = few_seeds_smem(probe1, W2);
     auto kernel = W2 % 4 == 0 ? k9_few_seeds<true> : k9_few_seeds<false>;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(kernel);
     const int64_t batch = rvq_seed_batch(m);
     for (int64_t q0 = 0; q0 < m; q0 += batch) {
         const int64_t c = std::min(batch, m - q0);
@@ -1082,7 +1082,7 @@ void launch_rvq_seeds(const float* w1T, int W1, const float* w2T, int W2, int D,
     LaunchScope ls("k9_seeds", s,
                    (double)m * (D * 4.0 + (double)(W1 + W2) * D * 4.0 + (double)probe1 * W2 * 12.0 + s_seeds * 8.0),
                    (double)m * (W1 + W2) * D * 2.0);
-    cudaFuncSetAttribute(k9_seeds, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k9_seeds);
     k9_seeds<<<(unsigned)m, kSdT, smem, s>>>(w1T, W1, w2T, W2, D, n1, n2, x12, off, ids, Q, probe1, P, s_seeds, S,
                                              status);
 }

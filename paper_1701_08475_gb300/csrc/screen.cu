@@ -950,7 +950,7 @@ bool launch_screen(const uint16_t* A, const uint16_t* B, int Dp, ScreenArgs& P, 
     const size_t smem = screen_smem(P.nk, MODE).total + 1024;
     const int64_t units = (int64_t)P.nrt * P.nstripe;
     LaunchScope ls(name, s, (double)(P.nrows + P.ncols) * (Dp * 2.0 + 8.0), (double)P.nrows * P.ncols * 2.0 * Dp);
-    cudaFuncSetAttribute(ks_screen<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(ks_screen<MODE>);
     ks_screen<MODE><<<(int)std::min<int64_t>(units, kScGrid), kScThreads, smem, s>>>(ta, tb, P);
     return true;
 }
@@ -1020,7 +1020,7 @@ bool launch_exact_screened(const float* X, int64_t n, int D, int k, const int32_
     const int64_t batch = exact_batch(s_rows);
     const int nsplit = exact_splits(n, batch);
     const size_t rank_smem = (size_t)kScreenCap * 12 + ((size_t)D + 3) / 4 * 16;
-    cudaFuncSetAttribute(k7_rank<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rank_smem);
+    allow_smem(k7_rank<true>);
     for (int64_t q0 = 0; q0 < s_rows; q0 += batch) {
         const int64_t rows = std::min(batch, s_rows - q0);
         ScreenArgs P{};

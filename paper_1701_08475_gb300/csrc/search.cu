@@ -257,7 +257,7 @@ template <bool VEC, int W>
 void launch_search_t(const float* X, int64_t n, int D, const int32_t* G, int k, const float* Q, int64_t m,
                      const int32_t* S, int s, int t0, int ks, int32_t* out_ids, float* out_d, cudaStream_t st) {
     const size_t smem = search_smem(D, W).total;
-    cudaFuncSetAttribute(k8_search<VEC, W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k8_search<VEC, W>);
     k8_search<VEC, W><<<(unsigned)m, 32 * W, smem, st>>>(X, n, D, G, k, Q, S, s, t0, ks, out_ids, out_d);
 }
 

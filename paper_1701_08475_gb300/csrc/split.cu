@@ -1515,7 +1515,7 @@ void run_split_level(const float* X, int64_t n_rows, int D, const LevelPlan& lp,
             LaunchScope ls("k1_project", s, rows + n * 8, 2.0 * n * D);
             SelState* st = lp.small ? nullptr : b.st;
             if (vec) {
-                cudaFuncSetAttribute(k1_project_pipe, cudaFuncAttributeMaxDynamicSharedMemorySize, kPpSmem);
+                allow_smem(k1_project_pipe);
                 const int grid = std::min(lp.nsweep, 2 * sm_count());
                 k1_project_pipe<<<grid, kPrRows, kPpSmem, s>>>(X, D, perm_in, lp.sweep, lp.nsweep, lp.seg_off, b.W,
                                                                bi.S, st, b.status, b.Xq, b.Dq, b.qtype, b.qflag,
@@ -1583,7 +1583,7 @@ void run_split_level(const float* X, int64_t n_rows, int D, const LevelPlan& lp,
             // the staged sums pay off on an exact narrow copy (when the host
             // does not know, as in a captured build, they decide on the device)
             if (vec && (b.Xq || b.Xb) && (b.u8_host || b.q16_host || b.capture)) {
-                cudaFuncSetAttribute(k1_sums_async, cudaFuncAttributeMaxDynamicSharedMemorySize, kSuSmem);
+                allow_smem(k1_sums_async);
                 k1_sums_async<<<lp.ntiles, kSuThreads, kSuSmem, s>>>(X, D, perm_in, lp.tiles, bi.S, lp.seg_off,
                                                                      bi.thr, lp.pos_bits, b.partial, b.status, b.Xq,
                                                                      b.Dq, b.qtype, b.qflag, b.Xb, b.Db, b.bflag, Sp,
