@@ -49,14 +49,16 @@ void cuda_check(cudaError_t e, const char* what) {
 void record_error(const char* msg) { g_last_error = msg; }
 
 // ---------------------------------------------------------------- fault injection
-// KNNG_FAULT=alloc|launch makes the next calls fail on the host, for tests of
+// KNNG_FAULT=alloc|launch|optional makes the next calls fail on the host, for tests of
 // the error paths (no device fault is ever made): "alloc" fails the workspace
 // allocation as if the pool were out of memory (KNNG_ENOMEM); "launch" adds,
 // before the call's first kernel, one launch the runtime refuses on the host
 // (more threads per block than any GPU allows), which the call's launch check
-// reports (KNNG_ECUDA).  The variable is read at the start of every call.
+// reports (KNNG_ECUDA).  "optional" refuses only the allocations that a call
+// can do without: it takes its smaller layout and succeeds.  The variable is
+// read at the start of every call.
 namespace {
-thread_local int g_fault = 0;  // 0 none, 1 alloc, 2 launch
+thread_local int g_fault = 0;  // 0 none, 1 alloc, 2 launch, 3 optional
 thread_local bool g_fault_fired = false;
 // The first launch error of the current call, taken right after the launch:
 // later runtime calls of the same call may clear the runtime's own record.
@@ -67,7 +69,7 @@ __global__ void k_refused() {}
 
 void fault_begin() {
     const char* e = getenv("KNNG_FAULT");
-    g_fault = !e ? 0 : strcmp(e, "alloc") == 0 ? 1 : strcmp(e, "launch") == 0 ? 2 : 0;
+    g_fault = !e ? 0 : strcmp(e, "alloc") == 0 ? 1 : strcmp(e, "launch") == 0 ? 2 : strcmp(e, "optional") == 0 ? 3 : 0;
     g_fault_fired = false;
     g_launch_error = cudaSuccess;
 }
@@ -78,6 +80,8 @@ cudaError_t launch_error() {
 }
 
 bool fault_alloc() { return g_fault == 1; }
+
+bool fault_optional() { return g_fault == 3; }
 
 void fault_launch_point(cudaStream_t s) {
     if (g_fault != 2 || g_fault_fired) return;
@@ -301,6 +305,7 @@ struct Workspace {
             return true;
         }
         void* p = nullptr;
+        if (fault_optional()) return false;
         if (cudaMallocFromPoolAsync(&p, used, device_pool(), stream) != cudaSuccess) {
             cudaGetLastError();
             return false;

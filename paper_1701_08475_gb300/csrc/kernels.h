@@ -22,12 +22,14 @@ struct LaunchScope {
 // Reads the event times of the launches timed since the last flush into the
 // statistics; call after the stream has been synchronised.
 void stats_flush();
-// Host-side fault injection for tests (KNNG_FAULT=alloc|launch, read by
-// fault_begin at the start of each call): fault_alloc() tells an allocation
-// to fail; fault_launch_point(s) issues, once per call, a launch the runtime
+// Host-side fault injection for tests (KNNG_FAULT=alloc|launch|optional, read
+// by fault_begin at the start of each call): fault_alloc() tells an allocation
+// to fail, fault_optional() one that the call can do without;
+// fault_launch_point(s) issues, once per call, a launch the runtime
 // refuses on the host (never on a capturing stream).
 void fault_begin();
 bool fault_alloc();
+bool fault_optional();
 void fault_launch_point(cudaStream_t s);
 // The first error of a launch made in this call (LaunchScope records it right
 // after each launch), else the runtime's last error; both are cleared.
