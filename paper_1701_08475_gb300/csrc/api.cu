@@ -49,16 +49,16 @@ void cuda_check(cudaError_t e, const char* what) {
 void record_error(const char* msg) { g_last_error = msg; }
 
 // ---------------------------------------------------------------- fault injection
-// KNNG_FAULT=alloc|launch|optional makes the next calls fail on the host, for tests of
+// KNNG_FAULT=alloc|launch|optional|optionals makes the next calls fail on the host, for tests of
 // the error paths (no device fault is ever made): "alloc" fails the workspace
 // allocation as if the pool were out of memory (KNNG_ENOMEM); "launch" adds,
 // before the call's first kernel, one launch the runtime refuses on the host
 // (more threads per block than any GPU allows), which the call's launch check
-// reports (KNNG_ECUDA).  "optional" refuses only the allocations that a call
-// can do without: it takes its smaller layout and succeeds.  The variable is
-// read at the start of every call.
+// reports (KNNG_ECUDA).  "optional" refuses the call's first allocation that
+// it can do without, "optionals" every such one: it takes a smaller layout and
+// succeeds.  The variable is read at the start of every call.
 namespace {
-thread_local int g_fault = 0;  // 0 none, 1 alloc, 2 launch, 3 optional
+thread_local int g_fault = 0;  // 0 none, 1 alloc, 2 launch, 3 optional, 4 optionals
 thread_local bool g_fault_fired = false;
 // The first launch error of the current call, taken right after the launch:
 // later runtime calls of the same call may clear the runtime's own record.
@@ -69,7 +69,8 @@ __global__ void k_refused() {}
 
 void fault_begin() {
     const char* e = getenv("KNNG_FAULT");
-    g_fault = !e ? 0 : strcmp(e, "alloc") == 0 ? 1 : strcmp(e, "launch") == 0 ? 2 : strcmp(e, "optional") == 0 ? 3 : 0;
+    g_fault = !e ? 0 : strcmp(e, "alloc") == 0 ? 1 : strcmp(e, "launch") == 0 ? 2 : strcmp(e, "optional") == 0 ? 3
+            : strcmp(e, "optionals") == 0 ? 4 : 0;
     g_fault_fired = false;
     g_launch_error = cudaSuccess;
 }
@@ -81,7 +82,11 @@ cudaError_t launch_error() {
 
 bool fault_alloc() { return g_fault == 1; }
 
-bool fault_optional() { return g_fault == 3; }
+bool fault_optional() {
+    const bool refuse = g_fault == 4 || (g_fault == 3 && !g_fault_fired);
+    g_fault_fired |= refuse;
+    return refuse;
+}
 
 void fault_launch_point(cudaStream_t s) {
     if (g_fault != 2 || g_fault_fired) return;
@@ -1936,8 +1941,9 @@ int knng_exact(const float* data, int64_t n, int D, int k, const int32_t* sample
         const size_t batch = (size_t)exact_batch(s_rows);
         const int nsplit = exact_splits(n, s_rows);
         // the screen's copy and candidate lists come on top of what the FP32
-        // kernel needs; where they do not fit, the FP32 kernel runs alone
-        bool screen = exact_screened(n);
+        // kernel needs; where they do not fit, the FP32 kernel runs alone, with
+        // its columns split when the partial lists fit
+        bool screen = exact_screened(n), split = nsplit > 1;
         for (int ps = 0; ps < 2; ++ps) {
             ws.used = 0;
             bind(ws, X, data, (size_t)n * D, ps);
@@ -1963,10 +1969,11 @@ int knng_exact(const float* data, int64_t n, int D, int k, const int32_t* sample
                 w.fb_list = ws.take<int32_t>(batch);
                 w.fb_flag = ws.take<int32_t>(batch);
                 w.part = ws.take<uint64_t>(batch * exact_splits(n, (int64_t)batch) * k);
-            } else if (nsplit > 1) {
-                part = ws.take<uint64_t>(sk * nsplit);
+            } else {
+                part = split ? ws.take<uint64_t>(sk * nsplit) : nullptr;
             }
-            if (ps == 0 && !ws.try_allocate(s, screen)) {
+            if (ps == 0 && !ws.try_allocate(s, screen || split)) {
+                if (!screen) split = false;
                 screen = false;
                 ps = -1;
             }

@@ -22,8 +22,8 @@ struct LaunchScope {
 // Reads the event times of the launches timed since the last flush into the
 // statistics; call after the stream has been synchronised.
 void stats_flush();
-// Host-side fault injection for tests (KNNG_FAULT=alloc|launch|optional, read
-// by fault_begin at the start of each call): fault_alloc() tells an allocation
+// Host-side fault injection for tests (KNNG_FAULT, read by fault_begin at the
+// start of each call): fault_alloc() tells an allocation
 // to fail, fault_optional() one that the call can do without;
 // fault_launch_point(s) issues, once per call, a launch the runtime
 // refuses on the host (never on a capturing stream).

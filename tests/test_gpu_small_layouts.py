@@ -1,6 +1,6 @@
 """Calls whose scratch does not fit take a smaller layout and give the same
-results: KNNG_FAULT=optional refuses, on the host, every allocation that a call
-can do without.  Exact lists by the FP32 kernel with its columns split, words
+results: KNNG_FAULT=optional refuses, on the host, the first allocation that a
+call can do without, KNNG_FAULT=optionals every one.  Exact lists by the FP32 kernel with its columns split, words
 and codes by the FP32 assignment with every word's mean summed in ascending
 order, and up to 32 seeds by the general ranking; the statistics say that those
 kernels ran."""
@@ -25,15 +25,15 @@ def knng():
 
 @pytest.fixture
 def kernels(knng, monkeypatch):
-    """Runs a call under the fault; its result and the names of the kernels that ran."""
-    def run(call):
-        monkeypatch.setenv("KNNG_FAULT", "optional")
+    """Runs a call under the fault; its result and the statistics of the kernels that ran."""
+    def run(call, mode="optional"):
+        monkeypatch.setenv("KNNG_FAULT", mode)
         knng.stats_reset()
         knng.stats_enable(True, False)
         try:
             out = call()
             torch.cuda.synchronize()
-            return out, set(knng.stats())
+            return out, knng.stats()
         finally:
             knng.stats_enable(False)
             monkeypatch.delenv("KNNG_FAULT")
@@ -55,6 +55,16 @@ def test_exact_lists(knng, kernels, n, D, k, s):
     assert "k7_exact" in ran and "ks_screen" not in ran
 
 
+def test_exact_lists_without_partial_lists(knng, kernels):
+    """The FP32 lists need no scratch beyond the keys when the partial lists of its column splits do not fit."""
+    X, rows = _dev(datagen.gaussian_mixture(30000, 60, 30, seed=1), datagen.sample_rows(30000, 200, seed=4))
+    (ids, d), ran = kernels(lambda: knng.knng_exact(X, 12, rows), "optional")
+    assert ran["k7_exact"]["launches"] == 2          # the splits, then their merge
+    (ids1, d1), ran = kernels(lambda: knng.knng_exact(X, 12, rows), "optionals")
+    assert ran["k7_exact"]["launches"] == 1
+    assert torch.equal(ids, ids1) and torch.equal(d, d1)
+
+
 @pytest.mark.parametrize("n,D,W1,W2", [(3000, 33, 16, 20), (2500, 128, 200, 129), (40, 5, 40, 3)])
 def test_words_and_index(knng, kernels, n, D, W1, W2):
     X = datagen.gaussian_mixture(n, D, 20, seed=n)
@@ -66,7 +76,7 @@ def test_words_and_index(knng, kernels, n, D, W1, W2):
     got, ran = kernels(lambda: knng.knng_rvq_index(Xd, w1, w2))
     for a, b in zip(got, oracle.rvq_index(X, o1, o2)):
         assert np.array_equal(a.cpu().numpy(), b)
-    assert {"k9_assign", "k9_assign_res"} <= ran and "ks_assign" not in ran
+    assert {"k9_assign", "k9_assign_res"} <= set(ran) and "ks_assign" not in ran
 
 
 @pytest.mark.parametrize("W1,W2,probe1,s,D,m", [(64, 256, 16, 32, 40, 65), (7, 13, 7, 20, 33, 200), (256, 30, 32, 1, 64, 3)])
