@@ -375,7 +375,8 @@ typedef struct knng_kernel_stat {
     double ms;       /* summed device time, 0 when timing is off */
     double bytes;    /* summed algorithmic bytes */
     double flops;    /* summed algorithmic flops */
-    double items;    /* summed work items where counted (k5_join: offers that passed the filter) */
+    double items;    /* summed work items where counted (k5_join: offers that passed the filter;
+                        k7_exact: rows of screened calls that took the FP32 kernel) */
 } knng_kernel_stat;
 
 KNNG_API int knng_stats_enable(int on, int timing);

@@ -810,11 +810,14 @@ int grid_1d(int64_t count) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, 152 * 16));
 }
 
-void check_status(const int* dstatus, cudaStream_t s) {
-    int st = 0;
-    cuda_check(cudaMemcpyAsync(&st, dstatus, sizeof st, cudaMemcpyDeviceToHost, s), "status read");
+// given_up: the kernel whose statistics count the rows in the second word.
+void check_status(const int* dstatus, cudaStream_t s, const char* given_up = nullptr) {
+    int hs[2] = {0, 0};
+    cuda_check(cudaMemcpyAsync(hs, dstatus, sizeof hs, cudaMemcpyDeviceToHost, s), "status read");
     cuda_check(cudaStreamSynchronize(s), "stream synchronize");
     reg().flush();
+    const int st = hs[0];
+    if (given_up) record_items(given_up, (double)hs[1]);
     if (st & kStatusTimeout) fail(KNNG_ETIMEOUT, "a bounded device wait ran out");
     if (st & kStatusNonFinite) fail(KNNG_EINVAL, "data holds a non-finite value");
     if (st & kStatusBadInput) fail(KNNG_EINVAL, "an id or offset given by the caller is out of range");
@@ -1994,7 +1997,7 @@ int knng_exact(const float* data, int64_t n, int D, int k, const int32_t* sample
         download(oi, s);
         download(od, s);
         cuda_check(launch_error(), "kernel launch");
-        check_status(status, s);
+        check_status(status, s, screen ? "k7_exact" : nullptr);
     });
 }
 

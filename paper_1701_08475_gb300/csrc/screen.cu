@@ -862,6 +862,7 @@ __global__ void __launch_bounds__(kRrThreads) k7_rank(ScreenArgs P, bool dump, i
         if (threadIdx.x == 0) {
             fb_flag[r] = 1;
             fb_list[atomicAdd(fb_count, 1)] = (int32_t)r;
+            atomicAdd(P.status + 1, 1);  // over all batches (statistics)
             rowA[r] = 0.f;
             rowR[r] = __int_as_float(0xff800000);
         }
