@@ -18,21 +18,31 @@
 // collected ids do not depend on the order.
 //
 // Visited ids are kept in a shared-memory hash table.  It is exact until it is
-// three quarters full; after that an id may be visited again, which the merge
-// drops when it is in the list, and which cannot enter the list when it was
-// turned away before (the ks-th key only falls).
+// three quarters full; from then on it is a cache: an id is looked for in eight
+// slots, and takes the place of another there when it is new.  So an id may be
+// visited again, which the merge drops when it is in the list, and which cannot
+// enter the list when it was turned away before (the ks-th key only falls).  The
+// ids met again are mostly recent ones: with the table frozen when it was full,
+// every later id went through long probes and was visited anew each time
+// (300,000 x 128, k = 20, ks = 32, 1,000 queries 0.85 ms, 0.46 so; 40,000 x 48,
+// k = 64, 305 queries 6.3 and 0.91; one query per warp with exact tables of twice
+// the visits in global memory 1.1).
 //
 // One CTA per query: one warp, or, for few queries, kSearchGroup warps, which
-// share the collecting and take a batch of rows each.
+// share the collecting and take a batch of rows each.  Rows of at least
+// kSearchWide dims are staged 128 dims at a time with one warp too (fewer round
+// trips to memory; the query then comes with each stage): 20,000 x 960, k = 16,
+// ks = 32, 305 queries 1.95 -> 1.25 ms, 10,000 queries 6.10 -> 5.88; at 512 dims
+// 10,000 queries 3.67 -> 3.88, at 256 2.21 -> 2.70.
 //
 // Measured (GB300), 1M x 128 integers, k = 20, 10,000 queries, t0 = 12, ks = 20:
 // the call took 2.54 ms with a lane per row in global memory, the visited
 // tables in global memory and every entry expanded in every iteration; 1.57
 // with entries expanded once, staged rows and shared tables (128 dims, two
 // queries per CTA: 10 warps per SM), 0.97 with one query per CTA and 32 dims,
-// 0.86 with far rows dropped.  What is left is issue slots and latency about
-// equally (47 % of issue slots used, 625 MB read from DRAM at n = 300,000).
-// One query, 100,000 x 96: the kernel 115 -> 28 us.
+// 0.86 with far rows dropped, 0.80 with a warp's ids queued by one atomic.  What
+// is left is issue slots and latency about equally.  One query, 100,000 x 96: the
+// kernel 115 -> 28 us.
 #include <algorithm>
 
 #include "common.cuh"
@@ -43,23 +53,27 @@ namespace knng {
 namespace {
 
 constexpr int kSearchGroup = 4;  // warps of a query when there are few
-// dims staged at once: narrow with one warp per query, so that more queries fit
-// an SM; wide with several, where one round trip to memory is what counts
-__host__ __device__ constexpr int search_dims(int W) { return W > 1 ? 128 : 32; }
 // floats per staged row: the 16-byte reads of 8 lanes cover all banks
-__host__ __device__ constexpr int search_stride(int W) { return search_dims(W) + 4; }
-constexpr int kSearchTab = 1024;             // visited table
-constexpr int kSearchFull = kSearchTab * 3 / 4;
+__host__ __device__ constexpr int search_stride(int dims) { return dims + 4; }
+// slots of the visited table (log2): one warp's is small, so that many queries
+// fit an SM; all layouts are compile-time constants (table sizes chosen at run
+// time cost 30 % of the bulk search)
+__host__ __device__ constexpr int search_tab(int W) { return W > 1 ? 12 : 10; }
+constexpr int kSearchNear = 8;     // slots that a full table is asked for an id
 constexpr int kSearchQueue = 256;
+constexpr int kSearchWide = 640;
+
+__host__ __device__ constexpr bool search_by_stage(int W, int dims) { return W == 1 && dims > 32; }
 
 struct SearchSmem {
     size_t stage, tab, queue, keys, entry, misc, total;
 };
-__host__ __device__ inline SearchSmem search_smem(int D, int W) {
+__host__ __device__ inline SearchSmem search_smem(int D, int W, int dims) {
     SearchSmem L;
-    L.stage = ((size_t)D * 4 + 15) & ~(size_t)15;  // the query first
-    L.tab = L.stage + (size_t)W * 32 * search_stride(W) * 4;
-    L.queue = L.tab + kSearchTab * 4;
+    // the query first; with one warp and wide stages, the dims of one stage
+    L.stage = ((size_t)(search_by_stage(W, dims) ? dims : D) * 4 + 15) & ~(size_t)15;
+    L.tab = L.stage + (size_t)W * 32 * search_stride(dims) * 4;
+    L.queue = L.tab + ((size_t)4 << search_tab(W));
     L.keys = L.queue + kSearchQueue * 4;
     L.entry = L.keys + (size_t)W * 32 * 8;
     L.misc = L.entry + 32 * 4;
@@ -74,16 +88,19 @@ __device__ __forceinline__ uint64_t list_key(float d, uint32_t id) {
 }
 __device__ __forceinline__ uint32_t list_id(uint64_t k) { return (uint32_t)k >> 1; }
 
-template <bool VEC, int W>
+// W: warps of the CTA; DIMS: dims staged at once.
+template <bool VEC, int W, int DIMS>
 __global__ void __launch_bounds__(32 * W) k8_search(
     const float* __restrict__ X, int64_t n, int D, const int32_t* __restrict__ G, int k, const float* __restrict__ Q,
     const int32_t* __restrict__ S, int s, int t0, int ks, int32_t* __restrict__ out_ids,
     float* __restrict__ out_d) {
-    constexpr int kDims = search_dims(W), kStride = search_stride(W);
+    constexpr int kDims = DIMS, kStride = search_stride(DIMS);
+    constexpr int tab_log2 = search_tab(W), full = 3 << (tab_log2 - 2);
+    constexpr uint32_t mask = (1u << tab_log2) - 1u;
     extern __shared__ __align__(16) uint8_t se_smem[];
     const int gt = threadIdx.x, gw = gt >> 5, lane = gt & 31;
     const int64_t qi = blockIdx.x;
-    const SearchSmem L = search_smem(D, W);
+    const SearchSmem L = search_smem(D, W, DIMS);
     uint8_t* base = se_smem;
     float* q = reinterpret_cast<float*>(base);
     float* stage = reinterpret_cast<float*>(base + L.stage) + (size_t)gw * 32 * kStride;
@@ -97,30 +114,47 @@ __global__ void __launch_bounds__(32 * W) k8_search(
         if (W > 1) __syncthreads();
         else __syncwarp();
     };
-    for (int j = gt; j < D; j += 32 * W) q[j] = Q[qi * D + j];
-    for (int j = gt; j < kSearchTab; j += 32 * W) tab[j] = -1;
+    constexpr bool kByStage = search_by_stage(W, DIMS);
+    for (int j = gt; j < D && !kByStage; j += 32 * W) q[j] = Q[qi * D + j];
+    for (int j = gt; j < (1 << tab_log2) / 4; j += 32 * W) reinterpret_cast<int4*>(tab)[j] = make_int4(-1, -1, -1, -1);
     if (gt < 3) misc[gt] = 0;
     if (gt == 0) *bound = __int_as_float(0x7f800000);
     sync();
     uint64_t list = kEmptyKey;  // entry `lane` of the list (in warp 0)
 
-    // queues an id (-1: none) that has not been visited
+    // queues the lanes' ids (-1: none) that have not been visited; by whole warps
     auto collect = [&](int32_t id) {
-        if (id < 0 || id >= n) return;
-        uint32_t h = ((uint32_t)id * 2654435761u) >> 22;
+        const uint32_t h = ((uint32_t)id * 2654435761u) >> (32 - tab_log2);
+        const bool room = __shfl_sync(0xffffffffu, *(volatile int*)(misc + 1), 0) < full;
         bool fresh = false;
-        const bool room = *(volatile int*)(misc + 1) < kSearchFull;
-        for (int probe = 0; probe < kSearchTab; ++probe) {
-            const int32_t old = room ? atomicCAS(tab + h, -1, id) : *(volatile int32_t*)(tab + h);
-            if (old == id) return;
-            if (old == -1) {
+        if (id >= 0 && id < n) {
+            if (room) {
+                uint32_t at = h;
+                for (uint32_t probe = 0; probe <= mask; ++probe) {
+                    const int32_t old = atomicCAS(tab + at, -1, id);
+                    fresh = old == -1;
+                    if (fresh || old == id) break;
+                    at = (at + 1u) & mask;
+                }
+            } else {
                 fresh = true;
-                break;
+#pragma unroll
+                for (int e = 0; e < kSearchNear; ++e) fresh &= *(volatile int32_t*)(tab + ((h + e) & mask)) != id;
             }
-            h = (h + 1u) & (kSearchTab - 1);
         }
-        if (room && fresh) atomicAdd(misc + 1, 1);
-        queue[atomicAdd(misc, 1)] = id;
+        const unsigned bal = __ballot_sync(0xffffffffu, fresh);
+        if (bal == 0) return;
+        int at = 0;
+        if (lane == 0) {
+            at = atomicAdd(misc, __popc(bal));
+            if (room) atomicAdd(misc + 1, __popc(bal));
+        }
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(bal & ((1u << lane) - 1u));
+        if (fresh) {
+            queue[at] = id;
+            // full: the id takes the place of an older one near its own
+            if (!room) *(volatile int32_t*)(tab + ((h + at % kSearchNear) & mask)) = id;
+        }
     };
     // distances of the queued ids, merged into the list; empties the queue
     auto process = [&] {
@@ -141,6 +175,12 @@ __global__ void __launch_bounds__(32 * W) k8_search(
                 // P pieces per row: a warp's lanes take 32 / P rows side by side
                 constexpr int P = VEC ? kDims / 4 : 32, R = 32 / P;
                 const int32_t* ids = queue + b + 32 * gw;
+                if (kByStage)
+                    for (int c = lane; c < dl; c += 32)
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(
+                                         (uint32_t)__cvta_generic_to_shared(q + c)),
+                                     "l"(Q + qi * D + d0 + c)
+                                     : "memory");
                 for (int r = lane / P; r < cnt; r += R) {
                     if (!((open >> r) & 1u)) continue;
                     const float* src = X + (int64_t)ids[r] * D + d0;
@@ -160,7 +200,7 @@ __global__ void __launch_bounds__(32 * W) k8_search(
                 __syncwarp();
                 if ((open >> lane) & 1u) {  // the canonical chain: dims ascending, t = x_j - q_j, acc = fmaf(t, t, acc)
                     const float* x = stage + lane * kStride;
-                    const float* y = q + d0;
+                    const float* y = kByStage ? q : q + d0;
                     if (VEC) {
 #pragma unroll 4
                         for (int j = 0; j < dl; j += 4) {
@@ -189,16 +229,22 @@ __global__ void __launch_bounds__(32 * W) k8_search(
             if (gw == 0) {
                 for (int v = 0; v < W && b + 32 * v < nq; ++v) {
                     uint64_t cand[1] = {keys[32 * v + lane]}, out;
-                    if (misc[1] >= kSearchFull) {
-                        // the table is no longer exact: drop ids the list
-                        // holds, and repeats
-                        const uint32_t cid = cand[0] == kEmptyKey ? 0xFFFFFFFFu : list_id(cand[0]);
+                    if (misc[1] >= full) {
+                        // the table is no longer exact: of the ids that could
+                        // enter drop those that the list holds, and repeats
+                        const uint64_t kth = shfl64(list, ks - 1);
+                        const bool in = cand[0] < kth;
+                        unsigned left = __ballot_sync(0xffffffffu, in);
+                        if (left == 0) continue;
+                        const uint32_t cid = in ? list_id(cand[0]) : 0x80000000u | (uint32_t)lane;  // ids are below 2^31
                         bool drop = (__match_any_sync(0xffffffffu, cid) & ((1u << lane) - 1u)) != 0;
-                        for (int e = 0; e < ks; ++e) {
-                            const uint64_t o = shfl64(list, e);
-                            drop |= o != kEmptyKey && list_id(o) == cid;
+                        const uint32_t have = list == kEmptyKey ? 0xFFFFFFFFu : list_id(list);
+                        for (; left; left &= left - 1) {
+                            const int src = __ffs(left) - 1;
+                            const bool held = __any_sync(0xffffffffu, have == __shfl_sync(0xffffffffu, cid, src));
+                            drop |= held && lane == src;
                         }
-                        if (drop) cand[0] = kEmptyKey;
+                        if (drop || !in) cand[0] = kEmptyKey;
                     }
                     __syncwarp();
                     bool changed;
@@ -253,12 +299,12 @@ __global__ void __launch_bounds__(32 * W) k8_search(
     }
 }
 
-template <bool VEC, int W>
+template <bool VEC, int W, int DIMS>
 void launch_search_t(const float* X, int64_t n, int D, const int32_t* G, int k, const float* Q, int64_t m,
                      const int32_t* S, int s, int t0, int ks, int32_t* out_ids, float* out_d, cudaStream_t st) {
-    const size_t smem = search_smem(D, W).total;
-    allow_smem(k8_search<VEC, W>);
-    k8_search<VEC, W><<<(unsigned)m, 32 * W, smem, st>>>(X, n, D, G, k, Q, S, s, t0, ks, out_ids, out_d);
+    const size_t smem = search_smem(D, W, DIMS).total;
+    allow_smem(k8_search<VEC, W, DIMS>);
+    k8_search<VEC, W, DIMS><<<(unsigned)m, 32 * W, smem, st>>>(X, n, D, G, k, Q, S, s, t0, ks, out_ids, out_d);
 }
 
 }  // namespace
@@ -274,16 +320,17 @@ void launch_search(const float* X, int64_t n, int D, const int32_t* G, int k, co
     const bool vec = D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
     // with less than two queries per SM the chip is idle anyway: four warps on each
     const bool few = m <= 2 * 152;
+    const bool wide = D >= kSearchWide;
     for (int64_t q0 = 0; q0 < m; q0 += (int64_t)1 << 30) {  // one CTA per query
         const int64_t c = std::min(m - q0, (int64_t)1 << 30);
         const float* Qc = Q + q0 * D;
         const int32_t* Sc = S ? S + q0 * s : nullptr;
         int32_t* ic = out_ids + q0 * ks;
         float* dc = out_d + q0 * ks;
-        if (few && vec) launch_search_t<true, kSearchGroup>(X, n, D, G, k, Qc, c, Sc, s, t0, ks, ic, dc, st);
-        else if (few) launch_search_t<false, kSearchGroup>(X, n, D, G, k, Qc, c, Sc, s, t0, ks, ic, dc, st);
-        else if (vec) launch_search_t<true, 1>(X, n, D, G, k, Qc, c, Sc, s, t0, ks, ic, dc, st);
-        else launch_search_t<false, 1>(X, n, D, G, k, Qc, c, Sc, s, t0, ks, ic, dc, st);
+        const auto launch = few ? (vec ? launch_search_t<true, kSearchGroup, 128> : launch_search_t<false, kSearchGroup, 128>)
+                          : wide ? (vec ? launch_search_t<true, 1, 128> : launch_search_t<false, 1, 128>)
+                                 : (vec ? launch_search_t<true, 1, 32> : launch_search_t<false, 1, 32>);
+        launch(X, n, D, G, k, Qc, c, Sc, s, t0, ks, ic, dc, st);
     }
 }
 
