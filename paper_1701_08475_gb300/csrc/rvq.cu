@@ -336,9 +336,25 @@ __global__ void __launch_bounds__(128) k9_pieces(const float* __restrict__ X, in
     }
 }
 
+// (double)x by integer operations: the conversion would take the FP64 units as
+// long as the addition that follows it.
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
+    if (m != 0 && m < 0x00800000u) return (double)x;  // subnormal
+    const uint32_t hi = m ? (m >> 3) + 0x38000000u : 0u;
+    return __hiloint2double((int)((u & 0x80000000u) | hi), (int)(m << 29));
+}
+
 // One CTA per word and 128 dims: the sum of its pieces, the proof that the
-// rounded mean is the defined one, and else the chain.
+// rounded mean is the defined one, and else the chain: one group adds 32 members
+// from shared memory while the others bring the next 32.  Its bound is then the
+// FP64 units: an addition of a warp has a latency of 64 cycles and takes 19 of
+// the SM's.  41,286 x 480 GIST-like rows in 64 uneven words (one of 37,571), 16
+// updates: 43.8 ms with one thread loading 32 values and then adding them, or
+// with a word's chunks of dims on one SM; 25.0 so.
 constexpr int kCbGroups = 4;  // the pieces of a word are read by this many threads per dim
+constexpr int kCbRows = 32;   // members staged at once
+constexpr int kCbShare = (kCbRows + kCbGroups - 2) / (kCbGroups - 1);  // of them per loading thread
 __global__ void __launch_bounds__(128 * kCbGroups) k9_combine(const float* __restrict__ X, int64_t N, int D,
                                                  const int32_t* __restrict__ order,
                                                  const int32_t* __restrict__ gofs, int nb, int W,
@@ -346,61 +362,80 @@ __global__ void __launch_bounds__(128 * kCbGroups) k9_combine(const float* __res
     __shared__ double gsum[kCbGroups][128];
     __shared__ float gabs[kCbGroups][128];
     __shared__ int glo[kCbGroups][128];
+    __shared__ float rows[2][kCbRows][128];
     const int dd = threadIdx.x & 127, g = threadIdx.x >> 7;
-    const int c = blockIdx.x, d = blockIdx.y * 128 + dd;
+    // a word's chunks of dims are neighbours in the grid, which go to different
+    // SMs: side by side on one their chains share its FP64 units
+    const int chunks = (D + 127) / 128, c = (int)(blockIdx.x / chunks), d = (int)(blockIdx.x % chunks) * 128 + dd;
     const int a = gofs[(int64_t)c * nb], b = c + 1 < W ? gofs[(int64_t)(c + 1) * nb] : (int)N;
-    if (b == a) return;  // no members: the word keeps its value
+    if (b == a) return;  // no members: the word keeps its value (the whole CTA)
     double sum = 0.0;
     const int m = b - a;
-    auto chain = [&] {  // the defined order, the loads of 32 members ahead of their additions
-        double s = 0.0;
-        for (int t = a; t < b; t += 32) {
-            float v[32];
-#pragma unroll
-            for (int q = 0; q < 32; ++q) v[q] = t + q < b ? __ldg(X + (int64_t)order[t + q] * D + d) : 0.f;
-#pragma unroll
-            for (int q = 0; q < 32; ++q)
-                if (t + q < b) s = __dadd_rn(s, (double)v[q]);
-        }
-        return s;
-    };
-    if (part == nullptr) {  // no room for pieces
-        if (g == 0 && d < D) words[(int64_t)c * D + d] = __double2float_rn(__ddiv_rn(chain(), (double)m));
-        return;
-    }
-    int lo = kUpNone;
-    float A = 0.f;
-    if (d < D) {
+    bool open = part == nullptr && g == 0;  // whether this sum has to be the chain's
+    if (part != nullptr) {
+        int lo = kUpNone;
+        float A = 0.f;
+        if (d < D) {
 #pragma unroll 4
-        for (int64_t u = a / kUpRows + g; u <= (b - 1) / kUpRows; u += kCbGroups) {
-            const double* o = up_slot(part, u + c, D);
-            const uint2 mg = reinterpret_cast<const uint2*>(o + D)[d];
-            sum = __dadd_rn(sum, o[d]);
-            lo = min(lo, (int)mg.x);
-            A = __fadd_ru(A, __uint_as_float(mg.y));
+            for (int64_t u = a / kUpRows + g; u <= (b - 1) / kUpRows; u += kCbGroups) {
+                const double* o = up_slot(part, u + c, D);
+                const uint2 mg = reinterpret_cast<const uint2*>(o + D)[d];
+                sum = __dadd_rn(sum, o[d]);
+                lo = min(lo, (int)mg.x);
+                A = __fadd_ru(A, __uint_as_float(mg.y));
+            }
+        }
+        gsum[g][dd] = sum;
+        gabs[g][dd] = A;
+        glo[g][dd] = lo;
+        __syncthreads();
+        if (g == 0) {
+#pragma unroll
+            for (int q = 1; q < kCbGroups; ++q) {
+                sum = __dadd_rn(sum, gsum[q][dd]);
+                A = __fadd_ru(A, gabs[q][dd]);
+                lo = min(lo, glo[q][dd]);
+            }
+            // every value is a multiple of 2^(lo - 150) and no partial sum is
+            // above A, which past FP32's range is no bound at all (then x and
+            // y below differ)
+            if (up_exp(A) > 53 + lo - 150 || isinf(A)) {
+                // the defined order is within m 2^-53 A, and a little, of the
+                // true sum; this one, which adds at most m / 128 + 48 times in
+                // a row, nearer
+                const double e = ldexp(((double)m * 1.0625 + 64.0) * (double)A, -53);
+                const float x = __double2float_rn(__ddiv_rn(sum - e, (double)m));
+                const float y = __double2float_rn(__ddiv_rn(sum + e, (double)m));
+                open = x != y || x == 0.f;
+            }
         }
     }
-    gsum[g][dd] = sum;
-    gabs[g][dd] = A;
-    glo[g][dd] = lo;
-    __syncthreads();
-    if (g > 0 || d >= D) return;
+    if (__syncthreads_or(open)) {
+        double s = 0.0;
+        for (int t = a - kCbRows; t < b; t += kCbRows) {  // members t .. are added, the next ones brought
+            const int buf = ((t - a) / kCbRows) & 1;
+            if (g > 0) {
+                float v[kCbShare];
 #pragma unroll
-    for (int q = 1; q < kCbGroups; ++q) {
-        sum = __dadd_rn(sum, gsum[q][dd]);
-        A = __fadd_ru(A, gabs[q][dd]);
-        lo = min(lo, glo[q][dd]);
+                for (int q = 0; q < kCbShare; ++q) {
+                    const int r = g - 1 + q * (kCbGroups - 1), p = t + kCbRows + r;
+                    v[q] = r < kCbRows && p < b && d < D ? __ldg(X + (int64_t)__ldg(order + p) * D + d) : 0.f;
+                }
+#pragma unroll
+                for (int q = 0; q < kCbShare; ++q) {
+                    const int r = g - 1 + q * (kCbGroups - 1);
+                    if (r < kCbRows) rows[buf ^ 1][r][dd] = v[q];
+                }
+            } else if (t >= a) {
+#pragma unroll
+                for (int r = 0; r < kCbRows; ++r)
+                    if (t + r < b) s = __dadd_rn(s, widen(rows[buf][r][dd]));
+            }
+            __syncthreads();
+        }
+        if (open) sum = s;
     }
-    // every value is a multiple of 2^(lo - 150) and no partial sum is above A,
-    // which past FP32's range is no bound at all (then x and y below differ)
-    if (up_exp(A) > 53 + lo - 150 || isinf(A)) {
-        // either order is within (m - 1) 2^-53 A, and a little, of the true sum
-        const double e = ldexp((double)m * (double)A, -51);
-        const float x = __double2float_rn(__ddiv_rn(sum - e, (double)m));
-        const float y = __double2float_rn(__ddiv_rn(sum + e, (double)m));
-        if (x != y || x == 0.f) sum = chain();
-    }
-    words[(int64_t)c * D + d] = __double2float_rn(__ddiv_rn(sum, (double)m));
+    if (g == 0 && d < D) words[(int64_t)c * D + d] = __double2float_rn(__ddiv_rn(sum, (double)m));
 }
 
 // words[c] = v_{pos[c]} (the initial words).
@@ -985,7 +1020,7 @@ void launch_rvq_update(const float* X, int64_t N, int D, const int32_t* order, c
     const bool vec = D % 4 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
     if (part && vec) k9_pieces<true><<<grid, 128, 0, s>>>(X, N, D, order, gofs, nb, W, part);
     if (part && !vec) k9_pieces<false><<<grid, 128, 0, s>>>(X, N, D, order, gofs, nb, W, part);
-    k9_combine<<<dim3((unsigned)W, (unsigned)((D + 127) / 128)), 128 * kCbGroups, 0, s>>>(X, N, D, order, gofs, nb, W, part,
+    k9_combine<<<(unsigned)(W * ((D + 127) / 128)), 128 * kCbGroups, 0, s>>>(X, N, D, order, gofs, nb, W, part,
                                                                              words);
 }
 
