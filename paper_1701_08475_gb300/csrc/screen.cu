@@ -120,22 +120,13 @@ __host__ __device__ inline ScreenSmem screen_smem(int nk, int mode) {
     return L;
 }
 
-// The canonical distance of one vector (x, minus w1 when given) to one word
-// (or to a point staged in shared memory).
-__device__ __forceinline__ float word_dist(const float* __restrict__ x, const float* __restrict__ w1,
-                                           const float* w, int D, bool vec) {
+// The canonical distance of a point to one staged in shared memory.
+__device__ __forceinline__ float point_dist(const float* __restrict__ x, const float* q, int D, bool vec) {
     float acc = 0.f;
     if (vec) {
         for (int d = 0; d < D; d += 4) {
-            float4 a = __ldg(reinterpret_cast<const float4*>(x + d));
-            const float4 b = *reinterpret_cast<const float4*>(w + d);
-            if (w1) {
-                const float4 r = __ldg(reinterpret_cast<const float4*>(w1 + d));
-                a.x = __fsub_rn(a.x, r.x);
-                a.y = __fsub_rn(a.y, r.y);
-                a.z = __fsub_rn(a.z, r.z);
-                a.w = __fsub_rn(a.w, r.w);
-            }
+            const float4 a = __ldg(reinterpret_cast<const float4*>(x + d));
+            const float4 b = *reinterpret_cast<const float4*>(q + d);
             float t = __fsub_rn(a.x, b.x);
             acc = __fmaf_rn(t, t, acc);
             t = __fsub_rn(a.y, b.y);
@@ -148,9 +139,7 @@ __device__ __forceinline__ float word_dist(const float* __restrict__ x, const fl
         return acc;
     }
     for (int d = 0; d < D; ++d) {
-        float a = __ldg(x + d);
-        if (w1) a = __fsub_rn(a, __ldg(w1 + d));
-        const float t = __fsub_rn(a, w[d]);
+        const float t = __fsub_rn(__ldg(x + d), q[d]);
         acc = __fmaf_rn(t, t, acc);
     }
     return acc;
@@ -332,8 +321,9 @@ __global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant
         int32_t* brow = reinterpret_cast<int32_t*>(base + L.list_off);
         int32_t* bid = brow + kScCand;
         float* bg = reinterpret_cast<float*>(bid + kScCand);
-        // nearest word: the words' c_j, then e_j (one column tile, loaded
-        // once), the greatest N_j and e_j, and each part's least value of a row
+        // nearest word: the words' c_j, then e_j, then N_j (1 + c) rounded up
+        // (one column tile, loaded once), the greatest e_j, and each part's
+        // least value of a row
         float* colf = reinterpret_cast<float*>(colc);
         uint32_t* cmax = reinterpret_cast<uint32_t*>(ncand);
         float* hmin = reinterpret_cast<float*>(base + L.row_off);  // [2][4][kScM]
@@ -388,10 +378,8 @@ __global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant
                 const float2 c = col_const(et);
                 colf[et] = c.x;
                 colf[kScN + et] = c.y;
-                if (et < P.ncols) {  // both at least 0: their bits have their order
-                    atomicMax(cmax, __float_as_uint(__ldg(P.cnrm + et)));
-                    atomicMax(cmax + 1, __float_as_uint(c.y));
-                }
+                colf[2 * kScN + et] = et < P.ncols ? __fmul_ru(__ldg(P.cnrm + et), __fadd_ru(1.f, c2)) : c.x;
+                if (et < P.ncols) atomicMax(cmax, __float_as_uint(c.y));  // at least 0: its bits have its order
             }
             epi_sync();
         }
@@ -492,9 +480,9 @@ __global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant
                         __syncwarp();
                     }
                 } else {
-                    // nearest word: the row's least approximate value gives an
-                    // upper bound tau of its least distance; every word that
-                    // could be within tau is a candidate
+                    // nearest word: the row's least upper bound of a distance
+                    // gives tau; every word that could be within tau is a
+                    // candidate
                     float va[32], vb[32];
                     tc::tmem_ld_issue(taddr, va);
                     tc::tmem_ld_issue(taddr + 32, vb);
@@ -505,11 +493,12 @@ __global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant
                     if (lane == 0) mbar_arrive(tempty0 + 8 * buf);
                     const float4* c4 = reinterpret_cast<const float4*>(colf + part * kScPart);
                     const float4* e4 = reinterpret_cast<const float4*>(colf + kScN + part * kScPart);
+                    const float4* u4 = reinterpret_cast<const float4*>(colf + 2 * kScN + part * kScPart);
                     float mn = __int_as_float(0x7f800000);
                     auto least = [&](const float (&v)[32], int b) {
 #pragma unroll
                         for (int q = 0; q < 8; ++q) {
-                            const float4 c = c4[8 * b + q];
+                            const float4 c = u4[8 * b + q];
                             mn = min_pair(fma_pair(v[4 * q], v[4 * q + 1], c.x, c.y), mn);
                             mn = min_pair(fma_pair(v[4 * q + 2], v[4 * q + 3], c.z, c.w), mn);
                         }
@@ -520,11 +509,10 @@ __global__ void __launch_bounds__(kScThreads, 1) ks_screen(const __grid_constant
                     epi_sync();
 #pragma unroll
                     for (int q = 0; q < 4; ++q) mn = fminf(mn, hmin[(buf * 4 + q) * kScM + rl]);
-                    // N_j - 2 g <= mn + c N_j + e_j^2 for the word that has it
-                    const float ne = __uint_as_float(cmax[0]), ee = __uint_as_float(cmax[1]);
+                    const float ee = __uint_as_float(cmax[0]);
                     float tau = __fadd_rn(ni, mn);
-                    if (!exact) {
-                        const float d = __fadd_ru(__fadd_ru(ni, mn), __fmaf_ru(c2, __fadd_ru(ni, __fmul_ru(2.f, ne)), __fmul_ru(ee, ee)));
+                    if (!exact) {  // mn: N_j (1 + c) - 2 g of some word, its own rounding covered by c's 2^-19
+                        const float d = __fadd_ru(mn, __fmul_ru(ni, __fadd_ru(1.f, c2)));
                         const float r = __fadd_ru(__fsqrt_ru(fmaxf(d, 0.f)), __fadd_ru(ei, ee));
                         tau = __fmul_ru(__fmul_ru(r, r), __fadd_ru(1.f, gamma));
                     }
@@ -720,17 +708,29 @@ __global__ void __launch_bounds__(256) ks_gather(const uint4* __restrict__ Xq, c
 // ---------------------------------------------------------------- nearest words
 // One warp per 32 rows: a row with one candidate word takes it; the others'
 // (row, word) pairs are spread over the lanes, which compute canonical
-// distances; ties go to the smaller word.
+// distances; ties go to the smaller word.  The rows and words of 32 pairs come
+// to shared memory kPickDims dims at a time, a row's pieces side by side, and
+// each lane walks its own pair there.  (A lane that walked its rows in global
+// memory took a sector of its own per 16 bytes: the index of 30,000 x 960 in 64
+// words, with 36 candidates a residue, 2.2 ms, staged 1.9; 1.4 with a word's own
+// norm in its upper bound instead of the largest, which leaves fewer.)
 constexpr int kPickPairs = 512;  // pairs a warp lists at once
-__global__ void __launch_bounds__(128) ks_pick(const uint32_t* __restrict__ mask, int64_t N, int W,
-                                              const float* __restrict__ X, int D, bool vec,
-                                              const float* __restrict__ W1, const int32_t* __restrict__ c1,
-                                              int c1_stride, const float* __restrict__ words,
-                                              int32_t* __restrict__ out, int out_stride) {
-    __shared__ uint16_t pairs[4][kPickPairs];
-    __shared__ unsigned long long best[4][32];
+constexpr int kPickWarps = 2, kPickDims = 32, kPickStride = kPickDims + 4;
+
+template <bool VEC, bool RES>
+__global__ void __launch_bounds__(32 * kPickWarps) ks_pick(const uint32_t* __restrict__ mask, int64_t N, int W,
+                                                          const float* __restrict__ X, int D,
+                                                          const float* __restrict__ W1,
+                                                          const int32_t* __restrict__ c1, int c1_stride,
+                                                          const float* __restrict__ words,
+                                                          int32_t* __restrict__ out, int out_stride) {
+    // staged rows: the vectors, the words and, for residues, the first words
+    __shared__ __align__(16) float stage[kPickWarps][RES ? 3 : 2][32 * kPickStride];
+    __shared__ uint16_t pairs[kPickWarps][kPickPairs];
+    __shared__ unsigned long long best[kPickWarps][32];
+    __shared__ int32_t code[kPickWarps][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t r0 = ((int64_t)blockIdx.x * 4 + w) * 32, row = r0 + lane;
+    const int64_t r0 = ((int64_t)blockIdx.x * kPickWarps + w) * 32, row = r0 + lane;
     if (r0 >= N) return;
     uint32_t m[8];
     int cnt = 0, first = 0;
@@ -742,6 +742,7 @@ __global__ void __launch_bounds__(128) ks_pick(const uint32_t* __restrict__ mask
         if (m[q]) first = 32 * q + __ffs(m[q]) - 1;
     }
     best[w][lane] = cnt > 1 ? kEmptyKey : (unsigned long long)first;
+    if (RES) code[w][lane] = cnt > 1 ? c1[row * c1_stride] : 0;
     __syncwarp();
     int left = cnt > 1 ? cnt : 0;  // pairs still to list
     int q = 0;
@@ -771,12 +772,60 @@ __global__ void __launch_bounds__(128) ks_pick(const uint32_t* __restrict__ mask
         }
         left -= take;
         __syncwarp();
-        for (int e = lane; e < total; e += 32) {
-            const int r = pairs[w][e] >> 8, c = pairs[w][e] & 255;
-            const int64_t i = r0 + r;
-            const float* w1 = W1 ? W1 + (int64_t)c1[i * c1_stride] * D : nullptr;
-            const float d = word_dist(X + i * D, w1, words + (int64_t)c * D, D, vec);
-            atomicMin(&best[w][r], (unsigned long long)make_key(d, (uint32_t)c));
+        for (int e = 0; e < total; e += 32) {
+            const int np = min(32, total - e);  // pairs of this turn, one per lane
+            const uint16_t* list = pairs[w] + e;
+            float acc = 0.f;
+            for (int d0 = 0; d0 < D; d0 += kPickDims) {
+                const int dl = min(kPickDims, D - d0);
+                // P pieces per row: a warp's lanes take 32 / P rows side by side
+                constexpr int P = VEC ? kPickDims / 4 : 32, S = VEC ? 4 : 1;
+                const int c = lane % P * S;
+                for (int p = lane / P; p < np; p += 32 / P) {
+                    if (c >= dl) continue;
+                    const int r = list[p] >> 8;
+                    const float* src[3] = {X + (r0 + r) * D, words + (int64_t)(list[p] & 255) * D,
+                                           RES ? W1 + (int64_t)code[w][r] * D : nullptr};
+#pragma unroll
+                    for (int u = 0; u < (RES ? 3 : 2); ++u) {
+                        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(stage[w][u] + p * kPickStride + c);
+                        if (VEC)
+                            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src[u] + d0 + c)
+                                         : "memory");
+                        else
+                            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src[u] + d0 + c)
+                                         : "memory");
+                    }
+                }
+                asm volatile("cp.async.wait_all;\n" ::: "memory");
+                __syncwarp();
+                if (lane < np) {  // the canonical chain: dims ascending
+                    const float* x = stage[w][0] + lane * kPickStride;
+                    const float* y = stage[w][1] + lane * kPickStride;
+                    const float* z = stage[w][RES ? 2 : 0] + lane * kPickStride;
+                    auto add = [&](float a, float b, float v) {
+                        const float t = __fsub_rn(RES ? __fsub_rn(a, v) : a, b);
+                        acc = __fmaf_rn(t, t, acc);
+                    };
+                    if (VEC) {
+#pragma unroll 4
+                        for (int d = 0; d < dl; d += 4) {
+                            const float4 a = *reinterpret_cast<const float4*>(x + d);
+                            const float4 b = *reinterpret_cast<const float4*>(y + d);
+                            const float4 v = RES ? *reinterpret_cast<const float4*>(z + d) : a;
+                            add(a.x, b.x, v.x);
+                            add(a.y, b.y, v.y);
+                            add(a.z, b.z, v.z);
+                            add(a.w, b.w, v.w);
+                        }
+                    } else {
+                        for (int d = 0; d < dl; ++d) add(x[d], y[d], z[d]);
+                    }
+                }
+                __syncwarp();  // the next stage overwrites
+            }
+            if (lane < np)
+                atomicMin(&best[w][list[lane] >> 8], (unsigned long long)make_key(acc, (uint32_t)(list[lane] & 255)));
         }
         __syncwarp();
     }
@@ -894,7 +943,7 @@ __global__ void __launch_bounds__(kRrThreads) k7_rank(ScreenArgs P, bool dump, i
     int Pk = 2;
     while (Pk < ns) Pk <<= 1;
     for (int e = threadIdx.x; e < Pk; e += kRrThreads)
-        keys[e] = e < ns ? make_key(word_dist(P.X + (int64_t)sid[e] * P.D, nullptr, q, P.D, P.vec), (uint32_t)sid[e])
+        keys[e] = e < ns ? make_key(point_dist(P.X + (int64_t)sid[e] * P.D, q, P.D, P.vec), (uint32_t)sid[e])
                          : kEmptyKey;
     __syncthreads();
     for (int kk = 2; kk <= Pk; kk <<= 1)
@@ -989,8 +1038,11 @@ bool launch_assign_screened(const float* X, int64_t N, int D, const float* W1, c
     const bool vec = D % 4 == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(words) |
                                      reinterpret_cast<uintptr_t>(W1)) & 15) == 0;
     LaunchScope ls("ks_pick", s, (double)N * 36.0, 0);
-    ks_pick<<<(unsigned)((N + 127) / 128), 128, 0, s>>>(w.mask, N, W, X, D, vec, W1, c1, c1_stride, words, out,
-                                                        out_stride);
+    const auto pick = W1 ? (vec ? ks_pick<true, true> : ks_pick<false, true>)
+                         : (vec ? ks_pick<true, false> : ks_pick<false, false>);
+    constexpr int kRows = 32 * kPickWarps;
+    pick<<<(unsigned)((N + kRows - 1) / kRows), kRows, 0, s>>>(w.mask, N, W, X, D, W1, c1, c1_stride, words, out,
+                                                              out_stride);
     return true;
 }
 
