@@ -394,6 +394,8 @@ struct AssignWork {
     uint32_t* mask;    // [N][8] candidate words
     int* flags;        // [2]
 };
+// assign_screened: whether N vectors against W words are worth it.
+bool assign_screened(int64_t N, int D, int W);
 void launch_screen_copy(const float* X, int64_t N, int D, const float* W1, const int32_t* c1, int c1_stride,
                         const AssignWork& w, int* status, cudaStream_t s);
 // launch_rvq_assign from the copies, the same codes; false when the tensor

@@ -1008,6 +1008,19 @@ bool launch_screen(const uint16_t* A, const uint16_t* B, int Dp, ScreenArgs& P, 
 }  // namespace
 
 // ---------------------------------------------------------------- nearest words
+// The FP32 kernel takes about 0.19 us a dim, tile of 128 words and wave of 9,728
+// vectors, the screen 25 us of short launches, plus rows of at least 64 dims to
+// copy and read.  Index of 10,000 vectors, two assignments, FP32 against the
+// screen (us): 64 words 16 dims 161 and 203, 64 dims 189 and 207, 128 dims 218 and
+// 225, 300 dims 324 and 302; 256 words 64 dims 231 and 213; 100,000 vectors, 16
+// dims: 64 words 222 and 248, 256 words 277 and 264.  With hardly more vectors than
+// words the vectors are the words, and most distances of the residues are ties
+// (300 x 300, 256 words: 418 and 1,800).
+bool assign_screened(int64_t N, int D, int W) {
+    const double tiles = (W + 127) / 128, waves = std::max(1.0, (double)N / 9728.0);
+    return N >= 4 * (int64_t)W && D * tiles * waves >= 140.0 * std::max(1.0, 32.0 / D);
+}
+
 void launch_screen_copy(const float* X, int64_t N, int D, const float* W1, const int32_t* c1, int c1_stride,
                         const AssignWork& w, int* status, cudaStream_t s) {
     cudaMemsetAsync(w.flags, 0, sizeof(int), s);
