@@ -1873,7 +1873,7 @@ int knng_rvq_seeds(const float* words1, int W1, const float* words2, int W2, int
         float *n1 = nullptr, *n2 = nullptr, *x12 = nullptr, *w1T = nullptr, *w2T = nullptr;
         SeedWork sw{};
         int* status = nullptr;
-        bool few = rvq_few_seeds(s);  // unless its products do not fit
+        bool few = rvq_few_seeds(W1, W2, D, m, probe1, s);  // unless its products do not fit
         for (int ps = 0; ps < 2; ++ps) {
             ws.used = 0;
             bind(ws, w1, words1, (size_t)W1 * D, ps);

@@ -342,7 +342,7 @@ struct SeedWork {
     float* dots;   // [rvq_seed_batch(m)][W1 + W2]
     float* qq;     // [rvq_seed_batch(m)]
 };
-bool rvq_few_seeds(int s_seeds);
+bool rvq_few_seeds(int W1, int W2, int D, int64_t m, int probe1, int s_seeds);
 int64_t rvq_seed_batch(int64_t m);
 void launch_rvq_few_seeds(const float* w1, int W1, const float* w2, int W2, int D, const int32_t* off,
                           const int32_t* ids, const float* Q, int64_t m, int probe1, int s_seeds,

@@ -1054,7 +1054,13 @@ void launch_rvq_tables(const float* w1, int W1, const float* w2, int W2, int D, 
     k9_tables<<<grid_for_count((int64_t)W1 * W2), 256, 0, s>>>(w1, W1, w2, W2, D, n1, n2, x12, w1T, w2T);
 }
 
-bool rvq_few_seeds(int s_seeds) { return s_seeds <= kSeedFew; }
+// Where few keys are ranked over short words, the general route's two launches
+// cost less than this one's four and two copies (us, 100 queries): 16 words of
+// one dim in both stages 89 and 102, 64 of 16 dims and one kept word 90 and 105,
+// 256 of 128 dims 169 and 115; 3,000 queries are even.
+bool rvq_few_seeds(int W1, int W2, int D, int64_t m, int probe1, int s_seeds) {
+    return s_seeds <= kSeedFew && (probe1 * W2 > 256 || (int64_t)(W1 + W2) * D > 8192 || m > 4096);
+}
 
 int64_t rvq_seed_batch(int64_t m) { return std::min<int64_t>(m, 65536); }
 
