@@ -1947,7 +1947,7 @@ int knng_exact(const float* data, int64_t n, int D, int k, const int32_t* sample
         // the screen's copy and candidate lists come on top of what the FP32
         // kernel needs; where they do not fit, the FP32 kernel runs alone, with
         // its columns split when the partial lists fit
-        bool screen = exact_screened(n), split = nsplit > 1;
+        bool screen = exact_screened(n, D, s_rows), split = nsplit > 1;
         for (int ps = 0; ps < 2; ++ps) {
             ws.used = 0;
             bind(ws, X, data, (size_t)n * D, ps);

@@ -368,8 +368,8 @@ void launch_exact(const float* X, int64_t n, int D, int k, const int32_t* sample
                   const int32_t* list, const int* list_count, int nsplit, uint64_t* part, uint64_t* out,
                   const int* status, cudaStream_t s);
 
-// Tensor-core screening (screen.cu).  exact_screened: whether exact lists
-// over n points are screened; exact_batch: rows screened at once; the lists equal
+// Tensor-core screening (screen.cu).  exact_screened: whether exact lists of
+// s_rows rows over n points of D dims are screened; exact_batch: rows screened at once; the lists equal
 // launch_exact's bit for bit.  Checks X for non-finite values on the way.
 struct ScreenWork {
     uint16_t *Xq, *Qq;      // BF16 copies of X and of a batch's rows
@@ -404,7 +404,7 @@ bool launch_assign_screened(const float* X, int64_t N, int D, const float* W1, c
                             const float* words, int W, const AssignWork& w, int32_t* out, int out_stride, int* status,
                             cudaStream_t s);
 constexpr int kScreenCap = 4096;
-bool exact_screened(int64_t n);
+bool exact_screened(int64_t n, int D, int64_t s_rows);
 int64_t exact_batch(int64_t s_rows);
 bool launch_exact_screened(const float* X, int64_t n, int D, int k, const int32_t* sample, int64_t s_rows,
                            const ScreenWork& w, uint64_t* out, int* status, cudaStream_t s);

@@ -1065,8 +1065,10 @@ bool launch_assign_screened(const float* X, int64_t N, int D, const float* W1, c
 // Measured (GB300): n = 500, D = 128, 15 rows 195 us against 95; n = 20,000,
 // D = 64, 7 rows 456 against 143; n = 1 M, D = 128, 1 row 5.7 ms against
 // 0.55, 2,000 rows 189 ms against 1.33 (0.94 of it the products).  Below one
-// column tile there is nothing to screen.
-bool exact_screened(int64_t n) { return n >= kScN; }
+// column tile there is nothing to screen; a few rows of few values take the
+// FP32 kernel less time than the launches (1 row of 256 x 32 93 us against 101,
+// of 300 x 2 85 against 104; 256 rows of 256 x 32 124 against 109).
+bool exact_screened(int64_t n, int D, int64_t s_rows) { return n >= kScN && (s_rows > 4 || n * D > 8192); }
 
 int64_t exact_batch(int64_t s_rows) { return std::min<int64_t>(s_rows, 8192); }
 

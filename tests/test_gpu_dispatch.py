@@ -51,6 +51,17 @@ def test_screened_rows(knng, kind, given_up):
     assert torch.equal(ids, ref_ids) and torch.equal(d, ref_d)
 
 
+@pytest.mark.parametrize("n,D,s,screened", [(255, 300, 200, False), (256, 32, 4, False), (256, 33, 4, True), (256, 32, 5, True),
+                                            (8192, 1, 1, False), (8193, 1, 1, True)])
+def test_small_exact_lists(knng, n, D, s, screened):
+    X = torch.from_numpy(datagen.gaussian_mixture(n, D, 10, seed=n)).cuda()
+    rows = torch.arange(s, dtype=torch.int32, device="cuda")
+    (ids, d), ran = _kernels(knng, lambda: knng.knng_exact(X, 7, rows))
+    assert ("ks_screen" in ran) == screened
+    ref_ids, ref_d = knng.knng_exact_noalloc(X, 7, rows)
+    assert torch.equal(ids, ref_ids) and torch.equal(d, ref_d)
+
+
 @pytest.mark.parametrize("leaf", [64, 128, 256])
 @pytest.mark.parametrize("data,exact", [("integer", ("bf16", "fp16")), ("wide", ("fp16",)), ("float", ())])
 def test_leaf_kernels(knng, data, exact, leaf):
