@@ -358,12 +358,14 @@ __device__ __forceinline__ float canon_dist(const float* __restrict__ xa, const 
     return acc;
 }
 
-// s / b rounded to nearest (FP64) from inv = RN(1 / b): the FMA residual
-// r = s - q0 b of q0 = RN(s inv) is exact, and q0 + r inv rounds to RN(s / b)
-// (Markstein's correction).  For integer s and b < 2^52 the quotient is never
-// within the correction's error of a rounding boundary, so the result equals
-// FP64 division bit for bit; it costs three FP64 operations, where GB300
-// issues FP64 at a small fraction of its FP32 rate.
+// s / b rounded to nearest (FP64) from inv = RN(1 / b), for any FP64 s and an
+// integer 1 <= b < 2^31, short of underflow.  q0 = RN(s inv) is within 1.5 ulp of
+// s / b, so the residual r = s - q0 b is a multiple of ulp(q0) below 2^33 of
+// them: the FMA gives it exactly.  r inv is then within 2^-52 ulp of the exact
+// correction (Markstein's), while s / b lies at least ulp / (2 b) from any
+// rounding boundary (a boundary has 54 bits, and no multiple of it by b fits
+// 53): the result is the FP64 division's, bit for bit.  It costs three FP64
+// operations, where GB300 issues FP64 at a small fraction of its FP32 rate.
 __device__ __forceinline__ double div_by(double s, double b, double inv) {
     const double q0 = __dmul_rn(s, inv);
     const double r = __fma_rn(-q0, b, s);

@@ -15,7 +15,10 @@
 // fmaf), the cut is by the (projection, position) key, and the sums are
 // compensated FP32 (TwoSum) per warp, FP64 across warps, CTAs and iterations
 // (integers: exact int64): split.cu's definitions, with the rows of a sum in
-// another fixed order.
+// another fixed order.  A warp adds up to a sixteenth of the CTA's rows before
+// FP64 (68 of 32 dims, about 150 of 8; the sweeps 32): r rows leave the low part
+// within r^2 2^-48 of their magnitudes' sum, 8e-11 at 150, against the 6e-8 of
+// the mean's own rounding to FP32.
 //
 // Its own bound is latency: 3 synchronisations and about four short dependent
 // phases per iteration, 8-15 us an iteration.
