@@ -682,6 +682,7 @@ __global__ void __launch_bounds__(256) k9_dots(const float* __restrict__ A, int6
                 *reinterpret_cast<float4*>(dst + r * kDotStride + c) = v;
             }
         } else {
+#pragma unroll 16  // that many loads in flight
             for (int e = tid; e < rows * kDotDims; e += 256) {
                 const int r = e / kDotDims, c = e % kDotDims;
                 dst[r * kDotStride + c] = first + r < count && d0 + c < D ? __ldg(src + (first + r) * D + d0 + c) : 0.f;
@@ -726,6 +727,13 @@ __global__ void __launch_bounds__(256) k9_dots(const float* __restrict__ A, int6
             if (r < M && c < W) out[r * W + c] = acc[i][j];
         }
     if (blockIdx.y == 0 && tid < kDotRows && r0 + tid < M) self[r0 + tid] = own;
+}
+
+// The na values of a, then the nb of b (one launch less than two copies).
+__global__ void __launch_bounds__(256) k9_stack(const float* __restrict__ a, int64_t na, const float* __restrict__ b,
+                                               int64_t nb, float* __restrict__ out) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < na + nb; e += (int64_t)gridDim.x * blockDim.x)
+        out[e] = e < na ? __ldg(a + e) : __ldg(b + e - na);
 }
 
 // part[a * W2 + b] = fmaf(2, w1_a . w2_b, |w2_b|^2), or kNoList when the key's
@@ -1055,7 +1063,7 @@ void launch_rvq_tables(const float* w1, int W1, const float* w2, int W2, int D, 
 }
 
 // Where few keys are ranked over short words, the general route's two launches
-// cost less than this one's four and two copies (us, 100 queries): 16 words of
+// cost less than this one's five (us, 100 queries): 16 words of
 // one dim in both stages 89 and 102, 64 of 16 dims and one kept word 90 and 105,
 // 256 of 128 dims 169 and 115; 3,000 queries are even.
 bool rvq_few_seeds(int W1, int W2, int D, int64_t m, int probe1, int s_seeds) {
@@ -1083,8 +1091,10 @@ void launch_rvq_few_seeds(const float* w1, int W1, const float* w2, int W2, int 
                           const int32_t* ids, const float* Q, int64_t m, int probe1, int s_seeds,
                           const SeedWork& w, int32_t* S, const int* status, cudaStream_t s) {
     const int W = W1 + W2;
-    cudaMemcpyAsync(w.words, w1, sizeof(float) * W1 * D, cudaMemcpyDeviceToDevice, s);
-    cudaMemcpyAsync(w.words + (size_t)W1 * D, w2, sizeof(float) * W2 * D, cudaMemcpyDeviceToDevice, s);
+    {
+        LaunchScope ls("k9_stack", s, (double)W * D * 8.0, 0);
+        k9_stack<<<grid_for_count((int64_t)W * D), 256, 0, s>>>(w1, (int64_t)W1 * D, w2, (int64_t)W2 * D, w.words);
+    }
     launch_dots(w.words, W, w.words, W, D, w.table, w.self, s);
     {
         LaunchScope ls("k9_keys", s, (double)W1 * W2 * 16.0, 0);
